@@ -92,15 +92,69 @@ __device__ __forceinline__ double drcp_newton(double y) {
     return fma(r, e, r);
 }
 
+// 1 / sqrt(x) of a positive finite double: the hardware's approximation y0
+// (PTX rsqrt.approx.ftz.f64) and one third-order step, y = y0 + y0 e (1/2 +
+// 3 e / 8) with e = 1 - x y0^2 (the series of (1 - e)^(-1/2); the next term,
+// 5 e^3 / 16, is below 2^-60).  5 FP64 instructions.  The callers take
+// square roots as x / sqrt(x) and reciprocals as (1 / sqrt(x))^2 from the
+// same value: CUDA's sqrt and a Newton reciprocal of the same x take 13.
+__device__ __forceinline__ double drsqrt_newton(double x) {
+    double y;
+    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+    const double e = fma(-(x * y), y, 1.0);
+    return fma(fma(0.375, e, 0.5), y * e, y);
+}
+
+// a / b, b > 0 finite and normal: the approximate quotient q0 = a r0 (r0
+// PTX rcp.approx.ftz.f64, e = 1 - b r0) times 1 + e + e^2 (next term below
+// 2^-57): 4 FP64 instructions, one fewer than a drcp_newton(b).
+__device__ __forceinline__ double ddiv_newton(double a, double b) {
+    double r;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(b));
+    const double e = fma(-b, r, 1.0);
+    const double q = a * r;
+    return fma(fma(e, e, e), q, q);
+}
+
+// 2^n x by an addition to the exponent field (binary64: bits 52-62) on the
+// integer pipes, |n| <= 2; exact for 2^-1020 <= |x| < 2^1020, x itself
+// otherwise (zero, infinities and NaN keep their value; magnitudes outside
+// that range do not occur in a physical state).
+template <int N>
+__device__ __forceinline__ double dscale2(double x) {
+    const int hi = __double2hiint(x);
+    const unsigned e = (unsigned)hi & 0x7ff00000u;
+    const bool in = e - 0x00300000u < 0x7fa00000u;
+    return __hiloint2double(in ? hi + N * 0x00100000 : hi, __double2loint(x));
+}
+
+// the larger of two non-negative doubles: they order like their bit
+// patterns, and an integer comparison leaves the FP64 pipe free (a NaN is
+// the larger one and is kept)
+__device__ __forceinline__ double dmax_nonneg(double a, double b) {
+    return __double_as_longlong(a) > __double_as_longlong(b) ? a : b;
+}
+
 template <> struct M<double> {
     static __device__ __forceinline__ double sqrt_(double x) { return sqrt(x); }
-    static __device__ __forceinline__ double div_(double a, double b) { return a * drcp_newton(b); }
+    static __device__ __forceinline__ double div_(double a, double b) { return ddiv_newton(a, b); }
     static __device__ __forceinline__ double rcp_(double x) { return drcp_newton(x); }
-    static __device__ __forceinline__ double rsqrt_(double x) { return rsqrt(x); }
+    static __device__ __forceinline__ double rsqrt_(double x) { return drsqrt_newton(x); }
     static __device__ __forceinline__ double abs_(double x) { return fabs(x); }
     static __device__ __forceinline__ double max_(double a, double b) { return fmax(a, b); }
+    static __device__ __forceinline__ double max_nonneg(double a, double b) { return dmax_nonneg(a, b); }
     static __device__ __forceinline__ double min_(double a, double b) { return fmin(a, b); }
-    static __device__ __forceinline__ bool finite_pos(double x) { return x > 0.0 && x < 1.0e308; }
+    static __device__ __forceinline__ double fma_(double a, double b, double c) { return fma(a, b, c); }
+    static __device__ __forceinline__ double half_(double x) { return dscale2<-1>(x); }
+    // comparisons on the bit patterns (order preserving for a positive right
+    // side; a comparison of doubles would issue on the FP64 pipe)
+    static __device__ __forceinline__ bool ge_pos(double x, double c) { return __double_as_longlong(x) >= __double_as_longlong(c); }
+    static __device__ __forceinline__ bool gt_pos(double x, double c) { return __double_as_longlong(x) > __double_as_longlong(c); }
+    static __device__ __forceinline__ bool nonneg(double x) { return __double2hiint(x) >= 0; }
+    static __device__ __forceinline__ bool normal_pos(double x) { return __double2hiint(x) >= 0x00200000; }
+    static __device__ __forceinline__ bool finite_pos(double x) {   // 0 < x < 1e308; false for NaN
+        return __double_as_longlong(x) > 0 && __double_as_longlong(x) < __double_as_longlong(1.0e308);
+    }
 };
 template <> struct M<float> {
     static __device__ __forceinline__ float sqrt_(float x) { return sqrtf(x); }
@@ -109,36 +163,39 @@ template <> struct M<float> {
     static __device__ __forceinline__ float rsqrt_(float x) { return rsqrtf(x); }
     static __device__ __forceinline__ float abs_(float x) { return fabsf(x); }
     static __device__ __forceinline__ float max_(float a, float b) { return fmaxf(a, b); }
+    static __device__ __forceinline__ float max_nonneg(float a, float b) { return fmaxf(a, b); }
     static __device__ __forceinline__ float min_(float a, float b) { return fminf(a, b); }
+    static __device__ __forceinline__ float fma_(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+    static __device__ __forceinline__ float half_(float x) { return 0.5f * x; }
+    static __device__ __forceinline__ bool ge_pos(float x, float c) { return x >= c; }
+    static __device__ __forceinline__ bool gt_pos(float x, float c) { return x > c; }
+    static __device__ __forceinline__ bool nonneg(float x) { return x >= 0.0f; }
+    static __device__ __forceinline__ bool normal_pos(float x) { return !(x < 1.17549435e-38f); }
     static __device__ __forceinline__ bool finite_pos(float x) { return x > 0.0f && x < 3.0e38f; }
 };
 
 // ---------------------------------------------------------------- wave speeds
 // c_f^2 - c_s^2 (fmc), c_s^2 - c_slow^2 (cms) without cancellation, and c_f^2.
 // The larger of the two differences is (sd + |aa|) / 2 (aa = c_A^2 + b_t^2 -
-// c_s^2), the other c_s^2 b_t^2 over it.  In float the two cases are formed
-// without branches (0.5% faster sweep), in double with them (0.5% faster
-// there); the results are the same bits.
+// c_s^2), the other c_s^2 b_t^2 over it; the discriminant is the same one as
+// (c_s^2 - c_A^2)^2 + b_t^2 (b_t^2 + 2 c_A^2 + 2 c_s^2), written as
+// aa^2 + 4 c_s^2 b_t^2: still a sum of non-negative terms, so nothing cancels.
 template <typename Real>
 __device__ __forceinline__ void speeds_fast(Real cs2, Real ca2, Real bt2, Real &fmc, Real &cms, Real &cf2) {
     using m = M<Real>;
-    const Real dd = (cs2 - ca2) * (cs2 - ca2) + bt2 * (bt2 + Real(2) * ca2 + Real(2) * cs2);
-    const Real sd = m::sqrt_(dd);
+    const Real q = cs2 * bt2;
     const Real aa = ca2 + bt2 - cs2;
-    if constexpr (float_based<Real>) {
-        const Real big = Real(0.5) * (sd + m::abs_(aa));
-        const Real oth = big > Real(0) ? m::div_(cs2 * bt2, big) : Real(0);
-        const bool fast_big = aa >= Real(0);
-        fmc = fast_big ? big : oth;
-        cms = fast_big ? oth : big;
+    const Real dd = m::fma_(aa, aa, Real(4) * q);
+    const Real sd = m::normal_pos(dd) ? dd * m::rsqrt_(dd) : Real(0);
+    const Real big = m::half_(sd + m::abs_(aa));
+    // a branch, not a select: the callers that use only fmc skip the division
+    // where it is the larger one
+    if (m::nonneg(aa)) {
+        fmc = big;
+        cms = m::normal_pos(big) ? m::div_(q, big) : Real(0);
     } else {
-        if (aa >= Real(0)) {
-            fmc = Real(0.5) * (aa + sd);
-            cms = fmc > Real(0) ? m::div_(cs2 * bt2, fmc) : Real(0);
-        } else {
-            cms = Real(0.5) * (sd - aa);
-            fmc = cms > Real(0) ? m::div_(cs2 * bt2, cms) : Real(0);
-        }
+        cms = big;
+        fmc = m::normal_pos(big) ? m::div_(q, big) : Real(0);
     }
     cf2 = cs2 + fmc;
 }
@@ -161,11 +218,12 @@ __device__ __forceinline__ void cell_fill_frame(Real *sm, int stride, Real rho, 
     using m = M<Real>;
     Real r = rho;
     if (K.floors && r < K.rho_min) { r = K.rho_min; hit = true; }
-    const Real ir = m::rcp_(r);
+    const Real isr = m::rsqrt_(r), ir = isr * isr;
     const Real vn = mn * ir, v1 = m1 * ir, v2 = m2 * ir;
     const Real vv = vn * vn + v1 * v1 + v2 * v2;
-    const Real BB = Bn * Bn + B1 * B1 + B2 * B2;
-    Real P = K.gm1 * (E - Real(0.5) * r * vv - Real(0.5) * BB);
+    const Real Bn2 = Bn * Bn, Bt2 = B1 * B1 + B2 * B2;
+    const Real BB = Bn2 + Bt2;
+    Real P = K.gm1 * (E - Real(0.5) * (r * vv + BB));
     if (K.floors && P < K.p_min) { P = K.p_min; hit = true; }
     if (!(r > Real(0)) || !m::finite_pos(P)) bad = true;
     const Real Pt = P + Real(0.5) * BB;
@@ -185,20 +243,21 @@ __device__ __forceinline__ void cell_fill_frame(Real *sm, int stride, Real rho, 
     sm[C_E * stride] = E;
     // rho v_n = m_n (v = m / rho with the same, possibly floored, rho)
     sm[C_F0 * stride] = mn;
-    sm[C_F1 * stride] = mn * vn + Pt - Bn * Bn;
+    sm[C_F1 * stride] = mn * vn + (Pt - Bn2);
     sm[C_F2 * stride] = mn * v1 - Bn * B1;
     sm[C_F3 * stride] = mn * v2 - Bn * B2;
     sm[C_F4 * stride] = B1 * vn - Bn * v1;
     sm[C_F5 * stride] = B2 * vn - Bn * v2;
     sm[C_F6 * stride] = (E + Pt) * vn - Bn * vB;
+    // c_f, c_A and c_slow = c_s c_A / c_f, from reciprocal square roots
     const Real cs2 = K.gamma * P * ir;
-    const Real ca2 = Bn * Bn * ir;
-    const Real bt2 = (B1 * B1 + B2 * B2) * ir;
-    Real fmc, cms, cf2, csl2;
-    speeds<Real>(cs2, ca2, bt2, fmc, cms, cf2, csl2);
-    sm[C_CF * stride] = m::sqrt_(cf2);
-    sm[C_CA * stride] = m::abs_(Bn) * m::rsqrt_(r);     // |B_n| / sqrt(rho)
-    sm[C_CSL * stride] = m::sqrt_(csl2);
+    Real fmc, cms, cf2;
+    speeds_fast<Real>(cs2, Bn2 * ir, Bt2 * ir, fmc, cms, cf2);
+    const Real icf = m::rsqrt_(cf2);
+    const Real ca = m::abs_(Bn) * isr;
+    sm[C_CF * stride] = cf2 * icf;
+    sm[C_CA * stride] = ca;
+    sm[C_CSL * stride] = cs2 * m::rsqrt_(cs2) * (ca * icf);
 }
 
 // cell_fill_frame for a sweep along axis AX (frame (n, t1, t2) = (AX, AX+1,
@@ -276,48 +335,53 @@ __device__ __forceinline__ Real signal_speed(Real r, Real vn, Real P, Real Bn, R
 // Two rewrites that leave phi_N unchanged up to rounding:
 // * the weights depend only on the ratios of eps + IS_k (JS: alpha_k =
 //   d_k / (eps + IS_k)^2 normalised; WENO-Z: tau_5 / (eps + IS_k)), so the
-//   smoothness indicators are evaluated as IS_k / 3 = (13/3) x^2 + y^2 with
-//   eps / 3 (the caller passes it);
+//   smoothness indicators are evaluated as IS_k / 12 with eps / 12 (the
+//   caller passes it);
 // * with w_k = a_k / D (D = a_0 + a_1 + a_2) and the second differences
 //   t1 = a - 2b + c = x0 - y0, t2 = b - 2c + d = y0 - z0 of the first ones
 //   (x0 = a - b, y0 = b - c, z0 = c - d, also those of the indicators),
 //   phi_N = w_0 t1 / 3 + (w_2 - 1/2) t2 / 6
-//         = [a_0 t1 + (a_2 / 2 - D / 4) t2] / (3 D);
+//         = [4 a_0 t1 + (2 a_2 - D) t2] / (12 D);
 //   in double each interpolant returns that numerator and D, and weno_field
 //   divides once for the two; in float the weights are normalised first
 //   (D = 1) and phi_N = Nn / 3.
 //
-// smoothness3 returns s_k = eps/3 + IS_k/3, the epsilon added inside the
-// last FMA of each indicator, and the first differences x0, y0, z0.
+// smoothness3 returns s_k = (eps + IS_k) / 12 and the first differences x0,
+// y0, z0.  With a = b + x0, b = c + y0, d = c - z0 the three indicators are
+// quadratics in one difference and b or c,
+//   IS_0 / 12 = x0 (4 x0 / 3 - b) + b^2,  IS_1 / 12 = y0 (4 y0 / 3 - b) + b^2,
+//   IS_2 / 12 = z0 (4 z0 / 3 + c) + c^2,
+// positive definite (the minimum over the difference is 13/16 of the square),
+// so nothing cancels: 11 operations with the differences, where 13 x^2 / 3 +
+// y^2 each takes 15.  eps12 = eps / 12 of the caller's epsilon.
 template <typename Real>
-__device__ __forceinline__ void smoothness3(Real a, Real b, Real c, Real d, Real eps3, Real &s0, Real &s1, Real &s2,
+__device__ __forceinline__ void smoothness3(Real a, Real b, Real c, Real d, Real eps12, Real &s0, Real &s1, Real &s2,
                                             Real &x0, Real &y0, Real &z0) {
-    const Real k = Real(13.0 / 3.0);
+    using m = M<Real>;
+    const Real k = Real(4.0 / 3.0);
     x0 = a - b;
-    const Real x1 = a - Real(3) * b;
-    s0 = (k * x0) * x0 + (x1 * x1 + eps3);
     y0 = b - c;
-    const Real y1 = b + c;
-    s1 = (k * y0) * y0 + (y1 * y1 + eps3);
     z0 = c - d;
-    const Real z1 = Real(3) * c - d;
-    s2 = (k * z0) * z0 + (z1 * z1 + eps3);
+    const Real bb = m::fma_(b, b, eps12), cc = m::fma_(c, c, eps12);
+    s0 = m::fma_(x0, m::fma_(k, x0, -b), bb);
+    s1 = m::fma_(y0, m::fma_(k, y0, -b), bb);
+    s2 = m::fma_(z0, m::fma_(k, z0, c), cc);
 }
 
 // float: phi_N = Nn / 3 with the weights normalised here by one reciprocal
 // (the WENO-Z ratio tau_5 / (eps + IS_k) is clamped at 1e18, so nothing
 // overflows; unnormalised WENO-Z weights reach 1e36 in float)
 template <int VAR>
-__device__ __forceinline__ float phi_nf(float a, float b, float c, float d, float eps3) {
+__device__ __forceinline__ float phi_nf(float a, float b, float c, float d, float eps12) {
     float s0, s1, s2, x0, y0, z0;
-    smoothness3<float>(a, b, c, d, eps3, s0, s1, s2, x0, y0, z0);
+    smoothness3<float>(a, b, c, d, eps12, s0, s1, s2, x0, y0, z0);
     float e0, e1, e2;   // alpha_k / d_k
     if constexpr (VAR == 0) {
         e0 = __fdividef(1.0f, s0 * s0);
         e1 = __fdividef(1.0f, s1 * s1);
         e2 = __fdividef(1.0f, s2 * s2);
     } else {
-        const float tau = fabsf(s0 - s2);   // |IS_0 - IS_2| / 3
+        const float tau = fabsf(s0 - s2);   // |IS_0 - IS_2| / 12
         const float r0 = fminf(tau * __fdividef(1.0f, s0), 1.0e18f);
         const float r1 = fminf(tau * __fdividef(1.0f, s1), 1.0e18f);
         const float r2 = fminf(tau * __fdividef(1.0f, s2), 1.0e18f);
@@ -331,36 +395,44 @@ __device__ __forceinline__ float phi_nf(float a, float b, float c, float d, floa
 }
 
 // double: the weights times the common factor (s_0 s_1 s_2)^2, so that no
-// weight needs a division; phi_N = Nn / (3 D), and the two interpolants of
-// one field share a single division in weno_field.  The linear weights
-// d = (1, 6, 3) enter the sum and the numerator by FMAs.
+// weight needs a division; phi_N = N / (12 D), and the two interpolants of
+// one field share a single division in weno_field.  29 FP64 instructions
+// (WENO-Z).
 template <int VAR>
-__device__ __forceinline__ void phi_nd(double a, double b, double c, double d, double eps3, double &Nn, double &Dn) {
+__device__ __forceinline__ void phi_nd(double a, double b, double c, double d, double eps12, double &N, double &D) {
     double s0, s1, s2, x0, y0, z0;
-    smoothness3<double>(a, b, c, d, eps3, s0, s1, s2, x0, y0, z0);
+    smoothness3<double>(a, b, c, d, eps12, s0, s1, s2, x0, y0, z0);
+    const double p0 = s1 * s2;
     double W0, V1, V2;   // alpha_k / d_k times the common factor
     if constexpr (VAR == 0) {
-        // alpha_k = d_k / s_k^2 times (s0 s1 s2)^2
-        const double p0 = s1 * s2, p1 = s0 * s2, p2 = s0 * s1;
+        // alpha_k / d_k = 1 / s_k^2
+        const double p1 = s0 * s2, p2 = s0 * s1;
         W0 = p0 * p0;
         V1 = p1 * p1;
         V2 = p2 * p2;
     } else {
-        // alpha_k = d_k (1 + tau^2 / s_k^2) times (s0 s1 s2)^2: with e_k =
-        // s_k^2 and E = e0 e1 e2, (e_k + tau^2) prod_{j != k} e_j = E + tau^2
-        // prod_{j != k} e_j, one FMA per weight
-        const double tau = fabs(s0 - s2);   // |IS_0 - IS_2| / 3
-        const double tt = tau * tau;
-        const double e0 = s0 * s0, e1 = s1 * s1, e2 = s2 * s2;
-        const double e12 = e1 * e2, e02 = e0 * e2, e01 = e0 * e1;
-        const double E = e0 * e12;
-        W0 = fma(tt, e12, E);
-        V1 = fma(tt, e02, E);
-        V2 = fma(tt, e01, E);
+        // alpha_k / d_k = 1 + tau^2 / s_k^2: (s0 s1 s2)^2 + (tau prod_{j != k} s_j)^2,
+        // tau = (IS_0 - IS_2) / 12 (its sign drops out)
+        const double tau = s0 - s2;
+        const double q = s0 * p0, t0 = tau * s0;
+        const double A = tau * p0, B = t0 * s2, C = t0 * s1;
+        const double Q = q * q;
+        W0 = fma(A, A, Q);
+        V1 = fma(B, B, Q);
+        V2 = fma(C, C, Q);
     }
-    Dn = fma(3.0, V2, fma(6.0, V1, W0));
-    // a_0 t1 + (a_2 / 2 - D / 4) t2 with a_2 = 3 V2
-    Nn = W0 * (x0 - y0) + fma(1.5, V2, -0.25 * Dn) * (y0 - z0);
+    // D = W0 + 6 V1 + 3 V2, N = 4 W0 t1 + (6 V2 - D) t2
+    const double Y = fma(6.0, V1, W0);
+    D = fma(3.0, V2, Y);
+    N = fma(W0, dscale2<2>(x0 - y0), fma(3.0, V2, -Y) * (y0 - z0));
+}
+
+// N_m / D_m - N_p / D_p where the product of the denominators leaves the
+// range of one shared reciprocal (flat data: D ~ eps^6; huge data).  Not
+// inlined: rare, and its IEEE divisions would be issued, predicated off, on
+// the FP64 pipe of every field.
+static __device__ __noinline__ double weno_quotients(double Np, double Dp, double Nm, double Dm) {
+    return Nm / Dm - Np / Dp;
 }
 
 // ---------------------------------------------------------------- double-word
@@ -515,202 +587,126 @@ __device__ __forceinline__ dw phi_dw(dw a, dw b, dw c, dw d, dw eps3) {
     return dw_add(dw_mul(w0, dw_sub(x0, y0)), dw_mul(w2, dw_sub(y0, z0)));
 }
 
-// Eq. (FWENO) for one characteristic field from its 11 projections:
-// P[0] = L.central, P[1..5] = L.dF at i-3/2 .. i+5/2, P[6..10] = L.du there.
+// ---------------------------------------------------------------- pairs
+// The stencil's flux difference and state difference at one position, (dF_j,
+// du_j), share every projection coefficient, so they are carried as a pair.
+// In float one packed two-lane FMA (sm_100 f32x2) acts on both; each lane
+// rounds exactly as the scalar FMA would.
+template <typename Real> struct Pair;
+template <> struct Pair<float> { float2 v; };
+template <> struct Pair<double> { double x, y; };
+
+__device__ __forceinline__ Pair<float> make_pair2(float x, float y) { return {make_float2(x, y)}; }
+__device__ __forceinline__ Pair<double> make_pair2(double x, double y) { return {x, y}; }
+__device__ __forceinline__ Pair<float> pmul(float s, Pair<float> a) { return {__fmul2_rn(make_float2(s, s), a.v)}; }
+__device__ __forceinline__ Pair<double> pmul(double s, Pair<double> a) { return {s * a.x, s * a.y}; }
+__device__ __forceinline__ Pair<float> pfma(float s, Pair<float> a, Pair<float> c) {
+    return {__ffma2_rn(make_float2(s, s), a.v, c.v)};
+}
+__device__ __forceinline__ Pair<double> pfma(double s, Pair<double> a, Pair<double> c) {
+    return {fma(s, a.x, c.x), fma(s, a.y, c.y)};
+}
+// dF + alpha du and dF - alpha du
+__device__ __forceinline__ float psplit(Pair<float> a, float al) { return __fmaf_rn(al, a.v.y, a.v.x); }
+__device__ __forceinline__ double psplit(Pair<double> a, double al) { return fma(al, a.y, a.x); }
+
+// The two members u = c + s, l = c - s of a mode pair, c the sign-free part
+// of the projection and s = c1 a + c2 b.  In double u is one chain on c and
+// l = 2 c - u (one instruction fewer than s, c + s, c - s); in float l is a
+// chain of its own (a packed negation of u would cost what it saves).
+__device__ __forceinline__ void mode_pair(Pair<double> c, double c1, Pair<double> a, double c2, Pair<double> b,
+                                          Pair<double> &u, Pair<double> &l) {
+    u = pfma(c1, a, pfma(c2, b, c));
+    l = {fma(2.0, c.x, -u.x), fma(2.0, c.y, -u.y)};
+}
+__device__ __forceinline__ void mode_pair(Pair<float> c, float c1, Pair<float> a, float c2, Pair<float> b,
+                                          Pair<float> &u, Pair<float> &l) {
+    u = pfma(c1, a, pfma(c2, b, c));
+    l = pfma(-c1, a, pfma(-c2, b, c));
+}
+
+// The WENO part of Eq. (FWENO) for one characteristic field: its flux is
+// L.central + kWenoScale weno_field(...), from the five pairs L.(dF_j, du_j) at
+// i-3/2 .. i+5/2.
 //
 // The split differences are (dF +- alpha dq)/2.  IS_k scales with the square
 // of its arguments and phi_N linearly, so phi_N(x/2; eps) = phi_N(x; 4 eps)/2
 // for both weight variants: the factor 1/2 is applied once to the result.
-// With the IS_k / 3 form above the epsilon passed in is eps43 = 4 eps / 3,
-// and F = P[0] + (phi_N^- - phi_N^+)/2 = P[0] + (Nm/Dm - Np/Dp)/6.
+// With the IS_k / 12 form above the epsilon passed in is eps3 = 4 eps / 12.
+// float: -N_p + N_m with phi_N = N / 3, times 1/6; double: phi_N = N / (12 D),
+// times 1/24.
 //
 // DWW (double only): the split differences, formed in double, go to
 // double-word, phi_dw evaluates both interpolants there, and their
-// difference returns to double for the last FMAs with P[0].
+// difference returns to double.
+template <typename Real>
+constexpr Real kWenoScale = std::is_same<Real, double>::value ? Real(1.0 / 24.0) : Real(1.0 / 6.0);
+
 template <typename Real, int VAR, bool DWW = false>
-__device__ __forceinline__ Real weno_field(const Real P[11], Real alpha, Real eps43) {
-    Real p[5], q[5];
+__device__ __forceinline__ Real weno_field(const Pair<Real> (&P)[5], Real alpha, Real eps3) {
+    Real p[4], q[4];
 #pragma unroll
-    for (int j = 0; j < 5; ++j) {
-        p[j] = P[1 + j] + alpha * P[6 + j];
-        q[j] = P[1 + j] - alpha * P[6 + j];
+    for (int j = 0; j < 4; ++j) {
+        p[j] = psplit(P[j], alpha);
+        q[j] = psplit(P[j + 1], -alpha);
     }
     if constexpr (std::is_same<Real, double>::value && DWW) {
-        dw pd[5], qd[5];
+        dw pd[4], qd[4];
 #pragma unroll
-        for (int j = 0; j < 5; ++j) {
+        for (int j = 0; j < 4; ++j) {
             pd[j] = dw_from_double(p[j]);
             qd[j] = dw_from_double(q[j]);
         }
-        const dw e3 = dw_from_double(eps43);
+        const dw e3 = dw_from_double(4.0 * eps3);
         const dw Np = phi_dw<VAR>(pd[0], pd[1], pd[2], pd[3], e3);
-        const dw Nm = phi_dw<VAR>(qd[4], qd[3], qd[2], qd[1], e3);
+        const dw Nm = phi_dw<VAR>(qd[3], qd[2], qd[1], qd[0], e3);
         const dw r = dw_sub(Nm, Np);
-        return fma(1.0 / 6.0, dw_f2d(r.hi), fma(1.0 / 6.0, dw_f2d(r.lo), P[0]));
+        return dw_f2d(4.0f * r.hi) + dw_f2d(4.0f * r.lo);
     }
     if constexpr (std::is_same<Real, double>::value) {
         double Np, Dp, Nm, Dm;
-        phi_nd<VAR>(p[0], p[1], p[2], p[3], eps43, Np, Dp);
-        phi_nd<VAR>(q[4], q[3], q[2], q[1], eps43, Nm, Dm);
+        phi_nd<VAR>(p[0], p[1], p[2], p[3], eps3, Np, Dp);
+        phi_nd<VAR>(q[3], q[2], q[1], q[0], eps3, Nm, Dm);
         const double prod = Dp * Dm;
-        if (prod > 1e-290 && prod < 1e290) {
-            // -Np/Dp + Nm/Dm over the common denominator: one reciprocal
-            return P[0] + (1.0 / 6.0) * ((Nm * Dp - Np * Dm) * drcp_newton(prod));
-        }
-        return P[0] + (1.0 / 6.0) * (Nm / Dm - Np / Dp);
+        // 2^-962 <= prod < 2^962 by its exponent field (positive, or NaN: outside)
+        if ((unsigned)__double2hiint(prod) - 0x03d00000u < 0x78400000u)
+            // -Np/Dp + Nm/Dm over the common denominator: one division
+            return ddiv_newton(fma(Nm, Dp, -(Np * Dm)), prod);
+        return weno_quotients(Np, Dp, Nm, Dm);
     } else {
         static_assert(std::is_same<Real, float>::value, "weno_field takes float or double");
-        const float Np = phi_nf<VAR>(p[0], p[1], p[2], p[3], eps43);
-        const float Nm = phi_nf<VAR>(q[4], q[3], q[2], q[1], eps43);
-        return __fmaf_rn(1.0f / 6.0f, Nm - Np, P[0]);
+        const float Np = phi_nf<VAR>(p[0], p[1], p[2], p[3], eps3);
+        const float Nm = phi_nf<VAR>(q[3], q[2], q[1], q[0], eps3);
+        return Nm - Np;
     }
-}
-
-// ---------------------------------------------------------------- float
-// In float the 11 stencil vectors are kept as the central one, X0, and the
-// five pairs X2[j] = (dF_j, du_j) (vectors 1 + j and 6 + j), which share
-// every projection coefficient: one packed two-lane FMA (sm_100 f32x2)
-// projects both.  Each lane rounds exactly as the scalar FMA would.
-__device__ __forceinline__ float2 bcast2(float a) { return make_float2(a, a); }
-__device__ __forceinline__ float2 neg2(float2 a) { return make_float2(-a.x, -a.y); }
-
-// P = sum_k L[k] X[ci[k]] for the 11 vectors (scalar central, packed pairs)
-template <int N>
-__device__ __forceinline__ void project_f(const float (&X0)[7], const float2 (&X2)[5][7], const int (&ci)[N],
-                                          const float (&L)[N], float &P0, float2 (&P2)[5]) {
-    float p = L[0] * X0[ci[0]];
-#pragma unroll
-    for (int k = 1; k < N; ++k) p = __fmaf_rn(L[k], X0[ci[k]], p);
-    P0 = p;
-    float2 Lb[N];
-#pragma unroll
-    for (int k = 0; k < N; ++k) Lb[k] = bcast2(L[k]);
-#pragma unroll
-    for (int j = 0; j < 5; ++j) {
-        float2 q = __fmul2_rn(Lb[0], X2[j][ci[0]]);
-#pragma unroll
-        for (int k = 1; k < N; ++k) q = __ffma2_rn(Lb[k], X2[j][ci[k]], q);
-        P2[j] = q;
-    }
-}
-
-// weno_field's 11 projections from the central value and the five pairs
-__device__ __forceinline__ void unpack11(float P0, const float2 (&P2)[5], float (&P)[11]) {
-    P[0] = P0;
-#pragma unroll
-    for (int j = 0; j < 5; ++j) {
-        P[1 + j] = P2[j].x;
-        P[6 + j] = P2[j].y;
-    }
-}
-
-// (P_c + P_s, P_c - P_s) of a mode pair, both packed halves at once
-__device__ __forceinline__ void split_pair_f(float Pc0, const float2 (&Pc2)[5], float Ps0, const float2 (&Ps2)[5],
-                                             float (&Pu)[11], float (&Pl)[11]) {
-    float2 U[5], D[5];
-#pragma unroll
-    for (int j = 0; j < 5; ++j) {
-        U[j] = __fadd2_rn(Pc2[j], Ps2[j]);
-        D[j] = __fadd2_rn(Pc2[j], neg2(Ps2[j]));
-    }
-    unpack11(Pc0 + Ps0, U, Pu);
-    unpack11(Pc0 - Ps0, D, Pl);
 }
 
 // ---------------------------------------------------------------- one face
-// Characteristic WENO flux at the face between stencil cells 2 and 3 of the
-// six cells at sm + k*st (k = 0..5); quantities are `ncell` elements apart.
-// Ff receives the frame flux (rho, m_n, m_t1, m_t2, B_t1, B_t2, E) and
-// s1, s2 the CT transport fluxes F_{B_t} + <B_n v_t> of Eqs. (fct1)-(fct6).
-template <typename Real, int VAR, bool DIFF = false, bool DWW = false>
-__device__ __forceinline__ void face_flux(const Real *__restrict__ sm, int ncell, int st, const Phys<Real> &K,
-                                          Real (&Ff)[7], Real &s1, Real &s2) {
-    using m = M<Real>;
-#define SMQ(q, k) sm[(q) * ncell + (k) * st]
-    // physical central combination and differences (projection is linear)
-    Real X[11][7];
-#pragma unroll
-    for (int c = 0; c < 7; ++c) {
-        if constexpr (DIFF) {
-            // from the box's forward differences (its difference pass):
-            // X[1 + j] = dF(j), X[6 + j] = du(j), j = 0..4, and the central
-            // combination (7 (f2 + f3) - (f1 + f4)) / 12 written as
-            // f2 + (6 dF(2) + dF(1) - dF(3)) / 12
-            const int qD = C_DF0 + c;
-            const int qU = c == 0 ? C_RHOQ : c == 1 ? C_MN : c == 2 ? C_MT1 : c == 3 ? C_MT2 : c == 4 ? C_DU4
-                           : c == 5 ? C_DU5 : C_E;
-#pragma unroll
-            for (int j = 0; j < 5; ++j) {
-                X[1 + j][c] = SMQ(qD, j);
-                X[6 + j][c] = SMQ(qU, j);
-            }
-            X[0][c] = SMQ(C_F0 + c, 2) + (Real(6) * X[3][c] + X[2][c] - X[4][c]) * Real(1.0 / 12.0);
-        } else {
-            const int qF = C_F0 + c;
-            const Real f0 = SMQ(qF, 0), f1 = SMQ(qF, 1), f2 = SMQ(qF, 2), f3 = SMQ(qF, 3), f4 = SMQ(qF, 4),
-                       f5 = SMQ(qF, 5);
-            X[1][c] = f1 - f0;
-            X[2][c] = f2 - f1;
-            X[3][c] = f3 - f2;
-            X[4][c] = f4 - f3;
-            X[5][c] = f5 - f4;
-            // (7 (f2 + f3) - (f1 + f4)) / 12 from the differences
-            X[0][c] = f2 + (Real(6) * X[3][c] + X[2][c] - X[4][c]) * Real(1.0 / 12.0);
-            const int qU = c == 0 ? C_RHOQ : c == 1 ? C_MN : c == 2 ? C_MT1 : c == 3 ? C_MT2 : c == 4 ? C_BT1
-                           : c == 5 ? C_BT2 : C_E;
-            const Real u0 = SMQ(qU, 0), u1 = SMQ(qU, 1), u2 = SMQ(qU, 2), u3 = SMQ(qU, 3), u4 = SMQ(qU, 4),
-                       u5 = SMQ(qU, 5);
-            X[6][c] = u1 - u0;
-            X[7][c] = u2 - u1;
-            X[8][c] = u3 - u2;
-            X[9][c] = u4 - u3;
-            X[10][c] = u5 - u4;
-        }
-    }
-    // float: the central vector and the pairs (dF_j, du_j) for the packed
-    // projection (the same values; only their grouping)
-    [[maybe_unused]] float X0f[7];
-    [[maybe_unused]] float2 X2f[5][7];
-    if constexpr (std::is_same<Real, float>::value) {
-#pragma unroll
-        for (int c = 0; c < 7; ++c) {
-            X0f[c] = X[0][c];
-#pragma unroll
-            for (int j = 0; j < 5; ++j) X2f[j][c] = make_float2(X[1 + j][c], X[6 + j][c]);
-        }
-    }
-    // interface state: mean of the primitives of cells i and i+1
-    const Real r = Real(0.5) * (SMQ(C_RHO, 2) + SMQ(C_RHO, 3));
-    const Real vn = Real(0.5) * (SMQ(C_VN, 2) + SMQ(C_VN, 3));
-    const Real vt1 = Real(0.5) * (SMQ(C_VT1, 2) + SMQ(C_VT1, 3));
-    const Real vt2 = Real(0.5) * (SMQ(C_VT2, 2) + SMQ(C_VT2, 3));
-    const Real Bn = Real(0.5) * (SMQ(C_BN, 2) + SMQ(C_BN, 3));
-    const Real Bt1 = Real(0.5) * (SMQ(C_BT1, 2) + SMQ(C_BT1, 3));
-    const Real Bt2 = Real(0.5) * (SMQ(C_BT2, 2) + SMQ(C_BT2, 3));
-    const Real P = Real(0.5) * (SMQ(C_P, 2) + SMQ(C_P, 3));
-    // Lax-Friedrichs speeds alpha(m) from the cell eigenvalues
-    const Real vL = SMQ(C_VN, 2), vR = SMQ(C_VN, 3);
-    const Real cfL = SMQ(C_CF, 2), cfR = SMQ(C_CF, 3);
-    const Real caL = SMQ(C_CA, 2), caR = SMQ(C_CA, 3);
-    const Real csL = SMQ(C_CSL, 2), csR = SMQ(C_CSL, 3);
-    const Real al_fm = m::max_(m::abs_(vL - cfL), m::abs_(vR - cfR));
-    const Real al_fp = m::max_(m::abs_(vL + cfL), m::abs_(vR + cfR));
-    const Real al_am = m::max_(m::abs_(vL - caL), m::abs_(vR - caR));
-    const Real al_ap = m::max_(m::abs_(vL + caL), m::abs_(vR + caR));
-    const Real al_sm = m::max_(m::abs_(vL - csL), m::abs_(vR - csR));
-    const Real al_sp = m::max_(m::abs_(vL + csL), m::abs_(vR + csR));
-    const Real al_e = m::max_(m::abs_(vL), m::abs_(vR));
-    // transport fluxes <B_n v_t> of the two cells
-    const Real bvt1 = Real(0.5) * (SMQ(C_BN, 2) * SMQ(C_VT1, 2) + SMQ(C_BN, 3) * SMQ(C_VT1, 3));
-    const Real bvt2 = Real(0.5) * (SMQ(C_BN, 2) * SMQ(C_VT2, 2) + SMQ(C_BN, 3) * SMQ(C_VT2, 3));
-#undef SMQ
 
-    // ---- eigen scalars at the interface state (Appendix A)
-    const Real ir = m::rcp_(r);
+// The scalars of Appendix A's eigenvectors at an interface state (the mean
+// of the two cells' primitives), from reciprocal square roots: 1 / sqrt(rho),
+// 1 / c_s, 1 / sqrt(d) (d the discriminant of the speeds, whose root is
+// c_f^2 - c_slow^2), 1 / |B_t|, 1 / c_f and one for the larger of (a_f, a_s).
+// With big = (sqrt(d) + |aa|) / 2 (aa = c_A^2 + b_t^2 - c_s^2) the larger of
+// a_f, a_s is sqrt(big / sqrt(d)) in [1/sqrt2, 1], and their product c_s b_t /
+// sqrt(d) gives the smaller one without a second root or a division.
+template <typename Real>
+struct FaceEigen {
+    Real sr, isr, cs, cs2, cf, cf2, csl, csl2, ics2, af, as, b1, b2, bt, sg;
+    bool apart;   // c_f > c_slow: a_f, a_s as above (else both 1, Appendix A)
+};
+
+template <typename Real>
+__device__ __forceinline__ FaceEigen<Real> face_eigen(Real r, Real v2, Real Bn, Real Bt1, Real Bt2, Real P,
+                                                      const Phys<Real> &K) {
+    using m = M<Real>;
+    FaceEigen<Real> e;
+    e.isr = m::rsqrt_(r);
+    const Real ir = e.isr * e.isr;
+    e.sr = r * e.isr;
     const Real ca2 = Bn * Bn * ir;
     const Real btm = Bt1 * Bt1 + Bt2 * Bt2;
     const Real bt2 = btm * ir;
-    const Real v2 = vn * vn + vt1 * vt1 + vt2 * vt2;
     // The slow and fast left eigenvectors carry 1/(2 c_s^2): the projection
     // amplifies the rounding of the data by about (v^2 + c_A^2 + b_t^2)/c_s^2.
     // In float, near a pressure floor, that reaches 1e9 and the split fluxes
@@ -718,200 +714,236 @@ __device__ __forceinline__ void face_flux(const Real *__restrict__ sm, int ncell
     // no smaller than cs2_rel times that sum.  L and R stay exact inverses, so
     // the flux stays consistent and conservative; only the basis in which
     // WENO reconstructs changes.  cs2_rel = 0 in double.
-    Real cs2 = K.gamma * P * ir;
-    if constexpr (float_based<Real>) cs2 = m::max_(cs2, K.cs2_rel * (v2 + ca2 + bt2));
-    Real fmc, cms, cf2, csl2;
-    speeds_fast<Real>(cs2, ca2, bt2, fmc, cms, cf2);
-    const Real sr = m::sqrt_(r);
-    const Real isr = sr * ir;
+    e.cs2 = K.gamma * P * ir;
+    if constexpr (float_based<Real>) e.cs2 = m::max_(e.cs2, K.cs2_rel * (v2 + ca2 + bt2));
+    const Real ics = m::rsqrt_(e.cs2);
+    e.cs = e.cs2 * ics;
+    e.ics2 = ics * ics;
+    const Real q = e.cs2 * bt2;
+    const Real aa = ca2 + bt2 - e.cs2;
+    const Real dd = m::fma_(aa, aa, Real(4) * q);
+    const bool some = m::normal_pos(dd);
+    const Real isd = some ? m::rsqrt_(dd) : Real(0);
+    const Real sd = dd * isd;
+    const Real big = m::half_(sd + m::abs_(aa));
+    const Real ibt = m::normal_pos(btm) ? m::rsqrt_(btm) : Real(0);
+    const Real bta = btm * ibt;   // |B_t|
+    const Real wb = big * isd;
+    const Real iwb = m::rsqrt_(wb);
+    const Real small_a = some ? (e.cs * (bta * e.isr)) * (isd * iwb) : Real(0);
+    e.apart = some && m::ge_pos(sd, K.eps_b2);
+    const Real ab = e.apart ? wb * iwb : Real(1), al = e.apart ? small_a : Real(1);
+    const bool fast_big = m::nonneg(aa);
+    e.as = fast_big ? ab : al;
+    e.af = fast_big ? al : ab;
+    // c_f^2 = c_s^2 + (c_f^2 - c_s^2), the difference a_s^2 sqrt(d)
+    e.cf2 = e.cs2 + (fast_big ? big : small_a * small_a * sd);
+    const Real icf = m::rsqrt_(e.cf2);
+    e.cf = e.cf2 * icf;
     // c_slow = c_s c_A / c_f (c_slow^2 = c_s^2 c_A^2 / c_f^2), c_A = |B_n| / sqrt(rho)
-    const Real cf = m::sqrt_(cf2), cs = m::sqrt_(cs2);
-    const Real csl = cf > Real(0) ? cs * (m::abs_(Bn) * isr) * m::rcp_(cf) : Real(0);
-    csl2 = csl * csl;
-    const Real dfs = fmc + cms;   // c_f^2 - c_slow^2
-    Real af, as;
-    if (dfs >= K.eps_b2) {
-        const Real idf = m::rcp_(dfs);
-        af = m::sqrt_(m::max_(cms * idf, Real(0)));
-        as = m::sqrt_(m::max_(fmc * idf, Real(0)));
+    e.csl = e.cs * (m::abs_(Bn) * e.isr) * icf;
+    e.csl2 = e.csl * e.csl;
+    if (m::gt_pos(btm, K.eps_b)) {   // b = B_t / |B_t|
+        e.b1 = Bt1 * ibt;
+        e.b2 = Bt2 * ibt;
+        e.bt = bta;
     } else {
-        af = Real(1);
-        as = Real(1);
+        e.b1 = Real(0.70710678118654752440);
+        e.b2 = Real(0.70710678118654752440);
+        e.bt = Real(0);
     }
-    Real b1, b2, bt;   // b = B_t / |B_t|, bt = |B_t|
-    if (btm > K.eps_b) {
-        const Real ib = m::rsqrt_(btm);
-        b1 = Bt1 * ib;
-        b2 = Bt2 * ib;
-        bt = btm * ib;
-    } else {
-        b1 = Real(0.70710678118654752440);
-        b2 = Real(0.70710678118654752440);
-        bt = Real(0);
-    }
-    const Real sg = (Bn >= K.eps_b) ? Real(1) : Real(-1);
-    const Real bv = b1 * vt1 + b2 * vt2;
-    const Real Gf = af * cf * vn - as * csl * sg * bv;
-    const Real Ga = sg * (b2 * vt1 - b1 * vt2);
-    const Real Gs = as * csl * vn + af * cf * sg * bv;
-    const Real ics2 = m::rcp_(cs2);
-    const Real pre = Real(0.5) * ics2;
-    const Real eps = Real(4.0 / 3.0) * K.eps_w;   // 4 eps / 3: see weno_field
+    e.sg = m::ge_pos(Bn, K.eps_b) ? Real(1) : Real(-1);
+    return e;
+}
 
-    // The sign-free parts of the fast and slow left eigenvectors and the
-    // entropy left eigenvector are combinations of two common vectors,
-    //   G = (v^2 / 2, -v_n, -v_t1, -v_t2, -B_t1, -B_t2, 1),
-    //   H = (0, 0, 0, 0, b_1, b_2, 0):
-    //   Lc_fast = pre ((gamma - 1) a_f G + sqrt(rho) c_s a_s H),
-    //   Lc_slow = pre ((gamma - 1) a_s G - sqrt(rho) c_s a_f H),
-    //   L_entropy = e_0 - (gamma - 1) G / c_s^2   (e_0: the density's unit vector),
-    // so each stencil vector is projected on G (its last component, 1, needs
-    // no product) and H once.  In double, G's field part -B_t = -|B_t| b is
-    // taken as -|B_t| (H.X): G.X = X_E + (v^2/2) X_rho - v.X_m - |B_t| H.X.
-    // (Where |B_t|^2 <= eps_B the default b is not B_t / |B_t|; there |B_t| is
-    // taken as 0, which leaves out at most |B_t| |X_B| <= 1e-15 |X_B| of G.X.)
-    const Real G[7] = {Real(0.5) * v2, -vn, -vt1, -vt2, -Bt1, -Bt2, Real(1)};
-    [[maybe_unused]] Real gX[11], hX[11];     // double: G.X, H.X
-    [[maybe_unused]] float g0, h0;            // float: the central vector's and
-    [[maybe_unused]] float2 g2[5], h2[5];     // the five pairs' projections
-    if constexpr (std::is_same<Real, float>::value) {
-        // (float: G projected in full -- the H form measured 0.7% slower, its
-        // longer-lived projections spilling more)
-        constexpr int cc[7] = {0, 1, 2, 3, 4, 5, 6};
-        constexpr int ch[2] = {4, 5};
-        const float Hc[2] = {b1, b2};
-        project_f<7>(X0f, X2f, cc, G, g0, g2);   // (the compiler drops the factor 1)
-        project_f<2>(X0f, X2f, ch, Hc, h0, h2);
-    } else {
+// Characteristic WENO flux at the face between stencil cells 2 and 3 of the
+// six cells at sm + k*st (k = 0..5); quantities are `ncell` elements apart.
+// Ff receives the frame flux (rho, m_n, m_t1, m_t2, B_t1, B_t2, E) and
+// s1, s2 the CT transport fluxes F_{B_t} + <B_n v_t> of Eqs. (fct1)-(fct6).
+//
+// The left and right eigenvectors of Appendix A are inverses (sum_m R_m L_m =
+// identity on the 7-vector), so the central part of Eq. (FWENO) needs no
+// projection: sum_m R_m (L_m . central + phi_m) = central + sum_m R_m phi_m.  Only
+// the five pairs of stencil differences are projected, and the flux keeps
+// the unprojected central combination (whose rounding no longer passes
+// through 1 / c_s^2).  The exception is Appendix A's fallback a_f = a_s = 1 at
+// c_f = c_slow, where L and R are not inverses: there the central part goes
+// through both, as printed.
+//
+// Bound: the FP64 pipe in double (2 lanes per SM and clock: one instruction
+// of a warp takes 16 clocks, in which 64 others can issue, hence the
+// comparisons, halvings and maxima on the integer pipes), the issue slots in
+// float.  Against the form that projected eleven vectors on Appendix A's rows
+// in the lab frame: 535.0 -> 416.7 ms per 256^3 FP64 step (WENO-Z), 15.57 ->
+// 14.46 ms in FP32-bulk, 56.6 -> 49.3 ms per 128^3 step with double-word
+// weights; no larger error against 64-bit values in any of them.
+template <typename Real, int VAR, bool DIFF = false, bool DWW = false>
+__device__ __forceinline__ void face_flux(const Real *__restrict__ sm, int ncell, int st, const Phys<Real> &K,
+                                          Real (&Ff)[7], Real &s1, Real &s2) {
+    using m = M<Real>;
+    using P2 = Pair<Real>;
+#define SMQ(q, k) sm[(q) * ncell + (k) * st]
+    // stencil differences X[c][j] = (dF_c, du_c) at position j, and the
+    // central combination (7 (f2 + f3) - (f1 + f4)) / 12 written as
+    // f2 + (6 dF(2) + dF(1) - dF(3)) / 12
+    P2 X[7][5];
+    Real X0[7];
 #pragma unroll
-        for (int x = 0; x < 11; ++x) {
-            const Real hx = b1 * X[x][4] + b2 * X[x][5];
-            Real gx = X[x][6] + G[0] * X[x][0];
+    for (int c = 0; c < 7; ++c) {
+        if constexpr (DIFF) {
+            // from the box's forward differences (its difference pass)
+            const int qD = C_DF0 + c;
+            const int qU = c == 0 ? C_RHOQ : c == 1 ? C_MN : c == 2 ? C_MT1 : c == 3 ? C_MT2 : c == 4 ? C_DU4
+                           : c == 5 ? C_DU5 : C_E;
+            Real dF[5];
 #pragma unroll
-            for (int c = 1; c < 4; ++c) gx += G[c] * X[x][c];
-            gX[x] = gx - bt * hx;
-            hX[x] = hx;
+            for (int j = 0; j < 5; ++j) {
+                dF[j] = SMQ(qD, j);
+                X[c][j] = make_pair2(dF[j], SMQ(qU, j));
+            }
+            X0[c] = SMQ(C_F0 + c, 2) + (Real(6) * dF[2] + dF[1] - dF[3]) * Real(1.0 / 12.0);
+        } else {
+            const int qF = C_F0 + c;
+            const int qU = c == 0 ? C_RHOQ : c == 1 ? C_MN : c == 2 ? C_MT1 : c == 3 ? C_MT2 : c == 4 ? C_BT1
+                           : c == 5 ? C_BT2 : C_E;
+            Real f[6], u[6];
+#pragma unroll
+            for (int j = 0; j < 6; ++j) {
+                f[j] = SMQ(qF, j);
+                u[j] = SMQ(qU, j);
+            }
+#pragma unroll
+            for (int j = 0; j < 5; ++j) X[c][j] = make_pair2(f[j + 1] - f[j], u[j + 1] - u[j]);
+            X0[c] = f[2] + (Real(6) * (f[3] - f[2]) + (f[2] - f[1]) - (f[4] - f[3])) * Real(1.0 / 12.0);
         }
     }
-    // The WENO fluxes (Fu for the left eigenvector Lc + Ls, Fl for Lc - Ls)
-    // of one magnetosonic pair: Lc = cg G + ch H, Ls non-zero in rows 0..3.
-    auto magnetosonic = [&](Real cg, Real ch, const Real (&Ls)[4], Real alu, Real all, Real &Fu, Real &Fl) {
-        Real Pu[11], Pl[11];
-        if constexpr (std::is_same<Real, float>::value) {
-            constexpr int cs4[4] = {0, 1, 2, 3};
-            const float pc0 = cg * g0 + ch * h0;
-            float2 pc2[5];
+    // interface state: mean of the primitives of cells i and i+1
+    auto mean = [&](int q) { return m::half_(SMQ(q, 2) + SMQ(q, 3)); };
+    const Real r = mean(C_RHO), vn = mean(C_VN), vt1 = mean(C_VT1), vt2 = mean(C_VT2);
+    const Real Bn = mean(C_BN), Bt1 = mean(C_BT1), Bt2 = mean(C_BT2), P = mean(C_P);
+    // Lax-Friedrichs speeds alpha(m) from the cell eigenvalues
+    const Real vL = SMQ(C_VN, 2), vR = SMQ(C_VN, 3);
+    auto alpha = [&](Real cL, Real cR) { return m::max_nonneg(m::abs_(vL + cL), m::abs_(vR + cR)); };
+    const Real cfL = SMQ(C_CF, 2), cfR = SMQ(C_CF, 3);
+    const Real caL = SMQ(C_CA, 2), caR = SMQ(C_CA, 3);
+    const Real csL = SMQ(C_CSL, 2), csR = SMQ(C_CSL, 3);
+    // twice the transport fluxes <B_n v_t> of the two cells
+    const Real bvt1 = SMQ(C_BN, 2) * SMQ(C_VT1, 2) + SMQ(C_BN, 3) * SMQ(C_VT1, 3);
+    const Real bvt2 = SMQ(C_BN, 2) * SMQ(C_VT2, 2) + SMQ(C_BN, 3) * SMQ(C_VT2, 3);
+#undef SMQ
+
+    // ---- eigen scalars at the interface state (Appendix A)
+    const Real v2 = vn * vn + vt1 * vt1 + vt2 * vt2;
+    const Real hv2 = m::half_(v2);
+    const FaceEigen<Real> e = face_eigen<Real>(r, v2, Bn, Bt1, Bt2, P, K);
+    const Real b1 = e.b1, b2 = e.b2, sg = e.sg;
+    const Real pre = m::half_(e.ics2);
+    const Real tau = K.gm1 * e.ics2;
+    const Real afcf = e.af * e.cf, ascl = e.as * e.csl;
+    const Real sas = sg * ascl, saf = sg * afcf;
+    const Real eps3 = Real(1.0 / 3.0) * K.eps_w;   // 4 eps / 12: see weno_field
+
+    // ---- projections.  With Y = X_m - v X_rho (the momentum differences in
+    // the frame of the interface) the left eigenvectors of Appendix A are
+    // combinations of
+    //   g = X_E - v^2/2 X_rho - v.Y - |B_t| h,   h = b.X_B,   k = b.Y_t,
+    //   L_fast    = pre ((gamma - 1) a_f g + sqrt(rho) c_s a_s h -+ a_f c_f Y_n +- sg a_s c_slow k),
+    //   L_slow    = pre ((gamma - 1) a_s g - sqrt(rho) c_s a_f h -+ a_s c_slow Y_n -+ sg a_f c_f k),
+    //   L_Alfven  = sg/2 (b x Y_t -+ ... ) = sg/2 [b_1 Y_t2 - b_2 Y_t1 +- sg sqrt(rho) (b_1 X_B2 - b_2 X_B1)],
+    //   L_entropy = X_rho - (gamma - 1) g / c_s^2.
+    // (g's field part -B_t is taken as -|B_t| b.  Where |B_t|^2 <= eps_B the
+    // default b is not B_t / |B_t|; there |B_t| is taken as 0, which leaves out
+    // at most |B_t| |X_B| <= 1e-15 |X_B|.)  The Alfven fields are carried
+    // without their factor sg/2: phi_N is linear up to epsilon, which scales
+    // by 4 with them, and the factor joins the back-projection.
+    P2 fu[5], fl[5], su[5], sl[5], au[5], al[5], en[5];
+    const Real cF = pre * (K.gm1 * e.af), cS = pre * (K.gm1 * e.as);
+    const Real srcs = pre * (e.sr * e.cs);
+    const Real hF = srcs * e.as, hS = -(srcs * e.af);
+    const Real nF = -(pre * afcf), nS = -(pre * ascl), kF = pre * sas, kS = -(pre * saf);
+    const Real ssr = sg * e.sr;
+    const Real a5 = ssr * b1, a4 = -(ssr * b2);
 #pragma unroll
-            for (int j = 0; j < 5; ++j) pc2[j] = __ffma2_rn(bcast2(cg), g2[j], __fmul2_rn(bcast2(ch), h2[j]));
-            float ps0;
-            float2 ps2[5];
-            project_f<4>(X0f, X2f, cs4, Ls, ps0, ps2);
-            split_pair_f(pc0, pc2, ps0, ps2, Pu, Pl);
-        } else {
-#pragma unroll
-            for (int x = 0; x < 11; ++x) {
-                const Real pc = cg * gX[x] + ch * hX[x];
-                Real ps = Ls[0] * X[x][0];
-#pragma unroll
-                for (int c = 1; c < 4; ++c) ps += Ls[c] * X[x][c];
-                Pu[x] = pc + ps;
-                Pl[x] = pc - ps;
-            }
-        }
-        Fu = weno_field<Real, VAR, DWW>(Pu, alu, eps);
-        Fl = weno_field<Real, VAR, DWW>(Pl, all, eps);
+    for (int j = 0; j < 5; ++j) {
+        const P2 Yn = pfma(-vn, X[0][j], X[1][j]);
+        const P2 Y1 = pfma(-vt1, X[0][j], X[2][j]);
+        const P2 Y2 = pfma(-vt2, X[0][j], X[3][j]);
+        const P2 h = pfma(b1, X[4][j], pmul(b2, X[5][j]));
+        const P2 k = pfma(b1, Y1, pmul(b2, Y2));
+        const P2 x = pfma(b1, Y2, pmul(-b2, Y1));
+        P2 g = pfma(-hv2, X[0][j], X[6][j]);
+        g = pfma(-vn, Yn, g);
+        g = pfma(-vt1, Y1, g);
+        g = pfma(-vt2, Y2, g);
+        g = pfma(-e.bt, h, g);
+        mode_pair(pfma(cF, g, pmul(hF, h)), nF, Yn, kF, k, fu[j], fl[j]);
+        mode_pair(pfma(cS, g, pmul(hS, h)), nS, Yn, kS, k, su[j], sl[j]);
+        mode_pair(x, a4, X[4][j], a5, X[5][j], au[j], al[j]);
+        en[j] = pfma(-tau, g, X[0][j]);
+    }
+
+    // ---- WENO parts of the fields: sums and differences of the pairs, upper
+    // members m = 1 (v - c_f), 3 (v - c_slow), 2 (v - c_A)
+    Real sf, df, ss, ds, sa, da, Fe;
+    auto fields = [&](const P2 (&u)[5], const P2 (&l)[5], Real cL, Real cR, Real ep, Real &sum, Real &dif) {
+        const Real Fu = weno_field<Real, VAR, DWW>(u, alpha(-cL, -cR), ep);
+        const Real Fl = weno_field<Real, VAR, DWW>(l, alpha(cL, cR), ep);
+        sum = Fu + Fl;
+        dif = Fu - Fl;
     };
+    fields(fu, fl, cfL, cfR, eps3, sf, df);
+    fields(su, sl, csL, csR, eps3, ss, ds);
+    fields(au, al, caL, caR, Real(4) * eps3, sa, da);
+    Fe = weno_field<Real, VAR, DWW>(en, m::max_nonneg(m::abs_(vL), m::abs_(vR)), eps3);
+    if (!e.apart) {
+        // Appendix A's fallback: the central part through L and R, in the
+        // units of the WENO parts, in place of the unprojected one
+        const Real u = Real(1) / kWenoScale<Real>;
+        const Real Yn = X0[1] - vn * X0[0], Y1 = X0[2] - vt1 * X0[0], Y2 = X0[3] - vt2 * X0[0];
+        const Real h = b1 * X0[4] + b2 * X0[5], k = b1 * Y1 + b2 * Y2;
+        const Real g = X0[6] - hv2 * X0[0] - vn * Yn - vt1 * Y1 - vt2 * Y2 - e.bt * h;
+        const Real u2 = Real(2) * u;
+        sf += u2 * (cF * g + hF * h);
+        df += u2 * (nF * Yn + kF * k);
+        ss += u2 * (cS * g + hS * h);
+        ds += u2 * (nS * Yn + kS * k);
+        sa += u2 * (b1 * Y2 - b2 * Y1);
+        da += u2 * (a4 * X0[4] + a5 * X0[5]);
+        Fe += u * (X0[0] - tau * g);
+#pragma unroll
+        for (int c = 0; c < 7; ++c) X0[c] = Real(0);
+    }
 
-    // ---- fast pair: m = 1 (v - c_f, upper sign) and m = 7 (v + c_f)
-    Real sf, df;
-    {
-        const Real Ls[4] = {pre * Gf, -pre * af * cf, pre * csl * as * b1 * sg, pre * csl * as * b2 * sg};
-        Real Fu, Fl;
-        magnetosonic(pre * (K.gm1 * af), pre * (sr * cs * as), Ls, al_fm, al_fp, Fu, Fl);
-        sf = Fu + Fl;
-        df = Fu - Fl;
-    }
-    // ---- slow pair: m = 3 (v - c_slow, upper sign) and m = 5 (v + c_slow)
-    Real ss, ds;
-    {
-        const Real Ls[4] = {pre * Gs, -pre * as * csl, -pre * cf * af * b1 * sg, -pre * cf * af * b2 * sg};
-        Real Fu, Fl;
-        magnetosonic(pre * (K.gm1 * as), -(pre * (sr * cs * af)), Ls, al_sm, al_sp, Fu, Fl);
-        ss = Fu + Fl;
-        ds = Fu - Fl;
-    }
-    // ---- Alfven pair: m = 2 (v - c_A, upper sign) and m = 6 (v + c_A)
-    //   L = (Ga/2, 0, -b2 sg/2, b1 sg/2, -+ sr b2/2, +- sr b1/2, 0)
-    //   R = (0, 0, -b2 sg, b1 sg, -+ b2/sr, +- b1/sr, -Ga)
-    Real sa, da;
-    {
-        const Real l0 = Real(0.5) * Ga, l2 = Real(-0.5) * b2 * sg, l3 = Real(0.5) * b1 * sg;
-        const Real l4 = Real(-0.5) * sr * b2, l5 = Real(0.5) * sr * b1;
-        Real Pu[11], Pl[11];
-        if constexpr (std::is_same<Real, float>::value) {
-            constexpr int cc[3] = {0, 2, 3};
-            constexpr int cs[2] = {4, 5};
-            const float Lc[3] = {l0, l2, l3}, Ls[2] = {l4, l5};
-            float pc0, ps0;
-            float2 pc2[5], ps2[5];
-            project_f<3>(X0f, X2f, cc, Lc, pc0, pc2);
-            project_f<2>(X0f, X2f, cs, Ls, ps0, ps2);
-            split_pair_f(pc0, pc2, ps0, ps2, Pu, Pl);
-        } else {
-#pragma unroll
-            for (int x = 0; x < 11; ++x) {
-                const Real pc = l0 * X[x][0] + l2 * X[x][2] + l3 * X[x][3];
-                const Real ps = l4 * X[x][4] + l5 * X[x][5];
-                Pu[x] = pc + ps;
-                Pl[x] = pc - ps;
-            }
-        }
-        const Real Fu = weno_field<Real, VAR, DWW>(Pu, al_am, eps);
-        const Real Fl = weno_field<Real, VAR, DWW>(Pl, al_ap, eps);
-        sa = Fu + Fl;
-        da = Fu - Fl;
-    }
-    // ---- entropy field: m = 4 (v), L = e_0 - (gamma - 1) G / c_s^2
-    Real Fe;
-    {
-        const Real tau = K.gm1 * ics2;
-        Real Pe[11];
-        if constexpr (std::is_same<Real, float>::value) {
-            float2 pe2[5];
-#pragma unroll
-            for (int j = 0; j < 5; ++j) pe2[j] = __ffma2_rn(bcast2(-tau), g2[j], X2f[j][0]);
-            unpack11(__fmaf_rn(-tau, g0, X0f[0]), pe2, Pe);
-        } else {
-#pragma unroll
-            for (int x = 0; x < 11; ++x) Pe[x] = X[x][0] - tau * gX[x];
-        }
-        Fe = weno_field<Real, VAR, DWW>(Pe, al_e, eps);
-    }
-    // ---- back-projection: F = sum over fields of (WENO flux) x (right
-    // eigenvector).  The right eigenvectors of the fast pair (Rc +- Rs),
-    //   Rc = (a_f, a_f v, c_s a_s b / sqrt(rho), a_f (v^2/2 + c_f^2 - g2 c_s^2)),
-    //   Rs = rows (1, 2, 3, 6): (-a_f c_f, c_slow a_s b sg, -Gf),
+    // ---- back-projection: central + sum over fields of (WENO part) x (right
+    // eigenvector).  The right eigenvectors of the fast pair (Rc +- Rs), seen
+    // from the frame of the interface (v = 0),
+    //   Rc = (a_f, 0, c_s a_s b / sqrt(rho), a_f (c_f^2 - g2 c_s^2)),
+    //   Rs = rows (1, 2, 3): (-a_f c_f, c_slow a_s b sg),
     // of the slow pair (a_f, c_f -> a_s, c_slow and a_s, c_slow -> -a_f, c_f
-    // in Rc's field rows and Rs) and of the entropy field (1, v, 0, v^2 / 2)
-    // share R1 = (1, v, 0, 0, v^2/2 - g2 c_s^2) and (0, 0, 0, 0, b_1, b_2, 0),
-    // so the sums (Fu + Fl) and differences (Fu - Fl) of the fields combine
-    // into a few scalars first.
+    // in Rc's field rows and Rs), of the Alfven pair and of the entropy field
+    // (1, 0, 0, 0) combine into a few scalars; the boost back to the lab adds
+    // v S1 to the momentum and v^2/2 S1 + v.T to the energy.
     {
-        const Real S1 = af * sf + as * ss + Fe;
-        const Real S2 = (cs * isr) * (as * sf - af * ss);
-        const Real T1 = -(af * cf * df + as * csl * ds);
-        const Real T2 = sg * (csl * as * df - cf * af * ds);
-        const Real w = Real(0.5) * v2 - K.g2 * cs2;
-        Ff[0] = S1;
-        Ff[1] = S1 * vn + T1;
-        Ff[2] = S1 * vt1 + T2 * b1 - sa * (b2 * sg);
-        Ff[3] = S1 * vt2 + T2 * b2 + sa * (b1 * sg);
-        Ff[4] = S2 * b1 - da * (b2 * isr);
-        Ff[5] = S2 * b2 + da * (b1 * isr);
-        Ff[6] = S1 * w + af * cf2 * sf + as * csl2 * ss + K.g2 * cs2 * Fe - (Gf * df + Gs * ds) - sa * Ga;
+        const Real kw = kWenoScale<Real>;
+        const Real mg = e.af * sf + e.as * ss;                     // magnetosonic density
+        const Real S1 = mg + Fe;
+        const Real S2 = (e.cs * e.isr) * (e.as * sf - e.af * ss);
+        const Real hsa = m::half_(sa), hda = m::half_(da) * (sg * e.isr);   // (sg/2)^2, sg/2 of the Alfven fields
+        const Real Tn = -(afcf * df + ascl * ds);
+        const Real Tk = sas * df - saf * ds;
+        const Real T1 = Tk * b1 - hsa * b2;
+        const Real T2 = Tk * b2 + hsa * b1;
+        const Real en6 = (afcf * e.cf) * sf + (ascl * e.csl) * ss - (K.g2 * e.cs2) * mg;
+        Ff[0] = X0[0] + kw * S1;
+        Ff[1] = X0[1] + kw * (S1 * vn + Tn);
+        Ff[2] = X0[2] + kw * (S1 * vt1 + T1);
+        Ff[3] = X0[3] + kw * (S1 * vt2 + T2);
+        Ff[4] = X0[4] + kw * (S2 * b1 - hda * b2);
+        Ff[5] = X0[5] + kw * (S2 * b2 + hda * b1);
+        Ff[6] = X0[6] + kw * (hv2 * S1 + vn * Tn + vt1 * T1 + vt2 * T2 + en6);
     }
-    s1 = Ff[4] + bvt1;
-    s2 = Ff[5] + bvt2;
+    s1 = m::fma_(Real(0.5), bvt1, Ff[4]);
+    s2 = m::fma_(Real(0.5), bvt2, Ff[5]);
 }
 
 }  // namespace w5ct
