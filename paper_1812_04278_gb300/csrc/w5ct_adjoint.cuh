@@ -22,798 +22,698 @@
 namespace w5ct {
 
 // ---------------------------------------------------------------- sweep adjoint
+//
+// Two kernels per axis and stage.  adj_face_kernel runs the face function's
+// reverse mode, one thread per face over the same shared-memory cell box as
+// the forward sweep, and writes the adjoints of what the face reads of its
+// cells: the five stencil differences of the flux and of the conserved vector
+// (70), the central flux (7), the interface primitives (8) and the wave
+// speeds of its two cells (2 x 4).  adj_cell_kernel sums them over the faces
+// of each cell in a fixed order and reverses the cell recovery once per cell.
+constexpr int kAdjDiff = 0;                    // plane (c * 5 + j) * 2 + (0: dF_c, 1: du_c) at position j
+constexpr int kAdjCentral = 70;                // central flux, component c
+constexpr int kAdjPrim = 77;                   // interface primitives (C_RHO .. C_P)
+constexpr int kAdjSide = 85;                   // (v_n, c_f, c_A, c_slow) of the lower cell, then of the upper
+constexpr int kAdjFacePlanes = 93;
+constexpr int kAdjFluxPlanes = 21;             // the first planes lie in the context's flux buffers
 
-template <typename B>
+template <typename Real>
 struct AdjSweepArgs {
     int nx, ny, nz;
-    const B *q[5];          // stage state (rho, m, E), arithmetic type
-    const B *bc[3];         // the stage's cell-centred field
-    const double *lamF[5];  // dL/dF of this axis' face fluxes (lab order)
-    const double *lamS[2];  // dL/dS of this axis' transport fluxes
-    double *cb;             // 48 planes: cb[(s * 8 + v) * n + p] = d(lam . out_p)/d(input v of stencil cell s)
-    Phys<B> K;
+    double rd;                 // 1 / spacing along the axis
+    const Real *q[5];          // stage state (rho, m, E), arithmetic type
+    const Real *bc[3];         // the stage's cell-centred field
+    const double *lamD;        // 5 planes: adjoint of the flux divergence
+    const double *lamO;        // 3 planes: adjoint of the corner EMFs
+    Real *fa, *fb;             // face adjoints: planes 0..20 in fa, the others in fb
+    double *outq, *outb;       // 5 planes of the state's adjoint, 3 of the cell field's
+    bool first;                // the first axis of the stage writes outq, outb, the others add
+    Phys<Real> K;
+    __device__ __forceinline__ Real *face_plane(int k) const {
+        const size_t n = (size_t)nx * ny * nz;
+        return k < kAdjFluxPlanes ? fa + (size_t)k * n : fb + (size_t)(k - kAdjFluxPlanes) * n;
+    }
 };
 
-// ---------------------------------------------------------------- reverse mode
-
-// The seven characteristic modes of Appendix A at the interface state w =
-// (rho, v_n, v_t1, v_t2, B_n, B_t1, B_t2, P) as full left and right
-// eigenvectors in the frame order (rho, m_n, m_t1, m_t2, B_t1, B_t2, E):
-// modes 0/1 fast (v -/+ c_f), 2/3 slow (v -/+ c_slow), 4/5 Alfven
-// (v -/+ c_A), 6 entropy.  The formulas (and branches) of face_flux, written
-// as whole vectors: the paired forms there are L = Lc +- Ls, R = Rc +- Rs.
-template <typename Real>
-__device__ __forceinline__ void eigen7(const Real (&w)[8], const Phys<Real> &K, Real (&L)[7][7], Real (&R)[7][7]) {
-    using m = M<Real>;
-    const Real r = w[0], vn = w[1], vt1 = w[2], vt2 = w[3], Bn = w[4], Bt1 = w[5], Bt2 = w[6], P = w[7];
-    const Real ir = m::rcp_(r);
-    const Real ca2 = Bn * Bn * ir;
-    const Real btm = Bt1 * Bt1 + Bt2 * Bt2;
-    const Real bt2 = btm * ir;
-    const Real v2 = vn * vn + vt1 * vt1 + vt2 * vt2;
-    Real cs2 = K.gamma * P * ir;
-    if constexpr (float_based<Real>) cs2 = m::max_(cs2, K.cs2_rel * (v2 + ca2 + bt2));
-    Real fmc, cms, cf2, csl2;
-    speeds<Real>(cs2, ca2, bt2, fmc, cms, cf2, csl2);
-    const Real cf = m::sqrt_(cf2), csl = m::sqrt_(csl2), cs = m::sqrt_(cs2);
-    const Real dfs = fmc + cms;
-    Real af, as;
-    if (dfs >= K.eps_b2) {
-        const Real idf = m::rcp_(dfs);
-        af = m::sqrt_(m::max_(cms * idf, Real(0)));
-        as = m::sqrt_(m::max_(fmc * idf, Real(0)));
-    } else {
-        af = Real(1);
-        as = Real(1);
-    }
-    Real b1, b2;
-    if (btm > K.eps_b) {
-        const Real ib = m::rsqrt_(btm);
-        b1 = Bt1 * ib;
-        b2 = Bt2 * ib;
-    } else {
-        b1 = Real(0.70710678118654752440);
-        b2 = Real(0.70710678118654752440);
-    }
-    const Real sg = (Bn >= K.eps_b) ? Real(1) : Real(-1);
-    const Real sr = m::sqrt_(r);
-    const Real isr = sr * ir;
-    const Real bv = b1 * vt1 + b2 * vt2;
-    const Real Gf = af * cf * vn - as * csl * sg * bv;
-    const Real Ga = sg * (b2 * vt1 - b1 * vt2);
-    const Real Gs = as * csl * vn + af * cf * sg * bv;
-    const Real ics2 = m::rcp_(cs2);
-    const Real pre = Real(0.5) * ics2;
-    const Real tau = K.gm1 * ics2;
-    auto pair = [&](int mu, const Real (&Lc)[7], const Real (&Ls)[4], const Real (&Rc)[7], const Real (&Rs)[4]) {
-#pragma unroll
-        for (int c = 0; c < 7; ++c) {
-            L[mu][c] = Lc[c];
-            L[mu + 1][c] = Lc[c];
-            R[mu][c] = Rc[c];
-            R[mu + 1][c] = Rc[c];
-        }
-#pragma unroll
-        for (int c = 0; c < 4; ++c) {
-            L[mu][c] = L[mu][c] + Ls[c];
-            L[mu + 1][c] = L[mu + 1][c] - Ls[c];
-        }
-        const int rows[4] = {1, 2, 3, 6};
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            R[mu][rows[k]] = R[mu][rows[k]] + Rs[k];
-            R[mu + 1][rows[k]] = R[mu + 1][rows[k]] - Rs[k];
-        }
-    };
-    {
-        const Real k1 = -K.gm1 * af;
-        const Real Lc[7] = {pre * K.g1 * af * v2, pre * k1 * vn, pre * k1 * vt1, pre * k1 * vt2,
-                            pre * (k1 * Bt1 + sr * cs * as * b1), pre * (k1 * Bt2 + sr * cs * as * b2), pre * K.gm1 * af};
-        const Real Ls[4] = {pre * Gf, -pre * af * cf, pre * csl * as * b1 * sg, pre * csl * as * b2 * sg};
-        const Real Rc[7] = {af, af * vn, af * vt1, af * vt2, cs * as * b1 * isr, cs * as * b2 * isr,
-                            af * (Real(0.5) * v2 + cf2 - K.g2 * cs2)};
-        const Real Rs[4] = {-af * cf, csl * as * b1 * sg, csl * as * b2 * sg, -Gf};
-        pair(0, Lc, Ls, Rc, Rs);
-    }
-    {
-        const Real k2 = -K.gm1 * as;
-        const Real Lc[7] = {pre * K.g1 * as * v2, pre * k2 * vn, pre * k2 * vt1, pre * k2 * vt2,
-                            pre * (k2 * Bt1 - sr * cs * af * b1), pre * (k2 * Bt2 - sr * cs * af * b2), pre * K.gm1 * as};
-        const Real Ls[4] = {pre * Gs, -pre * as * csl, -pre * cf * af * b1 * sg, -pre * cf * af * b2 * sg};
-        const Real Rc[7] = {as, as * vn, as * vt1, as * vt2, -cs * af * b1 * isr, -cs * af * b2 * isr,
-                            as * (Real(0.5) * v2 + csl2 - K.g2 * cs2)};
-        const Real Rs[4] = {-as * csl, -cf * af * b1 * sg, -cf * af * b2 * sg, -Gs};
-        pair(2, Lc, Ls, Rc, Rs);
-    }
-    {
-        const Real l0 = Real(0.5) * Ga, l2 = Real(-0.5) * b2 * sg, l3 = Real(0.5) * b1 * sg;
-        const Real l4 = Real(-0.5) * sr * b2, l5 = Real(0.5) * sr * b1;
-        const Real z = Real(0);
-        const Real La[7] = {l0, z, l2, l3, l4, l5, z}, Lb[7] = {l0, z, l2, l3, -l4, -l5, z};
-        const Real Ra[7] = {z, z, -b2 * sg, b1 * sg, -b2 * isr, b1 * isr, -Ga};
-        const Real Rb[7] = {z, z, -b2 * sg, b1 * sg, b2 * isr, -b1 * isr, -Ga};
-#pragma unroll
-        for (int c = 0; c < 7; ++c) {
-            L[4][c] = La[c];
-            L[5][c] = Lb[c];
-            R[4][c] = Ra[c];
-            R[5][c] = Rb[c];
-        }
-    }
-    {
-        const Real Le[7] = {Real(1) - Real(0.5) * tau * v2, tau * vn, tau * vt1, tau * vt2, tau * Bt1, tau * Bt2, -tau};
-        const Real Re[7] = {Real(1), vn, vt1, vt2, Real(0), Real(0), Real(0.5) * v2};
-#pragma unroll
-        for (int c = 0; c < 7; ++c) {
-            L[6][c] = Le[c];
-            R[6][c] = Re[c];
-        }
-    }
-}
-
-// Reverse of speeds(): adds to (lcs2, lca2, lbt2) the adjoints of its inputs
-// given those of (fmc, cms, cf2, csl2); the same branches and guards as the
-// forward formulas (Eqs. slow/fast), run backwards.
-template <typename B, typename A>
-__device__ __forceinline__ void speeds_rev(B cs2, B ca2, B bt2, A lfmc, A lcms, A lcf2, A lcsl2, A &lcs2, A &lca2,
-                                           A &lbt2) {
-    using m = M<B>;
-    const B dd = (cs2 - ca2) * (cs2 - ca2) + bt2 * (bt2 + B(2) * ca2 + B(2) * cs2);
-    const B sd = m::sqrt_(dd);
-    const B aa = ca2 + bt2 - cs2;
-    B fmc, cms;
-    if (aa >= B(0)) {
-        fmc = B(0.5) * (aa + sd);
-        cms = fmc > B(0) ? m::div_(cs2 * bt2, fmc) : B(0);
-    } else {
-        cms = B(0.5) * (sd - aa);
-        fmc = cms > B(0) ? m::div_(cs2 * bt2, cms) : B(0);
-    }
-    const B cf2 = cs2 + fmc;
-    if (cf2 > B(0)) {
-        const A icf = A(1) / (A)cf2;
-        const A csl2 = (A)m::div_(cs2 * ca2, cf2);
-        lcs2 += lcsl2 * (A)ca2 * icf;
-        lca2 += lcsl2 * (A)cs2 * icf;
-        lcf2 -= lcsl2 * csl2 * icf;
-    }
+// Reverse of speeds_fast and c_slow^2 = c_s^2 c_A^2 / c_f^2: adds to (lcs2,
+// lca2, lbt2) the adjoints of the inputs given those of (fmc, cms, cf2, csl2);
+// the same branches and guards as the forward formulas (Eqs. slow/fast).
+template <typename R>
+__device__ __forceinline__ void speeds_rev(R cs2, R ca2, R bt2, R lfmc, R lcms, R lcf2, R lcsl2, R &lcs2, R &lca2,
+                                           R &lbt2) {
+    using m = M<R>;
+    const R q = cs2 * bt2;
+    const R aa = ca2 + bt2 - cs2;
+    const R dd = m::fma_(aa, aa, R(4) * q);
+    const R isd = m::normal_pos(dd) ? m::rsqrt_(dd) : R(0);
+    const R big = m::half_(dd * isd + m::abs_(aa));
+    const R ibig = m::normal_pos(big) ? m::rcp3_(big) : R(0);
+    const R oth = q * ibig;
+    const bool fast_big = m::nonneg(aa);
+    const R cf2 = cs2 + (fast_big ? big : oth);
+    const R icf2 = m::normal_pos(cf2) ? m::rcp3_(cf2) : R(0);
+    lcs2 += lcsl2 * (ca2 * icf2);
+    lca2 += lcsl2 * (cs2 * icf2);
+    lcf2 -= lcsl2 * (cs2 * ca2 * icf2) * icf2;
     lcs2 += lcf2;
     lfmc += lcf2;
-    A laa = A(0), lsd = A(0);
-    if (aa >= B(0)) {
-        if (fmc > B(0)) {
-            const A ifm = A(1) / (A)fmc;
-            lcs2 += lcms * (A)bt2 * ifm;
-            lbt2 += lcms * (A)cs2 * ifm;
-            lfmc -= lcms * (A)cms * ifm;
-        }
-        laa += A(0.5) * lfmc;
-        lsd += A(0.5) * lfmc;
-    } else {
-        if (cms > B(0)) {
-            const A icm = A(1) / (A)cms;
-            lcs2 += lfmc * (A)bt2 * icm;
-            lbt2 += lfmc * (A)cs2 * icm;
-            lcms -= lfmc * (A)fmc * icm;
-        }
-        lsd += A(0.5) * lcms;
-        laa -= A(0.5) * lcms;
-    }
-    lca2 += laa;
-    lbt2 += laa;
-    lcs2 -= laa;
-    const A ldd = sd > B(0) ? lsd * A(0.5) / (A)sd : A(0);
-    lcs2 += ldd * (A(2) * ((A)cs2 - (A)ca2) + A(2) * (A)bt2);
-    lca2 += ldd * (A(-2) * ((A)cs2 - (A)ca2) + A(2) * (A)bt2);
-    lbt2 += ldd * (A(2) * (A)bt2 + A(2) * (A)ca2 + A(2) * (A)cs2);
+    // big = (sqrt(dd) + |aa|) / 2, oth = q / big
+    const R loth = fast_big ? lcms : lfmc;
+    R lbig = fast_big ? lfmc : lcms;
+    const R lq = loth * ibig;
+    lbig -= loth * oth * ibig;
+    lcs2 += lq * bt2;
+    lbt2 += lq * cs2;
+    const R laa = m::half_(fast_big ? lbig : -lbig);
+    const R ldd = m::half_(lbig) * m::half_(isd);
+    // dd = aa^2 + 4 q, aa = ca2 + bt2 - cs2
+    const R la = laa + R(2) * ldd * aa;
+    lca2 += la;
+    lbt2 += la + R(4) * ldd * cs2;
+    lcs2 += R(4) * ldd * bt2 - la;
 }
 
-// Reverse of eigen7: lw = d/dw of sum(lL * L) + sum(lR * R) at the
-// interface state w, written by hand from the forward formulas (recomputed
-// here in B; the adjoints in A).  Branches follow the primal values: the
-// epsilon_B switches and the WENO sign sg, the c_s^2 bound of the float
-// path, the sqrt of zero (subgradient 0): the derivative of the branch the
-// forward step takes.
-template <typename B, typename A>
-__device__ __forceinline__ void eigen7_rev(const B (&w)[8], const Phys<B> &K, const A (&lL)[7][7], const A (&lR)[7][7],
-                                           A (&lw)[8]) {
-    using m = M<B>;
-    const B r = w[0], vn = w[1], vt1 = w[2], vt2 = w[3], Bn = w[4], Bt1 = w[5], Bt2 = w[6], P = w[7];
-    // ---- forward values
-    const B ir = m::rcp_(r);
-    const B ca2 = Bn * Bn * ir;
-    const B btm = Bt1 * Bt1 + Bt2 * Bt2;
-    const B bt2 = btm * ir;
-    const B v2 = vn * vn + vt1 * vt1 + vt2 * vt2;
-    const B cs2a = K.gamma * P * ir;
-    B cs2 = cs2a;
+// One interpolant phi~ = N / D = 12 phi_N(a, b, c, d) (the weights of the
+// forward step: JS, or WENO-Z with the ratio clamped at 1e18 in float) and its
+// gradient, times the seed l: smoothness indicators -> weights, in the
+// normalised form e_k = alpha_k / d_k from one reciprocal per indicator ->
+// N / D, run backwards.  A reciprocal r = 1/x is reversed as -r (r l), never
+// with r^2, so that a tiny eps + IS times a zero adjoint stays 0 in float.
+template <typename R, int VAR>
+__device__ __forceinline__ void phi_rev(R a, R b, R c, R d, R eps12, R l, R &f, R (&g)[4]) {
+    using m = M<R>;
+    R s0, s1, s2, x0, y0, z0;
+    smoothness3<R>(a, b, c, d, eps12, s0, s1, s2, x0, y0, z0);
+    const R i0 = m::rcp3_(s0), i1 = m::rcp3_(s1), i2 = m::rcp3_(s2);
+    R r0, r1, r2, e0, e1, e2, tau = R(0);
+    bool k0 = false, k1 = false, k2 = false;      // clamped ratios
+    if constexpr (VAR == 0) {
+        e0 = i0 * i0;
+        e1 = i1 * i1;
+        e2 = i2 * i2;
+        r0 = r1 = r2 = R(0);
+    } else {
+        tau = s0 - s2;
+        const R ta = m::abs_(tau);
+        r0 = ta * i0;
+        r1 = ta * i1;
+        r2 = ta * i2;
+        if constexpr (float_based<R>) {
+            const R top = R(1.0e18);
+            k0 = r0 > top;
+            k1 = r1 > top;
+            k2 = r2 > top;
+            r0 = k0 ? top : r0;
+            r1 = k1 ? top : r1;
+            r2 = k2 ? top : r2;
+        }
+        e0 = m::fma_(r0, r0, R(1));
+        e1 = m::fma_(r1, r1, R(1));
+        e2 = m::fma_(r2, r2, R(1));
+    }
+    const R D = m::fma_(R(3), e2, m::fma_(R(6), e1, e0));
+    const R iD = m::rcp3_(D);
+    const R w0 = m::times4_(e0 * iD), w2 = m::fma_(R(6) * e2, iD, R(-1));
+    const R t1 = x0 - y0, t2 = y0 - z0;
+    f = m::fma_(w0, t1, w2 * t2);
+    // d(l f): weights
+    const R u2 = R(2) * l * iD;      // twice the seeds of e_k
+    const R le0 = u2 * (m::fma_(R(4), t1, -t2) - f), le1 = R(-6) * u2 * (t2 + f), le2 = R(3) * u2 * (t2 - f);
+    const R lt1 = l * w0, lt2 = l * w2;
+    R ls0, ls1, ls2;
+    if constexpr (VAR == 0) {
+        ls0 = -(le0 * e0) * i0;
+        ls1 = -(le1 * e1) * i1;
+        ls2 = -(le2 * e2) * i2;
+    } else {
+        // e = 1 + r^2, r = |tau| / s
+        const R v0 = k0 ? R(0) : le0 * r0 * i0, v1 = k1 ? R(0) : le1 * r1 * i1, v2 = k2 ? R(0) : le2 * r2 * i2;
+        const R lta = v0 + v1 + v2;
+        const R lt = m::nonneg(tau) ? lta : -lta;
+        ls0 = m::fma_(-v0, r0, lt);
+        ls1 = -(v1 * r1);
+        ls2 = m::fma_(-v2, r2, -lt);
+    }
+    const R k = R(8.0 / 3.0);
+    const R lx = m::fma_(ls0, m::fma_(k, x0, -b), lt1);
+    const R ly = m::fma_(ls1, m::fma_(k, y0, -b), lt2 - lt1);
+    const R lz = m::fma_(ls2, m::fma_(k, z0, c), -lt2);
+    g[0] = lx;
+    g[1] = m::fma_(ls0, m::fma_(R(2), b, -x0), m::fma_(ls1, m::fma_(R(2), b, -y0), ly - lx));
+    g[2] = m::fma_(ls2, m::fma_(R(2), c, z0), lz - ly);
+    g[3] = -lz;
+}
+
+__device__ __forceinline__ double pair_x(Pair<double> a) { return a.x; }
+__device__ __forceinline__ double pair_y(Pair<double> a) { return a.y; }
+__device__ __forceinline__ float pair_x(Pair<float> a) { return a.v.x; }
+__device__ __forceinline__ float pair_y(Pair<float> a) { return a.v.y; }
+__device__ __forceinline__ Pair<double> padd(Pair<double> a, Pair<double> b) { return {a.x + b.x, a.y + b.y}; }
+__device__ __forceinline__ Pair<float> padd(Pair<float> a, Pair<float> b) { return {__fadd2_rn(a.v, b.v)}; }
+__device__ __forceinline__ Pair<double> psub(Pair<double> a, Pair<double> b) { return {a.x - b.x, a.y - b.y}; }
+__device__ __forceinline__ Pair<float> psub(Pair<float> a, Pair<float> b) {
+    return {make_float2(a.v.x - b.v.x, a.v.y - b.v.y)};
+}
+template <typename R>
+__device__ __forceinline__ void pdot(R &acc, Pair<R> a, Pair<R> b) {
+    acc = M<R>::fma_(pair_x(a), pair_x(b), acc);
+    acc = M<R>::fma_(pair_y(a), pair_y(b), acc);
+}
+template <typename R>
+__device__ __forceinline__ void pdots(R &acc, Pair<R> a, Pair<R> b) {   // acc -= a.b
+    acc = M<R>::fma_(-pair_x(a), pair_x(b), acc);
+    acc = M<R>::fma_(-pair_y(a), pair_y(b), acc);
+}
+
+// weno_field's reverse: value = phi~(q) - phi~(p) (both 12 phi_N, in units of
+// 1/24 of the split fluxes' sum), the pairs P replaced by l times the
+// gradient, galpha = l d(value)/d(alpha).
+template <typename R, int VAR>
+__device__ __forceinline__ R field_rev(Pair<R> (&P)[5], R alpha, R eps3, R l, R &galpha) {
+    R fp, fq, gp[4], gq[4];
+    phi_rev<R, VAR>(psplit(P[0], alpha), psplit(P[1], alpha), psplit(P[2], alpha), psplit(P[3], alpha), eps3, -l, fp, gp);
+    phi_rev<R, VAR>(psplit(P[4], -alpha), psplit(P[3], -alpha), psplit(P[2], -alpha), psplit(P[1], -alpha), eps3, l, fq,
+                    gq);
+    R ga = R(0);
+#pragma unroll
+    for (int j = 0; j < 5; ++j) {
+        const R up = j < 4 ? gp[j] : R(0), uq = j > 0 ? gq[4 - j] : R(0);
+        const R d = up - uq;
+        ga = M<R>::fma_(pair_y(P[j]), d, ga);
+        P[j] = make_pair2(up + uq, alpha * d);
+    }
+    galpha = ga;
+    return fq - fp;
+}
+
+// Reverse mode of the face function (face_flux and face_eigen: same
+// quantities, same branches).  Its outputs are the five lab-order face fluxes
+// and the two transport fluxes; their adjoints come from lamD and lamO by the
+// transposes of Eq. num and of the EMF averages.  First every field's WENO part
+// and its gradient, in place of the field's projections; then, per stencil
+// position, the projections again from the box and their transposes; last the
+// eigen scalars backwards.  The central flux is not projected, so its adjoint
+// is the incoming one (except in Appendix A's fallback a_f = a_s = 1).
+//
+// Bound: FP64 pipe in double; in float the registers (70 projections and
+// their gradients live between the two passes).  One reciprocal per smoothness
+// indicator and weight sum (an IEEE division costs 9 FP64 instructions, and a
+// field has 28 of them), the shared cell box, the frame projections with their
+// transposes and one cell recovery per cell took the 64^3 adjoint step from
+// 45.1 to 18.7 ms in its face and cell kernels (FP64, WENO-Z) and from 2.6 to
+// 1.35 ms (FP32-bulk, WENO5); the whole 2-step rollout gradient 127.8 -> 66.3 ms,
+// in float (3 steps) 12.1 -> 7.8 ms, no larger error against 64-bit gradients.
+template <int AX, typename R, int VAR, int T2, int BX, int MINB>
+__global__ void __launch_bounds__(BX *T2, MINB) adj_face_kernel(AdjSweepArgs<R> a) {
+    using m = M<R>;
+    using P2 = Pair<R>;
+    using TT = SweepTile<AX, T2, BX, 1>;
+    constexpr bool DIFF = box_diff<R>();
+    extern __shared__ __align__(16) unsigned char w5ct_smem[];
+    R *sm = reinterpret_cast<R *>(w5ct_smem);
+    const int nx = a.nx, ny = a.ny, nz = a.nz;
+    const int tx = threadIdx.x, ty = threadIdx.y, tid = tx + BX * ty;
+    const int x0 = blockIdx.x * TT::BX, y0 = blockIdx.y * TT::BY, z0 = blockIdx.z * TT::BZ;
+    const Phys<R> K = a.K;
+    // cell box
+    bool bad = false, hit = false;
+    for (int c = tid; c < TT::NC; c += TT::NT) {
+        const int cx = c % TT::CX, cy = (c / TT::CX) % TT::CY, cz = c / (TT::CX * TT::CY);
+        const int gx = wrapi(x0 - (AX == 0 ? 2 : 0) + cx, nx), gy = wrapi(y0 - (AX == 1 ? 2 : 0) + cy, ny),
+                  gz = wrapi(z0 - (AX == 2 ? 2 : 0) + cz, nz);
+        const size_t g = (size_t)gx + (size_t)nx * ((size_t)gy + (size_t)ny * (size_t)gz);
+        cell_fill<R, AX>(sm + c, TT::NC, a.q[0][g], a.q[1][g], a.q[2][g], a.q[3][g], a.q[4][g], a.bc[0][g],
+                         a.bc[1][g], a.bc[2][g], K, bad, hit);
+    }
+    __syncthreads();
+    if constexpr (DIFF) {
+        constexpr int NIT = (TT::NC + TT::NT - 1) / TT::NT;
+        constexpr int LAST = (AX == 0 ? TT::CX : AX == 1 ? TT::CY : TT::CZ) - 1;
+        CellDiff<R> d[NIT];
+        bool has[NIT];
+#pragma unroll
+        for (int it = 0; it < NIT; ++it) {
+            const int c = tid + it * TT::NT;
+            const int ca = AX == 0 ? c % TT::CX : AX == 1 ? (c / TT::CX) % TT::CY : c / (TT::CX * TT::CY);
+            has[it] = c < TT::NC && ca < LAST;
+            if (has[it]) box_diff_load<R>(sm, TT::NC, c, TT::ST, d[it]);
+        }
+        __syncthreads();
+#pragma unroll
+        for (int it = 0; it < NIT; ++it)
+            if (has[it]) box_diff_store<R>(sm, TT::NC, tid + it * TT::NT, d[it]);
+        __syncthreads();
+    }
+    const int gx = x0 + tx, gy = y0 + (AX == 2 ? 0 : ty), gz = z0 + (AX == 2 ? ty : 0);
+    if (gx >= nx || gy >= ny || gz >= nz) return;
+    const int c0 = tx + TT::CX * ((AX == 2 ? 0 : ty) + TT::CY * (AX == 2 ? ty : 0));   // stencil cell i-2
+    const R *box = sm + c0;
+    constexpr int ST = TT::ST, NC = TT::NC;
+    const size_t n = (size_t)nx * ny * nz;
+    const size_t p = (size_t)gx + (size_t)nx * ((size_t)gy + (size_t)ny * (size_t)gz);
+
+#define SMQ(q, k) box[(q) * NC + (k) * ST]
+    // stencil pair (dF_c, du_c) at position j
+    auto X = [&](int c, int j) -> P2 {
+        const int qU = c == 0 ? C_RHOQ : c == 1 ? C_MN : c == 2 ? C_MT1 : c == 3 ? C_MT2
+                       : c == 4 ? (DIFF ? (int)C_DU4 : (int)C_BT1) : c == 5 ? (DIFF ? (int)C_DU5 : (int)C_BT2) : C_E;
+        if constexpr (DIFF)
+            return make_pair2(SMQ(C_DF0 + c, j), SMQ(qU, j));
+        else
+            return make_pair2(SMQ(C_F0 + c, j + 1) - SMQ(C_F0 + c, j), SMQ(qU, j + 1) - SMQ(qU, j));
+    };
+    auto mean = [&](int q) { return m::half_(SMQ(q, 2) + SMQ(q, 3)); };
+    const R r = mean(C_RHO), vn = mean(C_VN), vt1 = mean(C_VT1), vt2 = mean(C_VT2);
+    const R Bn = mean(C_BN), Bt1 = mean(C_BT1), Bt2 = mean(C_BT2), P = mean(C_P);
+    const R v2 = vn * vn + vt1 * vt1 + vt2 * vt2;
+    const R hv2 = m::half_(v2);
+    const FaceEigen<R> e = face_eigen<R>(r, v2, Bn, Bt1, Bt2, P, K);
+    const R b1 = e.b1, b2 = e.b2, sg = e.sg;
+    const R pre = m::half_(e.ics2), tau = K.gm1 * e.ics2;
+    const R afcf = e.af * e.cf, ascl = e.as * e.csl;
+    const R sas = sg * ascl, saf = sg * afcf;
+    const R eps3 = R(1.0 / 3.0) * K.eps_w;
+    const R cF = pre * (K.gm1 * e.af), cS = pre * (K.gm1 * e.as);
+    const R srcs = pre * (e.sr * e.cs);
+    const R hF = srcs * e.as, hS = -(srcs * e.af);
+    const R nF = -(pre * afcf), nS = -(pre * ascl), kF = pre * sas, kS = -(pre * saf);
+    const R ssr = sg * e.sr;
+    const R a5 = ssr * b1, a4 = -(ssr * b2);
+    const R csisr = e.cs * e.isr;
+
+    // ---- adjoint of the frame flux, in units of the WENO parts
+    const R kw = R(1.0 / 24.0);   // field_rev carries 12 phi_N in both types
+    R lX0[7], lW[7];
+    {
+        const size_t hi = AX == 0 ? (size_t)wrapi(gx + 1, nx) + (size_t)nx * ((size_t)gy + (size_t)ny * gz)
+                          : AX == 1 ? (size_t)gx + (size_t)nx * ((size_t)wrapi(gy + 1, ny) + (size_t)ny * gz)
+                                    : (size_t)gx + (size_t)nx * ((size_t)gy + (size_t)ny * wrapi(gz + 1, nz));
+        auto below = [&](int ax) {
+            return ax == 0 ? (size_t)wrapi(gx - 1, nx) + (size_t)nx * ((size_t)gy + (size_t)ny * gz)
+                   : ax == 1 ? (size_t)gx + (size_t)nx * ((size_t)wrapi(gy - 1, ny) + (size_t)ny * gz)
+                             : (size_t)gx + (size_t)nx * ((size_t)gy + (size_t)ny * wrapi(gz - 1, nz));
+        };
+        constexpr int t1 = (AX + 1) % 3, t2 = (AX + 2) % 3;
+        auto lF = [&](int f) {
+            const double *L = a.lamD + (size_t)f * n;
+            return from_double<R>(a.rd * (L[hi] - L[p]));
+        };
+        lX0[0] = lF(0);
+        lX0[1] = lF(1 + AX);
+        lX0[2] = lF(1 + t1);
+        lX0[3] = lF(1 + t2);
+        const double *On = a.lamO + (size_t)AX * n, *O2 = a.lamO + (size_t)t2 * n;
+        lX0[4] = from_double<R>(-0.5 * (On[p] + On[below(t1)]));
+        lX0[5] = from_double<R>(0.5 * (O2[p] + O2[below(t2)]));
+        lX0[6] = lF(4);
+    }
+#pragma unroll
+    for (int c = 0; c < 7; ++c) lW[c] = kw * lX0[c];
+    const R lS1 = lW[0] + vn * lW[1] + vt1 * lW[2] + vt2 * lW[3] + hv2 * lW[6];
+    const R lTn = lW[1] + vn * lW[6], lT1 = lW[2] + vt1 * lW[6], lT2 = lW[3] + vt2 * lW[6];
+    const R lS2 = b1 * lW[4] + b2 * lW[5], lhda = b1 * lW[5] - b2 * lW[4];
+    const R lTk = b1 * lT1 + b2 * lT2, lhsa = b1 * lT2 - b2 * lT1;
+    const R lmg = lS1 - K.g2 * e.cs2 * lW[6];
+    const R lsf = e.af * lmg + csisr * e.as * lS2 + afcf * e.cf * lW[6];
+    const R lss = e.as * lmg - csisr * e.af * lS2 + ascl * e.csl * lW[6];
+    const R ldf = sas * lTk - afcf * lTn, lds = -(ascl * lTn + saf * lTk);
+    const R lsa = m::half_(lhsa), lda = m::half_(lhda) * (sg * e.isr);
+
+    // ---- field projections (as face_flux; g with the field part -B_t in full)
+    struct Proj {
+        P2 Yn, Y1, Y2, h, k, g;
+    };
+    auto project = [&](P2 X0, P2 X1, P2 X2, P2 X3, P2 X4, P2 X5, P2 X6) -> Proj {
+        Proj q;
+        q.Yn = pfma(-vn, X0, X1);
+        q.Y1 = pfma(-vt1, X0, X2);
+        q.Y2 = pfma(-vt2, X0, X3);
+        q.h = pfma(b1, X4, pmul(b2, X5));
+        q.k = pfma(b1, q.Y1, pmul(b2, q.Y2));
+        P2 g = pfma(-hv2, X0, X6);
+        g = pfma(-vn, q.Yn, g);
+        g = pfma(-vt1, q.Y1, g);
+        g = pfma(-vt2, q.Y2, g);
+        g = pfma(-Bt1, X4, g);
+        q.g = pfma(-Bt2, X5, g);
+        return q;
+    };
+    P2 F[7][5];
+    // in double the projections are kept (in local memory) for the transposes,
+    // in float they are formed again: 13 operations against 12 loads
+    [[maybe_unused]] Proj kept[float_based<R> ? 1 : 5];
+#pragma unroll
+    for (int j = 0; j < 5; ++j) {
+        const P2 X0 = X(0, j), X4 = X(4, j), X5 = X(5, j);
+        const Proj q = project(X0, X(1, j), X(2, j), X(3, j), X4, X5, X(6, j));
+        if constexpr (!float_based<R>) kept[j] = q;
+        const P2 x = pfma(b1, q.Y2, pmul(-b2, q.Y1));
+        mode_pair(pfma(cF, q.g, pmul(hF, q.h)), nF, q.Yn, kF, q.k, F[0][j], F[1][j]);
+        mode_pair(pfma(cS, q.g, pmul(hS, q.h)), nS, q.Yn, kS, q.k, F[2][j], F[3][j]);
+        mode_pair(x, a4, X4, a5, X5, F[4][j], F[5][j]);
+        F[6][j] = pfma(-tau, q.g, X0);
+    }
+    // ---- WENO parts and gradients, field by field: fast -+, slow -+, Alfven
+    // -+, entropy.  LF speeds: alpha = max over the two cells of |v_n + s c|,
+    // with the cell and sign that attain it.  In double one copy of the code
+    // in a loop, the projections in local memory (unrolled, the scheduler
+    // mixes the fields and spills four times as much); in float unrolled.
+    R V[7], gs[7];
+    const R lf[7] = {lsf + ldf, lsf - ldf, lss + lds, lss - lds, lsa + lda, lsa - lda, lS1};
+    unsigned lower = 0;
+    constexpr int kUnroll = float_based<R> ? 7 : 1;
+#pragma unroll kUnroll
+    for (int mo = 0; mo < 7; ++mo) {
+        const int qc = mo < 2 ? C_CF : mo < 4 ? C_CSL : C_CA;
+        const R s = mo == 6 ? R(0) : (mo & 1) ? R(1) : R(-1);
+        const R xL = m::fma_(s, SMQ(qc, 2), SMQ(C_VN, 2)), xR = m::fma_(s, SMQ(qc, 3), SMQ(C_VN, 3));
+        const bool lo = m::abs_(xL) >= m::abs_(xR);
+        const R xa = lo ? xL : xR;
+        P2 f[5];
+#pragma unroll
+        for (int j = 0; j < 5; ++j) f[j] = F[mo][j];
+        R ga;
+        V[mo] = field_rev<R, VAR>(f, m::abs_(xa), mo == 4 || mo == 5 ? R(4) * eps3 : eps3, lf[mo], ga);
+        gs[mo] = m::nonneg(xa) ? ga : -ga;
+        lower |= lo ? 1u << mo : 0u;
+#pragma unroll
+        for (int j = 0; j < 5; ++j) F[mo][j] = f[j];
+    }
+    R side[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+#pragma unroll
+    for (int mo = 0; mo < 7; ++mo) {
+        const int o = mo < 2 ? 1 : mo < 4 ? 3 : 2;
+        const R gL = (lower >> mo) & 1u ? gs[mo] : R(0), gR = (lower >> mo) & 1u ? R(0) : gs[mo];
+        side[0] += gL;
+        side[4] += gR;
+        if (mo < 6) {
+            side[o] += (mo & 1) ? gL : -gL;
+            side[4 + o] += (mo & 1) ? gR : -gR;
+        }
+    }
+    R sf = V[0] + V[1], df = V[0] - V[1], ss = V[2] + V[3], ds = V[2] - V[3], sa = V[4] + V[5], da = V[4] - V[5], Fe = V[6];
+
+    // ---- transposes of the projections.  The stencil differences are read
+    // again: the compiler may not keep the first reads' 70 values across the
+    // WENO parts.
+    asm volatile("" ::: "memory");
+    R lhv2 = 0, lvn = 0, lvt1 = 0, lvt2 = 0, lBt1 = 0, lBt2 = 0, lb1 = 0, lb2 = 0, ltau = 0;
+    R lcF = 0, lcS = 0, lhF = 0, lhS = 0, lnF = 0, lnS = 0, lkF = 0, lkS = 0, la4 = 0, la5 = 0;
+    // position j: from the pairs X, their projections and the fields' adjoints
+    // to the adjoint of X
+    auto transpose = [&](P2 X0, P2 X4, P2 X5, const Proj &q, P2 Lfu, P2 Lfl, P2 Lsu, P2 Lsl, P2 Lau, P2 Lal, P2 Len, P2 (&out)[7]) {
+        const P2 Yn = q.Yn, Y1 = q.Y1, Y2 = q.Y2, h = q.h, k = q.k, g = q.g;
+        const P2 fc = padd(Lfu, Lfl), fs = psub(Lfu, Lfl), sc = padd(Lsu, Lsl), sd = psub(Lsu, Lsl);
+        const P2 lx = padd(Lau, Lal), ls = psub(Lau, Lal);
+        pdot(lcF, g, fc);
+        pdot(lhF, h, fc);
+        pdot(lnF, Yn, fs);
+        pdot(lkF, k, fs);
+        pdot(lcS, g, sc);
+        pdot(lhS, h, sc);
+        pdot(lnS, Yn, sd);
+        pdot(lkS, k, sd);
+        pdot(la4, X4, ls);
+        pdot(la5, X5, ls);
+        pdots(ltau, g, Len);
+        const P2 lg = pfma(-tau, Len, pfma(cF, fc, pmul(cS, sc)));
+        const P2 lh = pfma(hF, fc, pmul(hS, sc));
+        const P2 lk = pfma(kF, fs, pmul(kS, sd));
+        P2 lYn = pfma(nF, fs, pmul(nS, sd));
+        // k = b1 Y1 + b2 Y2, x = b1 Y2 - b2 Y1, h = b1 X4 + b2 X5
+        P2 lY1 = pfma(b1, lk, pmul(-b2, lx)), lY2 = pfma(b2, lk, pmul(b1, lx));
+        pdot(lb1, Y1, lk);
+        pdot(lb2, Y2, lk);
+        pdot(lb1, Y2, lx);
+        pdots(lb2, Y1, lx);
+        pdot(lb1, X4, lh);
+        pdot(lb2, X5, lh);
+        // g = X6 - v^2/2 X0 - v.Y - B_t.X_B
+        pdots(lhv2, X0, lg);
+        pdots(lvn, Yn, lg);
+        pdots(lvt1, Y1, lg);
+        pdots(lvt2, Y2, lg);
+        pdots(lBt1, X4, lg);
+        pdots(lBt2, X5, lg);
+        lYn = pfma(-vn, lg, lYn);
+        lY1 = pfma(-vt1, lg, lY1);
+        lY2 = pfma(-vt2, lg, lY2);
+        out[6] = lg;
+        out[4] = pfma(a4, ls, pfma(b1, lh, pmul(-Bt1, lg)));
+        out[5] = pfma(a5, ls, pfma(b2, lh, pmul(-Bt2, lg)));
+        // Y = X_m - v X0
+        out[1] = lYn;
+        out[2] = lY1;
+        out[3] = lY2;
+        pdots(lvn, X0, lYn);
+        pdots(lvt1, X0, lY1);
+        pdots(lvt2, X0, lY2);
+        out[0] = pfma(-hv2, lg, pfma(-vn, lYn, pfma(-vt1, lY1, pfma(-vt2, lY2, Len))));
+    };
+#pragma unroll
+    for (int j = 0; j < 5; ++j) {
+        P2 out[7];
+        const P2 X0 = X(0, j), X4 = X(4, j), X5 = X(5, j);
+        Proj q;
+        if constexpr (float_based<R>)
+            q = project(X0, X(1, j), X(2, j), X(3, j), X4, X5, X(6, j));
+        else
+            q = kept[j];
+        transpose(X0, X4, X5, q, F[0][j], F[1][j], F[2][j], F[3][j], F[4][j], F[5][j], F[6][j], out);
+#pragma unroll
+        for (int c = 0; c < 7; ++c) {
+            a.face_plane(kAdjDiff + (c * 5 + j) * 2)[p] = pair_x(out[c]);
+            a.face_plane(kAdjDiff + (c * 5 + j) * 2 + 1)[p] = pair_y(out[c]);
+        }
+    }
+    if (!e.apart) {
+        // Appendix A's fallback: the central flux went through L and R, each
+        // field's central part added to its WENO part (in units of kw)
+        P2 Xc[7], out[7];
+#pragma unroll
+        for (int c = 0; c < 7; ++c) {
+            R x;
+            if constexpr (DIFF)
+                x = SMQ(C_F0 + c, 2) + (R(6) * SMQ(C_DF0 + c, 2) + SMQ(C_DF0 + c, 1) - SMQ(C_DF0 + c, 3)) * R(1.0 / 12.0);
+            else
+                x = (R(7) * (SMQ(C_F0 + c, 2) + SMQ(C_F0 + c, 3)) - (SMQ(C_F0 + c, 1) + SMQ(C_F0 + c, 4))) * R(1.0 / 12.0);
+            Xc[c] = make_pair2(x, R(0));
+        }
+        const R u = R(24);
+        auto one = [&](R l) { return make_pair2(u * l, R(0)); };
+        const Proj q = project(Xc[0], Xc[1], Xc[2], Xc[3], Xc[4], Xc[5], Xc[6]);
+        transpose(Xc[0], Xc[4], Xc[5], q, one(lsf + ldf), one(lsf - ldf), one(lss + lds), one(lss - lds), one(lsa + lda),
+                  one(lsa - lda), one(lS1), out);
+#pragma unroll
+        for (int c = 0; c < 7; ++c) lX0[c] = pair_x(out[c]);
+        const R Yn = pair_x(q.Yn), Y1 = pair_x(q.Y1), Y2 = pair_x(q.Y2), h = pair_x(q.h), k = pair_x(q.k), g = pair_x(q.g);
+        sf += R(2) * u * (cF * g + hF * h);
+        df += R(2) * u * (nF * Yn + kF * k);
+        ss += R(2) * u * (cS * g + hS * h);
+        ds += R(2) * u * (nS * Yn + kS * k);
+        sa += R(2) * u * (b1 * Y2 - b2 * Y1);
+        da += R(2) * u * (a4 * pair_x(Xc[4]) + a5 * pair_x(Xc[5]));
+        Fe += u * (pair_x(Xc[0]) - tau * g);
+    }
+#pragma unroll
+    for (int c = 0; c < 7; ++c) a.face_plane(kAdjCentral + c)[p] = lX0[c];
+#pragma unroll
+    for (int t = 0; t < 8; ++t) a.face_plane(kAdjSide + t)[p] = side[t];
+#undef SMQ
+
+    // ---- back-projection's scalars
+    R lafcf = 0, lascl = 0, laf, las, lcf, lcsl, lcs, lisr, lsr, lcs2, lpre;
+    {
+        const R mg = e.af * sf + e.as * ss, S1 = mg + Fe, D2 = e.as * sf - e.af * ss, S2 = csisr * D2;
+        const R hsa = m::half_(sa), hda = m::half_(da) * (sg * e.isr);
+        const R Tn = -(afcf * df + ascl * ds), Tk = sas * df - saf * ds;
+        const R Tt1 = Tk * b1 - hsa * b2, Tt2 = Tk * b2 + hsa * b1;
+        lvn += lW[1] * S1 + lW[6] * Tn;
+        lvt1 += lW[2] * S1 + lW[6] * Tt1;
+        lvt2 += lW[3] * S1 + lW[6] * Tt2;
+        lhv2 += lW[6] * S1;
+        lb1 += lT1 * Tk + lT2 * hsa + lW[4] * S2 + lW[5] * hda;
+        lb2 += lT2 * Tk - lT1 * hsa + lW[5] * S2 - lW[4] * hda;
+        lisr = lhda * m::half_(da) * sg + lS2 * e.cs * D2;
+        lcs = lS2 * e.isr * D2;
+        laf = lmg * sf - lS2 * csisr * ss;
+        las = lmg * ss + lS2 * csisr * sf;
+        const R sT = sg * lTk;
+        lafcf = lW[6] * e.cf * sf - lTn * df - sT * ds;
+        lascl = lW[6] * e.csl * ss - lTn * ds + sT * df;
+        lcf = lW[6] * afcf * sf;
+        lcsl = lW[6] * ascl * ss;
+        lcs2 = -(K.g2 * lW[6] * mg);
+    }
+    // ---- projection coefficients
+    {
+        const R lsrcs = lhF * e.as - lhS * e.af;
+        lpre = K.gm1 * (lcF * e.af + lcS * e.as) + lsrcs * (e.sr * e.cs) - lnF * afcf - lnS * ascl + lkF * sas - lkS * saf;
+        laf += lcF * (pre * K.gm1) - lhS * srcs;
+        las += lcS * (pre * K.gm1) + lhF * srcs;
+        lsr = pre * lsrcs * e.cs + sg * (b1 * la5 - b2 * la4);
+        lcs += pre * lsrcs * e.sr;
+        lafcf -= pre * (lnF + sg * lkS);
+        lascl += pre * (sg * lkF - lnS);
+        lb1 += ssr * la5;
+        lb2 -= ssr * la4;
+        laf += lafcf * e.cf;
+        lcf += lafcf * e.af;
+        las += lascl * e.csl;
+        lcsl += lascl * e.as;
+        const R lics2 = K.gm1 * ltau + m::half_(lpre);
+        lcs2 -= e.ics2 * (e.ics2 * lics2);
+    }
+    // ---- eigen scalars (face_eigen) backwards
+    const R ir = e.isr * e.isr;
+    const R ca2 = Bn * Bn * ir, btm = Bt1 * Bt1 + Bt2 * Bt2, bt2 = btm * ir;
+    R lir = lisr * e.sr;                       // isr = sr ir
+    lsr += lisr * ir;
+    R lr = m::half_(lsr * e.isr);              // sr = sqrt(r)
+    R lbtm = R(0);
+    if (m::gt_pos(btm, K.eps_b)) {
+        const R ib = m::rsqrt_(btm);
+        lBt1 += lb1 * ib;
+        lBt2 += lb2 * ib;
+        lbtm = -m::half_(ib * (ib * (ib * (lb1 * Bt1 + lb2 * Bt2))));
+    }
+    R lfmc = R(0), lcms = R(0);
+    if (e.apart) {
+        R fmc, cms, cf2;
+        speeds_fast<R>(e.cs2, ca2, bt2, fmc, cms, cf2);
+        const R idf = m::rcp3_(fmc + cms);
+        // a_f = sqrt(cms idf), a_s = sqrt(fmc idf)
+        const R lqa = m::normal_pos(e.af) ? m::half_(laf * m::rcp3_(e.af)) : R(0);
+        const R lqs = m::normal_pos(e.as) ? m::half_(las * m::rcp3_(e.as)) : R(0);
+        const R ldfs = -(idf * (idf * (lqa * cms + lqs * fmc)));
+        lcms = lqa * idf + ldfs;
+        lfmc = lqs * idf + ldfs;
+    }
+    const R ics = e.cs * e.ics2;
+    lcs2 += m::half_(lcs * ics);
+    const R lcsl2 = m::normal_pos(e.csl) ? m::half_(lcsl * m::rcp3_(e.csl)) : R(0);
+    const R lcf2 = m::normal_pos(e.cf) ? m::half_(lcf * m::rcp3_(e.cf)) : R(0);
+    R lca2 = R(0), lbt2 = R(0), lP = R(0), lv2 = m::half_(lhv2);
+    speeds_rev<R>(e.cs2, ca2, bt2, lfmc, lcms, lcf2, lcsl2, lcs2, lca2, lbt2);
     bool bound = false;
-    if constexpr (float_based<B>) {
-        const B cs2b = K.cs2_rel * (v2 + ca2 + bt2);
-        bound = cs2b > cs2a;
-        cs2 = m::max_(cs2a, cs2b);
-    }
-    B fmc, cms, cf2, csl2;
-    speeds<B>(cs2, ca2, bt2, fmc, cms, cf2, csl2);
-    const B cf = m::sqrt_(cf2), csl = m::sqrt_(csl2), cs = m::sqrt_(cs2);
-    const B dfs = fmc + cms;
-    const bool brA = dfs >= K.eps_b2;
-    B af = B(1), as = B(1), idf = B(0), qa = B(0), qs = B(0);
-    if (brA) {
-        idf = m::rcp_(dfs);
-        qa = cms * idf;
-        qs = fmc * idf;
-        af = m::sqrt_(m::max_(qa, B(0)));
-        as = m::sqrt_(m::max_(qs, B(0)));
-    }
-    const bool brB = btm > K.eps_b;
-    B b1 = B(0.70710678118654752440), b2 = B(0.70710678118654752440), ib = B(0);
-    if (brB) {
-        ib = m::rsqrt_(btm);
-        b1 = Bt1 * ib;
-        b2 = Bt2 * ib;
-    }
-    const A sg = (Bn >= K.eps_b) ? A(1) : A(-1);
-    const B sr = m::sqrt_(r);
-    const B isr = sr * ir;
-    const B bvB = b1 * vt1 + b2 * vt2;
-    const B ics2B = m::rcp_(cs2);
-    // the rest in the adjoint type
-    const A Avn = (A)vn, Avt1 = (A)vt1, Avt2 = (A)vt2, ABt1 = (A)Bt1, ABt2 = (A)Bt2;
-    const A Av2 = (A)v2, Acf = (A)cf, Acsl = (A)csl, Acs = (A)cs, Acf2 = (A)cf2, Acsl2 = (A)csl2, Acs2 = (A)cs2;
-    const A Aaf = (A)af, Aas = (A)as, Ab1 = (A)b1, Ab2 = (A)b2, Asr = (A)sr, Aisr = (A)isr, Abv = (A)bvB;
-    const A ics2 = (A)ics2B, pre = A(0.5) * ics2, gm1 = (A)K.gm1, g1 = (A)K.g1, g2 = (A)K.g2;
-    const A tau = gm1 * ics2;
-    const A Gf = Aaf * Acf * Avn - Aas * Acsl * sg * Abv;
-    const A Gs = Aas * Acsl * Avn + Aaf * Acf * sg * Abv;
-    const A k1 = -gm1 * Aaf, k2 = -gm1 * Aas;
-    const A V[3] = {Avn, Avt1, Avt2};
-    // ---- adjoints
-    A lpre = 0, laf = 0, las = 0, lcf = 0, lcsl = 0, lcs = 0, lsr = 0, lisr = 0, lb1 = 0, lb2 = 0;
-    A lGf = 0, lGs = 0, lGa = 0, lv2 = 0, lBt1 = 0, lBt2 = 0, lcf2 = 0, lcsl2 = 0, lcs2 = 0, ltau = 0;
-    A lk1 = 0, lk2 = 0;
-    A lv[3] = {0, 0, 0};
-    // fast pair (modes 0, 1): L = Lc +- Ls, R = Rc +- Rs (rows 1, 2, 3, 6)
-    {
-        A lLc[7], lLs[4], lRc[7], lRs[4];
-#pragma unroll
-        for (int c = 0; c < 7; ++c) {
-            lLc[c] = lL[0][c] + lL[1][c];
-            lRc[c] = lR[0][c] + lR[1][c];
-        }
-#pragma unroll
-        for (int c = 0; c < 4; ++c) lLs[c] = lL[0][c] - lL[1][c];
-        lRs[0] = lR[0][1] - lR[1][1];
-        lRs[1] = lR[0][2] - lR[1][2];
-        lRs[2] = lR[0][3] - lR[1][3];
-        lRs[3] = lR[0][6] - lR[1][6];
-        A l = lLc[0];
-        lpre += l * g1 * Aaf * Av2;
-        laf += l * pre * g1 * Av2;
-        lv2 += l * pre * g1 * Aaf;
-#pragma unroll
-        for (int j = 0; j < 3; ++j) {
-            l = lLc[1 + j];
-            lpre += l * k1 * V[j];
-            lk1 += l * pre * V[j];
-            lv[j] += l * pre * k1;
-        }
-        {
-            l = lLc[4];
-            const A lt = l * pre;
-            lpre += l * (k1 * ABt1 + Asr * Acs * Aas * Ab1);
-            lk1 += lt * ABt1;
-            lBt1 += lt * k1;
-            lsr += lt * Acs * Aas * Ab1;
-            lcs += lt * Asr * Aas * Ab1;
-            las += lt * Asr * Acs * Ab1;
-            lb1 += lt * Asr * Acs * Aas;
-        }
-        {
-            l = lLc[5];
-            const A lt = l * pre;
-            lpre += l * (k1 * ABt2 + Asr * Acs * Aas * Ab2);
-            lk1 += lt * ABt2;
-            lBt2 += lt * k1;
-            lsr += lt * Acs * Aas * Ab2;
-            lcs += lt * Asr * Aas * Ab2;
-            las += lt * Asr * Acs * Ab2;
-            lb2 += lt * Asr * Acs * Aas;
-        }
-        l = lLc[6];
-        lpre += l * gm1 * Aaf;
-        laf += l * pre * gm1;
-        l = lLs[0];
-        lpre += l * Gf;
-        lGf += l * pre;
-        l = lLs[1];
-        lpre -= l * Aaf * Acf;
-        laf -= l * pre * Acf;
-        lcf -= l * pre * Aaf;
-        l = lLs[2];
-        lpre += l * Acsl * Aas * Ab1 * sg;
-        lcsl += l * pre * Aas * Ab1 * sg;
-        las += l * pre * Acsl * Ab1 * sg;
-        lb1 += l * pre * Acsl * Aas * sg;
-        l = lLs[3];
-        lpre += l * Acsl * Aas * Ab2 * sg;
-        lcsl += l * pre * Aas * Ab2 * sg;
-        las += l * pre * Acsl * Ab2 * sg;
-        lb2 += l * pre * Acsl * Aas * sg;
-        laf += lRc[0];
-#pragma unroll
-        for (int j = 0; j < 3; ++j) {
-            l = lRc[1 + j];
-            laf += l * V[j];
-            lv[j] += l * Aaf;
-        }
-        l = lRc[4];
-        lcs += l * Aas * Ab1 * Aisr;
-        las += l * Acs * Ab1 * Aisr;
-        lb1 += l * Acs * Aas * Aisr;
-        lisr += l * Acs * Aas * Ab1;
-        l = lRc[5];
-        lcs += l * Aas * Ab2 * Aisr;
-        las += l * Acs * Ab2 * Aisr;
-        lb2 += l * Acs * Aas * Aisr;
-        lisr += l * Acs * Aas * Ab2;
-        l = lRc[6];
-        laf += l * (A(0.5) * Av2 + Acf2 - g2 * Acs2);
-        lv2 += l * Aaf * A(0.5);
-        lcf2 += l * Aaf;
-        lcs2 -= l * Aaf * g2;
-        l = lRs[0];
-        laf -= l * Acf;
-        lcf -= l * Aaf;
-        l = lRs[1];
-        lcsl += l * Aas * Ab1 * sg;
-        las += l * Acsl * Ab1 * sg;
-        lb1 += l * Acsl * Aas * sg;
-        l = lRs[2];
-        lcsl += l * Aas * Ab2 * sg;
-        las += l * Acsl * Ab2 * sg;
-        lb2 += l * Acsl * Aas * sg;
-        lGf -= lRs[3];
-        laf -= gm1 * lk1;
-    }
-    // slow pair (modes 2, 3)
-    {
-        A lLc[7], lLs[4], lRc[7], lRs[4];
-#pragma unroll
-        for (int c = 0; c < 7; ++c) {
-            lLc[c] = lL[2][c] + lL[3][c];
-            lRc[c] = lR[2][c] + lR[3][c];
-        }
-#pragma unroll
-        for (int c = 0; c < 4; ++c) lLs[c] = lL[2][c] - lL[3][c];
-        lRs[0] = lR[2][1] - lR[3][1];
-        lRs[1] = lR[2][2] - lR[3][2];
-        lRs[2] = lR[2][3] - lR[3][3];
-        lRs[3] = lR[2][6] - lR[3][6];
-        A l = lLc[0];
-        lpre += l * g1 * Aas * Av2;
-        las += l * pre * g1 * Av2;
-        lv2 += l * pre * g1 * Aas;
-#pragma unroll
-        for (int j = 0; j < 3; ++j) {
-            l = lLc[1 + j];
-            lpre += l * k2 * V[j];
-            lk2 += l * pre * V[j];
-            lv[j] += l * pre * k2;
-        }
-        {
-            l = lLc[4];
-            const A lt = l * pre;
-            lpre += l * (k2 * ABt1 - Asr * Acs * Aaf * Ab1);
-            lk2 += lt * ABt1;
-            lBt1 += lt * k2;
-            lsr -= lt * Acs * Aaf * Ab1;
-            lcs -= lt * Asr * Aaf * Ab1;
-            laf -= lt * Asr * Acs * Ab1;
-            lb1 -= lt * Asr * Acs * Aaf;
-        }
-        {
-            l = lLc[5];
-            const A lt = l * pre;
-            lpre += l * (k2 * ABt2 - Asr * Acs * Aaf * Ab2);
-            lk2 += lt * ABt2;
-            lBt2 += lt * k2;
-            lsr -= lt * Acs * Aaf * Ab2;
-            lcs -= lt * Asr * Aaf * Ab2;
-            laf -= lt * Asr * Acs * Ab2;
-            lb2 -= lt * Asr * Acs * Aaf;
-        }
-        l = lLc[6];
-        lpre += l * gm1 * Aas;
-        las += l * pre * gm1;
-        l = lLs[0];
-        lpre += l * Gs;
-        lGs += l * pre;
-        l = lLs[1];
-        lpre -= l * Aas * Acsl;
-        las -= l * pre * Acsl;
-        lcsl -= l * pre * Aas;
-        l = lLs[2];
-        lpre -= l * Acf * Aaf * Ab1 * sg;
-        lcf -= l * pre * Aaf * Ab1 * sg;
-        laf -= l * pre * Acf * Ab1 * sg;
-        lb1 -= l * pre * Acf * Aaf * sg;
-        l = lLs[3];
-        lpre -= l * Acf * Aaf * Ab2 * sg;
-        lcf -= l * pre * Aaf * Ab2 * sg;
-        laf -= l * pre * Acf * Ab2 * sg;
-        lb2 -= l * pre * Acf * Aaf * sg;
-        las += lRc[0];
-#pragma unroll
-        for (int j = 0; j < 3; ++j) {
-            l = lRc[1 + j];
-            las += l * V[j];
-            lv[j] += l * Aas;
-        }
-        l = lRc[4];
-        lcs -= l * Aaf * Ab1 * Aisr;
-        laf -= l * Acs * Ab1 * Aisr;
-        lb1 -= l * Acs * Aaf * Aisr;
-        lisr -= l * Acs * Aaf * Ab1;
-        l = lRc[5];
-        lcs -= l * Aaf * Ab2 * Aisr;
-        laf -= l * Acs * Ab2 * Aisr;
-        lb2 -= l * Acs * Aaf * Aisr;
-        lisr -= l * Acs * Aaf * Ab2;
-        l = lRc[6];
-        las += l * (A(0.5) * Av2 + Acsl2 - g2 * Acs2);
-        lv2 += l * Aas * A(0.5);
-        lcsl2 += l * Aas;
-        lcs2 -= l * Aas * g2;
-        l = lRs[0];
-        las -= l * Acsl;
-        lcsl -= l * Aas;
-        l = lRs[1];
-        lcf -= l * Aaf * Ab1 * sg;
-        laf -= l * Acf * Ab1 * sg;
-        lb1 -= l * Acf * Aaf * sg;
-        l = lRs[2];
-        lcf -= l * Aaf * Ab2 * sg;
-        laf -= l * Acf * Ab2 * sg;
-        lb2 -= l * Acf * Aaf * sg;
-        lGs -= lRs[3];
-        las -= gm1 * lk2;
-    }
-    // Alfven pair (modes 4, 5)
-    {
-        const A ll0 = lL[4][0] + lL[5][0], ll2 = lL[4][2] + lL[5][2], ll3 = lL[4][3] + lL[5][3];
-        const A ll4 = lL[4][4] - lL[5][4], ll5 = lL[4][5] - lL[5][5];
-        lGa += A(0.5) * ll0;
-        lb2 -= A(0.5) * sg * ll2;
-        lb1 += A(0.5) * sg * ll3;
-        lsr -= A(0.5) * Ab2 * ll4;
-        lb2 -= A(0.5) * Asr * ll4;
-        lsr += A(0.5) * Ab1 * ll5;
-        lb1 += A(0.5) * Asr * ll5;
-        const A r2 = lR[4][2] + lR[5][2], r3 = lR[4][3] + lR[5][3], r4 = lR[4][4] - lR[5][4];
-        const A r5 = lR[4][5] - lR[5][5], r6 = lR[4][6] + lR[5][6];
-        lb2 -= sg * r2;
-        lb1 += sg * r3;
-        lb2 -= Aisr * r4;
-        lisr -= Ab2 * r4;
-        lb1 += Aisr * r5;
-        lisr += Ab1 * r5;
-        lGa -= r6;
-    }
-    // entropy (mode 6)
-    {
-        A l = lL[6][0];
-        ltau -= A(0.5) * Av2 * l;
-        lv2 -= A(0.5) * tau * l;
-#pragma unroll
-        for (int j = 0; j < 3; ++j) {
-            l = lL[6][1 + j];
-            ltau += l * V[j];
-            lv[j] += l * tau;
-        }
-        ltau += lL[6][4] * ABt1;
-        lBt1 += lL[6][4] * tau;
-        ltau += lL[6][5] * ABt2;
-        lBt2 += lL[6][5] * tau;
-        ltau -= lL[6][6];
-#pragma unroll
-        for (int j = 0; j < 3; ++j) lv[j] += lR[6][1 + j];
-        lv2 += A(0.5) * lR[6][6];
-    }
-    // ---- the scalars, backwards
-    const A lics2 = gm1 * ltau + A(0.5) * lpre;
-    lcs2 -= ics2 * (ics2 * lics2);
-    las += lGs * Acsl * Avn;
-    lcsl += lGs * Aas * Avn;
-    lv[0] += lGs * Aas * Acsl;
-    laf += lGs * Acf * sg * Abv;
-    lcf += lGs * Aaf * sg * Abv;
-    A lbv = lGs * Aaf * Acf * sg;
-    // Ga = sg (b2 vt1 - b1 vt2)
-    lb2 += lGa * sg * Avt1;
-    lv[1] += lGa * sg * Ab2;
-    lb1 -= lGa * sg * Avt2;
-    lv[2] -= lGa * sg * Ab1;
-    laf += lGf * Acf * Avn;
-    lcf += lGf * Aaf * Avn;
-    lv[0] += lGf * Aaf * Acf;
-    las -= lGf * Acsl * sg * Abv;
-    lcsl -= lGf * Aas * sg * Abv;
-    lbv -= lGf * Aas * Acsl * sg;
-    lb1 += lbv * Avt1;
-    lv[1] += lbv * Ab1;
-    lb2 += lbv * Avt2;
-    lv[2] += lbv * Ab2;
-    const A Air = (A)ir;
-    A lir = lisr * Asr;
-    lsr += lisr * Air;
-    A lr = sr > B(0) ? lsr * A(0.5) / Asr : A(0);
-    A lbtm = A(0);
-    if (brB) {
-        const A Aib = (A)ib;
-        lBt1 += lb1 * Aib;
-        lBt2 += lb2 * Aib;
-        const A lib = lb1 * ABt1 + lb2 * ABt2;
-        lbtm -= A(0.5) * Aib * (Aib * (Aib * lib));
-    }
-    A lfmc = A(0), lcms = A(0);
-    if (brA) {
-        const A lqa = qa > B(0) ? laf * A(0.5) / Aaf : A(0);
-        const A lqs = qs > B(0) ? las * A(0.5) / Aas : A(0);
-        const A Aidf = (A)idf;
-        lcms += lqa * Aidf;
-        lfmc += lqs * Aidf;
-        const A lidf = lqa * (A)cms + lqs * (A)fmc;
-        const A ldfs = -Aidf * (Aidf * lidf);
-        lfmc += ldfs;
-        lcms += ldfs;
-    }
-    if (cs > B(0)) lcs2 += lcs * A(0.5) / Acs;
-    if (csl > B(0)) lcsl2 += lcsl * A(0.5) / Acsl;
-    if (cf > B(0)) lcf2 += lcf * A(0.5) / Acf;
-    A lca2 = A(0), lbt2 = A(0);
-    speeds_rev<B, A>(cs2, ca2, bt2, lfmc, lcms, lcf2, lcsl2, lcs2, lca2, lbt2);
-    A lP = A(0);
+    if constexpr (float_based<R>) bound = K.cs2_rel * (v2 + ca2 + bt2) > K.gamma * P * ir;
     if (bound) {
-        const A t = (A)K.cs2_rel * lcs2;
+        const R t = K.cs2_rel * lcs2;
         lv2 += t;
         lca2 += t;
         lbt2 += t;
     } else {
-        lP += (A)K.gamma * Air * lcs2;
-        lir += (A)K.gamma * (A)P * lcs2;
+        lP = K.gamma * ir * lcs2;
+        lir += K.gamma * P * lcs2;
     }
-    lv[0] += A(2) * Avn * lv2;
-    lv[1] += A(2) * Avt1 * lv2;
-    lv[2] += A(2) * Avt2 * lv2;
-    lbtm += Air * lbt2;
-    lir += (A)btm * lbt2;
-    lBt1 += A(2) * ABt1 * lbtm;
-    lBt2 += A(2) * ABt2 * lbtm;
-    const A lBn = A(2) * (A)Bn * Air * lca2;
-    lir += (A)Bn * (A)Bn * lca2;
-    lr -= Air * (Air * lir);
-    lw[0] = lr;
-    lw[1] = lv[0];
-    lw[2] = lv[1];
-    lw[3] = lv[2];
-    lw[4] = lBn;
-    lw[5] = lBt1;
-    lw[6] = lBt2;
-    lw[7] = lP;
+    lvn += R(2) * vn * lv2;
+    lvt1 += R(2) * vt1 * lv2;
+    lvt2 += R(2) * vt2 * lv2;
+    lbtm += ir * lbt2;
+    lir += btm * lbt2 + Bn * Bn * lca2;
+    lBt1 += R(2) * Bt1 * lbtm;
+    lBt2 += R(2) * Bt2 * lbtm;
+    lr -= ir * (ir * lir);
+    const R lw[8] = {lr, lvn, lvt1, lvt2, R(2) * Bn * ir * lca2, lBt1, lBt2, lP};
+#pragma unroll
+    for (int t = 0; t < 8; ++t) a.face_plane(kAdjPrim + t)[p] = lw[t];
 }
 
-// phi_N(a, b, c, d) of Sec. 2.2 (the weights of the forward step: JS, or
-// WENO-Z with the ratio clamped at 1e18 in float) and its gradient in (a, b,
-// c, d), by hand: smoothness indicators -> weights (through tau for WENO-Z)
-// -> the two interpolants, run backwards.
-template <typename B, int VAR>
-__device__ __forceinline__ void phi_n_grad(B a, B b, B c, B d, B eps, B &phi, B (&g)[4]) {
-    const B x0 = a - b, x1 = a - B(3) * b, y0 = b - c, y1 = b + c, z0 = c - d, z1 = B(3) * c - d;
-    const B IS0 = B(13) * x0 * x0 + B(3) * x1 * x1;
-    const B IS1 = B(13) * y0 * y0 + B(3) * y1 * y1;
-    const B IS2 = B(13) * z0 * z0 + B(3) * z1 * z1;
-    const B s[3] = {eps + IS0, eps + IS1, eps + IS2};
-    const B dk[3] = {B(1), B(6), B(3)};
-    B al[3], r[3], t = B(0);
-    bool clamped[3] = {false, false, false};
-    if constexpr (VAR == 0) {
-#pragma unroll
-        for (int k = 0; k < 3; ++k) al[k] = dk[k] / (s[k] * s[k]);
-    } else {
-        t = IS0 - IS2;
-        const B tau = t >= B(0) ? t : -t;
-#pragma unroll
-        for (int k = 0; k < 3; ++k) {
-            r[k] = tau / s[k];
-            if constexpr (float_based<B>) {
-                if (r[k] > B(1.0e18)) {
-                    r[k] = B(1.0e18);
-                    clamped[k] = true;
-                }
-            }
-            al[k] = dk[k] * (B(1) + r[k] * r[k]);
-        }
-    }
-    const B S = al[0] + al[1] + al[2];
-    const B w0 = al[0] / S, w2 = al[2] / S;
-    const B t1 = a - B(2) * b + c, t2 = b - B(2) * c + d;
-    phi = w0 * B(1.0 / 3.0) * t1 + (w2 - B(0.5)) * B(1.0 / 6.0) * t2;
-    // backwards, with d(phi) = 1
-    const B lw0 = t1 * B(1.0 / 3.0), lw2 = t2 * B(1.0 / 6.0);
-    const B lt1 = w0 * B(1.0 / 3.0), lt2 = (w2 - B(0.5)) * B(1.0 / 6.0);
-    const B common = (lw0 * w0 + lw2 * w2) / S;
-    const B la[3] = {lw0 / S - common, -common, lw2 / S - common};
-    B lIS[3];
-    if constexpr (VAR == 0) {
-#pragma unroll
-        for (int k = 0; k < 3; ++k) lIS[k] = la[k] * (B(-2) * al[k] / s[k]);
-    } else {
-        B ltau = B(0);
-#pragma unroll
-        for (int k = 0; k < 3; ++k) {
-            const B lr = clamped[k] ? B(0) : la[k] * dk[k] * B(2) * r[k];
-            ltau = ltau + lr / s[k];
-            lIS[k] = -lr * r[k] / s[k];
-        }
-        const B lt = t >= B(0) ? ltau : -ltau;
-        lIS[0] = lIS[0] + lt;
-        lIS[2] = lIS[2] - lt;
-    }
-    g[0] = lIS[0] * (B(26) * x0 + B(6) * x1) + lt1;
-    g[1] = lIS[0] * (B(-26) * x0 - B(18) * x1) + lIS[1] * (B(26) * y0 + B(6) * y1) - B(2) * lt1 + lt2;
-    g[2] = lIS[1] * (B(-26) * y0 + B(6) * y1) + lIS[2] * (B(26) * z0 + B(18) * z1) + lt1 - B(2) * lt2;
-    g[3] = lIS[2] * (B(-26) * z0 - B(6) * z1) + lt2;
-}
-
-// weno_field (Eq. FWENO for one characteristic field) and its gradient in
-// its eleven projections and in alpha.
-template <typename B, int VAR>
-__device__ __forceinline__ void weno_field_grad(const B (&P)[11], B alpha, B eps4, B &phi, B (&gP)[11], B &galpha) {
-    B p[5], q[5];
-#pragma unroll
-    for (int j = 0; j < 5; ++j) {
-        p[j] = P[1 + j] + alpha * P[6 + j];
-        q[j] = P[1 + j] - alpha * P[6 + j];
-    }
-    B fp, fq, gpa[4], gqa[4];
-    phi_n_grad<B, VAR>(p[0], p[1], p[2], p[3], eps4, fp, gpa);
-    phi_n_grad<B, VAR>(q[4], q[3], q[2], q[1], eps4, fq, gqa);
-    phi = P[0] + B(0.5) * (fq - fp);
-    B gp[5], gq[5];
-#pragma unroll
-    for (int j = 0; j < 4; ++j) gp[j] = B(-0.5) * gpa[j];
-    gp[4] = B(0);
-    gq[0] = B(0);
-#pragma unroll
-    for (int j = 1; j < 5; ++j) gq[j] = B(0.5) * gqa[4 - j];
-    gP[0] = B(1);
-    galpha = B(0);
-#pragma unroll
-    for (int j = 0; j < 5; ++j) {
-        gP[1 + j] = gp[j] + gq[j];
-        gP[6 + j] = alpha * (gp[j] - gq[j]);
-        galpha = galpha + P[6 + j] * (gp[j] - gq[j]);
-    }
-}
-
-// Reverse of cell_fill<B, AX>: given the adjoints lq of a cell's 23
+// Reverse of cell_fill<R, AX>: given the adjoints lq of a cell's 23
 // quantities, the adjoints of its eight inputs (rho, m_x, m_y, m_z, E, B_x,
-// B_y, B_z) in out.  The primitives and the flux are differentiated by hand
-// (Eq. P and Eq. fluxes), and so are the three wave speeds when their
-// adjoints are not zero (the two cells next to the face), through
-// speeds_rev.  The floors, when they apply, cut the dependence as in the
-// forward step.
-template <typename B, typename A, int AX>
-__device__ __forceinline__ void cell_fill_adjoint(const B (&in)[8], const A (&lq)[NCQ], const Phys<B> &K,
-                                                  A (&out)[8]) {
+// B_y, B_z) in out: the primitives and the flux (Eq. P and Eq. fluxes), and
+// the three wave speeds through speeds_rev.  The floors, when they apply, cut
+// the dependence as in the forward step.
+template <typename R, int AX>
+__device__ __forceinline__ void cell_fill_adjoint(const R (&in)[8], const R (&lq)[NCQ], const Phys<R> &K, R (&out)[8]) {
+    using m = M<R>;
     constexpr int n = AX, t1 = (AX + 1) % 3, t2 = (AX + 2) % 3;
-    const B rho = in[0], mn = in[1 + n], m1 = in[1 + t1], m2 = in[1 + t2], E = in[4];
-    const B Bn = in[5 + n], B1 = in[5 + t1], B2 = in[5 + t2];
-    B r = rho;
+    const R rho = in[0], mn = in[1 + n], m1 = in[1 + t1], m2 = in[1 + t2], E = in[4];
+    const R Bn = in[5 + n], B1 = in[5 + t1], B2 = in[5 + t2];
+    R r = rho;
     bool rfloor = false, pfloor = false;
     if (K.floors && r < K.rho_min) {
         r = K.rho_min;
         rfloor = true;
     }
-    const B ir = M<B>::rcp_(r);
-    const A vn = (A)(mn * ir), v1 = (A)(m1 * ir), v2 = (A)(m2 * ir);
-    const A vv = vn * vn + v1 * v1 + v2 * v2;
-    const A BB = (A)Bn * (A)Bn + (A)B1 * (A)B1 + (A)B2 * (A)B2;
-    B P = K.gm1 * (E - B(0.5) * r * (B)vv - B(0.5) * (B)BB);
+    const R isr = m::rsqrt_(r), ir = isr * isr;
+    const R vn = mn * ir, v1 = m1 * ir, v2 = m2 * ir;
+    const R vv = vn * vn + v1 * v1 + v2 * v2;
+    const R Bn2 = Bn * Bn, Bt2 = B1 * B1 + B2 * B2;
+    const R BB = Bn2 + Bt2;
+    R P = K.gm1 * (E - R(0.5) * (r * vv + BB));
     if (K.floors && P < K.p_min) {
         P = K.p_min;
         pfloor = true;
     }
-    const A rA = (A)r, PA = (A)P, EA = (A)E, bn = (A)Bn, b1 = (A)B1, b2 = (A)B2;
-    const A Pt = PA + A(0.5) * BB;
-    const A vB = vn * bn + v1 * b1 + v2 * b2;
-    A lr = lq[C_RHO], lvn = lq[C_VN], lv1 = lq[C_VT1], lv2 = lq[C_VT2];
-    A lBn = lq[C_BN], lB1 = lq[C_BT1], lB2 = lq[C_BT2], lP = lq[C_P];
-    A lE = lq[C_E], lmn = lq[C_MN], lm1 = lq[C_MT1], lm2 = lq[C_MT2], lrho = lq[C_RHOQ];
-    A lPt = A(0), lvB = A(0);
-    {   // F0 = r vn, F1 = r vn^2 + Pt - Bn^2, F2 = r vn v1 - Bn B1, F3 = r vn v2 - Bn B2
-        const A f0 = lq[C_F0], f1 = lq[C_F1], f2 = lq[C_F2], f3 = lq[C_F3];
-        lr += f0 * vn + f1 * vn * vn + f2 * vn * v1 + f3 * vn * v2;
-        lvn += f0 * rA + f1 * A(2) * rA * vn + f2 * rA * v1 + f3 * rA * v2;
-        lPt += f1;
-        lBn -= f1 * A(2) * bn + f2 * b1 + f3 * b2;
-        lv1 += f2 * rA * vn;
-        lv2 += f3 * rA * vn;
-        lB1 -= f2 * bn;
-        lB2 -= f3 * bn;
-    }
-    {   // F4 = B1 vn - Bn v1, F5 = B2 vn - Bn v2, F6 = (E + Pt) vn - Bn vB
-        const A f4 = lq[C_F4], f5 = lq[C_F5], f6 = lq[C_F6];
-        lB1 += f4 * vn;
-        lB2 += f5 * vn;
-        lvn += f4 * b1 + f5 * b2 + f6 * (EA + Pt);
-        lBn -= f4 * v1 + f5 * v2 + f6 * vB;
-        lv1 -= f4 * bn;
-        lv2 -= f5 * bn;
-        lE += f6 * vn;
-        lPt += f6 * vn;
-        lvB -= f6 * bn;
-    }
+    const R Pt = P + R(0.5) * BB;
+    const R vB = vn * Bn + v1 * B1 + v2 * B2;
+    R lr = lq[C_RHO], lvn = lq[C_VN], lv1 = lq[C_VT1], lv2 = lq[C_VT2];
+    R lBn = lq[C_BN], lB1 = lq[C_BT1], lB2 = lq[C_BT2], lP = lq[C_P];
+    R lE = lq[C_E], lmn = lq[C_MN], lm1 = lq[C_MT1], lm2 = lq[C_MT2], lrho = lq[C_RHOQ];
+    // F0 = r vn, F1 = r vn^2 + Pt - Bn^2, F2 = r vn v1 - Bn B1, F3 = r vn v2 - Bn B2,
+    // F4 = B1 vn - Bn v1, F5 = B2 vn - Bn v2, F6 = (E + Pt) vn - Bn vB
+    const R f0 = lq[C_F0], f1 = lq[C_F1], f2 = lq[C_F2], f3 = lq[C_F3], f4 = lq[C_F4], f5 = lq[C_F5], f6 = lq[C_F6];
+    const R fv = f0 + f1 * vn + f2 * v1 + f3 * v2;      // adjoint of r vn times the rest
+    lr += fv * vn;
+    lvn += r * (fv + f1 * vn) + f4 * B1 + f5 * B2 + f6 * (E + Pt);
+    lv1 += r * (f2 * vn) - f4 * Bn;
+    lv2 += r * (f3 * vn) - f5 * Bn;
+    lBn -= R(2) * f1 * Bn + f2 * B1 + f3 * B2 + f4 * v1 + f5 * v2 + f6 * vB;
+    lB1 += f4 * vn - f2 * Bn;
+    lB2 += f5 * vn - f3 * Bn;
+    lE += f6 * vn;
+    const R lPt = f1 + f6 * vn, lvB = -(f6 * Bn);
     // vB = vn Bn + v1 B1 + v2 B2; Pt = P + BB/2
-    lvn += lvB * bn;
-    lv1 += lvB * b1;
-    lv2 += lvB * b2;
-    lBn += lvB * vn + lPt * bn;
-    lB1 += lvB * v1 + lPt * b1;
-    lB2 += lvB * v2 + lPt * b2;
+    lvn += lvB * Bn;
+    lv1 += lvB * B1;
+    lv2 += lvB * B2;
+    lBn += lvB * vn + lPt * Bn;
+    lB1 += lvB * v1 + lPt * B1;
+    lB2 += lvB * v2 + lPt * B2;
     lP += lPt;
-    // wave speeds c_f, c_A, c_slow of the cell from (r, P, Bn, B1, B2),
-    // reversed by hand (Eqs. slow/fast through speeds_rev; |Bn| and sqrt(0)
-    // take the sign of Bn and the subgradient 0)
-    const A lcf = lq[C_CF], lca = lq[C_CA], lcs = lq[C_CSL];
-    if (lcf != A(0) || lca != A(0) || lcs != A(0)) {
-        using mb = M<B>;
-        const B irr = mb::rcp_(r);
-        const B cs2 = K.gamma * P * irr, ca2 = Bn * Bn * irr, bt2 = (B1 * B1 + B2 * B2) * irr;
-        B fmc, cms, cf2, csl2;
-        speeds<B>(cs2, ca2, bt2, fmc, cms, cf2, csl2);
-        const B cf = mb::sqrt_(cf2), csl = mb::sqrt_(csl2), sr = mb::sqrt_(r);
-        const A lcf2 = cf > B(0) ? lcf * A(0.5) / (A)cf : A(0);
-        const A lcsl2 = csl > B(0) ? lcs * A(0.5) / (A)csl : A(0);
-        A lcs2 = A(0), lca2 = A(0), lbt2 = A(0);
-        speeds_rev<B, A>(cs2, ca2, bt2, A(0), A(0), lcf2, lcsl2, lcs2, lca2, lbt2);
-        // c_A = |Bn| (sqrt(r) / r)
-        const A Airr = (A)irr, Asr = (A)sr;
-        const A sgn = Bn >= B(0) ? A(1) : A(-1);
-        lBn += lca * sgn * Asr * Airr;
-        const A lq_ = lca * sgn * (A)Bn;              // adjoint of sqrt(r) / r
-        A lirr = lq_ * Asr;
-        const A lsr = lq_ * Airr;
-        if (sr > B(0)) lr += lsr * A(0.5) / Asr;
+    // wave speeds c_f, c_A, c_slow of the cell from (r, P, Bn, B1, B2); |Bn| and
+    // sqrt(0) take the sign of Bn and the subgradient 0
+    {
+        const R lcf = lq[C_CF], lca = lq[C_CA], lcs = lq[C_CSL];
+        const R cs2 = K.gamma * P * ir, ca2 = Bn2 * ir, bt2 = Bt2 * ir;
+        R fmc, cms, cf2;
+        speeds_fast<R>(cs2, ca2, bt2, fmc, cms, cf2);
+        const R icf2 = m::normal_pos(cf2) ? m::rcp3_(cf2) : R(0);
+        const R csl2 = cs2 * ca2 * icf2;
+        const R lcf2 = m::normal_pos(cf2) ? m::half_(lcf * m::rsqrt_(cf2)) : R(0);
+        const R lcsl2 = m::normal_pos(csl2) ? m::half_(lcs * m::rsqrt_(csl2)) : R(0);
+        R lcs2 = R(0), lca2 = R(0), lbt2 = R(0);
+        speeds_rev<R>(cs2, ca2, bt2, R(0), R(0), lcf2, lcsl2, lcs2, lca2, lbt2);
+        // c_A = |Bn| / sqrt(r)
+        const R g = Bn >= R(0) ? lca : -lca;
+        lBn += g * isr;
+        lr -= m::half_(g * Bn) * (isr * ir);
         // cs2 = gamma P / r, ca2 = Bn^2 / r, bt2 = (B1^2 + B2^2) / r
-        lP += (A)K.gamma * Airr * lcs2;
-        lirr += (A)K.gamma * (A)P * lcs2;
-        lBn += A(2) * (A)Bn * Airr * lca2;
-        lirr += (A)Bn * (A)Bn * lca2;
-        lB1 += A(2) * (A)B1 * Airr * lbt2;
-        lB2 += A(2) * (A)B2 * Airr * lbt2;
-        lirr += ((A)B1 * (A)B1 + (A)B2 * (A)B2) * lbt2;
-        lr -= Airr * (Airr * lirr);
+        lP += K.gamma * ir * lcs2;
+        lBn += R(2) * Bn * ir * lca2;
+        lB1 += R(2) * B1 * ir * lbt2;
+        lB2 += R(2) * B2 * ir * lbt2;
+        const R lirr = K.gamma * P * lcs2 + Bn2 * lca2 + Bt2 * lbt2;
+        lr -= ir * (ir * lirr);
     }
     // P = gm1 (E - r vv / 2 - BB / 2)
     if (!pfloor) {
-        const A gl = (A)K.gm1 * lP;
+        const R gl = K.gm1 * lP;
         lE += gl;
-        lr -= A(0.5) * vv * gl;
-        lvn -= rA * vn * gl;
-        lv1 -= rA * v1 * gl;
-        lv2 -= rA * v2 * gl;
-        lBn -= bn * gl;
-        lB1 -= b1 * gl;
-        lB2 -= b2 * gl;
+        lr -= R(0.5) * vv * gl;
+        lvn -= r * vn * gl;
+        lv1 -= r * v1 * gl;
+        lv2 -= r * v2 * gl;
+        lBn -= Bn * gl;
+        lB1 -= B1 * gl;
+        lB2 -= B2 * gl;
     }
     // v = m / r
-    const A irA = (A)ir;
-    lmn += lvn * irA;
-    lm1 += lv1 * irA;
-    lm2 += lv2 * irA;
-    lr -= (lvn * vn + lv1 * v1 + lv2 * v2) * irA;
+    lmn += lvn * ir;
+    lm1 += lv1 * ir;
+    lm2 += lv2 * ir;
+    lr -= (lvn * vn + lv1 * v1 + lv2 * v2) * ir;
     if (!rfloor) lrho += lr;
     out[0] = lrho;
     out[1 + n] = lmn;
@@ -825,224 +725,105 @@ __device__ __forceinline__ void cell_fill_adjoint(const B (&in)[8], const A (&lq
     out[5 + t2] = lB2;
 }
 
-// Reverse mode of the face function.  Face p (the interface between cell p
-// and its successor along AX) reads stencil cells p-2 .. p+3 (inputs rho,
-// m_x, m_y, m_z, E, B_x, B_y, B_z each); its outputs are the five lab-order
-// face fluxes and the two transport fluxes.  One primal evaluation (the
-// formulas of cell_fill and face_flux), then the transposes of the linear
-// parts (stencil combinations, projection on the left eigenvectors,
-// back-projection on the right ones), of phi_N (phi_n_grad) and of the cell
-// recovery (cell_fill_adjoint) and of the eigenvectors (eigen7_rev), all
-// written by hand.  Branches follow the primal values (the derivative of the
-// branch the forward step takes).  The 48 contributions
-// d(lam . outputs)/d(input) go to cb; adjoints accumulate in double (float
-// in the float path, whose Jacobians are float).
-template <int AX, typename B, int VAR>
-__global__ void __launch_bounds__(128) adj_face_kernel(AdjSweepArgs<B> a) {
-    using A = typename std::conditional<std::is_same<B, float>::value, float, double>::type;
+// Cell p of a 32 x 8 tile (x and the axis, or y for the x-sweep): the adjoint
+// of the difference between cells d and d + 1 is the sum of the face adjoints
+// at position j over the five faces d + 2 - j that read it, formed once per
+// difference (a tile's first cell also needs the one below it) and kept in
+// shared memory; a flux or conserved component of cell i then takes D(i-1) -
+// D(i), plus, for the flux, the central combinations of four faces.  Fixed
+// order throughout.
+template <int AX, typename R>
+__global__ void __launch_bounds__(256) adj_cell_kernel(AdjSweepArgs<R> a) {
+    constexpr int W = AX == 0 ? 33 : 32, H = AX == 0 ? 8 : 9;
+    __shared__ R acc[14][H][W];
     const int nx = a.nx, ny = a.ny, nz = a.nz;
-    const long long n = (long long)nx * ny * nz;
-    const long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-    if (p >= n) return;
-    const int i = (int)(p % nx);
-    const long long r = p / nx;
-    const int j = (int)(r % ny), k = (int)(r / ny);
-    B in[6][8];
+    const size_t n = (size_t)nx * ny * nz;
+    const int tx = threadIdx.x, ty = threadIdx.y;
+    const int gx = blockIdx.x * 32 + tx, gy = AX == 2 ? (int)blockIdx.y : (int)blockIdx.y * 8 + ty,
+              gz = AX == 2 ? (int)blockIdx.z * 8 + ty : (int)blockIdx.z;
+    // index of the cell `o` cells along the axis from (x, y, z)
+    auto at = [&](int x, int y, int z, int o) {
+        if (AX == 0) x = wrapi(x + o, nx);
+        if (AX == 1) y = wrapi(y + o, ny);
+        if (AX == 2) z = wrapi(z + o, nz);
+        return (size_t)x + (size_t)nx * ((size_t)y + (size_t)ny * (size_t)z);
+    };
+    auto differences = [&](int x, int y, int z, int o, int row, int col) {
+        size_t f[5];
 #pragma unroll
-    for (int s = 0; s < 6; ++s) {
-        const int ii = AX == 0 ? wrapi(i - 2 + s, nx) : i;
-        const int jj = AX == 1 ? wrapi(j - 2 + s, ny) : j;
-        const int kk = AX == 2 ? wrapi(k - 2 + s, nz) : k;
-        const size_t g = (size_t)ii + (size_t)nx * ((size_t)jj + (size_t)ny * (size_t)kk);
+        for (int j = 0; j < 5; ++j) f[j] = at(x, y, z, o + 2 - j);
 #pragma unroll
-        for (int f = 0; f < 5; ++f) in[s][f] = a.q[f][g];
+        for (int c = 0; c < 14; ++c) {
+            R s = R(0);
 #pragma unroll
-        for (int f = 0; f < 3; ++f) in[s][5 + f] = a.bc[f][g];
+            for (int j = 0; j < 5; ++j) s += a.face_plane(kAdjDiff + ((c % 7) * 5 + j) * 2 + c / 7)[f[j]];
+            acc[c][row][col] = s;
+        }
+    };
+    const bool in = gx < nx && gy < ny && gz < nz;
+    if (in) differences(gx, gy, gz, 0, AX == 0 ? ty : ty + 1, AX == 0 ? tx + 1 : tx);
+    if (ty == 0) {      // the differences below the tile: one warp
+        if (AX == 0) {
+            const int y = blockIdx.y * 8 + tx;
+            if (tx < 8 && y < ny) differences((int)blockIdx.x * 32, y, gz, -1, tx, 0);
+        } else if (in) {
+            differences(gx, gy, gz, -1, 0, tx);
+        }
     }
-    const A lam5 = from_double<A>(a.lamS[0][p]), lam6 = from_double<A>(a.lamS[1][p]);
-    // adjoint of the frame flux Ff (s1 = Ff[4] + bvt1, s2 = Ff[5] + bvt2)
-    A lFf[7];
-    lFf[0] = from_double<A>(a.lamF[0][p]);
-    lFf[1] = from_double<A>(a.lamF[1 + AX][p]);
-    lFf[2] = from_double<A>(a.lamF[1 + (AX + 1) % 3][p]);
-    lFf[3] = from_double<A>(a.lamF[1 + (AX + 2) % 3][p]);
-    lFf[4] = (A)lam5;
-    lFf[5] = (A)lam6;
-    lFf[6] = from_double<A>(a.lamF[4][p]);
-    const Phys<B> K = a.K;
-    bool bad = false, hit = false;
-    B cq[NCQ * 6];
-#pragma unroll 1
-    for (int c = 0; c < 6; ++c)
-        cell_fill<B, AX>(cq + c, 6, in[c][0], in[c][1], in[c][2], in[c][3], in[c][4], in[c][5], in[c][6], in[c][7], K,
-                         bad, hit);
-#define Q(q, kk) cq[(q) * 6 + (kk)]
+    __syncthreads();
+    if (!in) return;
+    const size_t p = at(gx, gy, gz, 0), pm = at(gx, gy, gz, -1), pm2 = at(gx, gy, gz, -2), pp = at(gx, gy, gz, 1);
+    constexpr int t1 = (AX + 1) % 3, t2 = (AX + 2) % 3;
+    R cell[8], lq[NCQ];
+#pragma unroll
+    for (int f = 0; f < 5; ++f) cell[f] = a.q[f][p];
+#pragma unroll
+    for (int f = 0; f < 3; ++f) cell[5 + f] = a.bc[f][p];
     constexpr int qU[7] = {C_RHOQ, C_MN, C_MT1, C_MT2, C_BT1, C_BT2, C_E};
-    B X[11][7];
-#pragma unroll
-    for (int c = 0; c < 7; ++c) {
-        const B f0 = Q(C_F0 + c, 0), f1 = Q(C_F0 + c, 1), f2 = Q(C_F0 + c, 2), f3 = Q(C_F0 + c, 3), f4 = Q(C_F0 + c, 4),
-                f5 = Q(C_F0 + c, 5);
-        X[0][c] = (B(7) * (f2 + f3) - (f1 + f4)) * B(1.0 / 12.0);
-        X[1][c] = f1 - f0;
-        X[2][c] = f2 - f1;
-        X[3][c] = f3 - f2;
-        X[4][c] = f4 - f3;
-        X[5][c] = f5 - f4;
-        const B u0 = Q(qU[c], 0), u1 = Q(qU[c], 1), u2 = Q(qU[c], 2), u3 = Q(qU[c], 3), u4 = Q(qU[c], 4),
-                u5 = Q(qU[c], 5);
-        X[6][c] = u1 - u0;
-        X[7][c] = u2 - u1;
-        X[8][c] = u3 - u2;
-        X[9][c] = u4 - u3;
-        X[10][c] = u5 - u4;
-    }
-    // LF speeds alpha(m) = max over cells 2, 3 of |v_n + sgn c|, with the
-    // cell and sign that attain it (the branch the forward step takes)
-    constexpr int cq_of_mode[7] = {C_CF, C_CF, C_CSL, C_CSL, C_CA, C_CA, -1};
-    constexpr int sgn_of_mode[7] = {-1, 1, -1, 1, -1, 1, 0};
-    B alpha[7];
-    int acell[7];
-    B asign[7];
-#pragma unroll
-    for (int mo = 0; mo < 7; ++mo) {
-        const B c2 = cq_of_mode[mo] >= 0 ? Q(cq_of_mode[mo], 2) : B(0);
-        const B c3 = cq_of_mode[mo] >= 0 ? Q(cq_of_mode[mo], 3) : B(0);
-        const B x2 = Q(C_VN, 2) + B(sgn_of_mode[mo]) * c2, x3 = Q(C_VN, 3) + B(sgn_of_mode[mo]) * c3;
-        const B a2 = x2 >= B(0) ? x2 : -x2, a3 = x3 >= B(0) ? x3 : -x3;
-        acell[mo] = a2 >= a3 ? 2 : 3;
-        alpha[mo] = a2 >= a3 ? a2 : a3;
-        asign[mo] = (a2 >= a3 ? x2 : x3) >= B(0) ? B(1) : B(-1);
-    }
-    // eigenvectors at the interface state (values); their dependence on the
-    // state is reversed by eigen7_rev after the mode loop
-    B wv[8];
-    const int prim[8] = {C_RHO, C_VN, C_VT1, C_VT2, C_BN, C_BT1, C_BT2, C_P};
-#pragma unroll
-    for (int t = 0; t < 8; ++t) wv[t] = B(0.5) * (Q(prim[t], 2) + Q(prim[t], 3));
-    B Lv[7][7], Rv[7][7];
-    eigen7<B>(wv, K, Lv, Rv);
-    A lLm[7][7], lRm[7][7];
-    const B eps4 = B(4) * K.eps_w;
-    A lX[11][7];
-#pragma unroll
-    for (int x = 0; x < 11; ++x)
-#pragma unroll
-        for (int c = 0; c < 7; ++c) lX[x][c] = A(0);
-    A lw[8];
-    A lalpha[7];
-#pragma unroll 1
-    for (int mo = 0; mo < 7; ++mo) {
-        B Pm[11];
-#pragma unroll
-        for (int x = 0; x < 11; ++x) {
-            B acc = Lv[mo][0] * X[x][0];
-#pragma unroll
-            for (int c = 1; c < 7; ++c) acc = acc + Lv[mo][c] * X[x][c];
-            Pm[x] = acc;
-        }
-        B phi, gP[11], ga;
-        weno_field_grad<B, VAR>(Pm, alpha[mo], eps4, phi, gP, ga);
-        A lphi = A(0);
-#pragma unroll
-        for (int c = 0; c < 7; ++c) lphi += (A)Rv[mo][c] * lFf[c];
-        lalpha[mo] = lphi * (A)ga;
-        A lL[7] = {0, 0, 0, 0, 0, 0, 0};
-#pragma unroll
-        for (int x = 0; x < 11; ++x) {
-            const A lp = lphi * (A)gP[x];
-#pragma unroll
-            for (int c = 0; c < 7; ++c) {
-                lX[x][c] += lp * (A)Lv[mo][c];
-                lL[c] += lp * (A)X[x][c];
-            }
-        }
-#pragma unroll
-        for (int c = 0; c < 7; ++c) {
-            lLm[mo][c] = lL[c];
-            lRm[mo][c] = (A)phi * lFf[c];
-        }
-    }
-    eigen7_rev<B, A>(wv, K, lLm, lRm, lw);
-    // adjoints of the cells' quantities
-    A lq[6][NCQ];
-#pragma unroll
-    for (int c = 0; c < 6; ++c)
-#pragma unroll
-        for (int q = 0; q < NCQ; ++q) lq[c][q] = A(0);
-#pragma unroll
-    for (int c = 0; c < 7; ++c) {
-        // X[0] = (7 (f2 + f3) - (f1 + f4)) / 12, X[1 + k] = f_{k+1} - f_k, X[6 + k] = u_{k+1} - u_k
-        const A l0 = lX[0][c] * A(1.0 / 12.0);
-        lq[1][C_F0 + c] -= l0;
-        lq[2][C_F0 + c] += A(7) * l0;
-        lq[3][C_F0 + c] += A(7) * l0;
-        lq[4][C_F0 + c] -= l0;
-#pragma unroll
-        for (int kk = 0; kk < 5; ++kk) {
-            lq[kk + 1][C_F0 + c] += lX[1 + kk][c];
-            lq[kk][C_F0 + c] -= lX[1 + kk][c];
-            lq[kk + 1][qU[c]] += lX[6 + kk][c];
-            lq[kk][qU[c]] -= lX[6 + kk][c];
-        }
-    }
+    constexpr int prim[8] = {C_RHO, C_VN, C_VT1, C_VT2, C_BN, C_BT1, C_BT2, C_P};
 #pragma unroll
     for (int t = 0; t < 8; ++t) {
-        lq[2][prim[t]] += A(0.5) * lw[t];
-        lq[3][prim[t]] += A(0.5) * lw[t];
+        const R *L = a.face_plane(kAdjPrim + t);
+        lq[prim[t]] = R(0.5) * (L[p] + L[pm]);
     }
+    auto D = [&](int c) {
+        return AX == 0 ? acc[c][ty][tx] - acc[c][ty][tx + 1] : acc[c][ty][tx] - acc[c][ty + 1][tx];
+    };
 #pragma unroll
-    for (int mo = 0; mo < 7; ++mo) {
-        const A g = lalpha[mo] * (A)asign[mo];
-        lq[acell[mo]][C_VN] += g;
-        if (cq_of_mode[mo] >= 0) lq[acell[mo]][cq_of_mode[mo]] += g * A(sgn_of_mode[mo]);
+    for (int c = 0; c < 7; ++c) {
+        const R *L = a.face_plane(kAdjCentral + c);
+        lq[C_F0 + c] = D(c) + (R(7) * (L[p] + L[pm]) - (L[pp] + L[pm2])) * R(1.0 / 12.0);
+        if (c == 4 || c == 5)
+            lq[qU[c]] += D(7 + c);
+        else
+            lq[qU[c]] = D(7 + c);
     }
-    // transport fluxes bvt = (B_n v_t (cell 2) + B_n v_t (cell 3)) / 2
-#pragma unroll
-    for (int c = 2; c <= 3; ++c) {
-        lq[c][C_BN] += A(0.5) * (lam5 * (A)Q(C_VT1, c) + lam6 * (A)Q(C_VT2, c));
-        lq[c][C_VT1] += A(0.5) * lam5 * (A)Q(C_BN, c);
-        lq[c][C_VT2] += A(0.5) * lam6 * (A)Q(C_BN, c);
+    // lower cell of its face, upper cell of the one before
+    lq[C_VN] += a.face_plane(kAdjSide)[p] + a.face_plane(kAdjSide + 4)[pm];
+    lq[C_CF] = a.face_plane(kAdjSide + 1)[p] + a.face_plane(kAdjSide + 5)[pm];
+    lq[C_CA] = a.face_plane(kAdjSide + 2)[p] + a.face_plane(kAdjSide + 6)[pm];
+    lq[C_CSL] = a.face_plane(kAdjSide + 3)[p] + a.face_plane(kAdjSide + 7)[pm];
+    // transport fluxes <B_n v_t>: half the sum of the two faces' adjoints
+    {
+        auto below = [&](int ax, int o) {
+            const int x = ax == 0 ? wrapi(gx - 1, nx) : gx, y = ax == 1 ? wrapi(gy - 1, ny) : gy,
+                      z = ax == 2 ? wrapi(gz - 1, nz) : gz;
+            return at(x, y, z, o);
+        };
+        const double *On = a.lamO + (size_t)AX * n, *O2 = a.lamO + (size_t)t2 * n;
+        const R l1 = from_double<R>(-0.25 * ((On[p] + On[below(t1, 0)]) + (On[pm] + On[below(t1, -1)])));
+        const R l2 = from_double<R>(0.25 * ((O2[p] + O2[below(t2, 0)]) + (O2[pm] + O2[below(t2, -1)])));
+        const R ir = M<R>::rcp3_(a.K.floors ? M<R>::max_(cell[0], a.K.rho_min) : cell[0]);
+        lq[C_BN] += (l1 * cell[1 + t1] + l2 * cell[1 + t2]) * ir;
+        lq[C_VT1] += l1 * cell[5 + AX];
+        lq[C_VT2] += l2 * cell[5 + AX];
     }
-#undef Q
-    // each cell's quantities back to its eight inputs
-#pragma unroll 1
-    for (int c = 0; c < 6; ++c) {
-        A g[8];
-        cell_fill_adjoint<B, A, AX>(in[c], lq[c], K, g);
-#pragma unroll
-        for (int v = 0; v < 8; ++v) a.cb[(size_t)(c * 8 + v) * (size_t)n + (size_t)p] = to_double(g[v]);
-    }
-}
-
-// Cell p collects, in a fixed order, the contributions of the six faces whose
-// stencils hold it (face p - s + 2 holds it as stencil cell s):
-// lamq[v] += ... (v < 5), lambc[v - 5] += ... (v >= 5).
-template <int AX>
-__global__ void __launch_bounds__(256) adj_gather_kernel(int nx, int ny, int nz, const double *__restrict__ cb,
-                                                         double *lq0, double *lq1, double *lq2, double *lq3,
-                                                         double *lq4, double *lb0, double *lb1, double *lb2) {
-    const long long n = (long long)nx * ny * nz;
-    const long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-    if (p >= n) return;
-    const int i = (int)(p % nx);
-    const long long r = p / nx;
-    const int j = (int)(r % ny), k = (int)(r / ny);
-    size_t face[6];
-#pragma unroll
-    for (int s = 0; s < 6; ++s) {
-        const int ii = AX == 0 ? wrapi(i + 2 - s, nx) : i;
-        const int jj = AX == 1 ? wrapi(j + 2 - s, ny) : j;
-        const int kk = AX == 2 ? wrapi(k + 2 - s, nz) : k;
-        face[s] = (size_t)ii + (size_t)nx * ((size_t)jj + (size_t)ny * (size_t)kk);
-    }
-    double *out[8] = {lq0, lq1, lq2, lq3, lq4, lb0, lb1, lb2};
+    R g[8];
+    cell_fill_adjoint<R, AX>(cell, lq, a.K, g);
 #pragma unroll
     for (int v = 0; v < 8; ++v) {
-        double acc = 0.0;
-#pragma unroll
-        for (int s = 0; s < 6; ++s) acc += cb[(size_t)(s * 8 + v) * (size_t)n + face[s]];
-        out[v][p] += acc;
+        double *o = v < 5 ? a.outq + (size_t)v * n : a.outb + (size_t)(v - 5) * n;
+        o[p] = a.first ? to_double(g[v]) : o[p] + to_double(g[v]);
     }
 }
 
@@ -1068,74 +849,44 @@ __device__ __forceinline__ bool adj_cell(const AdjGrid &g, int &i, int &j, int &
     return true;
 }
 
-// stage sources: lamD = cf lamq_fin + cn lamq_next, mu = cf lamb_fin + cn lamb_next
-// (mu is the adjoint of the stage's face-field increment dt-scaled curl Omega)
-static __global__ void __launch_bounds__(256) adj_sources_kernel(long long n, double cf, double cn,
+// Stage sources: lamD = cf lamq_fin + cn lamq_next (the adjoint of the flux
+// divergence) and lamO = curl^T mu, mu = cf lamb_fin + cn lamb_next, for the
+// face update of Sec. 2.3:
+//   db_x = -(O_x - O_x(j-1)) rdy + (O_z - O_z(k-1)) rdz
+//   db_y = -(O_y - O_y(k-1)) rdz + (O_x - O_x(i-1)) rdx
+//   db_z = -(O_z - O_z(i-1)) rdx + (O_y - O_y(j-1)) rdy
+// The flux adjoints follow from them face by face (adj_face_kernel):
+//   lamF_d = (lamD(+1 along d) - lamD) / dx_d  (transpose of Eq. num),
+// and, from the EMF averages of Eqs. ox1-ox3
+//   O_x = (g*_x + g*_x(i+1))/2 - (f*_y + f*_y(j+1))/2
+//   O_y = (h*_y + h*_y(j+1))/2 - (g*_z + g*_z(k+1))/2
+//   O_z = (f*_z + f*_z(k+1))/2 - (h*_x + h*_x(i+1))/2,
+// the sweep along d (t1, t2 the next axes, cyclic) has lamS_1 = -(lamO_d +
+// lamO_d(-1 along t1))/2 and lamS_2 = (lamO_t2 + lamO_t2(-1 along t2))/2.
+static __global__ void __launch_bounds__(256) adj_sources_kernel(AdjGrid g, double cf, double cn,
                                                                  const double *__restrict__ lq_fin,
                                                                  const double *__restrict__ lb_fin,
                                                                  const double *__restrict__ lq_next,
                                                                  const double *__restrict__ lb_next, double *lamD,
-                                                                 double *mu) {
-    const long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-    if (p >= n) return;
+                                                                 double *lamO) {
+    int i, j, k;
+    size_t p;
+    if (!adj_cell(g, i, j, k, p)) return;
+    const size_t n = (size_t)g.nx * g.ny * g.nz;
 #pragma unroll
     for (int f = 0; f < 5; ++f) {
-        const size_t o = (size_t)f * (size_t)n + (size_t)p;
+        const size_t o = (size_t)f * n + p;
         lamD[o] = cf * lq_fin[o] + (lq_next ? cn * lq_next[o] : 0.0);
     }
-#pragma unroll
-    for (int f = 0; f < 3; ++f) {
-        const size_t o = (size_t)f * (size_t)n + (size_t)p;
-        mu[o] = cf * lb_fin[o] + (lb_next ? cn * lb_next[o] : 0.0);
-    }
-}
-
-// lamO = curl^T mu for the face update of Sec. 2.3:
-//   db_x = -(O_x - O_x(j-1)) rdy + (O_z - O_z(k-1)) rdz
-//   db_y = -(O_y - O_y(k-1)) rdz + (O_x - O_x(i-1)) rdx
-//   db_z = -(O_z - O_z(i-1)) rdx + (O_y - O_y(j-1)) rdy
-static __global__ void __launch_bounds__(256) adj_curl_kernel(AdjGrid g, const double *__restrict__ mu, double *lamO) {
-    int i, j, k;
-    size_t p;
-    if (!adj_cell(g, i, j, k, p)) return;
-    const size_t n = (size_t)g.nx * g.ny * g.nz;
-    const double *mx = mu, *my = mu + n, *mz = mu + 2 * n;
-    lamO[p] = g.rdy * (mx[g.at(i, j + 1, k)] - mx[p]) + g.rdx * (my[p] - my[g.at(i + 1, j, k)]);
-    lamO[n + p] = g.rdz * (my[g.at(i, j, k + 1)] - my[p]) + g.rdy * (mz[p] - mz[g.at(i, j + 1, k)]);
-    lamO[2 * n + p] = g.rdz * (mx[p] - mx[g.at(i, j, k + 1)]) + g.rdx * (mz[g.at(i + 1, j, k)] - mz[p]);
-}
-
-// Flux adjoints from lamD (transpose of Eq. num) and lamO (transpose of the
-// EMF averages of Eqs. ox1-ox3):
-//   O_x = (g*_x + g*_x(i+1))/2 - (f*_y + f*_y(j+1))/2
-//   O_y = (h*_y + h*_y(j+1))/2 - (g*_z + g*_z(k+1))/2
-//   O_z = (f*_z + f*_z(k+1))/2 - (h*_x + h*_x(i+1))/2
-// lamF: 15 planes (axis-major: x fields 0..4, y, z); lamS: 6 planes
-// (f*_y, f*_z, g*_z, g*_x, h*_x, h*_y, the storage order of the sweeps).
-static __global__ void __launch_bounds__(256) adj_flux_kernel(AdjGrid g, const double *__restrict__ lamD,
-                                                              const double *__restrict__ lamO, double *lamF,
-                                                              double *lamS) {
-    int i, j, k;
-    size_t p;
-    if (!adj_cell(g, i, j, k, p)) return;
-    const size_t n = (size_t)g.nx * g.ny * g.nz;
+    auto mu = [&](int f, size_t q) {
+        const size_t o = (size_t)f * n + q;
+        return cf * lb_fin[o] + (lb_next ? cn * lb_next[o] : 0.0);
+    };
     const size_t px = g.at(i + 1, j, k), py = g.at(i, j + 1, k), pz = g.at(i, j, k + 1);
-#pragma unroll
-    for (int f = 0; f < 5; ++f) {
-        const double *L = lamD + (size_t)f * n;
-        const double c = L[p];
-        lamF[(size_t)f * n + p] = g.rdx * (L[px] - c);
-        lamF[(size_t)(5 + f) * n + p] = g.rdy * (L[py] - c);
-        lamF[(size_t)(10 + f) * n + p] = g.rdz * (L[pz] - c);
-    }
-    const double *Ox = lamO, *Oy = lamO + n, *Oz = lamO + 2 * n;
-    const double ox = Ox[p], oy = Oy[p], oz = Oz[p];
-    lamS[p] = -0.5 * (ox + Ox[g.at(i, j - 1, k)]);              // f*_y
-    lamS[n + p] = 0.5 * (oz + Oz[g.at(i, j, k - 1)]);           // f*_z
-    lamS[2 * n + p] = -0.5 * (oy + Oy[g.at(i, j, k - 1)]);      // g*_z
-    lamS[3 * n + p] = 0.5 * (ox + Ox[g.at(i - 1, j, k)]);       // g*_x
-    lamS[4 * n + p] = -0.5 * (oz + Oz[g.at(i - 1, j, k)]);      // h*_x
-    lamS[5 * n + p] = 0.5 * (oy + Oy[g.at(i, j - 1, k)]);       // h*_y
+    const double mx = mu(0, p), my = mu(1, p), mz = mu(2, p);
+    lamO[p] = g.rdy * (mu(0, py) - mx) + g.rdx * (my - mu(1, px));
+    lamO[n + p] = g.rdz * (mu(1, pz) - my) + g.rdy * (mz - mu(2, py));
+    lamO[2 * n + p] = g.rdz * (mx - mu(0, pz)) + g.rdx * (mu(2, px) - mz);
 }
 
 // Transpose of the fourth-order face -> centre interpolation of Sec. 2.3,
@@ -1312,22 +1063,53 @@ static __global__ void __launch_bounds__(256) ic_curl_adjoint_kernel(AdjGrid g, 
     lA[2 * n + p] = (bx[p] - bx[g.at(i, j + 1, k)]) * g.rdy - (by[p] - by[g.at(i + 1, j, k)]) * g.rdx;
 }
 
-// Defined in w5ct_adjoint{32,64}{js,z}.cu (one translation unit per
-// arithmetic type and WENO variant, compiled in parallel).
-template <typename B, int VAR>
-cudaError_t launch_adj_sweep(int axis, const AdjSweepArgs<B> &a, cudaStream_t s);
+// Tiles of the face kernel, one face per thread at up to 255 registers, eight
+// warps per SM: in double 256 threads (32 x 8 faces along x, 16 x 16 in the
+// other two sweeps), in float two blocks of 128 (32 x 4 and 8 x 16).  64^3
+// WENO5 rollout in float, three steps: 7.76 ms; one block of 256 threads 7.82,
+// three blocks of 128 (168 registers) 7.96, four (128 registers) 8.49.
+template <int AX, typename R, int VAR>
+struct AdjFace {
+    static constexpr bool kF = float_based<R>;
+    static constexpr int BX = AX == 0 ? 32 : kF ? 8 : 16, T2 = AX == 0 ? (kF ? 4 : 8) : 16, MINB = kF ? 2 : 1;
+    using TT = SweepTile<AX, T2, BX, 1>;
+    static constexpr size_t smem = (size_t)TT::NC * box_quantities<R>() * sizeof(R);
+    static cudaError_t prepare() {
+        return cudaFuncSetAttribute(adj_face_kernel<AX, R, VAR, T2, BX, MINB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    (int)smem);
+    }
+    static cudaError_t launch(const AdjSweepArgs<R> &a, cudaStream_t s) {
+        const dim3 grid = AX == 2 ? dim3((a.nx + BX - 1) / BX, a.ny, (a.nz + T2 - 1) / T2)
+                                  : dim3((a.nx + BX - 1) / BX, (a.ny + T2 - 1) / T2, a.nz);
+        adj_face_kernel<AX, R, VAR, T2, BX, MINB><<<grid, dim3(BX, T2), smem, s>>>(a);
+        const dim3 cells = AX == 2 ? dim3((a.nx + 31) / 32, a.ny, (a.nz + 7) / 8)
+                                   : dim3((a.nx + 31) / 32, (a.ny + 7) / 8, a.nz);
+        adj_cell_kernel<AX, R><<<cells, dim3(32, 8), 0, s>>>(a);
+        return cudaGetLastError();
+    }
+};
 
-template <typename B, int VAR>
-cudaError_t launch_adj_sweep_impl(int axis, const AdjSweepArgs<B> &a, cudaStream_t s) {
-    const long long n = (long long)a.nx * a.ny * a.nz;
-    const unsigned nb = (unsigned)((n + 127) / 128);
-    if (axis == 0)
-        adj_face_kernel<0, B, VAR><<<nb, 128, 0, s>>>(a);
-    else if (axis == 1)
-        adj_face_kernel<1, B, VAR><<<nb, 128, 0, s>>>(a);
-    else
-        adj_face_kernel<2, B, VAR><<<nb, 128, 0, s>>>(a);
-    return cudaGetLastError();
+// Defined in w5ct_adjoint{32,64}{js,z}.cu (one translation unit per
+// arithmetic type and WENO variant, compiled in parallel): the face and cell
+// kernels along `axis`, and their shared-memory allowance.
+template <typename R, int VAR>
+cudaError_t launch_adj_sweep(int axis, const AdjSweepArgs<R> &a, cudaStream_t s);
+template <typename R, int VAR>
+cudaError_t prepare_adj_sweep();
+
+template <typename R, int VAR>
+cudaError_t launch_adj_sweep_impl(int axis, const AdjSweepArgs<R> &a, cudaStream_t s) {
+    if (axis == 0) return AdjFace<0, R, VAR>::launch(a, s);
+    if (axis == 1) return AdjFace<1, R, VAR>::launch(a, s);
+    return AdjFace<2, R, VAR>::launch(a, s);
+}
+
+template <typename R, int VAR>
+cudaError_t prepare_adj_sweep_impl() {
+    cudaError_t e = AdjFace<0, R, VAR>::prepare();
+    if (e == cudaSuccess) e = AdjFace<1, R, VAR>::prepare();
+    if (e == cudaSuccess) e = AdjFace<2, R, VAR>::prepare();
+    return e;
 }
 
 }  // namespace w5ct

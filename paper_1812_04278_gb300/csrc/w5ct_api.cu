@@ -825,6 +825,7 @@ int w5ct_init_grid(w5ct_ctx *c, int npatch, const int *n3, const double *dx3) {
     auto take = [&](size_t bytes) { size_t o = bytes_total; bytes_total += align256(bytes); return o; };
     const size_t o_q0 = take(5 * n * 8), o_b0 = take(3 * n * 8), o_acc = take(5 * n * 8), o_oacc = take(3 * n * 8);
     const size_t o_qs = take(5 * n * rs), o_bs = take(3 * n * rs), o_bc = take(3 * n * rs);
+    // Fx .. Sz: 21 planes in one run (the adjoint step uses them as such)
     const size_t o_Fx = take(5 * n * rs), o_Fy = take(5 * n * rs), o_Fz = take(5 * n * rs);
     const size_t o_Sx = take(2 * n * rs), o_Sy = take(2 * n * rs), o_Sz = take(2 * n * rs);
     const bool fp32 = !ctx_fp64(c);
@@ -1257,16 +1258,19 @@ int autotune_measure(w5ct_ctx *c, int reps) {
 
 // ---------------------------------------------------------------- adjoint
 
-// Work buffers of the adjoint step, in one allocation: stage states
-// (4 x 8 planes of Real), then double planes: two sets of stage adjoints
-// (5 + 3 each), lamD (5), mu (3), lamO (3), lamF (15), lamS (6), lamBc (3),
-// face contributions (48).
-constexpr int kAdjDoublePlanes = 2 * 8 + 5 + 3 + 3 + 15 + 6 + 3 + 48;
+// Work buffers of the adjoint step, in one allocation: stage states (4 x 8
+// planes of Real) and the face adjoints that do not fit the context's flux
+// buffers (free between the forward stages and the next step), then double
+// planes: two sets of stage adjoints (5 + 3 each), lamD (5), lamO (3), lamBc (3).
+constexpr int kAdjRealPlanes = 32 + kAdjFacePlanes - kAdjFluxPlanes;
+constexpr int kAdjDoublePlanes = 2 * 8 + 5 + 3 + 3;
 
+template <typename Real>
 int ensure_adj(w5ct_ctx *c) {
     if (c->adj_slab) return W5CT_OK;
+    W5_CUDA(c, c->cfg.weno_variant == W5CT_WENO_JS ? (prepare_adj_sweep<Real, 0>()) : (prepare_adj_sweep<Real, 1>()));
     const size_t n = (size_t)c->n;
-    const size_t bytes = align256(32 * n * c->real_size) + (size_t)kAdjDoublePlanes * n * 8;
+    const size_t bytes = align256(kAdjRealPlanes * n * sizeof(Real)) + (size_t)kAdjDoublePlanes * n * 8;
     W5_CUDA(c, cudaMalloc(&c->adj_slab, bytes));
     return W5CT_OK;
 }
@@ -1274,16 +1278,15 @@ int ensure_adj(w5ct_ctx *c) {
 template <typename Real>
 int adjoint_step_impl(w5ct_ctx *c, double dt, const double *lq_fin, const double *lb_fin, double *lq_out,
                       double *lb_out) {
-    int rc = ensure_adj(c);
+    int rc = ensure_adj<Real>(c);
     if (rc) return rc;
     const long long nl = c->n;
     const size_t n = (size_t)nl;
     cudaStream_t st = c->stream;
     Real *stage = reinterpret_cast<Real *>(c->adj_slab);
-    double *w = reinterpret_cast<double *>((char *)c->adj_slab + align256(32 * n * sizeof(Real)));
+    double *w = reinterpret_cast<double *>((char *)c->adj_slab + align256(kAdjRealPlanes * n * sizeof(Real)));
     double *set[2] = {w, w + 8 * n};           // stage adjoints: q (5 planes) then b (3 planes)
-    double *lamD = w + 16 * n, *mu = lamD + 5 * n, *lamO = mu + 3 * n, *lamF = lamO + 3 * n;
-    double *lamS = lamF + 15 * n, *lamBc = lamS + 6 * n, *cb = lamBc + 3 * n;
+    double *lamD = w + 16 * n, *lamO = lamD + 5 * n, *lamBc = lamO + 3 * n;
 
     unsigned long long hits0 = 0;
     int flag0 = 0;
@@ -1310,45 +1313,38 @@ int adjoint_step_impl(w5ct_ctx *c, double dt, const double *lq_fin, const double
     double *next = nullptr;
     for (int s = 3; s >= 0; --s) {
         double *cur = set[s & 1];
-        adj_sources_kernel<<<nb, 256, 0, st>>>(nl, dt * wc[s], s < 3 ? cs[s] * dt : 0.0, lq_fin, lb_fin,
-                                               next, next ? next + 5 * n : nullptr, lamD, mu);
-        adj_curl_kernel<<<nb, 256, 0, st>>>(g, mu, lamO);
-        adj_flux_kernel<<<nb, 256, 0, st>>>(g, lamD, lamO, lamF, lamS);
+        adj_sources_kernel<<<nb, 256, 0, st>>>(g, dt * wc[s], s < 3 ? cs[s] * dt : 0.0, lq_fin, lb_fin, next,
+                                               next ? next + 5 * n : nullptr, lamD, lamO);
         // the stage's cell field from its stored face field
         const Real *sq = stage + (size_t)s * 8 * n, *sb = sq + 5 * n;
         cellb_kernel<Real><<<cellb_grid(c->nx, c->ny, c->nz), dim3(32, 8), 0, st>>>(
             c->nx, c->ny, c->nz, cellb_chunk(c->nx, c->ny, c->nz), sb, sb + n, sb + 2 * n,
             plane<Real>(c->bc, nl, 0), plane<Real>(c->bc, nl, 1), plane<Real>(c->bc, nl, 2));
-        W5_CUDA(c, cudaMemsetAsync(cur, 0, 5 * n * 8, st));
-        W5_CUDA(c, cudaMemsetAsync(lamBc, 0, 3 * n * 8, st));
+        const double rd[3] = {g.rdx, g.rdy, g.rdz};
         for (int ax = 0; ax < 3; ++ax) {
             AdjSweepArgs<Real> aa;
             aa.nx = c->nx;
             aa.ny = c->ny;
             aa.nz = c->nz;
+            aa.rd = rd[ax];
             for (int f = 0; f < 5; ++f) aa.q[f] = sq + (size_t)f * n;
             for (int f = 0; f < 3; ++f) aa.bc[f] = plane<Real>(c->bc, nl, f);
-            for (int f = 0; f < 5; ++f) aa.lamF[f] = lamF + (size_t)(5 * ax + f) * n;
-            for (int f = 0; f < 2; ++f) aa.lamS[f] = lamS + (size_t)(2 * ax + f) * n;
-            aa.cb = cb;
+            aa.lamD = lamD;
+            aa.lamO = lamO;
+            aa.fa = reinterpret_cast<Real *>(c->Fx);
+            aa.fb = stage + 32 * n;
+            aa.outq = cur;
+            aa.outb = lamBc;
+            aa.first = ax == 0;
             aa.K = K;
             const cudaError_t ea = c->cfg.weno_variant == W5CT_WENO_JS ? launch_adj_sweep<Real, 0>(ax, aa, st)
                                                                        : launch_adj_sweep<Real, 1>(ax, aa, st);
             W5_CUDA(c, ea);
-            double *q[5], *b[3];
-            for (int f = 0; f < 5; ++f) q[f] = cur + (size_t)f * n;
-            for (int f = 0; f < 3; ++f) b[f] = lamBc + (size_t)f * n;
-            if (ax == 0)
-                adj_gather_kernel<0><<<nb, 256, 0, st>>>(c->nx, c->ny, c->nz, cb, q[0], q[1], q[2], q[3], q[4], b[0], b[1], b[2]);
-            else if (ax == 1)
-                adj_gather_kernel<1><<<nb, 256, 0, st>>>(c->nx, c->ny, c->nz, cb, q[0], q[1], q[2], q[3], q[4], b[0], b[1], b[2]);
-            else
-                adj_gather_kernel<2><<<nb, 256, 0, st>>>(c->nx, c->ny, c->nz, cb, q[0], q[1], q[2], q[3], q[4], b[0], b[1], b[2]);
             c->launches += 2;
         }
         // stage face-field adjoint; both added into the step's outputs
         adj_interp_kernel<<<nb, 256, 0, st>>>(g, lamBc, cur, cur + 5 * n, lq_out, lb_out);
-        c->launches += 5;
+        c->launches += 3;
         W5_CUDA(c, cudaGetLastError());
         next = cur;
     }

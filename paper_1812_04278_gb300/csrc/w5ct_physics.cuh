@@ -116,6 +116,14 @@ __device__ __forceinline__ double ddiv_newton(double a, double b) {
     return fma(fma(e, e, e), q, q);
 }
 
+// 1 / b, b > 0 finite and normal, the same way: 3 FP64 instructions
+__device__ __forceinline__ double drcp_third(double b) {
+    double r;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(b));
+    const double e = fma(-b, r, 1.0);
+    return fma(fma(e, e, e), r, r);
+}
+
 // 2^n x by an addition to the exponent field (binary64: bits 52-62) on the
 // integer pipes, |n| <= 2; exact for 2^-1020 <= |x| < 2^1020, x itself
 // otherwise (zero, infinities and NaN keep their value; magnitudes outside
@@ -139,6 +147,8 @@ template <> struct M<double> {
     static __device__ __forceinline__ double sqrt_(double x) { return sqrt(x); }
     static __device__ __forceinline__ double div_(double a, double b) { return ddiv_newton(a, b); }
     static __device__ __forceinline__ double rcp_(double x) { return drcp_newton(x); }
+    static __device__ __forceinline__ double rcp3_(double x) { return drcp_third(x); }
+    static __device__ __forceinline__ double times4_(double x) { return dscale2<2>(x); }
     static __device__ __forceinline__ double rsqrt_(double x) { return drsqrt_newton(x); }
     static __device__ __forceinline__ double abs_(double x) { return fabs(x); }
     static __device__ __forceinline__ double max_(double a, double b) { return fmax(a, b); }
@@ -160,6 +170,8 @@ template <> struct M<float> {
     static __device__ __forceinline__ float sqrt_(float x) { return sqrtf(x); }
     static __device__ __forceinline__ float div_(float a, float b) { return __fdividef(a, b); }
     static __device__ __forceinline__ float rcp_(float x) { return __fdividef(1.0f, x); }
+    static __device__ __forceinline__ float rcp3_(float x) { return __fdividef(1.0f, x); }
+    static __device__ __forceinline__ float times4_(float x) { return 4.0f * x; }
     static __device__ __forceinline__ float rsqrt_(float x) { return rsqrtf(x); }
     static __device__ __forceinline__ float abs_(float x) { return fabsf(x); }
     static __device__ __forceinline__ float max_(float a, float b) { return fmaxf(a, b); }

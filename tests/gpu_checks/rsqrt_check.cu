@@ -1,5 +1,5 @@
 // Errors of the FP64 sweep's reciprocal square root and division
-// (drsqrt_newton, ddiv_newton in w5ct_physics.cuh) against the correctly
+// (drsqrt_newton, ddiv_newton, drcp_third in w5ct_physics.cuh) against the correctly
 // rounded 1 / sqrt(x) (from a quotient and one correction in twice the
 // working precision) and IEEE a / b, and of the exact scaling dscale2 and the
 // integer comparisons.  Prints the largest errors in units in the last place,
@@ -37,7 +37,7 @@ __global__ void check(long long n, unsigned long long *worst) {
         const double h = x * y, hl = fma(x, y, -h), e = fma(-h, y, 1.0) - hl * y;
         y = fma(0.5 * y, e, y);
         ws = max(ws, ulps(w5ct::drsqrt_newton(x), y));
-        wd = max(wd, ulps(w5ct::ddiv_newton(a, b), a / b));
+        wd = max(wd, max(ulps(w5ct::ddiv_newton(a, b), a / b), ulps(w5ct::drcp_third(x), 1.0 / x)));
         const double s = (r & 64) ? -a : a, t = (r2 & 64) ? -b : b;
         using m = w5ct::M<double>;
         bad += w5ct::dscale2<2>(s) != 4.0 * s;
