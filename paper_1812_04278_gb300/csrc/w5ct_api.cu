@@ -2,6 +2,7 @@
 // device memory, state transfer, the RK4 + CT step driver, reductions.
 #include <algorithm>
 #include <cstdarg>
+#include <cstdint>
 #include <cstdio>
 #include <cstring>
 #include <map>
@@ -84,6 +85,7 @@ struct w5ct_ctx {
     cudaStream_t cap_stream = nullptr;
     cudaGraphExec_t gexec = nullptr;
     long long graph_kernels = 0;
+    int *host_flag = nullptr;        // mapped host copy of the flag (store_state_kernel)
     // timing and accounting
     bool timing = false;
     std::vector<cudaEvent_t> ev;
@@ -703,6 +705,58 @@ int speeds_impl(w5ct_ctx *c, double *out) {
     return W5CT_OK;
 }
 
+// Whether [p, p + bytes) lies in one device allocation of the current device
+// and p is aligned to 8 bytes, so that a kernel may touch it.  Anything else
+// (another kind of memory, a range that runs past its allocation, an odd
+// address) goes through cudaMemcpyAsync, which takes it or returns an error.
+bool kernel_may_access(const void *p, size_t bytes) {
+    if (((uintptr_t)p & 7) != 0) return false;
+    cudaPointerAttributes at;
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || cudaPointerGetAttributes(&at, p) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    if (at.type != cudaMemoryTypeDevice || at.device != dev) return false;
+    using RangeFn = int (*)(unsigned long long *, size_t *, unsigned long long);
+    static const RangeFn range = [] {
+        void *f = nullptr;
+        cudaDriverEntryPointQueryResult r;
+        if (cudaGetDriverEntryPointByVersion("cuMemGetAddressRange", &f, 12000, cudaEnableDefault, &r) != cudaSuccess ||
+            r != cudaDriverEntryPointSuccess) {
+            cudaGetLastError();
+            f = nullptr;
+        }
+        return (RangeFn)f;
+    }();
+    unsigned long long base = 0;
+    size_t size = 0;
+    if (!range || range(&base, &size, (unsigned long long)(uintptr_t)p) != 0) return false;
+    return (unsigned long long)(uintptr_t)p + bytes <= base + size;
+}
+
+// what a synchronising call reports of the device flag
+int flag_status(w5ct_ctx *c, int flag) {
+    if (flag & 2) return fail(c, W5CT_ERR_TIMEOUT, "a wait of the fused step expired; the state is not valid");
+    if (flag) return fail(c, W5CT_ERR_NONPHYSICAL, "non-physical state (rho <= 0, P <= 0 or NaN) met in a step");
+    return W5CT_OK;
+}
+
+unsigned transfer_blocks(size_t np) {
+    const size_t nb = (np + 255) / 256;
+    return (unsigned)(nb < 16 * 152 ? nb : 16 * 152);
+}
+
+template <typename Real>
+int launch_load_state(w5ct_ctx *c, size_t off, size_t np, const double *cons, const double *bface, bool there) {
+    load_state_kernel<Real><<<transfer_blocks(np), 256, 0, c->stream>>>(
+        c->n, (long long)off, (long long)np, there ? c->q0 + off : cons, there ? c->b0 + off : bface, there, c->q0, c->b0,
+        (Real *)c->qs, (Real *)c->bs, (Real *)c->q0r, (Real *)c->b0r, c->flag, c->hits);
+    c->launches++;
+    W5_CUDA(c, cudaGetLastError());
+    return W5CT_OK;
+}
+
 int check_patch(w5ct_ctx *c, int patch) {
     if (patch < 0 || patch >= c->npatch) return fail(c, W5CT_ERR_ARG, "patch index %d out of range", patch);
     return W5CT_OK;
@@ -756,6 +810,7 @@ int w5ct_destroy(w5ct_ctx *c) {
     if (c->have_grid) cudaStreamSynchronize(c->stream);
     free_grid(c);
     if (c->cap_stream) cudaStreamDestroy(c->cap_stream);
+    if (c->host_flag) cudaFreeHost(c->host_flag);
     for (cudaEvent_t e : c->ev) cudaEventDestroy(e);
     delete c;
     return W5CT_OK;
@@ -905,42 +960,21 @@ int w5ct_set_state(w5ct_ctx *c, int patch, const double *cons, const double *bfa
     const PatchGeom g = patch_of(c, patch);
     const size_t np = (size_t)g.nx * g.ny * g.nz, off = (size_t)g.off;
     const cudaMemcpyKind kind = on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
-    if (c->npatch == 1) {
-        W5_CUDA(c, cudaMemcpyAsync(c->q0, cons, 5 * n * sizeof(double), kind, c->stream));
-        W5_CUDA(c, cudaMemcpyAsync(c->b0, bface, 3 * n * sizeof(double), kind, c->stream));
-    } else {
-        for (int f = 0; f < 5; ++f)
-            W5_CUDA(c, cudaMemcpyAsync(c->q0 + f * n + off, cons + f * np, np * sizeof(double), kind, c->stream));
-        for (int f = 0; f < 3; ++f)
-            W5_CUDA(c, cudaMemcpyAsync(c->b0 + f * n + off, bface + f * np, np * sizeof(double), kind, c->stream));
-    }
-    if (ctx_fp64(c)) {
-        for (int f = 0; f < 5; ++f)
-            W5_CUDA(c, cudaMemcpyAsync((double *)c->qs + f * n + off, c->q0 + f * n + off, np * 8,
-                                       cudaMemcpyDeviceToDevice, c->stream));
-        for (int f = 0; f < 3; ++f)
-            W5_CUDA(c, cudaMemcpyAsync((double *)c->bs + f * n + off, c->b0 + f * n + off, np * 8,
-                                       cudaMemcpyDeviceToDevice, c->stream));
-    } else {
-        long long nb = ((long long)np + 255) / 256;
-        if (nb > 8 * 152) nb = 8 * 152;
-        for (int f = 0; f < 5; ++f) {
-            to_real_kernel<float><<<(unsigned)nb, 256, 0, c->stream>>>((long long)np, c->q0 + f * n + off,
-                                                                      (float *)c->qs + f * n + off);
-            to_real_kernel<float><<<(unsigned)nb, 256, 0, c->stream>>>((long long)np, c->q0 + f * n + off,
-                                                                      (float *)c->q0r + f * n + off);
+    const bool direct = on_device && kernel_may_access(cons, 5 * np * 8) && kernel_may_access(bface, 3 * np * 8);
+    if (!direct) {
+        if (c->npatch == 1) {
+            W5_CUDA(c, cudaMemcpyAsync(c->q0, cons, 5 * n * sizeof(double), kind, c->stream));
+            W5_CUDA(c, cudaMemcpyAsync(c->b0, bface, 3 * n * sizeof(double), kind, c->stream));
+        } else {
+            for (int f = 0; f < 5; ++f)
+                W5_CUDA(c, cudaMemcpyAsync(c->q0 + f * n + off, cons + f * np, np * sizeof(double), kind, c->stream));
+            for (int f = 0; f < 3; ++f)
+                W5_CUDA(c, cudaMemcpyAsync(c->b0 + f * n + off, bface + f * np, np * sizeof(double), kind, c->stream));
         }
-        for (int f = 0; f < 3; ++f) {
-            to_real_kernel<float><<<(unsigned)nb, 256, 0, c->stream>>>((long long)np, c->b0 + f * n + off,
-                                                                      (float *)c->bs + f * n + off);
-            to_real_kernel<float><<<(unsigned)nb, 256, 0, c->stream>>>((long long)np, c->b0 + f * n + off,
-                                                                      (float *)c->b0r + f * n + off);
-        }
-        c->launches += 16;
-        W5_CUDA(c, cudaGetLastError());
     }
-    W5_CUDA(c, cudaMemsetAsync(c->flag, 0, 4, c->stream));
-    W5_CUDA(c, cudaMemsetAsync(c->hits, 0, 8, c->stream));
+    const int rc = ctx_fp64(c) ? launch_load_state<double>(c, off, np, cons, bface, !direct)
+                               : launch_load_state<float>(c, off, np, cons, bface, !direct);
+    if (rc) return rc;
     if (!on_device) W5_CUDA(c, cudaStreamSynchronize(c->stream));
     c->have_state = true;
     return W5CT_OK;
@@ -954,6 +988,18 @@ int w5ct_get_state(w5ct_ctx *c, int patch, double *cons, double *bface, double *
     const PatchGeom g = patch_of(c, patch);
     const size_t np = (size_t)g.nx * g.ny * g.nz, off = (size_t)g.off;
     const cudaMemcpyKind kind = on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost;
+    if (on_device && !bcell && (!cons || kernel_may_access(cons, 5 * np * 8)) &&
+        (!bface || kernel_may_access(bface, 3 * np * 8))) {
+        if (!c->host_flag) W5_CUDA(c, cudaHostAlloc(&c->host_flag, sizeof(int), cudaHostAllocMapped));
+        int *hf = nullptr;
+        W5_CUDA(c, cudaHostGetDevicePointer(&hf, c->host_flag, 0));
+        store_state_kernel<<<transfer_blocks(np), 256, 0, c->stream>>>(c->n, (long long)off, (long long)np, c->q0, c->b0,
+                                                                      cons, bface, c->flag, hf);
+        c->launches++;
+        W5_CUDA(c, cudaGetLastError());
+        W5_CUDA(c, cudaStreamSynchronize(c->stream));
+        return flag_status(c, *(volatile int *)c->host_flag);
+    }
     if (cons)
         for (int f = 0; f < 5; ++f)
             W5_CUDA(c, cudaMemcpyAsync(cons + f * np, c->q0 + f * n + off, np * 8, kind, c->stream));
@@ -973,9 +1019,7 @@ int w5ct_get_state(w5ct_ctx *c, int patch, double *cons, double *bface, double *
     int flag = 0;
     rc = read_flag(c, &flag);
     if (rc) return rc;
-    if (flag & 2) return fail(c, W5CT_ERR_TIMEOUT, "a wait of the fused step expired; the state is not valid");
-    if (flag) return fail(c, W5CT_ERR_NONPHYSICAL, "non-physical state (rho <= 0, P <= 0 or NaN) met in a step");
-    return W5CT_OK;
+    return flag_status(c, flag);
 }
 
 int w5ct_step(w5ct_ctx *c, double dt) {

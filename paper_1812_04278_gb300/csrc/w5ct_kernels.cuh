@@ -882,11 +882,63 @@ static __global__ void __launch_bounds__(kRedThreads) finalize_kernel(const doub
         for (int q = 0; q < nval; ++q) out[q] = v[q];
 }
 
-// double -> Real copy of a plane
+// ======================================================================
+// state transfer
+// ======================================================================
+
+// The state of one patch (np cells at `off` of n-cell planes) into every
+// buffer a step reads: q0, b0 in double, the stage state in the arithmetic
+// type and, in float, the float copies of q^n, b^n; the floor counter and the
+// non-physical flag are cleared.  cons / bface: the caller's planes, or q0 +
+// off / b0 + off with plane stride n when a copy has already put them there
+// (`there`).  One pass over HBM (float: 8 B read, 16 B written per value)
+// instead of 8 copies and 16 conversions: 512^3 FP32-bulk 8.0 -> 4.2 ms, and
+// one launch per patch of a batch instead of 26 operations.
 template <typename Real>
-__global__ void __launch_bounds__(256) to_real_kernel(long long n, const double *src, Real *dst) {
-    for (long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x; p < n; p += (long long)gridDim.x * blockDim.x)
-        dst[p] = (Real)src[p];
+__global__ void __launch_bounds__(256) load_state_kernel(long long n, long long off, long long np, const double *cons,
+                                                         const double *bface, bool there, double *q0, double *b0,
+                                                         Real *qs, Real *bs, Real *q0r, Real *b0r, int *flag,
+                                                         unsigned long long *hits) {
+    constexpr bool kCopy = !std::is_same<Real, double>::value;
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        *flag = 0;
+        *hits = 0;
+    }
+    const long long st = there ? n : np;
+    for (long long i = blockIdx.x * 256LL + threadIdx.x; i < np; i += 256LL * gridDim.x) {
+        double v[8];
+#pragma unroll
+        for (int f = 0; f < 5; ++f) v[f] = cons[f * st + i];
+#pragma unroll
+        for (int f = 0; f < 3; ++f) v[5 + f] = bface[f * st + i];
+#pragma unroll
+        for (int f = 0; f < 8; ++f) {
+            const long long o = (f < 5 ? f : f - 5) * n + off + i;
+            const Real r = from_double<Real>(v[f]);
+            if (!there) (f < 5 ? q0 : b0)[o] = v[f];
+            (f < 5 ? qs : bs)[o] = r;
+            if (kCopy) (f < 5 ? q0r : b0r)[o] = r;
+        }
+    }
+}
+
+// The state of one patch into the caller's device planes (either may be
+// NULL), and the non-physical flag into mapped host memory: one launch
+// instead of 9 copies.
+static __global__ void __launch_bounds__(256) store_state_kernel(long long n, long long off, long long np,
+                                                                 const double *__restrict__ q0,
+                                                                 const double *__restrict__ b0, double *cons,
+                                                                 double *bface, const int *flag, int *host_flag) {
+    if (blockIdx.x == 0 && threadIdx.x == 0) *host_flag = *flag;
+    for (long long i = blockIdx.x * 256LL + threadIdx.x; i < np; i += 256LL * gridDim.x) {
+        double v[8];
+#pragma unroll
+        for (int f = 0; f < 8; ++f)
+            if (f < 5 ? cons != nullptr : bface != nullptr) v[f] = (f < 5 ? q0 : b0)[(f < 5 ? f : f - 5) * n + off + i];
+#pragma unroll
+        for (int f = 0; f < 8; ++f)
+            if (f < 5 ? cons != nullptr : bface != nullptr) (f < 5 ? cons : bface)[(f < 5 ? f : f - 5) * np + i] = v[f];
+    }
 }
 
 }  // namespace w5ct
