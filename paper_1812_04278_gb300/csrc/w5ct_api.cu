@@ -50,7 +50,6 @@ struct w5ct_ctx {
     unsigned long long *hits = nullptr;
     double *part = nullptr;          // kRedBlocks x 8
     double *red_out = nullptr;       // 8
-    const double **planes = nullptr; // 8 device pointers
     // several patches (npatch > 1): planes hold the patches back to back
     int npatch = 0;
     std::vector<PatchGeom> pg;       // host copy of the patch table
@@ -311,9 +310,9 @@ int launch_speed(w5ct_ctx *c) {
             plane<Real>(c->bc, n, 2), make_phys<Real>(c->cfg), c->smax, c->flag);
     } else {
         long long nb = (n + kRedThreads - 1) / kRedThreads;
-        if (nb > 4 * 152) nb = 4 * 152;
+        if (nb > 8 * 152) nb = 8 * 152;
         speed_kernel<Real><<<(unsigned)nb, kRedThreads, 0, c->stream>>>(
-            n, c->nx, c->ny, plane<Real>(c->qs, n, 0), plane<Real>(c->qs, n, 1), plane<Real>(c->qs, n, 2),
+            n, plane<Real>(c->qs, n, 0), plane<Real>(c->qs, n, 1), plane<Real>(c->qs, n, 2),
             plane<Real>(c->qs, n, 3), plane<Real>(c->qs, n, 4), plane<Real>(c->bc, n, 0), plane<Real>(c->bc, n, 1),
             plane<Real>(c->bc, n, 2), make_phys<Real>(c->cfg), c->smax, c->flag);
     }
@@ -887,7 +886,7 @@ int w5ct_init_grid(w5ct_ctx *c, int npatch, const int *n3, const double *dx3) {
     const size_t o_q0r = fp32 ? take(5 * n * rs) : 0, o_b0r = fp32 ? take(3 * n * rs) : 0;
     const size_t np = (size_t)npatch;
     const size_t o_dt = take(8 * np), o_smax = take(24 * np), o_flag = take(4), o_hits = take(8);
-    const size_t o_part = take((size_t)kRedBlocks * 8 * 8), o_red = take(64), o_pl = take(64);
+    const size_t o_part = take((size_t)kRedBlocks * 8 * 8), o_red = take(64);
     const size_t o_pg = take(sizeof(PatchGeom) * np);
     const size_t o_pc = take(sizeof(int) * 4 * kMaxTileVariants);
     size_t o_cells = 0;
@@ -918,7 +917,6 @@ int w5ct_init_grid(w5ct_ctx *c, int npatch, const int *n3, const double *dx3) {
     c->hits = (unsigned long long *)(b + o_hits);
     c->part = (double *)(b + o_part);
     c->red_out = (double *)(b + o_red);
-    c->planes = (const double **)(b + o_pl);
     c->pg_dev = (PatchGeom *)(b + o_pg);
     c->pcounters = (int *)(b + o_pc);
     W5_CUDA(c, cudaMemcpy(c->pg_dev, c->pg.data(), sizeof(PatchGeom) * np, cudaMemcpyHostToDevice));
@@ -1116,11 +1114,10 @@ int w5ct_conserved_totals(w5ct_ctx *c, int patch, double out[8]) {
     const PatchGeom g = patch_of(c, patch);
     const size_t off = (size_t)g.off;
     const long long np = (long long)g.nx * g.ny * g.nz;
-    const double *pl[8];
-    for (int f = 0; f < 5; ++f) pl[f] = c->q0 + f * n + off;
-    for (int f = 0; f < 3; ++f) pl[5 + f] = c->b0 + f * n + off;
-    W5_CUDA(c, cudaMemcpyAsync((void *)c->planes, pl, sizeof(pl), cudaMemcpyHostToDevice, c->stream));
-    sums_partial_kernel<<<kRedBlocks, kRedThreads, 0, c->stream>>>(np, 8, c->planes, c->part);
+    Planes8 pl;
+    for (int f = 0; f < 5; ++f) pl.p[f] = c->q0 + f * n + off;
+    for (int f = 0; f < 3; ++f) pl.p[5 + f] = c->b0 + f * n + off;
+    sums_partial_kernel<<<kRedBlocks, kRedThreads, 0, c->stream>>>(np, pl, c->part);
     finalize_kernel<<<1, kRedThreads, 0, c->stream>>>(c->part, kRedBlocks, 8, 8, 0u, c->red_out);
     c->launches += 2;
     W5_CUDA(c, cudaGetLastError());

@@ -216,10 +216,9 @@ __device__ __forceinline__ void fused_cellb(const PatchGeom &g, int i, int j, in
                     yp1 = (wrapi(j + 1, g.ny) - j) * sy;
     const long long zm2 = (wrapi(k - 2, g.nz) - k) * sz, zm1 = (wrapi(k - 1, g.nz) - k) * sz,
                     zp1 = (wrapi(k + 1, g.nz) - k) * sz;
-    const Real s = Real(1.0 / 16.0);
-    Bx[p] = (Real(9) * (bx[p + xm1] + bx[p]) - (bx[p + xm2] + bx[p + xp1])) * s;
-    By[p] = (Real(9) * (by[p + ym1] + by[p]) - (by[p + ym2] + by[p + yp1])) * s;
-    Bz[p] = (Real(9) * (bz[p + zm1] + bz[p]) - (bz[p + zm2] + bz[p + zp1])) * s;
+    Bx[p] = face_to_cell<Real>(bx[p + xm2], bx[p + xm1], bx[p], bx[p + xp1]);
+    By[p] = face_to_cell<Real>(by[p + ym2], by[p + ym1], by[p], by[p + yp1]);
+    Bz[p] = face_to_cell<Real>(bz[p + zm2], bz[p + zm1], bz[p], bz[p + zp1]);
 }
 
 template <typename Real, int VAR>
@@ -318,7 +317,7 @@ __global__ void __launch_bounds__(FusedBlock<Real>::NT, FusedBlock<Real>::MINB) 
                 done = C.cellb(stage, p);
             } else if (type == FI_SPEED) {
                 if (A.cfl) {
-                    double v[3] = {0.0, 0.0, 0.0};
+                    Real v[3] = {Real(0), Real(0), Real(0)};
                     bool bad = false;
 #pragma unroll 1
                     for (int r = 0; r < kFusedCells / NT; ++r) {
@@ -331,22 +330,7 @@ __global__ void __launch_bounds__(FusedBlock<Real>::NT, FusedBlock<Real>::MINB) 
                         }
                     }
                     if (bad) atomicOr(A.a[0].flag, 1);
-                    // maxima over the block's NT / 32 warps
-#pragma unroll
-                    for (int d = 0; d < 3; ++d)
-#pragma unroll
-                        for (int o = 16; o > 0; o >>= 1) v[d] = fmax(v[d], __shfl_xor_sync(0xffffffffu, v[d], o));
-                    if ((tid & 31) == 0)
-                        for (int d = 0; d < 3; ++d) s_red[d * 32 + (tid >> 5)] = v[d];
-                    __syncthreads();
-                    if (tid < 32) {
-                        for (int d = 0; d < 3; ++d) {
-                            double x = tid < NT / 32 ? s_red[d * 32 + tid] : 0.0;
-#pragma unroll
-                            for (int o = 16; o > 0; o >>= 1) x = fmax(x, __shfl_xor_sync(0xffffffffu, x, o));
-                            if (tid == 0) atomicMax(&A.smax[3 * p + d], (unsigned long long)__double_as_longlong(x));
-                        }
-                    }
+                    block_speeds<Real, NT / 32>(v, reinterpret_cast<Real *>(s_red), tid, A.smax + 3 * (size_t)p);
                 }
                 done = C.speed(p);
             } else {

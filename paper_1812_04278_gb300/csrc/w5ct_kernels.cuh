@@ -299,6 +299,14 @@ __global__ void __launch_bounds__(SweepTile<AX, T2, BX, FPT>::NT, MINB)
 // cell-centred field: fourth-order interpolation of the faces (Sec. 2.3)
 // ======================================================================
 
+// (9 (f_{-1/2} + f_{1/2}) - (f_{-3/2} + f_{3/2})) / 16: in double 3 FP64
+// instructions, the scaling of the outer sum being exact on the integer pipes
+template <typename Real>
+__device__ __forceinline__ Real face_to_cell(Real fm3, Real fm1, Real fp1, Real fp3) {
+    using m = M<Real>;
+    return m::fma_(Real(9.0 / 16.0), fm1 + fp1, -m::sixteenth_(fm3 + fp3));
+}
+
 template <typename Real>
 __device__ __forceinline__ void cellb_cell(int nx, int ny, int nz, size_t off, int i, int j, int k,
                                            const Real *__restrict__ bx, const Real *__restrict__ by,
@@ -311,10 +319,9 @@ __device__ __forceinline__ void cellb_cell(int nx, int ny, int nz, size_t off, i
     const long long xm2 = wrapi(i - 2, nx) - i, xm1 = wrapi(i - 1, nx) - i, xp1 = wrapi(i + 1, nx) - i;
     const long long ym2 = (wrapi(j - 2, ny) - j) * sy, ym1 = (wrapi(j - 1, ny) - j) * sy, yp1 = (wrapi(j + 1, ny) - j) * sy;
     const long long zm2 = (wrapi(k - 2, nz) - k) * sz, zm1 = (wrapi(k - 1, nz) - k) * sz, zp1 = (wrapi(k + 1, nz) - k) * sz;
-    const Real s = Real(1.0 / 16.0);
-    Bx[p] = (Real(9) * (bx[p + xm1] + bx[p]) - (bx[p + xm2] + bx[p + xp1])) * s;
-    By[p] = (Real(9) * (by[p + ym1] + by[p]) - (by[p + ym2] + by[p + yp1])) * s;
-    Bz[p] = (Real(9) * (bz[p + zm1] + bz[p]) - (bz[p + zm2] + bz[p + zp1])) * s;
+    Bx[p] = face_to_cell<Real>(bx[p + xm2], bx[p + xm1], bx[p], bx[p + xp1]);
+    By[p] = face_to_cell<Real>(by[p + ym2], by[p + ym1], by[p], by[p + yp1]);
+    Bz[p] = face_to_cell<Real>(bz[p + zm2], bz[p + zm1], bz[p], bz[p + zp1]);
 }
 
 // The cell field of one patch: a block of 32 x 8 (x, y) columns marches
@@ -347,15 +354,14 @@ __global__ void __launch_bounds__(256) cellb_kernel(int nx, int ny, int nz, int 
     const long long xm2 = wrapi(i - 2, nx) - i, xm1 = wrapi(i - 1, nx) - i, xp1 = wrapi(i + 1, nx) - i;
     const long long ym2 = (wrapi(j - 2, ny) - j) * sy, ym1 = (wrapi(j - 1, ny) - j) * sy, yp1 = (wrapi(j + 1, ny) - j) * sy;
     const long long col = i + sy * j;
-    const Real s = Real(1.0 / 16.0);
     Real z0 = bz[col + sz * wrapi(k0 - 2, nz)], z1 = bz[col + sz * wrapi(k0 - 1, nz)], z2 = bz[col + sz * k0];
 #pragma unroll 4
     for (int k = k0; k < k1; ++k) {
         const long long p = col + sz * k;
         const Real z3 = bz[col + sz * (k + 1 < nz ? k + 1 : 0)];
-        Bx[p] = (Real(9) * (bx[p + xm1] + bx[p]) - (bx[p + xm2] + bx[p + xp1])) * s;
-        By[p] = (Real(9) * (by[p + ym1] + by[p]) - (by[p + ym2] + by[p + yp1])) * s;
-        Bz[p] = (Real(9) * (z1 + z2) - (z0 + z3)) * s;
+        Bx[p] = face_to_cell<Real>(bx[p + xm2], bx[p + xm1], bx[p], bx[p + xp1]);
+        By[p] = face_to_cell<Real>(by[p + ym2], by[p + ym1], by[p], by[p + yp1]);
+        Bz[p] = face_to_cell<Real>(z0, z1, z2, z3);
         z0 = z1;
         z1 = z2;
         z2 = z3;
@@ -653,7 +659,7 @@ __global__ void __launch_bounds__(256, UpdTuning<Real>::MINB) update_kernel(Upda
 // Several patches: block b updates the cells of cell block cells[b] (see
 // cell_of_block) with that patch's dt, dts[patch].
 template <typename Real, int STAGE>
-__global__ void __launch_bounds__(kCellBlock, W5CT_UPD_MINB) update_batched_kernel(UpdateArgs<Real> a,
+__global__ void __launch_bounds__(kCellBlock, UpdTuning<Real>::MINB) update_batched_kernel(UpdateArgs<Real> a,
                                                                                    const PatchGeom *__restrict__ pgs,
                                                                                    const int4 *__restrict__ cells,
                                                                                    const double *__restrict__ dts) {
@@ -704,41 +710,203 @@ __device__ __forceinline__ void block_reduce(T (&v)[N], bool is_max[N], T *red /
     }
 }
 
-// |v_d| + c_f^d of one cell for d = x, y, z folded into v (Eq. cfl)
-template <typename Real>
-__device__ __forceinline__ void cell_speeds(Real r, Real m0, Real m1, Real m2, Real E, Real bx, Real by, Real bz,
-                                            const Phys<Real> &K, double (&v)[3], bool &bad) {
-    if (K.floors && r < K.rho_min) r = K.rho_min;
-    const Real ir = M<Real>::rcp_(r);
-    const Real vx = m0 * ir, vy = m1 * ir, vz = m2 * ir;
-    Real P = K.gm1 * (E - Real(0.5) * r * (vx * vx + vy * vy + vz * vz) - Real(0.5) * (bx * bx + by * by + bz * bz));
-    if (K.floors && P < K.p_min) P = K.p_min;
-    if (!(r > Real(0)) || !M<Real>::finite_pos(P)) bad = true;
-    v[0] = fmax(v[0], (double)signal_speed<Real>(r, vx, P, bx, by, bz, K));
-    v[1] = fmax(v[1], (double)signal_speed<Real>(r, vy, P, by, bz, bx, K));
-    v[2] = fmax(v[2], (double)signal_speed<Real>(r, vz, P, bz, bx, by, K));
+// fast signal speed |v_n| + c_f of a cell along one axis (Eq. cfl), float
+__device__ __forceinline__ float signal_speed(float r, float vn, float P, float Bn, float B1, float B2,
+                                              const Phys<float> &K) {
+    using m = M<float>;
+    const float ir = m::rcp_(r);
+    const float cs2 = K.gamma * P * ir;
+    const float ca2 = Bn * Bn * ir;
+    const float bt2 = (B1 * B1 + B2 * B2) * ir;
+    const float dd = (cs2 - ca2) * (cs2 - ca2) + bt2 * (bt2 + 2.0f * ca2 + 2.0f * cs2);
+    const float sd = m::sqrt_(dd);
+    const float aa = ca2 + bt2 - cs2;
+    const float big = 0.5f * (sd + m::abs_(aa));
+    const float oth = big > 0.0f ? m::div_(cs2 * bt2, big) : 0.0f;
+    const float cf2 = cs2 + (aa >= 0.0f ? big : oth);
+    return m::abs_(vn) + m::sqrt_(cf2);
 }
 
-// |v_d| + c_f^d maxima of the stage state (Eq. cfl)
+// |v_d| + c_f^d of one cell for d = x, y, z folded into v (Eq. cfl); a NaN is
+// dropped (bad is set).  In double the squares and reciprocals are shared by
+// the three axes (110 FP64 instructions instead of 180).
 template <typename Real>
-__global__ void __launch_bounds__(kRedThreads) speed_kernel(long long n, int nx, int ny, const Real *q0, const Real *q1,
-                                                            const Real *q2, const Real *q3, const Real *q4,
-                                                            const Real *B0, const Real *B1, const Real *B2,
-                                                            Phys<Real> K, unsigned long long *smax, int *flag) {
-    __shared__ double red[3 * 32];
-    double v[3] = {0.0, 0.0, 0.0};
-    bool bad = false;
-    for (long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x; p < n; p += (long long)gridDim.x * blockDim.x)
-        cell_speeds<Real>(q0[p], q1[p], q2[p], q3[p], q4[p], B0[p], B1[p], B2[p], K, v, bad);
-    if (bad) atomicOr(flag, 1);
-    bool ismax[3] = {true, true, true};
-    block_reduce<double, 3>(v, ismax, red);
-    if (threadIdx.x == 0) {
-        // non-negative doubles order like their bit patterns
-        atomicMax(&smax[0], (unsigned long long)__double_as_longlong(v[0]));
-        atomicMax(&smax[1], (unsigned long long)__double_as_longlong(v[1]));
-        atomicMax(&smax[2], (unsigned long long)__double_as_longlong(v[2]));
+__device__ __forceinline__ void cell_speeds(Real r, Real m0, Real m1, Real m2, Real E, Real bx, Real by, Real bz,
+                                            const Phys<Real> &K, Real (&v)[3], bool &bad) {
+    using m = M<Real>;
+    if (K.floors && r < K.rho_min) r = K.rho_min;
+    if constexpr (float_based<Real>) {
+        const Real ir = m::rcp_(r);
+        const Real vx = m0 * ir, vy = m1 * ir, vz = m2 * ir;
+        Real P = K.gm1 * (E - Real(0.5) * r * (vx * vx + vy * vy + vz * vz) - Real(0.5) * (bx * bx + by * by + bz * bz));
+        if (K.floors && P < K.p_min) P = K.p_min;
+        if (!(r > Real(0)) || !m::finite_pos(P)) bad = true;
+        v[0] = fmaxf(v[0], signal_speed(r, vx, P, bx, by, bz, K));
+        v[1] = fmaxf(v[1], signal_speed(r, vy, P, by, bz, bx, K));
+        v[2] = fmaxf(v[2], signal_speed(r, vz, P, bz, bx, by, K));
+    } else {
+        const Real ir = m::rcp3_(r);
+        const Real u[3] = {m0 * ir, m1 * ir, m2 * ir};
+        const Real B2[3] = {bx * bx, by * by, bz * bz};
+        Real P = K.gm1 * (E - Real(0.5) * (r * (u[0] * u[0] + u[1] * u[1] + u[2] * u[2]) + (B2[0] + B2[1] + B2[2])));
+        if (K.floors && P < K.p_min) P = K.p_min;
+        if (!(r > Real(0)) || !m::finite_pos(P)) bad = true;
+        const Real cs2 = K.gamma * P * ir;
+        const Real a2[3] = {B2[0] * ir, B2[1] * ir, B2[2] * ir};
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+            Real fmc, cms, cf2;
+            speeds_fast<Real>(cs2, a2[d], a2[(d + 1) % 3] + a2[(d + 2) % 3], fmc, cms, cf2);
+            const Real s = m::abs_(u[d]) + cf2 * m::rsqrt_(cf2);
+            v[d] = s > v[d] ? s : v[d];
+        }
     }
+}
+
+// non-negative floats and doubles order like their bit patterns: maxima on
+// the integer pipes
+__device__ __forceinline__ float warp_max(float v) {
+    return __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(v)));
+}
+__device__ __forceinline__ double warp_max(double v) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v = dmax_nonneg(v, __shfl_xor_sync(0xffffffffu, v, o));
+    return v;
+}
+
+// the block's maxima (NW warps) into smax[0..2] (bits of doubles)
+template <typename Real, int NW>
+__device__ __forceinline__ void block_speeds(const Real (&v)[3], Real *red /* 3 x NW */, int tid,
+                                             unsigned long long *smax) {
+#pragma unroll
+    for (int q = 0; q < 3; ++q) {
+        const Real x = warp_max(v[q]);
+        if ((tid & 31) == 0) red[q * NW + (tid >> 5)] = x;
+    }
+    __syncthreads();
+    if (tid < 3) {
+        Real x = red[tid * NW];
+        for (int w = 1; w < NW; ++w) x = M<Real>::max_nonneg(x, red[tid * NW + w]);
+        atomicMax(&smax[tid], (unsigned long long)__double_as_longlong((double)x));
+    }
+}
+
+// x truncated to a float (24 significant bits) on the integer pipes; below
+// float's normal range 0, above it an infinity
+__device__ __forceinline__ float d2f_trunc(double x) {
+    const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
+    const int e = (int)((hi >> 20) & 0x7ffu) - 896;
+    unsigned b = (hi & 0x80000000u) | ((unsigned)e << 23) | (__funnelshift_l(lo, hi, 3) & 0x7fffffu);
+    b = e <= 0 ? 0u : e >= 255 ? (hi & 0x80000000u) | 0x7f800000u : b;
+    return __uint_as_float(b);
+}
+
+// Float bounds on a cell's double signal speeds: S_d lies in [lo[d], up[d]].
+// Returns false where float cannot tell (a pressure that is a small
+// difference, a state that is not physical or out of float's range).
+// With h = 2^-18, more than 8 float roundings (inputs truncated to 2^-23,
+// then at most 8 operations each on positive terms): the pressure is off by
+// at most h (gamma - 1)(|E| + kinetic + magnetic energy) =: ep P, v, c_A^2 and
+// b_t^2 by h.  c_f^2 is increasing and homogeneous of degree 1 in (c_s^2,
+// c_A^2, b_t^2), so it is off by at most a factor 1 + ep + 2 h, plus h for its
+// own evaluation, whose error is a few roundings of c_s^2 + c_A^2 + b_t^2 <= 2 c_f^2.
+struct FloatPhys {
+    float gamma, gm1, rho_min, p_min;   // rho_min, p_min: 0 without floors
+};
+__device__ __forceinline__ bool float_speeds(const double (&q)[8], const FloatPhys &K, float (&lo)[3], float (&up)[3]) {
+    const float h = 3.8146973e-6f;
+    const float r = fmaxf(d2f_trunc(q[0]), K.rho_min);
+    const float gm1 = K.gm1;
+    const float ir = __fdividef(1.0f, r);
+    float u[3], a2[3], ke = 0.0f, me = 0.0f;
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+        const float m = d2f_trunc(q[1 + d]), b = d2f_trunc(q[5 + d]);
+        u[d] = m * ir;
+        ke = __fmaf_rn(m, u[d], ke);
+        me = __fmaf_rn(b, b, me);
+        a2[d] = b * b * ir;
+    }
+    const float E = d2f_trunc(q[4]), half = 0.5f * (ke + me);
+    const float P = fmaxf(gm1 * (E - half), K.p_min);
+    const float ep = h * gm1 * (fabsf(E) + half) / P;
+    const bool ok = r > 1e-30f && r < 1e30f && P > 1e-30f && P < 1e30f && ep < 0.25f;
+    const float cs2 = K.gamma * P * ir;
+    const float w = ep + 4.0f * h;
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+        const float ca2 = a2[d], bt2 = a2[(d + 1) % 3] + a2[(d + 2) % 3];
+        const float aa = ca2 + bt2 - cs2;
+        const float cf2 = 0.5f * (cs2 + ca2 + bt2 + sqrtf(__fmaf_rn(aa, aa, 4.0f * cs2 * bt2)));
+        const float s = fabsf(u[d]) + sqrtf(cf2);
+        lo[d] = ok ? s * (1.0f - w) : 0.0f;
+        up[d] = s * (1.0f + w);
+    }
+    return ok && up[0] < 1e18f && up[1] < 1e18f && up[2] < 1e18f;
+}
+
+// |v_d| + c_f^d maxima of the stage state (Eq. cfl).  In float HBM-bound.  In
+// double the FP64 pipe would bound it (about 110 instructions per cell: 3.9
+// ms at 256^3 with 180 of them, where reading the 8 planes takes 0.16 ms), so
+// a cell is evaluated in double only if its float upper bound reaches the
+// largest float lower bound its warp has met and the largest value any warp
+// has published; the maxima are those of all cells.  256^3: 3.93 -> 0.24 ms.
+template <typename Real>
+__global__ void __launch_bounds__(kRedThreads, 4) speed_kernel(long long n, const Real *q0, const Real *q1, const Real *q2,
+                                                            const Real *q3, const Real *q4, const Real *B0,
+                                                            const Real *B1, const Real *B2, Phys<Real> K,
+                                                            unsigned long long *smax, int *flag) {
+    [[maybe_unused]] __shared__ Real red[3 * 8];
+    Real v[3] = {Real(0), Real(0), Real(0)};
+    [[maybe_unused]] float top[3] = {0.0f, 0.0f, 0.0f};
+    [[maybe_unused]] unsigned long long s[3] = {0, 0, 0};
+    [[maybe_unused]] int it = 0;
+    bool bad = false;
+    [[maybe_unused]] const FloatPhys KF = {(float)K.gamma, (float)K.gm1, K.floors ? (float)K.rho_min : 0.0f,
+                                           K.floors ? (float)K.p_min : 0.0f};
+    // whole warps iterate together (the bounds are shared by shuffles)
+    for (long long p0 = (blockIdx.x * (long long)blockDim.x + threadIdx.x) & ~31LL; p0 < n;
+         p0 += (long long)gridDim.x * blockDim.x) {
+        const long long p = p0 + (threadIdx.x & 31);
+        const bool in = p < n;
+        const long long c = in ? p : n - 1;
+        const Real q[8] = {q0[c], q1[c], q2[c], q3[c], q4[c], B0[c], B1[c], B2[c]};
+        bool eval = in;
+        if constexpr (std::is_same<Real, double>::value) {
+            // the largest published values so far (truncated: a lower bound),
+            // read in iterations 0, 1, 2, 4, 8, ... (every warp reads the same
+            // three words, and their L2 slice would bound the kernel)
+            if ((it & (it - 1)) == 0)
+#pragma unroll
+                for (int d = 0; d < 3; ++d) {
+                    s[d] = __ldcg(smax + d);
+                    top[d] = fmaxf(top[d], d2f_trunc(__longlong_as_double((long long)s[d])));
+                }
+            ++it;
+            float lo[3], up[3];
+            const bool ok = float_speeds(q, KF, lo, up);
+            eval = !ok;
+#pragma unroll
+            for (int d = 0; d < 3; ++d) {
+                top[d] = fmaxf(top[d], warp_max(lo[d]));
+                eval = eval || !(up[d] < top[d]);
+            }
+            eval = eval && in;
+            if (__any_sync(0xffffffffu, eval)) {
+                if (eval) cell_speeds<Real>(q[0], q[1], q[2], q[3], q[4], q[5], q[6], q[7], K, v, bad);
+#pragma unroll
+                for (int d = 0; d < 3; ++d) {
+                    const double x = warp_max(v[d]);
+                    const unsigned long long b = (unsigned long long)__double_as_longlong(x);
+                    if ((threadIdx.x & 31) == 0 && b > s[d]) atomicMax(smax + d, b);
+                }
+            }
+        } else if (eval) {
+            cell_speeds<Real>(q[0], q[1], q[2], q[3], q[4], q[5], q[6], q[7], K, v, bad);
+        }
+    }
+    if (bad) atomicOr(flag, 1);
+    if constexpr (!std::is_same<Real, double>::value) block_speeds<Real, kRedThreads / 32>(v, red, threadIdx.x, smax);
 }
 
 // Several patches: block b covers the cells of cell block cells[b] (see
@@ -751,10 +919,11 @@ __global__ void __launch_bounds__(kCellBlock) speed_batched_kernel(const PatchGe
                                                                    const Real *q4, const Real *B0, const Real *B1,
                                                                    const Real *B2, Phys<Real> K,
                                                                    unsigned long long *smax, int *flag) {
+    __shared__ Real red[3 * 8];
     const int4 t = cells[blockIdx.x];
     const PatchGeom pg = pgs[t.x];
     const int tid = threadIdx.x;
-    double v[3] = {0.0, 0.0, 0.0};
+    Real v[3] = {Real(0), Real(0), Real(0)};
     bool bad = false;
     if (t.y + tid < pg.nx * pg.ny * pg.nz) {
         // storage order: the block's cells are consecutive in the patch
@@ -762,24 +931,7 @@ __global__ void __launch_bounds__(kCellBlock) speed_batched_kernel(const PatchGe
         cell_speeds<Real>(q0[p], q1[p], q2[p], q3[p], q4[p], B0[p], B1[p], B2[p], K, v, bad);
     }
     if (bad) atomicOr(flag, 1);
-    // block maxima over the 8 warps of the 256-thread block
-    __shared__ double red2[3 * 32];
-#pragma unroll
-    for (int q = 0; q < 3; ++q)
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) v[q] = fmax(v[q], __shfl_xor_sync(0xffffffffu, v[q], o));
-    if ((tid & 31) == 0)
-        for (int q = 0; q < 3; ++q) red2[q * 32 + (tid >> 5)] = v[q];
-    __syncthreads();
-    if (tid < 32) {
-#pragma unroll
-        for (int q = 0; q < 3; ++q) {
-            double x = tid < 8 ? red2[q * 32 + tid] : 0.0;
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) x = fmax(x, __shfl_xor_sync(0xffffffffu, x, o));
-            if (tid == 0) atomicMax(&smax[3 * t.x + q], (unsigned long long)__double_as_longlong(x));
-        }
-    }
+    block_speeds<Real, kCellBlock / 32>(v, red, tid, smax + 3 * (size_t)t.x);
 }
 
 // dt of every patch, as dt_kernel: dts[p] = CFL / sum_d (S_d / dx_d)
@@ -825,14 +977,24 @@ static __global__ void __launch_bounds__(kRedThreads) divb_partial_kernel(int nx
     const long long n = (long long)nx * ny * nz;
     double v[2] = {0.0, 0.0};
     for (long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x; p < n; p += (long long)gridDim.x * blockDim.x) {
-        const int i = (int)(p % nx);
-        const long long r = p / nx;
-        const int j = (int)(r % ny), k = (int)(r / ny);
+        // (a 64-bit division costs more than the rest of the cell)
+        int i, j, k;
+        if (n <= 0x7fffffffLL) {
+            const unsigned r = (unsigned)p / (unsigned)nx;
+            i = (int)((unsigned)p - r * (unsigned)nx);
+            k = (int)(r / (unsigned)ny);
+            j = (int)(r - (unsigned)k * (unsigned)ny);
+        } else {
+            const long long r = p / nx;
+            i = (int)(p - r * nx);
+            k = (int)(r / ny);
+            j = (int)(r - (long long)k * ny);
+        }
         const long long pxm = p - i + (i > 0 ? i - 1 : nx - 1);
         const long long pym = p + (long long)nx * ((j > 0 ? j - 1 : ny - 1) - j);
         const long long pzm = p + (long long)nx * ny * ((k > 0 ? k - 1 : nz - 1) - k);
         const double d = (bx[p] - bx[pxm]) * rdx + (by[p] - by[pym]) * rdy + (bz[p] - bz[pzm]) * rdz;
-        v[0] = fmax(v[0], fabs(d));
+        v[0] = dmax_nonneg(v[0], fabs(d));   // (a NaN is kept)
         v[1] += d * d;
     }
     bool ismax[2] = {true, false};
@@ -843,20 +1005,22 @@ static __global__ void __launch_bounds__(kRedThreads) divb_partial_kernel(int nx
     }
 }
 
-// per-block sums of up to 8 planes
-static __global__ void __launch_bounds__(kRedThreads) sums_partial_kernel(long long n, int nplanes, const double *const *planes,
-                                                                   double *part) {
+// per-block sums of 8 planes (their addresses by value: read from memory they
+// headed every load of the loop)
+struct Planes8 {
+    const double *p[8];
+};
+static __global__ void __launch_bounds__(kRedThreads) sums_partial_kernel(long long n, Planes8 planes, double *part) {
     __shared__ double red[8 * 32];
     double v[8] = {0, 0, 0, 0, 0, 0, 0, 0};
     for (long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x; p < n; p += (long long)gridDim.x * blockDim.x) {
 #pragma unroll
-        for (int f = 0; f < 8; ++f)
-            if (f < nplanes) v[f] += planes[f][p];
+        for (int f = 0; f < 8; ++f) v[f] += planes.p[f][p];
     }
     bool ismax[8] = {false, false, false, false, false, false, false, false};
     block_reduce<double, 8>(v, ismax, red);
     if (threadIdx.x == 0)
-        for (int f = 0; f < nplanes; ++f) part[8 * blockIdx.x + f] = v[f];
+        for (int f = 0; f < 8; ++f) part[8 * blockIdx.x + f] = v[f];
 }
 
 // one block: combine nblk partial records of `stride` values in a fixed order;

@@ -125,14 +125,14 @@ __device__ __forceinline__ double drcp_third(double b) {
 }
 
 // 2^n x by an addition to the exponent field (binary64: bits 52-62) on the
-// integer pipes, |n| <= 2; exact for 2^-1020 <= |x| < 2^1020, x itself
+// integer pipes, |n| <= 4; exact for 2^-1018 <= |x| < 2^1018, x itself
 // otherwise (zero, infinities and NaN keep their value; magnitudes outside
 // that range do not occur in a physical state).
 template <int N>
 __device__ __forceinline__ double dscale2(double x) {
     const int hi = __double2hiint(x);
     const unsigned e = (unsigned)hi & 0x7ff00000u;
-    const bool in = e - 0x00300000u < 0x7fa00000u;
+    const bool in = e - 0x00500000u < 0x7f400000u;
     return __hiloint2double(in ? hi + N * 0x00100000 : hi, __double2loint(x));
 }
 
@@ -156,6 +156,7 @@ template <> struct M<double> {
     static __device__ __forceinline__ double min_(double a, double b) { return fmin(a, b); }
     static __device__ __forceinline__ double fma_(double a, double b, double c) { return fma(a, b, c); }
     static __device__ __forceinline__ double half_(double x) { return dscale2<-1>(x); }
+    static __device__ __forceinline__ double sixteenth_(double x) { return dscale2<-4>(x); }
     // comparisons on the bit patterns (order preserving for a positive right
     // side; a comparison of doubles would issue on the FP64 pipe)
     static __device__ __forceinline__ bool ge_pos(double x, double c) { return __double_as_longlong(x) >= __double_as_longlong(c); }
@@ -179,6 +180,7 @@ template <> struct M<float> {
     static __device__ __forceinline__ float min_(float a, float b) { return fminf(a, b); }
     static __device__ __forceinline__ float fma_(float a, float b, float c) { return __fmaf_rn(a, b, c); }
     static __device__ __forceinline__ float half_(float x) { return 0.5f * x; }
+    static __device__ __forceinline__ float sixteenth_(float x) { return 0.0625f * x; }
     static __device__ __forceinline__ bool ge_pos(float x, float c) { return x >= c; }
     static __device__ __forceinline__ bool gt_pos(float x, float c) { return x > c; }
     static __device__ __forceinline__ bool nonneg(float x) { return x >= 0.0f; }
@@ -210,13 +212,6 @@ __device__ __forceinline__ void speeds_fast(Real cs2, Real ca2, Real bt2, Real &
         fmc = m::normal_pos(big) ? m::div_(q, big) : Real(0);
     }
     cf2 = cs2 + fmc;
-}
-
-// speeds_fast and c_slow^2 = c_s^2 c_A^2 / c_f^2.
-template <typename Real>
-__device__ __forceinline__ void speeds(Real cs2, Real ca2, Real bt2, Real &fmc, Real &cms, Real &cf2, Real &csl2) {
-    speeds_fast<Real>(cs2, ca2, bt2, fmc, cms, cf2);
-    csl2 = cf2 > Real(0) ? M<Real>::div_(cs2 * ca2, cf2) : Real(0);
 }
 
 // ---------------------------------------------------------------- one cell
@@ -325,19 +320,6 @@ __device__ __forceinline__ void box_diff_store(Real *sm, int stride, int i, cons
     constexpr int qD[7] = {C_RHOQ, C_MN, C_MT1, C_MT2, C_DU4, C_DU5, C_E};
 #pragma unroll
     for (int c = 0; c < 7; ++c) a[qD[c] * stride] = d.dU[c];
-}
-
-// fast signal speed |v_d| + c_f^d of a cell along axis d (Eq. cfl)
-template <typename Real>
-__device__ __forceinline__ Real signal_speed(Real r, Real vn, Real P, Real Bn, Real B1, Real B2, const Phys<Real> &K) {
-    using m = M<Real>;
-    const Real ir = m::rcp_(r);
-    const Real cs2 = K.gamma * P * ir;
-    const Real ca2 = Bn * Bn * ir;
-    const Real bt2 = (B1 * B1 + B2 * B2) * ir;
-    Real fmc, cms, cf2, csl2;
-    speeds<Real>(cs2, ca2, bt2, fmc, cms, cf2, csl2);
-    return m::abs_(vn) + m::sqrt_(cf2);
 }
 
 // ---------------------------------------------------------------- WENO
