@@ -61,7 +61,7 @@ struct w5ct_ctx {
     int4 *tiles_buf = nullptr;
     int seg_off[3][kMaxTileVariants] = {};
     int seg_n[3][kMaxTileVariants] = {};
-    int sweep_t2[3] = {0, 0, 0};     // single patch: tile height of the sweep along each axis
+    bool sweeps_in_one = false;      // single patch: the three sweeps of a stage in one launch
     int schedule = 0;                // batched sweeps: 0 = one launch per axis and variant, 1 = persistent,
                                      // 2 = the whole step in one persistent launch (fused)
     // fused step (schedule 2): work items, per-patch targets and counters in one allocation
@@ -611,7 +611,6 @@ int run_step(w5ct_ctx *c, const double *dt_dev, bool cellb_done, int last_stage 
     a.K = make_phys<Real>(c->cfg);
     a.flag = c->flag;
     a.hits = c->hits;
-    a.dw = c->cfg.precision == W5CT_FP64_DW;
 
     const UpdateArgs<Real> u = update_args<Real>(c, dt_dev);
 
@@ -633,25 +632,24 @@ int run_step(w5ct_ctx *c, const double *dt_dev, bool cellb_done, int last_stage 
             int rc = launch_cellb<Real>(c);
             if (rc) return rc;
         }
+        SweepArgs<Real> a3[3] = {a, a, a};
+        for (int ax = 0; ax < 3; ++ax) {
+            for (int f = 0; f < 5; ++f) a3[ax].F[f] = plane<Real>(Fax[ax], n, f);
+            for (int f = 0; f < 2; ++f) a3[ax].S[f] = plane<Real>(Sax[ax], n, f);
+        }
         if (c->npatch > 1) {
-            SweepArgs<Real> a3[3] = {a, a, a};
-            for (int ax = 0; ax < 3; ++ax) {
-                for (int f = 0; f < 5; ++f) a3[ax].F[f] = plane<Real>(Fax[ax], n, f);
-                for (int f = 0; f < 2; ++f) a3[ax].S[f] = plane<Real>(Sax[ax], n, f);
-            }
             int rc = launch_batched_sweeps<Real>(c, a3, c->schedule, c->pcounters + s * kMaxTileVariants);
             if (rc) return rc;
         } else {
-            for (int ax = 0; ax < 3; ++ax) {
-                for (int f = 0; f < 5; ++f) a.F[f] = plane<Real>(Fax[ax], n, f);
-                for (int f = 0; f < 2; ++f) a.S[f] = plane<Real>(Sax[ax], n, f);
+            for (int ax = 0; ax < (c->sweeps_in_one ? 1 : 3); ++ax) {
                 int rc = record_event(c);
                 if (rc) return rc;
-                W5_CUDA(c, launch_sweep<Real>(ax, variant, c->sweep_t2[ax], a, c->stream));
+                W5_CUDA(c, c->sweeps_in_one ? launch_sweep_all<Real>(variant, a3, c->stream)
+                                            : launch_sweep<Real>(ax, variant, a3[ax], c->stream));
                 c->launches++;
                 rc = record_event(c);
                 if (rc) return rc;
-                if (c->timing) c->sweep_units += 1;
+                if (c->timing) c->sweep_units += c->sweeps_in_one ? 3 : 1;
             }
         }
         switch (s) {
@@ -932,9 +930,8 @@ int w5ct_init_grid(w5ct_ctx *c, int npatch, const int *n3, const double *dx3) {
         int dev = 0, sms = 0;
         W5_CUDA(c, cudaGetDevice(&dev));
         W5_CUDA(c, cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-        for (int ax = 0; ax < 3; ++ax)
-            c->sweep_t2[ax] = ctx_fp64(c) ? choose_sweep_t2<double>(ax, c->nx, c->ny, c->nz, sms)
-                                                            : choose_sweep_t2<float>(ax, c->nx, c->ny, c->nz, sms);
+        c->sweeps_in_one = ctx_fp64(c) ? sweeps_in_one<double>(c->nx, c->ny, c->nz, sms, c->cfg.precision == W5CT_FP64_DW)
+                                       : sweeps_in_one<float>(c->nx, c->ny, c->nz, sms, false);
     }
     c->schedule = 0;
     for (int v = 0; v < n_variants(c); ++v) {
@@ -1148,7 +1145,6 @@ SweepArgs<Real> sweep_args(w5ct_ctx *c, int ax) {
     a.K = make_phys<Real>(c->cfg);
     a.flag = c->flag;
     a.hits = c->hits;
-    a.dw = c->cfg.precision == W5CT_FP64_DW;
     return a;
 }
 

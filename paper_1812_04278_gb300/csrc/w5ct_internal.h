@@ -10,17 +10,18 @@ namespace w5ct {
 void set_global_error(const char *text);
 
 // Launch the characteristic sweep along `axis` (0, 1, 2) with WENO variant
-// `variant` (0 = JS, 1 = Z) over one patch, in tiles `t2` faces or pencils
-// high (0: the type's default, SweepTuning; the FP64 sweep also takes the
-// shorter tiles of small_tile_heights).  Defined in w5ct_sweep32.cu /
-// w5ct_sweep64.cu.
+// `variant` (0 = JS, 1 = Z) over one patch in the type's default tile
+// (SweepTuning; double: the double-word sweeps), and all three sweeps in one
+// launch (sweep_all_kernel).
+// Defined in w5ct_sweep32.cu / w5ct_sweep64.cu.
 template <typename Real>
-cudaError_t launch_sweep(int axis, int variant, int t2, const SweepArgs<Real> &a, cudaStream_t s);
+cudaError_t launch_sweep(int axis, int variant, const SweepArgs<Real> &a, cudaStream_t s);
+template <typename Real>
+cudaError_t launch_sweep_all(int variant, const SweepArgs<Real> (&a)[3], cudaStream_t s);
 
-// The FP64 single-patch sweeps of the default tiles with the WENO part of
-// every flux in double-word arithmetic (launch_sweep takes them when a.dw is
-// set and the tile is the default one), and the shared-memory allowance of
-// their kernels.  Defined in w5ct_sweep64dw.cu.
+// The FP64 single-patch sweeps with the WENO part of every flux in
+// double-word arithmetic, and the shared-memory allowance of their kernels.
+// Defined in w5ct_sweep64dw.cu.
 cudaError_t launch_sweep_f64dw(int axis, int variant, const SweepArgs<double> &a, cudaStream_t s);
 cudaError_t prepare_sweeps_f64dw();
 
@@ -30,20 +31,22 @@ cudaError_t prepare_sweeps_f64dw();
 template <typename Real>
 struct SweepTuning;
 
-// Defaults measured on GB300 (FP32 at 256^3: 2 blocks/SM of 16-high tiles,
-// 1.6x faster than 1 block of 8-high tiles; 3 blocks/SM or 32-high y/z tiles
-// are slower.  FP64 at 256^3: FP64-pipe bound, one 256-thread block of
-// 16-high tiles per SM; its cell box with the forward differences (NBQ
-// planes) leaves no room for 32-high tiles, which without the differences
-// were 1% faster; 384- or 512-thread blocks measured within 0.5%).
+// Defaults measured on GB300.  FP32: 128-thread blocks, two faces per thread,
+// four blocks per SM, 32 x 8 tiles along x and 16 x 16 in the other two sweeps:
+// 27.36 ms for two 256^3 WENO-Z steps and 109.8 ms for a 512^3 WENO5 step, against
+// 27.95 and 113.1 for 256-thread blocks of 32 x 16 (a barrier stalls half an
+// SM's warps there), 27.47 and 110.8 for 8 x 32, 28.17 and 113.9 for one face
+// per thread, 28.1 and 112.8 for three, 28.7 and 116.2 for four.
+// FP64 (the double-word sweeps and, through sweep_all_kernel, smaller tiles):
+// FP64-pipe bound, eight warps per SM at up to 255 registers.
 #ifndef W5CT_F32_T2X
-#define W5CT_F32_T2X 16
+#define W5CT_F32_T2X 8
 #endif
 #ifndef W5CT_F32_T2YZ
 #define W5CT_F32_T2YZ 16
 #endif
 #ifndef W5CT_F32_MINB
-#define W5CT_F32_MINB 2
+#define W5CT_F32_MINB 4
 #endif
 #ifndef W5CT_F64_T2X
 #define W5CT_F64_T2X 16
@@ -67,25 +70,32 @@ struct SweepTuning;
 #ifndef W5CT_F32_FPT
 #define W5CT_F32_FPT 2
 #endif
+#ifndef W5CT_F32_BXX
+#define W5CT_F32_BXX 32
+#endif
+#ifndef W5CT_F32_BXYZ
+#define W5CT_F32_BXYZ 16
+#endif
 template <>
 struct SweepTuning<float> {
-    static constexpr int T2X = W5CT_F32_T2X, T2YZ = W5CT_F32_T2YZ, MINB = W5CT_F32_MINB, FPT = W5CT_F32_FPT;
+    static constexpr int T2X = W5CT_F32_T2X, T2YZ = W5CT_F32_T2YZ, MINB = W5CT_F32_MINB, FPT = W5CT_F32_FPT,
+                         BXX = W5CT_F32_BXX, BXYZ = W5CT_F32_BXYZ;
 };
 template <>
 struct SweepTuning<double> {
     static constexpr int T2X = W5CT_F64_T2X, T2YZ = W5CT_F64_T2YZ, MINB = W5CT_F64_MINB, FPT = W5CT_F64_T2X / 8,
-                         BXYZ = W5CT_F64_BXYZ;
+                         BXX = 32, BXYZ = W5CT_F64_BXYZ;
 };
 
 template <int AX, typename Real>
 struct SweepCfg {
     static constexpr bool kNarrow = sizeof(Real) == 8 && AX != 0;   // FP64 y/z: 16 x 32
     static constexpr int T2 = AX == 0 ? SweepTuning<Real>::T2X : kNarrow ? W5CT_F64_T2YZ_NARROW : SweepTuning<Real>::T2YZ;
-    static constexpr int BX = kNarrow ? W5CT_F64_BXYZ : 32;
+    static constexpr int BX = AX == 0 ? SweepTuning<Real>::BXX : SweepTuning<Real>::BXYZ;
     static constexpr int MINB = SweepTuning<Real>::MINB;
     static constexpr int FPT = SweepTuning<Real>::FPT;
     using TT = SweepTile<AX, T2, BX, FPT>;
-    static constexpr size_t smem = (size_t)TT::NC * box_quantities<Real>() * sizeof(Real);
+    static constexpr size_t smem = (size_t)TT::template cells<Real> * box_quantities<Real>() * sizeof(Real);
 };
 
 // Single-patch sweep in tiles of BX x T2 faces, FPT per thread (the block
@@ -93,7 +103,7 @@ struct SweepCfg {
 template <int AX, typename Real, int VAR, int T2, int MINB, int FPT, int BX = 32, bool DW = false>
 struct SinglePatchSweep {
     using TT = SweepTile<AX, T2, BX, FPT>;
-    static constexpr size_t smem = (size_t)TT::NC * box_quantities<Real>() * sizeof(Real);
+    static constexpr size_t smem = (size_t)TT::template cells<Real> * box_quantities<Real>() * sizeof(Real);
     static cudaError_t prepare() {
         return cudaFuncSetAttribute(sweep_kernel<AX, Real, VAR, T2, MINB, FPT, BX, DW>,
                                     cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -117,13 +127,15 @@ struct SinglePatchSweep {
 // blocks per SM = 512 / threads per block.
 constexpr int kMaxTileVariants = 4;
 
+#ifndef W5CT_ALL_WAVES32
+#define W5CT_ALL_WAVES32 8
+#endif
+
 template <int AX, typename Real, int V>
 struct TileV;
-constexpr int kBatchedF64T2 = 16;
 template <int AX, typename Real>
 struct TileV<AX, Real, 0> {
-    static constexpr int T2 = sizeof(Real) == 8 ? kBatchedF64T2 : SweepCfg<AX, Real>::T2, BX = 32, FPT = T2 / 8,
-                         MINB = SweepCfg<AX, Real>::MINB;
+    static constexpr int T2 = 16, BX = 32, FPT = 2, MINB = sizeof(Real) == 8 ? 1 : 2;
 };
 template <int AX, typename Real>
 struct TileV<AX, Real, 1> {
@@ -148,7 +160,7 @@ template <typename Real>
 inline void tile_shape(int axis, int v, int &bx, int &t2) {
     if (v == 0) {
         bx = 32;
-        t2 = sizeof(Real) == 8 ? kBatchedF64T2 : axis == 0 ? SweepTuning<Real>::T2X : SweepTuning<Real>::T2YZ;
+        t2 = 16;
     } else {
         bx = v == 1 ? 16 : 8;
         t2 = v == 3 ? 8 : 16;
@@ -159,7 +171,7 @@ template <int AX, typename Real, int VAR, int V>
 struct BatchedSweep {
     using C = TileV<AX, Real, V>;
     using TT = SweepTile<AX, C::T2, C::BX, C::FPT>;
-    static constexpr size_t smem = (size_t)TT::NC * box_quantities<Real>() * sizeof(Real);
+    static constexpr size_t smem = (size_t)TT::template cells<Real> * box_quantities<Real>() * sizeof(Real);
     static cudaError_t prepare() {
         return cudaFuncSetAttribute(sweep_batched_kernel<AX, Real, VAR, C::T2, C::MINB, C::BX, C::FPT>,
                                     cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -190,9 +202,9 @@ struct PersistentSweep {
     static_assert(T0::NT == T1::NT && T1::NT == T2_::NT && C0::BX == C1::BX && C1::BX == C2::BX,
                   "one block shape for the three axes");
     static constexpr int NT = T0::NT, BX = C0::BX, ROWS = T0::ROWS, MINB = C0::MINB;
-    static constexpr size_t smem0 = (size_t)T0::NC * box_quantities<Real>() * sizeof(Real);
-    static constexpr size_t smem1 = (size_t)T1::NC * box_quantities<Real>() * sizeof(Real);
-    static constexpr size_t smem2 = (size_t)T2_::NC * box_quantities<Real>() * sizeof(Real);
+    static constexpr size_t smem0 = (size_t)T0::template cells<Real> * box_quantities<Real>() * sizeof(Real);
+    static constexpr size_t smem1 = (size_t)T1::template cells<Real> * box_quantities<Real>() * sizeof(Real);
+    static constexpr size_t smem2 = (size_t)T2_::template cells<Real> * box_quantities<Real>() * sizeof(Real);
     static constexpr size_t smem = smem0 > smem1 ? (smem0 > smem2 ? smem0 : smem2) : (smem1 > smem2 ? smem1 : smem2);
 };
 
@@ -248,16 +260,40 @@ struct PersistentLaunch {
     }
 };
 
+// The three sweeps of a stage in one launch (sweep_all_kernel).
+template <typename Real, int VAR>
+struct AllSweeps {
+    template <int AX>
+    static constexpr size_t smem_of = (size_t)SweepTile<AX, AllTile<AX>::T2, AllTile<AX>::BX, 1>::template cells<Real> *
+                                      box_quantities<Real>() * sizeof(Real);
+    static constexpr size_t smem = smem_of<0> > smem_of<1> ? smem_of<0> : smem_of<1>;   // (y and z alike)
+    static cudaError_t prepare() {
+        return cudaFuncSetAttribute(sweep_all_kernel<Real, VAR>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    }
+    static cudaError_t launch(const SweepArgs<Real> (&a)[3], cudaStream_t st) {
+        SweepAll<Real> s;
+        const int n[3] = {a[0].nx, a[0].ny, a[0].nz};
+        s.first[0] = 0;
+        for (int ax = 0; ax < 3; ++ax) {
+            s.a[ax] = a[ax];
+            const int bx = ax == 0 ? AllTile<0>::BX : AllTile<1>::BX, t2 = ax == 0 ? AllTile<0>::T2 : AllTile<1>::T2;
+            s.nbx[ax] = (n[0] + bx - 1) / bx;
+            s.nb2[ax] = (n[ax == 2 ? 2 : 1] + t2 - 1) / t2;
+            s.first[ax + 1] = s.first[ax] + s.nbx[ax] * s.nb2[ax] * n[ax == 2 ? 1 : 2];
+        }
+        sweep_all_kernel<Real, VAR><<<s.first[3], kAllThreads, smem, st>>>(s);
+        return cudaGetLastError();
+    }
+};
+
 // allow the dynamic shared memory of every sweep kernel of this type
 template <int AX, typename Real, int VAR>
 cudaError_t prepare_sweep_axis() {
-    using C = SweepCfg<AX, Real>;
-    cudaError_t e = cudaFuncSetAttribute(sweep_kernel<AX, Real, VAR, C::T2, C::MINB, C::FPT, C::BX>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::smem);
-    if (e != cudaSuccess) return e;
-    if constexpr (std::is_same<Real, double>::value) {
-        if ((e = SinglePatchSweep<AX, Real, VAR, 8, C::MINB, 1>::prepare()) != cudaSuccess) return e;
-        if ((e = SinglePatchSweep<AX, Real, VAR, 4, C::MINB, 1>::prepare()) != cudaSuccess) return e;
+    cudaError_t e = cudaSuccess;
+    if constexpr (std::is_same<Real, float>::value) {
+        using C = SweepCfg<AX, Real>;
+        e = SinglePatchSweep<AX, Real, VAR, C::T2, C::MINB, C::FPT, C::BX>::prepare();
+        if (e != cudaSuccess) return e;
     }
     if ((e = BatchedSweep<AX, Real, VAR, 0>::prepare()) != cudaSuccess) return e;
     if constexpr (sizeof(Real) == 4) {
@@ -266,6 +302,7 @@ cudaError_t prepare_sweep_axis() {
         if ((e = BatchedSweep<AX, Real, VAR, 3>::prepare()) != cudaSuccess) return e;
     }
     if constexpr (AX == 0) {
+        if ((e = AllSweeps<Real, VAR>::prepare()) != cudaSuccess) return e;
         if ((e = PersistentLaunch<Real, VAR, 0>::prepare()) != cudaSuccess) return e;
         if constexpr (sizeof(Real) == 4) {
             if ((e = PersistentLaunch<Real, VAR, 1>::prepare()) != cudaSuccess) return e;
@@ -353,12 +390,6 @@ cudaError_t launch_sweep_batched_impl(int axis, int variant, int tv, const Sweep
     return launch_sweep_batched_axis<2, Real, 1>(tv, a, pgs, tiles, ntiles, s);
 }
 
-// The FP64 sweep keeps one block of 256 threads per SM (its registers), so a
-// small patch fills the GPU only with shorter tiles: 8 high (256 threads, one
-// face each) or 4 high (128 threads, two blocks per SM).  The float sweep
-// always uses its default tile.
-constexpr int kSmallTileHeights[2] = {8, 4};
-
 // blocks of the single-patch sweep along `axis` in tiles of bx lanes x t2
 inline long long sweep_blocks(int axis, int t2, int bx, int nx, int ny, int nz) {
     const long long nbx = (nx + bx - 1) / bx;
@@ -366,44 +397,51 @@ inline long long sweep_blocks(int axis, int t2, int bx, int nx, int ny, int nz) 
     return nbx * ((ny + t2 - 1) / t2) * nz;     // x- and y-sweeps: t2 pencils or faces along y
 }
 
-// Tile height of the single-patch sweep along `axis`: the default, or for
-// FP64 the tallest of the shorter (32-lane) tiles that gives every SM at
-// least two blocks (the shortest if none does).
+// Whether the three sweeps of a single patch go in one launch
+// (sweep_all_kernel).
+// FP64: always.  The small blocks balance the SMs better than they lose by
+// their larger boxes: step of 32^3 1.93 -> 1.01 ms against three launches of the
+// 32 x 16 and 16 x 32 tiles, 64^3 7.68 -> 6.60, 100 x 70 x 50 10.26 -> 9.80 (WENO5),
+// 160^3 101.4 -> 100.4, 256^3 413.4 -> 411.4 ms.
+// FP32: below 8 waves of the default tiles' blocks on the device, where the
+// tails of three launches cost more than the one face per thread: 32^3 0.140 ->
+// 0.092 ms, 64^3 0.279 -> 0.255, 96^3 (5.7 waves) 0.798 -> 0.790, but 112^3 (9
+// waves) 1.260 -> 1.262 and 160^3 3.26 -> 3.37.
+// The double-word sweeps (dw) have no such kernel: they keep their own
+// launches unless one of them has fewer than two blocks per SM.
 template <typename Real>
-inline int choose_sweep_t2(int axis, int nx, int ny, int nz, int sms) {
-    const int t2d = axis == 0 ? SweepCfg<0, Real>::T2 : SweepCfg<1, Real>::T2;
-    const int bxd = axis == 0 ? SweepCfg<0, Real>::BX : SweepCfg<1, Real>::BX;
-    if (!std::is_same<Real, double>::value) return t2d;
-    if (sweep_blocks(axis, t2d, bxd, nx, ny, nz) >= 2LL * sms) return t2d;
-    for (int h : kSmallTileHeights)
-        if (sweep_blocks(axis, h, 32, nx, ny, nz) >= 2LL * sms) return h;
-    return kSmallTileHeights[1];
+inline bool sweeps_in_one(int nx, int ny, int nz, int sms, bool dw) {
+    if (std::is_same<Real, double>::value && !dw) return true;
+    const long long least = dw ? 2LL * sms : (long long)W5CT_ALL_WAVES32 * sms * SweepTuning<Real>::MINB;
+    for (int ax = 0; ax < 3; ++ax) {
+        const long long b = ax == 0 ? sweep_blocks(0, SweepCfg<0, Real>::T2, SweepCfg<0, Real>::BX, nx, ny, nz)
+                                    : sweep_blocks(ax, SweepCfg<1, Real>::T2, SweepCfg<1, Real>::BX, nx, ny, nz);
+        if (b < least) return true;
+    }
+    return false;
 }
 
 template <int AX, typename Real, int VAR>
-cudaError_t launch_sweep_axis(int t2, const SweepArgs<Real> &a, cudaStream_t s) {
-    using C = SweepCfg<AX, Real>;
+cudaError_t launch_sweep_axis(const SweepArgs<Real> &a, cudaStream_t s) {
+    // (their shared memory is allowed by prepare_sweeps() at w5ct_init_grid)
     if constexpr (std::is_same<Real, double>::value) {
-        if (t2 == 8) return SinglePatchSweep<AX, Real, VAR, 8, C::MINB, 1>::launch(a, s);
-        if (t2 == 4) return SinglePatchSweep<AX, Real, VAR, 4, C::MINB, 1>::launch(a, s);
+        return launch_sweep_f64dw(AX, VAR, a, s);
+    } else {
+        using C = SweepCfg<AX, Real>;
+        return SinglePatchSweep<AX, Real, VAR, C::T2, C::MINB, C::FPT, C::BX>::launch(a, s);
     }
-    if (t2 != 0 && t2 != C::T2) return cudaErrorInvalidValue;
-    if constexpr (std::is_same<Real, double>::value)
-        if (a.dw) return launch_sweep_f64dw(AX, VAR, a, s);
-    // the default tile; its shared memory is allowed by prepare_sweeps() at w5ct_init_grid
-    return SinglePatchSweep<AX, Real, VAR, C::T2, C::MINB, C::FPT, C::BX>::launch(a, s);
 }
 
 template <typename Real>
-cudaError_t launch_sweep_impl(int axis, int variant, int t2, const SweepArgs<Real> &a, cudaStream_t s) {
+cudaError_t launch_sweep_impl(int axis, int variant, const SweepArgs<Real> &a, cudaStream_t s) {
     if (variant == 0) {
-        if (axis == 0) return launch_sweep_axis<0, Real, 0>(t2, a, s);
-        if (axis == 1) return launch_sweep_axis<1, Real, 0>(t2, a, s);
-        return launch_sweep_axis<2, Real, 0>(t2, a, s);
+        if (axis == 0) return launch_sweep_axis<0, Real, 0>(a, s);
+        if (axis == 1) return launch_sweep_axis<1, Real, 0>(a, s);
+        return launch_sweep_axis<2, Real, 0>(a, s);
     }
-    if (axis == 0) return launch_sweep_axis<0, Real, 1>(t2, a, s);
-    if (axis == 1) return launch_sweep_axis<1, Real, 1>(t2, a, s);
-    return launch_sweep_axis<2, Real, 1>(t2, a, s);
+    if (axis == 0) return launch_sweep_axis<0, Real, 1>(a, s);
+    if (axis == 1) return launch_sweep_axis<1, Real, 1>(a, s);
+    return launch_sweep_axis<2, Real, 1>(a, s);
 }
 
 }  // namespace w5ct

@@ -36,7 +36,6 @@ struct SweepArgs {
     Phys<Real> K;
     int *flag;
     unsigned long long *hits;
-    int dw = 0;   // host-side choice: FP64 single-patch sweeps with the double-word WENO
 };
 
 // Cells whose loads a thread of a single-axis sweep kernel issues together
@@ -44,13 +43,25 @@ struct SweepArgs {
 // cell at a time: their larger code measured slower with the batch).
 constexpr int kStageBatch = 3;
 
-// Tile of one block: BX lanes along x (coalesced loads and stores; every
-// tile has x fastest), T2 faces or pencils in the second direction, each
-// thread computing FPT of them (the block is BX x T2/FPT threads).
+// Tile of one block: up to BX cells along x, T2 faces or pencils in the
+// second direction, computed by BX T2 / FPT threads.
 //  x-sweep: BX faces along x  x  T2 pencils along y
 //  y-sweep: BX pencils along x  x  T2 faces along y
 //  z-sweep: BX pencils along x  x  T2 faces along z
-// The cell box adds the 2 + 3 stencil cells along the sweep axis.
+// The cell box adds the 2 + 3 stencil cells along the sweep axis; its rows
+// are `pitch` cells apart (x fastest).
+//
+// In double (FlatTile) a patch is cut along x into ceil(nx / BX) tiles of
+// nearly equal width w, and the tile's faces and box cells are numbered row
+// after row over the actual extents, so that whatever nx is a warp's lanes are
+// full but for a tile's last one (100 cells: four tiles of 25, not three of 32
+// and one of 4): an FP64 instruction costs the same for one lane as for 32.
+// 100 x 70 x 50 step 11.69 -> 10.26 ms, 48 uneven patches 67.2 -> 54.8 ms, 256^3
+// unchanged.  In float the same numbering was 3-4% slower (its divisions, and
+// rows of a warp meeting in a shared-memory bank, which in double the FP64 pipe
+// hides), also where it fills lanes, so a float tile takes whole BX-wide rows,
+// its narrower tiles' x-boxes with a pitch that puts a warp's rows in different
+// banks.
 template <int AX, int T2, int BX_ = 32, int FPT_ = T2 / 8>
 struct SweepTile {
     static_assert(T2 % FPT_ == 0, "faces per thread must divide the tile height");
@@ -64,9 +75,21 @@ struct SweepTile {
     static constexpr int CX = BX + (AX == 0 ? 5 : 0);
     static constexpr int CY = BY + (AX == 1 ? 5 : 0);
     static constexpr int CZ = BZ + (AX == 2 ? 5 : 0);
-    static constexpr int NC = CX * CY * CZ;
-    static constexpr int ST = (AX == 0) ? 1 : (AX == 1) ? CX : CX * CY;
+    // elements between rows of the box and between quantities, and the stencil
+    // stride
+    static constexpr int PITCH_F = AX != 0 || BX >= 32 ? CX : BX == 8 ? 24 : 48;
+    template <typename Real>
+    static constexpr int pitch = std::is_same<Real, float>::value ? PITCH_F : CX;
+    static constexpr int NC = CX * CY * CZ;          // cells of the full box
+    template <typename Real>
+    static constexpr int cells = pitch<Real> *CY *CZ;
+    static constexpr int ST = (AX == 0) ? 1 : CX;
 };
+
+// q / d for 0 <= q < 1024, 0 < d <= 64, with inv = div_inv(d): q (inv - 65536 / d)
+// < 1024, under 65536 / d
+__device__ __forceinline__ int div_inv(int d) { return (65536 + d - 1) / d; }
+__device__ __forceinline__ int div_by(int q, int inv) { return (q * inv) >> 16; }
 
 // Patch geometry: cell counts, the patch's first cell in every plane (several
 // patches share the planes back to back) and the inverse spacings.
@@ -78,17 +101,26 @@ struct PatchGeom {
 };
 
 // One sweep tile (tile indices tbx, tby, tbz) of the patch described by g,
-// computed by the block's NT threads, numbered (tx, ty) in [0, BX) x
-// [0, ROWS).  sm: shared memory of box_quantities<Real>() * NC elements.  SB: cells whose loads
-// a thread issues together when it stages the cell box.
+// computed by the block's NT threads, numbered tx + BX ty.  sm: shared memory
+// of box_quantities<Real>() * cells<Real> elements.  SB: cells whose loads a
+// thread issues together when it stages the cell box.
 template <int AX, typename Real, int VAR, int T2, int BX, int FPT, int SB = kStageBatch, bool DWW = false>
 __device__ __forceinline__ void sweep_tile_at(const SweepArgs<Real> &a, const PatchGeom &pg, int tbx, int tby, int tbz,
                                               Real *sm, int tx, int ty) {
     using TT = SweepTile<AX, T2, BX, FPT>;
+    constexpr int NC = TT::template cells<Real>;      // elements between quantities
+    constexpr bool kFlat = std::is_same<Real, double>::value;
+    constexpr int pitch = TT::template pitch<Real>, st = TT::ST;
     const int nx = pg.nx, ny = pg.ny, nz = pg.nz;
     const size_t off = (size_t)pg.off;
-    const int x0 = tbx * TT::BX, y0 = tby * TT::BY, z0 = tbz * TT::BZ;
-    const int ox = x0 - (AX == 0 ? 2 : 0), oy = y0 - (AX == 1 ? 2 : 0), oz = z0 - (AX == 2 ? 2 : 0);
+    const int ntx = (nx + BX - 1) / BX, w0 = kFlat ? (nx + ntx - 1) / ntx : BX;
+    const int x0 = tbx * w0, y0 = tby * TT::BY, z0 = tbz * TT::BZ;
+    // extents of the faces and of the box, and the numbering's row length
+    const int w = kFlat ? min(w0, nx - x0) : BX;
+    const int h = !kFlat ? T2 : AX == 2 ? min(TT::BZ, nz - z0) : min(TT::BY, ny - y0);
+    const int cw = w + (AX == 0 ? 5 : 0), ncell = cw * (h + (AX == 0 ? 0 : 5));
+    const int cinv = kFlat ? div_inv(cw) : 0, finv = kFlat ? div_inv(w) : 0;
+    auto row_of = [&](int q, int d, int inv) { return kFlat ? div_by(q, inv) : q / d; };
     const int tid = tx + TT::BX * ty;
 
     // phase 1: per-cell primitives, flux and speeds of the cell box.  A
@@ -101,14 +133,16 @@ __device__ __forceinline__ void sweep_tile_at(const SweepArgs<Real> &a, const Pa
 #pragma unroll
     for (int it0 = 0; it0 < NIT; it0 += B) {
         Real v[B][8];
+        int at[B];
 #pragma unroll
         for (int j = 0; j < B; ++j) {
             const int c = tid + (it0 + j) * TT::NT;
-            if (it0 + j < NIT && c < TT::NC) {
-                const int cx = c % TT::CX;
-                const int cy = (c / TT::CX) % TT::CY;
-                const int cz = c / (TT::CX * TT::CY);
-                const int gx = wrapi(ox + cx, nx), gy = wrapi(oy + cy, ny), gz = wrapi(oz + cz, nz);
+            if (it0 + j < NIT && c < ncell) {
+                const int cr = row_of(c, cw, cinv), cx = c - cr * cw;
+                at[j] = cx + pitch * cr;
+                const int gx = wrapi(x0 + cx - (AX == 0 ? 2 : 0), nx);
+                const int gy = AX == 0 ? (kFlat ? y0 + cr : wrapi(y0 + cr, ny)) : AX == 1 ? wrapi(y0 + cr - 2, ny) : y0;
+                const int gz = AX == 2 ? wrapi(z0 + cr - 2, nz) : z0;
                 const size_t g = off + (size_t)gx + (size_t)nx * ((size_t)gy + (size_t)ny * (size_t)gz);
 #pragma unroll
                 for (int f = 0; f < 5; ++f) v[j][f] = a.q[f][g];
@@ -119,8 +153,8 @@ __device__ __forceinline__ void sweep_tile_at(const SweepArgs<Real> &a, const Pa
 #pragma unroll
         for (int j = 0; j < B; ++j) {
             const int c = tid + (it0 + j) * TT::NT;
-            if (it0 + j < NIT && c < TT::NC)
-                cell_fill<Real, AX>(sm + c, TT::NC, v[j][0], v[j][1], v[j][2], v[j][3], v[j][4], v[j][5], v[j][6],
+            if (it0 + j < NIT && c < ncell)
+                cell_fill<Real, AX>(sm + at[j], NC, v[j][0], v[j][1], v[j][2], v[j][3], v[j][4], v[j][5], v[j][6],
                                     v[j][7], a.K, bad, hit);
         }
     }
@@ -135,36 +169,44 @@ __device__ __forceinline__ void sweep_tile_at(const SweepArgs<Real> &a, const Pa
     // cell that has a successor along the sweep axis (the last one has none
     // and no stencil needs it)
     if constexpr (box_diff<Real>()) {
-        constexpr int NIT = (TT::NC + TT::NT - 1) / TT::NT;
-        constexpr int LAST = (AX == 0 ? TT::CX : AX == 1 ? TT::CY : TT::CZ) - 1;
         CellDiff<Real> d[NIT];
+        int at[NIT];
         bool has[NIT];
 #pragma unroll
         for (int it = 0; it < NIT; ++it) {
             const int c = tid + it * TT::NT;
-            const int ca = AX == 0 ? c % TT::CX : AX == 1 ? (c / TT::CX) % TT::CY : c / (TT::CX * TT::CY);
-            has[it] = c < TT::NC && ca < LAST;
-            if (has[it]) box_diff_load<Real>(sm, TT::NC, c, TT::ST, d[it]);
+            const int cr = row_of(c, cw, cinv), cx = c - cr * cw;
+            at[it] = cx + pitch * cr;
+            has[it] = c < ncell && (AX == 0 ? cx < cw - 1 : cr < h + 4);
+            if (has[it]) box_diff_load<Real>(sm, NC, at[it], st, d[it]);
         }
         __syncthreads();
 #pragma unroll
         for (int it = 0; it < NIT; ++it)
-            if (has[it]) box_diff_store<Real>(sm, TT::NC, tid + it * TT::NT, d[it]);
+            if (has[it]) box_diff_store<Real>(sm, NC, at[it], d[it]);
         __syncthreads();
     }
 
-    // phase 2: FPT interfaces per thread
+    // phase 2: up to FPT interfaces per thread
 #pragma unroll 1
     for (int r = 0; r < TT::FPT; ++r) {
-        const int t2 = ty + TT::ROWS * r;
-        const int bx = tx;
+        int t2, bx;
+        if constexpr (kFlat) {
+            const int f = tid + TT::NT * r;
+            if (f >= w * h) break;
+            t2 = div_by(f, finv);
+            bx = f - t2 * w;
+        } else {
+            t2 = ty + TT::ROWS * r;
+            bx = tx;
+        }
         const int by = (AX == 2) ? 0 : t2;
         const int bz = (AX == 2) ? t2 : 0;
         const int gx = x0 + bx, gy = y0 + by, gz = z0 + bz;
-        if (gx < nx && gy < ny && gz < nz) {
-            const int c0 = bx + TT::CX * (by + TT::CY * bz);   // stencil cell i-2
+        if (kFlat || (gx < nx && gy < ny && gz < nz)) {
             Real Ff[7], s1, s2;
-            face_flux<Real, VAR, box_diff<Real>(), DWW>(sm + c0, TT::NC, TT::ST, a.K, Ff, s1, s2);
+            // stencil cell i-2 of the face at bx + pitch t2
+            face_flux<Real, VAR, box_diff<Real>(), DWW>(sm + bx + pitch * t2, NC, st, a.K, Ff, s1, s2);
             const size_t g = off + (size_t)gx + (size_t)nx * ((size_t)gy + (size_t)ny * (size_t)gz);
             a.F[0][g] = Ff[0];
             a.F[1 + AX][g] = Ff[1];
@@ -278,6 +320,45 @@ __global__ void __launch_bounds__(SweepTile<AX, T2, BX, FPT>::NT, MINB) sweep_ke
     pg.off = 0;
     sweep_tile<AX, Real, VAR, T2, BX, FPT, kStageBatch, DW>(a, pg, blockIdx.x, blockIdx.y, blockIdx.z,
                                                             reinterpret_cast<Real *>(w5ct_smem));
+}
+
+// The three sweeps of a stage over a single patch in one launch, in tiles of
+// 128 faces (32 x 4 along x, 8 x 16 in the other two sweeps, one face per
+// thread; box cells per face 1.16 and 1.31).  They are independent, and a
+// patch of fewer than a few hundred thousand cells does not fill the GPU with
+// one of them: one launch has three times the blocks, one tail and one launch
+// latency.  first[ax] is the first block of axis ax.
+template <typename Real>
+struct SweepAll {
+    SweepArgs<Real> a[3];
+    int first[4];
+    int nbx[3], nb2[3];          // tiles along x and along the second direction
+};
+constexpr int kAllThreads = 128;
+template <int AX>
+struct AllTile {
+    static constexpr int BX = AX == 0 ? 32 : 8, T2 = AX == 0 ? 4 : 16;
+};
+
+template <typename Real, int VAR>
+__global__ void __launch_bounds__(kAllThreads, sizeof(Real) == 8 ? 2 : 4) sweep_all_kernel(SweepAll<Real> s) {
+    extern __shared__ __align__(16) unsigned char w5ct_smem[];
+    Real *sm = reinterpret_cast<Real *>(w5ct_smem);
+    const int b = blockIdx.x, tid = threadIdx.x;
+    const int ax = b < s.first[1] ? 0 : b < s.first[2] ? 1 : 2;
+    const int q = b - s.first[ax], r = q / s.nbx[ax], tbx = q - r * s.nbx[ax];
+    const int t2 = r / s.nb2[ax], t1 = r - t2 * s.nb2[ax];
+    PatchGeom pg;
+    pg.nx = s.a[0].nx;
+    pg.ny = s.a[0].ny;
+    pg.nz = s.a[0].nz;
+    pg.off = 0;
+    if (ax == 0)
+        sweep_tile_at<0, Real, VAR, AllTile<0>::T2, AllTile<0>::BX, 1>(s.a[0], pg, tbx, t1, t2, sm, tid % AllTile<0>::BX, tid / AllTile<0>::BX);
+    else if (ax == 1)
+        sweep_tile_at<1, Real, VAR, AllTile<1>::T2, AllTile<1>::BX, 1>(s.a[1], pg, tbx, t1, t2, sm, tid % AllTile<1>::BX, tid / AllTile<1>::BX);
+    else
+        sweep_tile_at<2, Real, VAR, AllTile<2>::T2, AllTile<2>::BX, 1>(s.a[2], pg, tbx, t2, t1, sm, tid % AllTile<2>::BX, tid / AllTile<2>::BX);
 }
 
 // Tile tables hold int4 (patch | axis << 28, tile x, tile y, tile z).

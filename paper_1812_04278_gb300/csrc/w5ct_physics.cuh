@@ -227,14 +227,14 @@ __device__ __forceinline__ void cell_fill_frame(Real *sm, int stride, Real rho, 
     if (K.floors && r < K.rho_min) { r = K.rho_min; hit = true; }
     const Real isr = m::rsqrt_(r), ir = isr * isr;
     const Real vn = mn * ir, v1 = m1 * ir, v2 = m2 * ir;
-    const Real vv = vn * vn + v1 * v1 + v2 * v2;
-    const Real Bn2 = Bn * Bn, Bt2 = B1 * B1 + B2 * B2;
+    const Real vv = m::fma_(v2, v2, m::fma_(v1, v1, vn * vn));
+    const Real Bn2 = Bn * Bn, Bt2 = m::fma_(B2, B2, B1 * B1);
     const Real BB = Bn2 + Bt2;
-    Real P = K.gm1 * (E - Real(0.5) * (r * vv + BB));
+    Real P = K.gm1 * m::fma_(Real(-0.5), m::fma_(r, vv, BB), E);
     if (K.floors && P < K.p_min) { P = K.p_min; hit = true; }
     if (!(r > Real(0)) || !m::finite_pos(P)) bad = true;
-    const Real Pt = P + Real(0.5) * BB;
-    const Real vB = vn * Bn + v1 * B1 + v2 * B2;
+    const Real Pt = m::fma_(Real(0.5), BB, P);
+    const Real vB = m::fma_(v2, B2, m::fma_(v1, B1, vn * Bn));
     sm[C_RHO * stride] = r;
     sm[C_VN * stride] = vn;
     sm[C_VT1 * stride] = v1;
@@ -250,12 +250,12 @@ __device__ __forceinline__ void cell_fill_frame(Real *sm, int stride, Real rho, 
     sm[C_E * stride] = E;
     // rho v_n = m_n (v = m / rho with the same, possibly floored, rho)
     sm[C_F0 * stride] = mn;
-    sm[C_F1 * stride] = mn * vn + (Pt - Bn2);
-    sm[C_F2 * stride] = mn * v1 - Bn * B1;
-    sm[C_F3 * stride] = mn * v2 - Bn * B2;
-    sm[C_F4 * stride] = B1 * vn - Bn * v1;
-    sm[C_F5 * stride] = B2 * vn - Bn * v2;
-    sm[C_F6 * stride] = (E + Pt) * vn - Bn * vB;
+    sm[C_F1 * stride] = m::fma_(mn, vn, Pt - Bn2);
+    sm[C_F2 * stride] = m::fma_(mn, v1, -(Bn * B1));
+    sm[C_F3 * stride] = m::fma_(mn, v2, -(Bn * B2));
+    sm[C_F4 * stride] = m::fma_(B1, vn, -(Bn * v1));
+    sm[C_F5 * stride] = m::fma_(B2, vn, -(Bn * v2));
+    sm[C_F6 * stride] = m::fma_(E + Pt, vn, -(Bn * vB));
     // c_f, c_A and c_slow = c_s c_A / c_f, from reciprocal square roots
     const Real cs2 = K.gamma * P * ir;
     Real fmc, cms, cf2;
@@ -385,7 +385,7 @@ __device__ __forceinline__ float phi_nf(float a, float b, float c, float d, floa
     }
     // D = e0 + 6 e1 + 3 e2; a_2 / 2 = 1.5 e2
     const float inv = __fdividef(1.0f, __fmaf_rn(3.0f, e2, __fmaf_rn(6.0f, e1, e0)));
-    return (e0 * inv) * (x0 - y0) + __fmaf_rn(e2, 1.5f * inv, -0.25f) * (y0 - z0);
+    return __fmaf_rn(e0 * inv, x0 - y0, __fmaf_rn(e2, 1.5f * inv, -0.25f) * (y0 - z0));
 }
 
 // double: the weights times the common factor (s_0 s_1 s_2)^2, so that no
@@ -699,7 +699,7 @@ __device__ __forceinline__ FaceEigen<Real> face_eigen(Real r, Real v2, Real Bn, 
     const Real ir = e.isr * e.isr;
     e.sr = r * e.isr;
     const Real ca2 = Bn * Bn * ir;
-    const Real btm = Bt1 * Bt1 + Bt2 * Bt2;
+    const Real btm = m::fma_(Bt2, Bt2, Bt1 * Bt1);
     const Real bt2 = btm * ir;
     // The slow and fast left eigenvectors carry 1/(2 c_s^2): the projection
     // amplifies the rounding of the data by about (v^2 + c_A^2 + b_t^2)/c_s^2.
@@ -731,7 +731,7 @@ __device__ __forceinline__ FaceEigen<Real> face_eigen(Real r, Real v2, Real Bn, 
     e.as = fast_big ? ab : al;
     e.af = fast_big ? al : ab;
     // c_f^2 = c_s^2 + (c_f^2 - c_s^2), the difference a_s^2 sqrt(d)
-    e.cf2 = e.cs2 + (fast_big ? big : small_a * small_a * sd);
+    e.cf2 = e.cs2 + (fast_big ? big : (small_a * small_a) * sd);
     const Real icf = m::rsqrt_(e.cf2);
     e.cf = e.cf2 * icf;
     // c_slow = c_s c_A / c_f (c_slow^2 = c_s^2 c_A^2 / c_f^2), c_A = |B_n| / sqrt(rho)
@@ -795,7 +795,7 @@ __device__ __forceinline__ void face_flux(const Real *__restrict__ sm, int ncell
                 dF[j] = SMQ(qD, j);
                 X[c][j] = make_pair2(dF[j], SMQ(qU, j));
             }
-            X0[c] = SMQ(C_F0 + c, 2) + (Real(6) * dF[2] + dF[1] - dF[3]) * Real(1.0 / 12.0);
+            X0[c] = m::fma_(m::fma_(Real(6), dF[2], dF[1]) - dF[3], Real(1.0 / 12.0), SMQ(C_F0 + c, 2));
         } else {
             const int qF = C_F0 + c;
             const int qU = c == 0 ? C_RHOQ : c == 1 ? C_MN : c == 2 ? C_MT1 : c == 3 ? C_MT2 : c == 4 ? C_BT1
@@ -808,7 +808,7 @@ __device__ __forceinline__ void face_flux(const Real *__restrict__ sm, int ncell
             }
 #pragma unroll
             for (int j = 0; j < 5; ++j) X[c][j] = make_pair2(f[j + 1] - f[j], u[j + 1] - u[j]);
-            X0[c] = f[2] + (Real(6) * (f[3] - f[2]) + (f[2] - f[1]) - (f[4] - f[3])) * Real(1.0 / 12.0);
+            X0[c] = m::fma_(m::fma_(Real(6), f[3] - f[2], f[2] - f[1]) - (f[4] - f[3]), Real(1.0 / 12.0), f[2]);
         }
     }
     // interface state: mean of the primitives of cells i and i+1
@@ -822,12 +822,12 @@ __device__ __forceinline__ void face_flux(const Real *__restrict__ sm, int ncell
     const Real caL = SMQ(C_CA, 2), caR = SMQ(C_CA, 3);
     const Real csL = SMQ(C_CSL, 2), csR = SMQ(C_CSL, 3);
     // twice the transport fluxes <B_n v_t> of the two cells
-    const Real bvt1 = SMQ(C_BN, 2) * SMQ(C_VT1, 2) + SMQ(C_BN, 3) * SMQ(C_VT1, 3);
-    const Real bvt2 = SMQ(C_BN, 2) * SMQ(C_VT2, 2) + SMQ(C_BN, 3) * SMQ(C_VT2, 3);
+    const Real bvt1 = m::fma_(SMQ(C_BN, 2), SMQ(C_VT1, 2), SMQ(C_BN, 3) * SMQ(C_VT1, 3));
+    const Real bvt2 = m::fma_(SMQ(C_BN, 2), SMQ(C_VT2, 2), SMQ(C_BN, 3) * SMQ(C_VT2, 3));
 #undef SMQ
 
     // ---- eigen scalars at the interface state (Appendix A)
-    const Real v2 = vn * vn + vt1 * vt1 + vt2 * vt2;
+    const Real v2 = m::fma_(vt2, vt2, m::fma_(vt1, vt1, vn * vn));
     const Real hv2 = m::half_(v2);
     const FaceEigen<Real> e = face_eigen<Real>(r, v2, Bn, Bt1, Bt2, P, K);
     const Real b1 = e.b1, b2 = e.b2, sg = e.sg;
@@ -919,22 +919,22 @@ __device__ __forceinline__ void face_flux(const Real *__restrict__ sm, int ncell
     // v S1 to the momentum and v^2/2 S1 + v.T to the energy.
     {
         const Real kw = kWenoScale<Real>;
-        const Real mg = e.af * sf + e.as * ss;                     // magnetosonic density
+        const Real mg = m::fma_(e.af, sf, e.as * ss);              // magnetosonic density
         const Real S1 = mg + Fe;
-        const Real S2 = (e.cs * e.isr) * (e.as * sf - e.af * ss);
+        const Real S2 = (e.cs * e.isr) * m::fma_(e.as, sf, -(e.af * ss));
         const Real hsa = m::half_(sa), hda = m::half_(da) * (sg * e.isr);   // (sg/2)^2, sg/2 of the Alfven fields
-        const Real Tn = -(afcf * df + ascl * ds);
-        const Real Tk = sas * df - saf * ds;
-        const Real T1 = Tk * b1 - hsa * b2;
-        const Real T2 = Tk * b2 + hsa * b1;
-        const Real en6 = (afcf * e.cf) * sf + (ascl * e.csl) * ss - (K.g2 * e.cs2) * mg;
-        Ff[0] = X0[0] + kw * S1;
-        Ff[1] = X0[1] + kw * (S1 * vn + Tn);
-        Ff[2] = X0[2] + kw * (S1 * vt1 + T1);
-        Ff[3] = X0[3] + kw * (S1 * vt2 + T2);
-        Ff[4] = X0[4] + kw * (S2 * b1 - hda * b2);
-        Ff[5] = X0[5] + kw * (S2 * b2 + hda * b1);
-        Ff[6] = X0[6] + kw * (hv2 * S1 + vn * Tn + vt1 * T1 + vt2 * T2 + en6);
+        const Real Tn = -m::fma_(afcf, df, ascl * ds);
+        const Real Tk = m::fma_(sas, df, -(saf * ds));
+        const Real T1 = m::fma_(Tk, b1, -(hsa * b2));
+        const Real T2 = m::fma_(Tk, b2, hsa * b1);
+        const Real en6 = m::fma_(afcf * e.cf, sf, m::fma_(ascl * e.csl, ss, -((K.g2 * e.cs2) * mg)));
+        Ff[0] = m::fma_(kw, S1, X0[0]);
+        Ff[1] = m::fma_(kw, m::fma_(S1, vn, Tn), X0[1]);
+        Ff[2] = m::fma_(kw, m::fma_(S1, vt1, T1), X0[2]);
+        Ff[3] = m::fma_(kw, m::fma_(S1, vt2, T2), X0[3]);
+        Ff[4] = m::fma_(kw, m::fma_(S2, b1, -(hda * b2)), X0[4]);
+        Ff[5] = m::fma_(kw, m::fma_(S2, b2, hda * b1), X0[5]);
+        Ff[6] = m::fma_(kw, m::fma_(hv2, S1, m::fma_(vn, Tn, m::fma_(vt1, T1, m::fma_(vt2, T2, en6)))), X0[6]);
     }
     s1 = m::fma_(Real(0.5), bvt1, Ff[4]);
     s2 = m::fma_(Real(0.5), bvt2, Ff[5]);

@@ -5,8 +5,13 @@
 namespace w5ct {
 
 template <>
-cudaError_t launch_sweep<float>(int axis, int variant, int t2, const SweepArgs<float> &a, cudaStream_t s) {
-    return launch_sweep_impl<float>(axis, variant, t2, a, s);
+cudaError_t launch_sweep<float>(int axis, int variant, const SweepArgs<float> &a, cudaStream_t s) {
+    return launch_sweep_impl<float>(axis, variant, a, s);
+}
+
+template <>
+cudaError_t launch_sweep_all<float>(int variant, const SweepArgs<float> (&a)[3], cudaStream_t s) {
+    return variant == 0 ? AllSweeps<float, 0>::launch(a, s) : AllSweeps<float, 1>::launch(a, s);
 }
 
 template <>
