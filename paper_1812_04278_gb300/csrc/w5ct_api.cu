@@ -62,6 +62,7 @@ struct w5ct_ctx {
     int seg_off[3][kMaxTileVariants] = {};
     int seg_n[3][kMaxTileVariants] = {};
     bool sweeps_in_one = false;      // single patch: the three sweeps of a stage in one launch
+    bool dw = false;                 // single patch: the sweeps with the double-word WENO
     int schedule = 0;                // batched sweeps: 0 = one launch per axis and variant, 1 = persistent,
                                      // 2 = the whole step in one persistent launch (fused)
     // fused step (schedule 2): work items, per-patch targets and counters in one allocation
@@ -599,6 +600,16 @@ int launch_batched_sweeps(w5ct_ctx *c, const SweepArgs<Real> (&a3)[3], int sched
     return W5CT_OK;
 }
 
+// Single patch: the sweep along ax, or all three of them in one launch.
+inline cudaError_t launch_sweeps(w5ct_ctx *c, int ax, const SweepArgs<float> (&a)[3]) {
+    return c->sweeps_in_one ? launch_sweep_all<float>(c->cfg.weno_variant, a, c->stream)
+                            : launch_sweep_f32(ax, c->cfg.weno_variant, a[ax], c->stream);
+}
+inline cudaError_t launch_sweeps(w5ct_ctx *c, int, const SweepArgs<double> (&a)[3]) {
+    return c->dw ? launch_sweep_all_f64dw(c->cfg.weno_variant, a, c->stream)
+                 : launch_sweep_all<double>(c->cfg.weno_variant, a, c->stream);
+}
+
 template <typename Real>
 int run_step(w5ct_ctx *c, const double *dt_dev, bool cellb_done, int last_stage = 3, void *stage_store = nullptr) {
     const long long n = c->n;
@@ -616,7 +627,6 @@ int run_step(w5ct_ctx *c, const double *dt_dev, bool cellb_done, int last_stage 
 
     void *Fax[3] = {c->Fx, c->Fy, c->Fz};
     void *Sax[3] = {c->Sx, c->Sy, c->Sz};
-    const int variant = c->cfg.weno_variant;
     if (c->npatch > 1 && c->schedule == 1)
         W5_CUDA(c, cudaMemsetAsync(c->pcounters, 0, 4 * kMaxTileVariants * sizeof(int), c->stream));
     for (int s = 0; s < 4; ++s) {
@@ -644,8 +654,7 @@ int run_step(w5ct_ctx *c, const double *dt_dev, bool cellb_done, int last_stage 
             for (int ax = 0; ax < (c->sweeps_in_one ? 1 : 3); ++ax) {
                 int rc = record_event(c);
                 if (rc) return rc;
-                W5_CUDA(c, c->sweeps_in_one ? launch_sweep_all<Real>(variant, a3, c->stream)
-                                            : launch_sweep<Real>(ax, variant, a3[ax], c->stream));
+                W5_CUDA(c, launch_sweeps(c, ax, a3));
                 c->launches++;
                 rc = record_event(c);
                 if (rc) return rc;
@@ -930,8 +939,8 @@ int w5ct_init_grid(w5ct_ctx *c, int npatch, const int *n3, const double *dx3) {
         int dev = 0, sms = 0;
         W5_CUDA(c, cudaGetDevice(&dev));
         W5_CUDA(c, cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-        c->sweeps_in_one = ctx_fp64(c) ? sweeps_in_one<double>(c->nx, c->ny, c->nz, sms, c->cfg.precision == W5CT_FP64_DW)
-                                       : sweeps_in_one<float>(c->nx, c->ny, c->nz, sms, false);
+        c->sweeps_in_one = ctx_fp64(c) || sweeps_in_one_f32(c->nx, c->ny, c->nz, sms);
+        c->dw = c->cfg.precision == W5CT_FP64_DW && dw_applies(c->nx, c->ny, c->nz, sms);
     }
     c->schedule = 0;
     for (int v = 0; v < n_variants(c); ++v) {

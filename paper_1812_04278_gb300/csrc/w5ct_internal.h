@@ -9,20 +9,18 @@ namespace w5ct {
 // Record the text that w5ct_last_error(NULL) returns (calls without a context).
 void set_global_error(const char *text);
 
-// Launch the characteristic sweep along `axis` (0, 1, 2) with WENO variant
-// `variant` (0 = JS, 1 = Z) over one patch in the type's default tile
-// (SweepTuning; double: the double-word sweeps), and all three sweeps in one
-// launch (sweep_all_kernel).
-// Defined in w5ct_sweep32.cu / w5ct_sweep64.cu.
-template <typename Real>
-cudaError_t launch_sweep(int axis, int variant, const SweepArgs<Real> &a, cudaStream_t s);
+// Launch the FP32 characteristic sweep along `axis` (0, 1, 2) with WENO
+// variant `variant` (0 = JS, 1 = Z) over one patch in the default tile
+// (SweepTuning), and, in either type, all three sweeps in one launch
+// (sweep_all_kernel).  Defined in w5ct_sweep32.cu / w5ct_sweep64.cu.
+cudaError_t launch_sweep_f32(int axis, int variant, const SweepArgs<float> &a, cudaStream_t s);
 template <typename Real>
 cudaError_t launch_sweep_all(int variant, const SweepArgs<Real> (&a)[3], cudaStream_t s);
 
-// The FP64 single-patch sweeps with the WENO part of every flux in
-// double-word arithmetic, and the shared-memory allowance of their kernels.
-// Defined in w5ct_sweep64dw.cu.
-cudaError_t launch_sweep_f64dw(int axis, int variant, const SweepArgs<double> &a, cudaStream_t s);
+// The three FP64 single-patch sweeps in one launch with the WENO part of every
+// flux in double-word arithmetic, and the shared-memory allowance of its
+// kernels.  Defined in w5ct_sweep64dw.cu.
+cudaError_t launch_sweep_all_f64dw(int variant, const SweepArgs<double> (&a)[3], cudaStream_t s);
 cudaError_t prepare_sweeps_f64dw();
 
 // Sweep tiling per arithmetic type: faces per block in the second tile
@@ -37,8 +35,6 @@ struct SweepTuning;
 // 27.95 and 113.1 for 256-thread blocks of 32 x 16 (a barrier stalls half an
 // SM's warps there), 27.47 and 110.8 for 8 x 32, 28.17 and 113.9 for one face
 // per thread, 28.1 and 112.8 for three, 28.7 and 116.2 for four.
-// FP64 (the double-word sweeps and, through sweep_all_kernel, smaller tiles):
-// FP64-pipe bound, eight warps per SM at up to 255 registers.
 #ifndef W5CT_F32_T2X
 #define W5CT_F32_T2X 8
 #endif
@@ -48,25 +44,6 @@ struct SweepTuning;
 #ifndef W5CT_F32_MINB
 #define W5CT_F32_MINB 4
 #endif
-#ifndef W5CT_F64_T2X
-#define W5CT_F64_T2X 16
-#endif
-#ifndef W5CT_F64_T2YZ
-#define W5CT_F64_T2YZ 16
-#endif
-#ifndef W5CT_F64_MINB
-#define W5CT_F64_MINB 1
-#endif
-// FP64 y- and z-sweeps: tiles of 16 pencils x 32 faces, whose cell box (37 x
-// 16 cells) stages 1.16 cells per face instead of the 1.31 of 32 x 16 (21 x
-// 32 cells); the x-sweep's 32 x 16 tile already stages 37 x 16.
-#ifndef W5CT_F64_BXYZ
-#define W5CT_F64_BXYZ 16
-#endif
-#ifndef W5CT_F64_T2YZ_NARROW
-#define W5CT_F64_T2YZ_NARROW 32
-#endif
-
 #ifndef W5CT_F32_FPT
 #define W5CT_F32_FPT 2
 #endif
@@ -81,16 +58,9 @@ struct SweepTuning<float> {
     static constexpr int T2X = W5CT_F32_T2X, T2YZ = W5CT_F32_T2YZ, MINB = W5CT_F32_MINB, FPT = W5CT_F32_FPT,
                          BXX = W5CT_F32_BXX, BXYZ = W5CT_F32_BXYZ;
 };
-template <>
-struct SweepTuning<double> {
-    static constexpr int T2X = W5CT_F64_T2X, T2YZ = W5CT_F64_T2YZ, MINB = W5CT_F64_MINB, FPT = W5CT_F64_T2X / 8,
-                         BXX = 32, BXYZ = W5CT_F64_BXYZ;
-};
-
 template <int AX, typename Real>
 struct SweepCfg {
-    static constexpr bool kNarrow = sizeof(Real) == 8 && AX != 0;   // FP64 y/z: 16 x 32
-    static constexpr int T2 = AX == 0 ? SweepTuning<Real>::T2X : kNarrow ? W5CT_F64_T2YZ_NARROW : SweepTuning<Real>::T2YZ;
+    static constexpr int T2 = AX == 0 ? SweepTuning<Real>::T2X : SweepTuning<Real>::T2YZ;
     static constexpr int BX = AX == 0 ? SweepTuning<Real>::BXX : SweepTuning<Real>::BXYZ;
     static constexpr int MINB = SweepTuning<Real>::MINB;
     static constexpr int FPT = SweepTuning<Real>::FPT;
@@ -100,12 +70,12 @@ struct SweepCfg {
 
 // Single-patch sweep in tiles of BX x T2 faces, FPT per thread (the block
 // is BX x T2 / FPT threads).
-template <int AX, typename Real, int VAR, int T2, int MINB, int FPT, int BX = 32, bool DW = false>
+template <int AX, typename Real, int VAR, int T2, int MINB, int FPT, int BX = 32>
 struct SinglePatchSweep {
     using TT = SweepTile<AX, T2, BX, FPT>;
     static constexpr size_t smem = (size_t)TT::template cells<Real> * box_quantities<Real>() * sizeof(Real);
     static cudaError_t prepare() {
-        return cudaFuncSetAttribute(sweep_kernel<AX, Real, VAR, T2, MINB, FPT, BX, DW>,
+        return cudaFuncSetAttribute(sweep_kernel<AX, Real, VAR, T2, MINB, FPT, BX>,
                                     cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     }
     static dim3 grid(int nx, int ny, int nz) {
@@ -113,18 +83,21 @@ struct SinglePatchSweep {
         return dim3((nx + BX - 1) / BX, ny, (nz + TT::BZ - 1) / TT::BZ);
     }
     static cudaError_t launch(const SweepArgs<Real> &a, cudaStream_t s) {
-        sweep_kernel<AX, Real, VAR, T2, MINB, FPT, BX, DW><<<grid(a.nx, a.ny, a.nz), dim3(BX, TT::ROWS), smem, s>>>(a);
+        sweep_kernel<AX, Real, VAR, T2, MINB, FPT, BX><<<grid(a.nx, a.ny, a.nz), dim3(BX, TT::ROWS), smem, s>>>(a);
         return cudaGetLastError();
     }
 };
 
 // Tile shapes of the batched sweeps (chosen per patch and axis by the
-// autotuner).  Variant 0 is SweepCfg's tile (32 lanes) in float and 32 x 16
-// in double (patches are 16 to 64 cells across); the float path also
-// has narrower tiles that waste fewer lanes on patches whose sizes are not
-// multiples of 32 or of 16: (BX, T2, faces per thread) = (16, 16, 1),
-// (8, 16, 1), (8, 8, 1).  Every variant keeps 128 registers per thread: min
-// blocks per SM = 512 / threads per block.
+// autotuner).  Variant 0 is 32 x 16; the float path also has narrower tiles
+// that waste fewer lanes on patches whose sizes are not multiples of 32 or of
+// 16: (BX, T2, faces per thread) = (16, 16, 2), (8, 16, 1), (8, 8, 1).  Every
+// variant keeps 128 registers per thread in float: min blocks per SM = 512 /
+// threads per block.  One launch per axis and variant computes a float 32 x 16
+// tile as two halves, in blocks of 128 threads like the single-patch tiles.
+// Step of the 512-patch workload with one variant forced on every patch: 24.7,
+// 25.2, 24.0, 23.4 ms (model choice 23.6); 27.6 for whole 32 x 16 tiles in 256-thread blocks and 26.3 for 16 x 16
+// with one face per thread.
 constexpr int kMaxTileVariants = 4;
 
 #ifndef W5CT_ALL_WAVES32
@@ -139,7 +112,7 @@ struct TileV<AX, Real, 0> {
 };
 template <int AX, typename Real>
 struct TileV<AX, Real, 1> {
-    static constexpr int T2 = 16, BX = 16, FPT = 1, MINB = 2;
+    static constexpr int T2 = 16, BX = 16, FPT = 2, MINB = 4;
 };
 template <int AX, typename Real>
 struct TileV<AX, Real, 2> {
@@ -170,16 +143,19 @@ inline void tile_shape(int axis, int v, int &bx, int &t2) {
 template <int AX, typename Real, int VAR, int V>
 struct BatchedSweep {
     using C = TileV<AX, Real, V>;
-    using TT = SweepTile<AX, C::T2, C::BX, C::FPT>;
+    static constexpr bool kHalves = std::is_same<Real, float>::value && V == 0;
+    static constexpr int BX = kHalves && AX != 0 ? C::BX / 2 : C::BX, T2 = kHalves && AX == 0 ? C::T2 / 2 : C::T2,
+                         MINB = kHalves ? 2 * C::MINB : C::MINB;
+    using TT = SweepTile<AX, T2, BX, C::FPT>;
     static constexpr size_t smem = (size_t)TT::template cells<Real> * box_quantities<Real>() * sizeof(Real);
     static cudaError_t prepare() {
-        return cudaFuncSetAttribute(sweep_batched_kernel<AX, Real, VAR, C::T2, C::MINB, C::BX, C::FPT>,
+        return cudaFuncSetAttribute(sweep_batched_kernel<AX, Real, VAR, T2, MINB, BX, C::FPT, kHalves>,
                                     cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     }
     static cudaError_t launch(const SweepArgs<Real> &a, const PatchGeom *pgs, const int4 *tiles, int ntiles,
                               cudaStream_t s) {
-        sweep_batched_kernel<AX, Real, VAR, C::T2, C::MINB, C::BX, C::FPT>
-            <<<ntiles, dim3(C::BX, TT::ROWS), smem, s>>>(a, pgs, tiles);
+        sweep_batched_kernel<AX, Real, VAR, T2, MINB, BX, C::FPT, kHalves>
+            <<<(unsigned)ntiles * (kHalves ? 2u : 1u), dim3(BX, TT::ROWS), smem, s>>>(a, pgs, tiles);
         return cudaGetLastError();
     }
 };
@@ -261,14 +237,14 @@ struct PersistentLaunch {
 };
 
 // The three sweeps of a stage in one launch (sweep_all_kernel).
-template <typename Real, int VAR>
+template <typename Real, int VAR, bool DW = false>
 struct AllSweeps {
     template <int AX>
     static constexpr size_t smem_of = (size_t)SweepTile<AX, AllTile<AX>::T2, AllTile<AX>::BX, 1>::template cells<Real> *
                                       box_quantities<Real>() * sizeof(Real);
     static constexpr size_t smem = smem_of<0> > smem_of<1> ? smem_of<0> : smem_of<1>;   // (y and z alike)
     static cudaError_t prepare() {
-        return cudaFuncSetAttribute(sweep_all_kernel<Real, VAR>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        return cudaFuncSetAttribute(sweep_all_kernel<Real, VAR, DW>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     }
     static cudaError_t launch(const SweepArgs<Real> (&a)[3], cudaStream_t st) {
         SweepAll<Real> s;
@@ -281,7 +257,7 @@ struct AllSweeps {
             s.nb2[ax] = (n[ax == 2 ? 2 : 1] + t2 - 1) / t2;
             s.first[ax + 1] = s.first[ax] + s.nbx[ax] * s.nb2[ax] * n[ax == 2 ? 1 : 2];
         }
-        sweep_all_kernel<Real, VAR><<<s.first[3], kAllThreads, smem, st>>>(s);
+        sweep_all_kernel<Real, VAR, DW><<<s.first[3], kAllThreads, smem, st>>>(s);
         return cudaGetLastError();
     }
 };
@@ -397,51 +373,38 @@ inline long long sweep_blocks(int axis, int t2, int bx, int nx, int ny, int nz) 
     return nbx * ((ny + t2 - 1) / t2) * nz;     // x- and y-sweeps: t2 pencils or faces along y
 }
 
-// Whether the three sweeps of a single patch go in one launch
-// (sweep_all_kernel).
-// FP64: always.  The small blocks balance the SMs better than they lose by
-// their larger boxes: step of 32^3 1.93 -> 1.01 ms against three launches of the
-// 32 x 16 and 16 x 32 tiles, 64^3 7.68 -> 6.60, 100 x 70 x 50 10.26 -> 9.80 (WENO5),
-// 160^3 101.4 -> 100.4, 256^3 413.4 -> 411.4 ms.
+// Whether the three FP32 sweeps of a single patch go in one launch
+// (sweep_all_kernel; the FP64 ones always do).
+// FP64: the small blocks balance the SMs better than they lose by their larger
+// boxes: step of 32^3 1.93 -> 1.01 ms against three launches of 32 x 16 and 16 x
+// 32 tiles, 64^3 7.68 -> 6.60, 100 x 70 x 50 10.26 -> 9.80 (WENO5), 160^3 101.4 ->
+// 100.4, 256^3 413.4 -> 411.4 ms.
 // FP32: below 8 waves of the default tiles' blocks on the device, where the
 // tails of three launches cost more than the one face per thread: 32^3 0.140 ->
 // 0.092 ms, 64^3 0.279 -> 0.255, 96^3 (5.7 waves) 0.798 -> 0.790, but 112^3 (9
 // waves) 1.260 -> 1.262 and 160^3 3.26 -> 3.37.
-// The double-word sweeps (dw) have no such kernel: they keep their own
-// launches unless one of them has fewer than two blocks per SM.
-template <typename Real>
-inline bool sweeps_in_one(int nx, int ny, int nz, int sms, bool dw) {
-    if (std::is_same<Real, double>::value && !dw) return true;
-    const long long least = dw ? 2LL * sms : (long long)W5CT_ALL_WAVES32 * sms * SweepTuning<Real>::MINB;
-    for (int ax = 0; ax < 3; ++ax) {
-        const long long b = ax == 0 ? sweep_blocks(0, SweepCfg<0, Real>::T2, SweepCfg<0, Real>::BX, nx, ny, nz)
-                                    : sweep_blocks(ax, SweepCfg<1, Real>::T2, SweepCfg<1, Real>::BX, nx, ny, nz);
-        if (b < least) return true;
-    }
-    return false;
+inline bool sweeps_in_one_f32(int nx, int ny, int nz, int sms) {
+    using X = SweepCfg<0, float>;
+    using YZ = SweepCfg<1, float>;
+    const long long least = (long long)W5CT_ALL_WAVES32 * sms * X::MINB;
+    return sweep_blocks(0, X::T2, X::BX, nx, ny, nz) < least || sweep_blocks(1, YZ::T2, YZ::BX, nx, ny, nz) < least ||
+           sweep_blocks(2, YZ::T2, YZ::BX, nx, ny, nz) < least;
 }
 
-template <int AX, typename Real, int VAR>
-cudaError_t launch_sweep_axis(const SweepArgs<Real> &a, cudaStream_t s) {
-    // (their shared memory is allowed by prepare_sweeps() at w5ct_init_grid)
-    if constexpr (std::is_same<Real, double>::value) {
-        return launch_sweep_f64dw(AX, VAR, a, s);
-    } else {
-        using C = SweepCfg<AX, Real>;
-        return SinglePatchSweep<AX, Real, VAR, C::T2, C::MINB, C::FPT, C::BX>::launch(a, s);
-    }
+// Whether W5CT_FP64_DW sweeps a patch in double-word arithmetic: where each
+// sweep has at least two blocks of 512 faces (32 x 16 along x, 16 x 32 in the
+// others) per SM.
+inline bool dw_applies(int nx, int ny, int nz, int sms) {
+    const long long least = 2LL * sms;
+    return sweep_blocks(0, 16, 32, nx, ny, nz) >= least && sweep_blocks(1, 32, 16, nx, ny, nz) >= least &&
+           sweep_blocks(2, 32, 16, nx, ny, nz) >= least;
 }
 
-template <typename Real>
-cudaError_t launch_sweep_impl(int axis, int variant, const SweepArgs<Real> &a, cudaStream_t s) {
-    if (variant == 0) {
-        if (axis == 0) return launch_sweep_axis<0, Real, 0>(a, s);
-        if (axis == 1) return launch_sweep_axis<1, Real, 0>(a, s);
-        return launch_sweep_axis<2, Real, 0>(a, s);
-    }
-    if (axis == 0) return launch_sweep_axis<0, Real, 1>(a, s);
-    if (axis == 1) return launch_sweep_axis<1, Real, 1>(a, s);
-    return launch_sweep_axis<2, Real, 1>(a, s);
+template <int AX, int VAR>
+cudaError_t launch_sweep_axis(const SweepArgs<float> &a, cudaStream_t s) {
+    using C = SweepCfg<AX, float>;
+    // (its shared memory is allowed by prepare_sweeps() at w5ct_init_grid)
+    return SinglePatchSweep<AX, float, VAR, C::T2, C::MINB, C::FPT, C::BX>::launch(a, s);
 }
 
 }  // namespace w5ct

@@ -300,17 +300,15 @@ __device__ __forceinline__ void sweep_tile_rt(const SweepArgs<Real> &a, const Pa
 }
 
 // One tile computed by the whole block, blockDim = (BX, ROWS).
-template <int AX, typename Real, int VAR, int T2, int BX = 32, int FPT = T2 / 8, int SB = kStageBatch,
-          bool DWW = false>
+template <int AX, typename Real, int VAR, int T2, int BX = 32, int FPT = T2 / 8, int SB = kStageBatch>
 __device__ __forceinline__ void sweep_tile(const SweepArgs<Real> &a, const PatchGeom &pg, int tbx, int tby, int tbz,
                                            Real *sm) {
-    sweep_tile_at<AX, Real, VAR, T2, BX, FPT, SB, DWW>(a, pg, tbx, tby, tbz, sm, (int)threadIdx.x, (int)threadIdx.y);
+    sweep_tile_at<AX, Real, VAR, T2, BX, FPT, SB>(a, pg, tbx, tby, tbz, sm, (int)threadIdx.x, (int)threadIdx.y);
 }
 
 // One tile per block over a single patch: BX x T2 / FPT threads (at most
-// 256), FPT faces per thread.  DW (double only): the WENO part of every
-// field's flux in double-word arithmetic (weno_field).
-template <int AX, typename Real, int VAR, int T2, int MINB, int FPT = T2 / 8, int BX = 32, bool DW = false>
+// 256), FPT faces per thread.
+template <int AX, typename Real, int VAR, int T2, int MINB, int FPT = T2 / 8, int BX = 32>
 __global__ void __launch_bounds__(SweepTile<AX, T2, BX, FPT>::NT, MINB) sweep_kernel(SweepArgs<Real> a) {
     extern __shared__ __align__(16) unsigned char w5ct_smem[];
     PatchGeom pg;
@@ -318,8 +316,7 @@ __global__ void __launch_bounds__(SweepTile<AX, T2, BX, FPT>::NT, MINB) sweep_ke
     pg.ny = a.ny;
     pg.nz = a.nz;
     pg.off = 0;
-    sweep_tile<AX, Real, VAR, T2, BX, FPT, kStageBatch, DW>(a, pg, blockIdx.x, blockIdx.y, blockIdx.z,
-                                                            reinterpret_cast<Real *>(w5ct_smem));
+    sweep_tile<AX, Real, VAR, T2, BX, FPT>(a, pg, blockIdx.x, blockIdx.y, blockIdx.z, reinterpret_cast<Real *>(w5ct_smem));
 }
 
 // The three sweeps of a stage over a single patch in one launch, in tiles of
@@ -327,7 +324,8 @@ __global__ void __launch_bounds__(SweepTile<AX, T2, BX, FPT>::NT, MINB) sweep_ke
 // thread; box cells per face 1.16 and 1.31).  They are independent, and a
 // patch of fewer than a few hundred thousand cells does not fill the GPU with
 // one of them: one launch has three times the blocks, one tail and one launch
-// latency.  first[ax] is the first block of axis ax.
+// latency.  first[ax] is the first block of axis ax.  DW (double only): the
+// WENO part of every field's flux in double-word arithmetic (weno_field).
 template <typename Real>
 struct SweepAll {
     SweepArgs<Real> a[3];
@@ -340,8 +338,12 @@ struct AllTile {
     static constexpr int BX = AX == 0 ? 32 : 8, T2 = AX == 0 ? 4 : 16;
 };
 
-template <typename Real, int VAR>
-__global__ void __launch_bounds__(kAllThreads, sizeof(Real) == 8 ? 2 : 4) sweep_all_kernel(SweepAll<Real> s) {
+// Blocks per SM: float 4 (128 registers); double 2 (255 registers; three blocks
+// of 168 spill: 256^3 step 416.4 against 413.4 ms); double-word 3, whose chains
+// of dependent FP32 operations want the warps (128^3 step 37.0 -> 33.9 ms; four
+// blocks no faster).
+template <typename Real, int VAR, bool DW>
+__global__ void __launch_bounds__(kAllThreads, sizeof(Real) == 4 ? 4 : DW ? 3 : 2) sweep_all_kernel(SweepAll<Real> s) {
     extern __shared__ __align__(16) unsigned char w5ct_smem[];
     Real *sm = reinterpret_cast<Real *>(w5ct_smem);
     const int b = blockIdx.x, tid = threadIdx.x;
@@ -354,11 +356,11 @@ __global__ void __launch_bounds__(kAllThreads, sizeof(Real) == 8 ? 2 : 4) sweep_
     pg.nz = s.a[0].nz;
     pg.off = 0;
     if (ax == 0)
-        sweep_tile_at<0, Real, VAR, AllTile<0>::T2, AllTile<0>::BX, 1>(s.a[0], pg, tbx, t1, t2, sm, tid % AllTile<0>::BX, tid / AllTile<0>::BX);
+        sweep_tile_at<0, Real, VAR, AllTile<0>::T2, AllTile<0>::BX, 1, kStageBatch, DW>(s.a[0], pg, tbx, t1, t2, sm, tid % AllTile<0>::BX, tid / AllTile<0>::BX);
     else if (ax == 1)
-        sweep_tile_at<1, Real, VAR, AllTile<1>::T2, AllTile<1>::BX, 1>(s.a[1], pg, tbx, t1, t2, sm, tid % AllTile<1>::BX, tid / AllTile<1>::BX);
+        sweep_tile_at<1, Real, VAR, AllTile<1>::T2, AllTile<1>::BX, 1, kStageBatch, DW>(s.a[1], pg, tbx, t1, t2, sm, tid % AllTile<1>::BX, tid / AllTile<1>::BX);
     else
-        sweep_tile_at<2, Real, VAR, AllTile<2>::T2, AllTile<2>::BX, 1>(s.a[2], pg, tbx, t2, t1, sm, tid % AllTile<2>::BX, tid / AllTile<2>::BX);
+        sweep_tile_at<2, Real, VAR, AllTile<2>::T2, AllTile<2>::BX, 1, kStageBatch, DW>(s.a[2], pg, tbx, t2, t1, sm, tid % AllTile<2>::BX, tid / AllTile<2>::BX);
 }
 
 // Tile tables hold int4 (patch | axis << 28, tile x, tile y, tile z).
@@ -366,13 +368,20 @@ constexpr int kItemAxisShift = 28;
 constexpr int kItemPatchMask = (1 << kItemAxisShift) - 1;
 
 // Several patches: block b computes tile tiles[b] = (patch, tbx, tby, tbz)
-// of shape SweepTile<AX, T2, BX, FPT>.
-template <int AX, typename Real, int VAR, int T2, int MINB, int BX, int FPT>
+// of shape SweepTile<AX, T2, BX, FPT>; HALVES: half b & 1 of tile tiles[b / 2],
+// which is two such shapes side by side (along y for the x-sweep, along x for
+// the others), the second one possibly outside the patch.
+template <int AX, typename Real, int VAR, int T2, int MINB, int BX, int FPT, bool HALVES>
 __global__ void __launch_bounds__(SweepTile<AX, T2, BX, FPT>::NT, MINB)
     sweep_batched_kernel(SweepArgs<Real> a, const PatchGeom *__restrict__ pgs, const int4 *__restrict__ tiles) {
     extern __shared__ __align__(16) unsigned char w5ct_smem[];
-    const int4 t = tiles[blockIdx.x];
+    int4 t = tiles[HALVES ? blockIdx.x >> 1 : blockIdx.x];
     const PatchGeom pg = pgs[t.x & kItemPatchMask];
+    if constexpr (HALVES) {
+        int &i = AX == 0 ? t.z : t.y;
+        i = 2 * i + (blockIdx.x & 1);
+        if (i * (AX == 0 ? T2 : BX) >= (AX == 0 ? pg.ny : pg.nx)) return;   // the whole block
+    }
     sweep_tile<AX, Real, VAR, T2, BX, FPT>(a, pg, t.y, t.z, t.w, reinterpret_cast<Real *>(w5ct_smem));
 }
 

@@ -879,16 +879,51 @@ __device__ __forceinline__ void face_flux(const Real *__restrict__ sm, int ncell
     // ---- WENO parts of the fields: sums and differences of the pairs, upper
     // members m = 1 (v - c_f), 3 (v - c_slow), 2 (v - c_A)
     Real sf, df, ss, ds, sa, da, Fe;
-    auto fields = [&](const P2 (&u)[5], const P2 (&l)[5], Real cL, Real cR, Real ep, Real &sum, Real &dif) {
-        const Real Fu = weno_field<Real, VAR, DWW>(u, alpha(-cL, -cR), ep);
-        const Real Fl = weno_field<Real, VAR, DWW>(l, alpha(cL, cR), ep);
+    [[maybe_unused]] auto fields = [&](const P2 (&u)[5], const P2 (&l)[5], Real cL, Real cR, Real ep, Real &sum, Real &dif) {
+        const Real Fu = weno_field<Real, VAR>(u, alpha(-cL, -cR), ep);
+        const Real Fl = weno_field<Real, VAR>(l, alpha(cL, cR), ep);
         sum = Fu + Fl;
         dif = Fu - Fl;
     };
-    fields(fu, fl, cfL, cfR, eps3, sf, df);
-    fields(su, sl, csL, csR, eps3, ss, ds);
-    fields(au, al, caL, caR, Real(4) * eps3, sa, da);
-    Fe = weno_field<Real, VAR, DWW>(en, m::max_nonneg(m::abs_(vL), m::abs_(vR)), eps3);
+    if constexpr (!DWW) {
+        fields(fu, fl, cfL, cfR, eps3, sf, df);
+        fields(su, sl, csL, csR, eps3, ss, ds);
+        fields(au, al, caL, caR, Real(4) * eps3, sa, da);
+        Fe = weno_field<Real, VAR>(en, m::max_nonneg(m::abs_(vL), m::abs_(vR)), eps3);
+    } else {
+        // double-word: one copy of the interpolants (about 1800 instructions
+        // for the two sides) in a loop over the fields, the projections in
+        // local memory.  Unrolled, the face function was 215 KB of code, which
+        // no instruction cache of an SM holds: 128^3 step 49.0 -> 39.7 ms.  (The
+        // IEEE form, 20 KB, is 1.6% faster unrolled.)
+        P2 F[7][5];
+        Real V[7];
+        const Real cL[7] = {-cfL, cfL, -csL, csL, -caL, caL, Real(0)}, cR[7] = {-cfR, cfR, -csR, csR, -caR, caR, Real(0)};
+#pragma unroll
+        for (int j = 0; j < 5; ++j) {
+            F[0][j] = fu[j];
+            F[1][j] = fl[j];
+            F[2][j] = su[j];
+            F[3][j] = sl[j];
+            F[4][j] = au[j];
+            F[5][j] = al[j];
+            F[6][j] = en[j];
+        }
+#pragma unroll 1
+        for (int mo = 0; mo < 7; ++mo) {
+            P2 f[5];
+#pragma unroll
+            for (int j = 0; j < 5; ++j) f[j] = F[mo][j];
+            V[mo] = weno_field<Real, VAR, true>(f, alpha(cL[mo], cR[mo]), mo == 4 || mo == 5 ? Real(4) * eps3 : eps3);
+        }
+        sf = V[0] + V[1];
+        df = V[0] - V[1];
+        ss = V[2] + V[3];
+        ds = V[2] - V[3];
+        sa = V[4] + V[5];
+        da = V[4] - V[5];
+        Fe = V[6];
+    }
     if (!e.apart) {
         // Appendix A's fallback: the central part through L and R, in the
         // units of the WENO parts, in place of the unprojected one

@@ -4,9 +4,15 @@
 
 namespace w5ct {
 
-template <>
-cudaError_t launch_sweep<float>(int axis, int variant, const SweepArgs<float> &a, cudaStream_t s) {
-    return launch_sweep_impl<float>(axis, variant, a, s);
+cudaError_t launch_sweep_f32(int axis, int variant, const SweepArgs<float> &a, cudaStream_t s) {
+    if (variant == 0) {
+        if (axis == 0) return launch_sweep_axis<0, 0>(a, s);
+        if (axis == 1) return launch_sweep_axis<1, 0>(a, s);
+        return launch_sweep_axis<2, 0>(a, s);
+    }
+    if (axis == 0) return launch_sweep_axis<0, 1>(a, s);
+    if (axis == 1) return launch_sweep_axis<1, 1>(a, s);
+    return launch_sweep_axis<2, 1>(a, s);
 }
 
 template <>

@@ -5,11 +5,6 @@
 namespace w5ct {
 
 template <>
-cudaError_t launch_sweep<double>(int axis, int variant, const SweepArgs<double> &a, cudaStream_t s) {
-    return launch_sweep_impl<double>(axis, variant, a, s);
-}
-
-template <>
 cudaError_t launch_sweep_all<double>(int variant, const SweepArgs<double> (&a)[3], cudaStream_t s) {
     return variant == 0 ? AllSweeps<double, 0>::launch(a, s) : AllSweeps<double, 1>::launch(a, s);
 }

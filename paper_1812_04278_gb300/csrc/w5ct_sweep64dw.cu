@@ -1,5 +1,4 @@
-// w5ct_sweep64dw.cu -- the FP64 single-patch sweep kernels of the default
-// tiles with the WENO part of every characteristic field's flux in
+// w5ct_sweep64dw.cu -- the FP64 single-patch sweeps with the WENO part of every characteristic field's flux in
 // double-word arithmetic (w5ct_physics.cuh, weno_field): the smoothness
 // indicators, the nonlinear weights and the two interpolants of the LF-split
 // differences run on the FP32 pipe, while the cell box, the eigenvectors,
@@ -10,31 +9,13 @@
 
 namespace w5ct {
 
-namespace {
-template <int AX, int VAR>
-using DwSweep = SinglePatchSweep<AX, double, VAR, SweepCfg<AX, double>::T2, SweepCfg<AX, double>::MINB,
-                                 SweepCfg<AX, double>::FPT, SweepCfg<AX, double>::BX, true>;
-}  // namespace
-
-cudaError_t launch_sweep_f64dw(int axis, int variant, const SweepArgs<double> &a, cudaStream_t s) {
-    if (variant == 0) {
-        if (axis == 0) return DwSweep<0, 0>::launch(a, s);
-        if (axis == 1) return DwSweep<1, 0>::launch(a, s);
-        return DwSweep<2, 0>::launch(a, s);
-    }
-    if (axis == 0) return DwSweep<0, 1>::launch(a, s);
-    if (axis == 1) return DwSweep<1, 1>::launch(a, s);
-    return DwSweep<2, 1>::launch(a, s);
+cudaError_t launch_sweep_all_f64dw(int variant, const SweepArgs<double> (&a)[3], cudaStream_t s) {
+    return variant == 0 ? AllSweeps<double, 0, true>::launch(a, s) : AllSweeps<double, 1, true>::launch(a, s);
 }
 
 cudaError_t prepare_sweeps_f64dw() {
-    cudaError_t e;
-    if ((e = DwSweep<0, 0>::prepare()) != cudaSuccess) return e;
-    if ((e = DwSweep<1, 0>::prepare()) != cudaSuccess) return e;
-    if ((e = DwSweep<2, 0>::prepare()) != cudaSuccess) return e;
-    if ((e = DwSweep<0, 1>::prepare()) != cudaSuccess) return e;
-    if ((e = DwSweep<1, 1>::prepare()) != cudaSuccess) return e;
-    return DwSweep<2, 1>::prepare();
+    const cudaError_t e = AllSweeps<double, 0, true>::prepare();
+    return e == cudaSuccess ? AllSweeps<double, 1, true>::prepare() : e;
 }
 
 }  // namespace w5ct
