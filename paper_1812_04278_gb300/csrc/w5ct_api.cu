@@ -46,6 +46,7 @@ struct w5ct_ctx {
     // small device scalars
     double *dt_dev = nullptr;
     unsigned long long *smax = nullptr;
+    unsigned *speed_count = nullptr;
     int *flag = nullptr;
     unsigned long long *hits = nullptr;
     double *part = nullptr;          // kRedBlocks x 8
@@ -289,49 +290,47 @@ int launch_cellb(w5ct_ctx *c) {
             c->pg_dev, c->cells_dev, plane<Real>(c->bs, n, 0), plane<Real>(c->bs, n, 1), plane<Real>(c->bs, n, 2),
             plane<Real>(c->bc, n, 0), plane<Real>(c->bc, n, 1), plane<Real>(c->bc, n, 2));
     } else {
-        cellb_kernel<Real><<<cellb_grid(c->nx, c->ny, c->nz), dim3(32, 8), 0, c->stream>>>(
-            c->nx, c->ny, c->nz, cellb_chunk(c->nx, c->ny, c->nz), plane<Real>(c->bs, n, 0),
-            plane<Real>(c->bs, n, 1), plane<Real>(c->bs, n, 2), plane<Real>(c->bc, n, 0), plane<Real>(c->bc, n, 1),
-            plane<Real>(c->bc, n, 2));
+        W5_CUDA(c, launch_chained(cellb_kernel<Real>, cellb_grid(c->nx, c->ny, c->nz), dim3(32, 8), 0, c->stream, c->nx,
+                                  c->ny, c->nz, cellb_chunk(c->nx, c->ny, c->nz), plane<Real>(c->bs, n, 0),
+                                  plane<Real>(c->bs, n, 1), plane<Real>(c->bs, n, 2), plane<Real>(c->bc, n, 0),
+                                  plane<Real>(c->bc, n, 1), plane<Real>(c->bc, n, 2)));
     }
     c->launches++;
     W5_CUDA(c, cudaGetLastError());
     return W5CT_OK;
 }
 
-// maxima S_d of every patch into smax[3 p + d]
+// maxima S_d of every patch into smax[3 p + d]; with a single patch and
+// cfl, instead its dt into dt_dev (and dt_copy).  smax is zero on entry and
+// left so by the latter; a batch clears it here.
 template <typename Real>
-int launch_speed(w5ct_ctx *c) {
+int launch_speed(w5ct_ctx *c, bool cfl, double *dt_copy) {
     const long long n = c->n;
-    W5_CUDA(c, cudaMemsetAsync(c->smax, 0, 3 * sizeof(unsigned long long) * (size_t)c->npatch, c->stream));
     if (c->npatch > 1) {
+        W5_CUDA(c, cudaMemsetAsync(c->smax, 0, 3 * sizeof(unsigned long long) * (size_t)c->npatch, c->stream));
         speed_batched_kernel<Real><<<c->ncells, kCellBlock, 0, c->stream>>>(
             c->pg_dev, c->cells_dev, plane<Real>(c->qs, n, 0), plane<Real>(c->qs, n, 1), plane<Real>(c->qs, n, 2),
             plane<Real>(c->qs, n, 3), plane<Real>(c->qs, n, 4), plane<Real>(c->bc, n, 0), plane<Real>(c->bc, n, 1),
             plane<Real>(c->bc, n, 2), make_phys<Real>(c->cfg), c->smax, c->flag);
-    } else {
-        long long nb = (n + kRedThreads - 1) / kRedThreads;
-        if (nb > 8 * 152) nb = 8 * 152;
-        speed_kernel<Real><<<(unsigned)nb, kRedThreads, 0, c->stream>>>(
-            n, plane<Real>(c->qs, n, 0), plane<Real>(c->qs, n, 1), plane<Real>(c->qs, n, 2),
-            plane<Real>(c->qs, n, 3), plane<Real>(c->qs, n, 4), plane<Real>(c->bc, n, 0), plane<Real>(c->bc, n, 1),
-            plane<Real>(c->bc, n, 2), make_phys<Real>(c->cfg), c->smax, c->flag);
+        c->launches++;
+        W5_CUDA(c, cudaGetLastError());
+        if (cfl) {
+            dt_batched_kernel<<<(c->npatch + 127) / 128, 128, 0, c->stream>>>(c->pg_dev, c->npatch, c->smax, c->cfg.cfl,
+                                                                            c->dt_dev, dt_copy);
+            c->launches++;
+            W5_CUDA(c, cudaGetLastError());
+        }
+        return W5CT_OK;
     }
+    long long nb = (n + kRedThreads - 1) / kRedThreads;
+    if (nb > 8 * 152) nb = 8 * 152;
+    const CflOut out = {cfl ? c->dt_dev : nullptr, dt_copy, c->cfg.cfl, c->dx, c->dy, c->dz, c->speed_count};
+    W5_CUDA(c, launch_chained(speed_kernel<Real>, dim3((unsigned)nb), dim3(kRedThreads), 0, c->stream, n,
+                              plane<Real>(c->qs, n, 0), plane<Real>(c->qs, n, 1), plane<Real>(c->qs, n, 2),
+                              plane<Real>(c->qs, n, 3), plane<Real>(c->qs, n, 4), plane<Real>(c->bc, n, 0),
+                              plane<Real>(c->bc, n, 1), plane<Real>(c->bc, n, 2), make_phys<Real>(c->cfg), c->smax,
+                              c->flag, out));
     c->launches++;
-    W5_CUDA(c, cudaGetLastError());
-    return W5CT_OK;
-}
-
-// dt of every patch from the maxima (one launch)
-int launch_dt(w5ct_ctx *c, double *dt_copy) {
-    if (c->npatch > 1) {
-        dt_batched_kernel<<<(c->npatch + 127) / 128, 128, 0, c->stream>>>(c->pg_dev, c->npatch, c->smax, c->cfg.cfl,
-                                                                        c->dt_dev, dt_copy);
-    } else {
-        dt_kernel<<<1, 1, 0, c->stream>>>(c->smax, c->cfg.cfl, c->dx, c->dy, c->dz, c->dt_dev, dt_copy);
-    }
-    c->launches++;
-    W5_CUDA(c, cudaGetLastError());
     return W5CT_OK;
 }
 
@@ -340,7 +339,7 @@ void launch_update_stage(w5ct_ctx *c, const UpdateArgs<Real> &u) {
     if (c->npatch > 1)
         update_batched_kernel<Real, S><<<c->ncells, kCellBlock, 0, c->stream>>>(u, c->pg_dev, c->cells_dev, u.dt);
     else
-        update_kernel<Real, S><<<cell_grid(c), dim3(32, 8), 0, c->stream>>>(u);
+        launch_chained(update_kernel<Real, S>, cell_grid(c), dim3(32, 8), 0, c->stream, u);   // (the caller checks)
 }
 
 // The stage-update arguments of the context's buffers (dt from dt_dev).
@@ -697,11 +696,12 @@ int read_flag(w5ct_ctx *c, int *flag_out) {
 int speeds_impl(w5ct_ctx *c, double *out) {
     int rc = ctx_fp64(c) ? launch_cellb<double>(c) : launch_cellb<float>(c);
     if (rc) return rc;
-    rc = ctx_fp64(c) ? launch_speed<double>(c) : launch_speed<float>(c);
+    rc = ctx_fp64(c) ? launch_speed<double>(c, false, nullptr) : launch_speed<float>(c, false, nullptr);
     if (rc) return rc;
     std::vector<unsigned long long> bits(3 * (size_t)c->npatch);
     W5_CUDA(c, cudaMemcpyAsync(bits.data(), c->smax, bits.size() * sizeof(unsigned long long), cudaMemcpyDeviceToHost,
                                c->stream));
+    W5_CUDA(c, cudaMemsetAsync(c->smax, 0, bits.size() * sizeof(unsigned long long), c->stream));
     int flag = 0;
     rc = read_flag(c, &flag);
     if (rc) return rc;
@@ -755,11 +755,11 @@ unsigned transfer_blocks(size_t np) {
 
 template <typename Real>
 int launch_load_state(w5ct_ctx *c, size_t off, size_t np, const double *cons, const double *bface, bool there) {
-    load_state_kernel<Real><<<transfer_blocks(np), 256, 0, c->stream>>>(
-        c->n, (long long)off, (long long)np, there ? c->q0 + off : cons, there ? c->b0 + off : bface, there, c->q0, c->b0,
-        (Real *)c->qs, (Real *)c->bs, (Real *)c->q0r, (Real *)c->b0r, c->flag, c->hits);
+    W5_CUDA(c, launch_chained(load_state_kernel<Real>, dim3(transfer_blocks(np)), dim3(256), 0, c->stream, c->n,
+                              (long long)off, (long long)np, there ? c->q0 + off : cons, there ? c->b0 + off : bface, there,
+                              c->q0, c->b0, (Real *)c->qs, (Real *)c->bs, (Real *)c->q0r, (Real *)c->b0r, c->flag,
+                              c->hits));
     c->launches++;
-    W5_CUDA(c, cudaGetLastError());
     return W5CT_OK;
 }
 
@@ -892,7 +892,7 @@ int w5ct_init_grid(w5ct_ctx *c, int npatch, const int *n3, const double *dx3) {
     const bool fp32 = !ctx_fp64(c);
     const size_t o_q0r = fp32 ? take(5 * n * rs) : 0, o_b0r = fp32 ? take(3 * n * rs) : 0;
     const size_t np = (size_t)npatch;
-    const size_t o_dt = take(8 * np), o_smax = take(24 * np), o_flag = take(4), o_hits = take(8);
+    const size_t o_dt = take(8 * np), o_smax = take(24 * np), o_count = take(4), o_flag = take(4), o_hits = take(8);
     const size_t o_part = take((size_t)kRedBlocks * 8 * 8), o_red = take(64);
     const size_t o_pg = take(sizeof(PatchGeom) * np);
     const size_t o_pc = take(sizeof(int) * 4 * kMaxTileVariants);
@@ -920,6 +920,7 @@ int w5ct_init_grid(w5ct_ctx *c, int npatch, const int *n3, const double *dx3) {
     c->b0r = fp32 ? (void *)(b + o_b0r) : (void *)c->b0;
     c->dt_dev = (double *)(b + o_dt);
     c->smax = (unsigned long long *)(b + o_smax);
+    c->speed_count = (unsigned *)(b + o_count);
     c->flag = (int *)(b + o_flag);
     c->hits = (unsigned long long *)(b + o_hits);
     c->part = (double *)(b + o_part);
@@ -948,6 +949,8 @@ int w5ct_init_grid(w5ct_ctx *c, int npatch, const int *n3, const double *dx3) {
                                                              : persistent_grid<float>(c->cfg.weno_variant, v, c->pgrid[v]);
         W5_CUDA(c, eg);
     }
+    W5_CUDA(c, cudaMemsetAsync(c->smax, 0, 24 * np, c->stream));
+    W5_CUDA(c, cudaMemsetAsync(c->speed_count, 0, 4, c->stream));
     W5_CUDA(c, cudaMemsetAsync(c->flag, 0, 4, c->stream));
     W5_CUDA(c, cudaMemsetAsync(c->hits, 0, 8, c->stream));
     W5_CUDA(c, cudaStreamSynchronize(c->stream));
@@ -997,10 +1000,10 @@ int w5ct_get_state(w5ct_ctx *c, int patch, double *cons, double *bface, double *
         if (!c->host_flag) W5_CUDA(c, cudaHostAlloc(&c->host_flag, sizeof(int), cudaHostAllocMapped));
         int *hf = nullptr;
         W5_CUDA(c, cudaHostGetDevicePointer(&hf, c->host_flag, 0));
-        store_state_kernel<<<transfer_blocks(np), 256, 0, c->stream>>>(c->n, (long long)off, (long long)np, c->q0, c->b0,
-                                                                      cons, bface, c->flag, hf);
+        W5_CUDA(c, launch_chained(store_state_kernel, dim3(transfer_blocks(np)), dim3(256), 0, c->stream, c->n,
+                                  (long long)off, (long long)np, (const double *)c->q0, (const double *)c->b0, cons, bface,
+                                  (const int *)c->flag, hf));
         c->launches++;
-        W5_CUDA(c, cudaGetLastError());
         W5_CUDA(c, cudaStreamSynchronize(c->stream));
         return flag_status(c, *(volatile int *)c->host_flag);
     }
@@ -1054,9 +1057,7 @@ int w5ct_step_cfl(w5ct_ctx *c, double *dt_dev_out) {
     if (c->npatch > 1 && c->schedule == 2) return fused_step(c, nullptr, dt_dev_out);
     rc = ctx_fp64(c) ? launch_cellb<double>(c) : launch_cellb<float>(c);
     if (rc) return rc;
-    rc = ctx_fp64(c) ? launch_speed<double>(c) : launch_speed<float>(c);
-    if (rc) return rc;
-    rc = launch_dt(c, dt_dev_out);
+    rc = ctx_fp64(c) ? launch_speed<double>(c, true, dt_dev_out) : launch_speed<float>(c, true, dt_dev_out);
     if (rc) return rc;
     return step_impl(c, c->dt_dev, true);
 }

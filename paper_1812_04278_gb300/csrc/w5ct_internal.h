@@ -9,6 +9,27 @@ namespace w5ct {
 // Record the text that w5ct_last_error(NULL) returns (calls without a context).
 void set_global_error(const char *text);
 
+// Launch a kernel of a single-patch step so that its blocks may be scheduled
+// before the kernel ahead of it in the stream has drained (programmatic
+// dependent launch; the kernel waits for it in chain_begin).  A 32^3 step is 13
+// kernels of 3 to 10 us, and their launch latencies do not overlap otherwise:
+// two 32^3 FP32-bulk steps with their state loaded and read back 250 -> 186 us
+// (of that, dt formed by the CFL kernel's last block: two operations a step).
+template <typename... P, typename... A>
+cudaError_t launch_chained(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
 // Launch the FP32 characteristic sweep along `axis` (0, 1, 2) with WENO
 // variant `variant` (0 = JS, 1 = Z) over one patch in the default tile
 // (SweepTuning), and, in either type, all three sweeps in one launch
@@ -83,8 +104,8 @@ struct SinglePatchSweep {
         return dim3((nx + BX - 1) / BX, ny, (nz + TT::BZ - 1) / TT::BZ);
     }
     static cudaError_t launch(const SweepArgs<Real> &a, cudaStream_t s) {
-        sweep_kernel<AX, Real, VAR, T2, MINB, FPT, BX><<<grid(a.nx, a.ny, a.nz), dim3(BX, TT::ROWS), smem, s>>>(a);
-        return cudaGetLastError();
+        return launch_chained(sweep_kernel<AX, Real, VAR, T2, MINB, FPT, BX>, grid(a.nx, a.ny, a.nz), dim3(BX, TT::ROWS),
+                              smem, s, a);
     }
 };
 
@@ -257,8 +278,7 @@ struct AllSweeps {
             s.nb2[ax] = (n[ax == 2 ? 2 : 1] + t2 - 1) / t2;
             s.first[ax + 1] = s.first[ax] + s.nbx[ax] * s.nb2[ax] * n[ax == 2 ? 1 : 2];
         }
-        sweep_all_kernel<Real, VAR, DW><<<s.first[3], kAllThreads, smem, st>>>(s);
-        return cudaGetLastError();
+        return launch_chained(sweep_all_kernel<Real, VAR, DW>, dim3(s.first[3]), dim3(kAllThreads), smem, st, s);
     }
 };
 

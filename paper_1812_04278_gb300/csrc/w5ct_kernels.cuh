@@ -22,6 +22,18 @@ __device__ __forceinline__ int wrapi(int g, int n) {
     return r < 0 ? r + n : r;
 }
 
+// The kernels of a single-patch step follow one another in a stream through
+// programmatic dependent launches (launch_chained, w5ct_internal.h): each
+// begins with a wait for the kernel before it to be complete and its writes
+// visible, then lets the next one's blocks be scheduled as soon as its own have
+// all come this far (so at most one kernel waits).  Every global access lies after chain_begin(); data the kernel
+// before may write is read by ordinary loads (no __restrict__, which would
+// allow the non-coherent path).
+__device__ __forceinline__ void chain_begin() {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
 // ======================================================================
 // characteristic sweep (Sec. 2.2 + Appendix A + Eqs. fct1-fct6)
 // ======================================================================
@@ -311,6 +323,7 @@ __device__ __forceinline__ void sweep_tile(const SweepArgs<Real> &a, const Patch
 template <int AX, typename Real, int VAR, int T2, int MINB, int FPT = T2 / 8, int BX = 32>
 __global__ void __launch_bounds__(SweepTile<AX, T2, BX, FPT>::NT, MINB) sweep_kernel(SweepArgs<Real> a) {
     extern __shared__ __align__(16) unsigned char w5ct_smem[];
+    chain_begin();
     PatchGeom pg;
     pg.nx = a.nx;
     pg.ny = a.ny;
@@ -345,6 +358,7 @@ struct AllTile {
 template <typename Real, int VAR, bool DW>
 __global__ void __launch_bounds__(kAllThreads, sizeof(Real) == 4 ? 4 : DW ? 3 : 2) sweep_all_kernel(SweepAll<Real> s) {
     extern __shared__ __align__(16) unsigned char w5ct_smem[];
+    chain_begin();
     Real *sm = reinterpret_cast<Real *>(w5ct_smem);
     const int b = blockIdx.x, tid = threadIdx.x;
     const int ax = b < s.first[1] ? 0 : b < s.first[2] ? 1 : 2;
@@ -434,9 +448,9 @@ inline dim3 cellb_grid(int nx, int ny, int nz) {
 }
 
 template <typename Real>
-__global__ void __launch_bounds__(256) cellb_kernel(int nx, int ny, int nz, int chunk, const Real *__restrict__ bx,
-                                                    const Real *__restrict__ by, const Real *__restrict__ bz,
-                                                    Real *__restrict__ Bx, Real *__restrict__ By, Real *__restrict__ Bz) {
+__global__ void __launch_bounds__(256) cellb_kernel(int nx, int ny, int nz, int chunk, const Real *bx,
+                                                    const Real *by, const Real *bz, Real *Bx, Real *By, Real *Bz) {
+    chain_begin();
     const int i = blockIdx.x * 32 + threadIdx.x, j = blockIdx.y * 8 + threadIdx.y;
     const int k0 = blockIdx.z * chunk, k1 = min(k0 + chunk, nz);
     if (i >= nx || j >= ny) return;
@@ -449,8 +463,10 @@ __global__ void __launch_bounds__(256) cellb_kernel(int nx, int ny, int nz, int 
     for (int k = k0; k < k1; ++k) {
         const long long p = col + sz * k;
         const Real z3 = bz[col + sz * (k + 1 < nz ? k + 1 : 0)];
-        Bx[p] = face_to_cell<Real>(bx[p + xm2], bx[p + xm1], bx[p], bx[p + xp1]);
-        By[p] = face_to_cell<Real>(by[p + ym2], by[p + ym1], by[p], by[p + yp1]);
+        const Real x = face_to_cell<Real>(bx[p + xm2], bx[p + xm1], bx[p], bx[p + xp1]);
+        const Real y = face_to_cell<Real>(by[p + ym2], by[p + ym1], by[p], by[p + yp1]);
+        Bx[p] = x;
+        By[p] = y;
         Bz[p] = face_to_cell<Real>(z0, z1, z2, z3);
         z0 = z1;
         z1 = z2;
@@ -740,6 +756,7 @@ __device__ __forceinline__ void update_cell(const UpdateArgs<Real> &a, const Upd
 
 template <typename Real, int STAGE>
 __global__ void __launch_bounds__(256, UpdTuning<Real>::MINB) update_kernel(UpdateArgs<Real> a) {
+    chain_begin();
     const int i = blockIdx.x * 32 + threadIdx.x, j = blockIdx.y * 8 + threadIdx.y, k = blockIdx.z;
     if (i >= a.nx || j >= a.ny) return;
     const UpdGeom<Real> ug = {a.nx, a.ny, a.nz, 0, a.rdx, a.rdy, a.rdz, a.drdx, a.drdy, a.drdz};
@@ -800,57 +817,38 @@ __device__ __forceinline__ void block_reduce(T (&v)[N], bool is_max[N], T *red /
     }
 }
 
-// fast signal speed |v_n| + c_f of a cell along one axis (Eq. cfl), float
-__device__ __forceinline__ float signal_speed(float r, float vn, float P, float Bn, float B1, float B2,
-                                              const Phys<float> &K) {
-    using m = M<float>;
-    const float ir = m::rcp_(r);
-    const float cs2 = K.gamma * P * ir;
-    const float ca2 = Bn * Bn * ir;
-    const float bt2 = (B1 * B1 + B2 * B2) * ir;
-    const float dd = (cs2 - ca2) * (cs2 - ca2) + bt2 * (bt2 + 2.0f * ca2 + 2.0f * cs2);
-    const float sd = m::sqrt_(dd);
-    const float aa = ca2 + bt2 - cs2;
-    const float big = 0.5f * (sd + m::abs_(aa));
-    const float oth = big > 0.0f ? m::div_(cs2 * bt2, big) : 0.0f;
-    const float cf2 = cs2 + (aa >= 0.0f ? big : oth);
+// fast signal speed |v_n| + c_f of a cell along one axis (Eq. cfl)
+template <typename Real>
+__device__ __forceinline__ Real signal_speed(Real r, Real vn, Real P, Real Bn, Real B1, Real B2, const Phys<Real> &K) {
+    using m = M<Real>;
+    const Real ir = m::rcp_(r);
+    const Real cs2 = K.gamma * P * ir;
+    const Real ca2 = Bn * Bn * ir;
+    const Real bt2 = (B1 * B1 + B2 * B2) * ir;
+    const Real dd = (cs2 - ca2) * (cs2 - ca2) + bt2 * (bt2 + Real(2) * ca2 + Real(2) * cs2);
+    const Real sd = m::sqrt_(dd);
+    const Real aa = ca2 + bt2 - cs2;
+    const Real big = Real(0.5) * (sd + m::abs_(aa));
+    const Real oth = big > Real(0) ? cs2 * bt2 * m::rcp_(big) : Real(0);
+    const Real cf2 = cs2 + (aa >= Real(0) ? big : oth);
     return m::abs_(vn) + m::sqrt_(cf2);
 }
 
 // |v_d| + c_f^d of one cell for d = x, y, z folded into v (Eq. cfl); a NaN is
-// dropped (bad is set).  In double the squares and reciprocals are shared by
-// the three axes (110 FP64 instructions instead of 180).
+// dropped (bad is set)
 template <typename Real>
 __device__ __forceinline__ void cell_speeds(Real r, Real m0, Real m1, Real m2, Real E, Real bx, Real by, Real bz,
                                             const Phys<Real> &K, Real (&v)[3], bool &bad) {
     using m = M<Real>;
     if (K.floors && r < K.rho_min) r = K.rho_min;
-    if constexpr (float_based<Real>) {
-        const Real ir = m::rcp_(r);
-        const Real vx = m0 * ir, vy = m1 * ir, vz = m2 * ir;
-        Real P = K.gm1 * (E - Real(0.5) * r * (vx * vx + vy * vy + vz * vz) - Real(0.5) * (bx * bx + by * by + bz * bz));
-        if (K.floors && P < K.p_min) P = K.p_min;
-        if (!(r > Real(0)) || !m::finite_pos(P)) bad = true;
-        v[0] = fmaxf(v[0], signal_speed(r, vx, P, bx, by, bz, K));
-        v[1] = fmaxf(v[1], signal_speed(r, vy, P, by, bz, bx, K));
-        v[2] = fmaxf(v[2], signal_speed(r, vz, P, bz, bx, by, K));
-    } else {
-        const Real ir = m::rcp3_(r);
-        const Real u[3] = {m0 * ir, m1 * ir, m2 * ir};
-        const Real B2[3] = {bx * bx, by * by, bz * bz};
-        Real P = K.gm1 * (E - Real(0.5) * (r * (u[0] * u[0] + u[1] * u[1] + u[2] * u[2]) + (B2[0] + B2[1] + B2[2])));
-        if (K.floors && P < K.p_min) P = K.p_min;
-        if (!(r > Real(0)) || !m::finite_pos(P)) bad = true;
-        const Real cs2 = K.gamma * P * ir;
-        const Real a2[3] = {B2[0] * ir, B2[1] * ir, B2[2] * ir};
-#pragma unroll
-        for (int d = 0; d < 3; ++d) {
-            Real fmc, cms, cf2;
-            speeds_fast<Real>(cs2, a2[d], a2[(d + 1) % 3] + a2[(d + 2) % 3], fmc, cms, cf2);
-            const Real s = m::abs_(u[d]) + cf2 * m::rsqrt_(cf2);
-            v[d] = s > v[d] ? s : v[d];
-        }
-    }
+    const Real ir = m::rcp_(r);
+    const Real vx = m0 * ir, vy = m1 * ir, vz = m2 * ir;
+    Real P = K.gm1 * (E - Real(0.5) * r * (vx * vx + vy * vy + vz * vz) - Real(0.5) * (bx * bx + by * by + bz * bz));
+    if (K.floors && P < K.p_min) P = K.p_min;
+    if (!(r > Real(0)) || !m::finite_pos(P)) bad = true;
+    v[0] = m::max_(v[0], signal_speed<Real>(r, vx, P, bx, by, bz, K));
+    v[1] = m::max_(v[1], signal_speed<Real>(r, vy, P, by, bz, bx, K));
+    v[2] = m::max_(v[2], signal_speed<Real>(r, vz, P, bz, bx, by, K));
 }
 
 // non-negative floats and doubles order like their bit patterns: maxima on
@@ -935,9 +933,23 @@ __device__ __forceinline__ bool float_speeds(const double (&q)[8], const FloatPh
     return ok && up[0] < 1e18f && up[1] < 1e18f && up[2] < 1e18f;
 }
 
+// dt = CFL / sum_d (S_d / dx_d), with the same rounded operations as the
+// host-side w5ct_cfl_dt (no contraction), so both give the same dt
+__device__ __forceinline__ double cfl_dt(double s0, double s1, double s2, double cfl, double dx, double dy, double dz) {
+    return __ddiv_rn(cfl, __dadd_rn(__dadd_rn(__ddiv_rn(s0, dx), __ddiv_rn(s1, dy)), __ddiv_rn(s2, dz)));
+}
+
+// Where speed_kernel's last block writes dt (dt = NULL: it leaves the maxima
+// for the host instead).  count: blocks done, wraps to 0.
+struct CflOut {
+    double *dt, *dt_copy;
+    double cfl, dx, dy, dz;
+    unsigned *count;
+};
+
 // |v_d| + c_f^d maxima of the stage state (Eq. cfl).  In float HBM-bound.  In
-// double the FP64 pipe would bound it (about 110 instructions per cell: 3.9
-// ms at 256^3 with 180 of them, where reading the 8 planes takes 0.16 ms), so
+// double the FP64 pipe would bound it (180 instructions per cell: 3.9 ms at
+// 256^3, where reading the 8 planes takes 0.16 ms), so
 // a cell is evaluated in double only if its float upper bound reaches the
 // largest float lower bound its warp has met and the largest value any warp
 // has published; the maxima are those of all cells.  256^3: 3.93 -> 0.24 ms.
@@ -945,7 +957,8 @@ template <typename Real>
 __global__ void __launch_bounds__(kRedThreads, 4) speed_kernel(long long n, const Real *q0, const Real *q1, const Real *q2,
                                                             const Real *q3, const Real *q4, const Real *B0,
                                                             const Real *B1, const Real *B2, Phys<Real> K,
-                                                            unsigned long long *smax, int *flag) {
+                                                            unsigned long long *smax, int *flag, CflOut out) {
+    chain_begin();
     [[maybe_unused]] __shared__ Real red[3 * 8];
     Real v[3] = {Real(0), Real(0), Real(0)};
     [[maybe_unused]] float top[3] = {0.0f, 0.0f, 0.0f};
@@ -997,6 +1010,17 @@ __global__ void __launch_bounds__(kRedThreads, 4) speed_kernel(long long n, cons
     }
     if (bad) atomicOr(flag, 1);
     if constexpr (!std::is_same<Real, double>::value) block_speeds<Real, kRedThreads / 32>(v, red, threadIdx.x, smax);
+    if (!out.dt) return;
+    // the last block to finish forms dt from the maxima and clears them
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0 && atomicInc(out.count, gridDim.x - 1) == gridDim.x - 1) {
+        double s[3];
+        for (int d = 0; d < 3; ++d) s[d] = __longlong_as_double((long long)atomicExch(smax + d, 0ULL));
+        const double v1 = cfl_dt(s[0], s[1], s[2], out.cfl, out.dx, out.dy, out.dz);
+        *out.dt = v1;
+        if (out.dt_copy) *out.dt_copy = v1;
+    }
 }
 
 // Several patches: block b covers the cells of cell block cells[b] (see
@@ -1024,7 +1048,7 @@ __global__ void __launch_bounds__(kCellBlock) speed_batched_kernel(const PatchGe
     block_speeds<Real, kCellBlock / 32>(v, red, tid, smax + 3 * (size_t)t.x);
 }
 
-// dt of every patch, as dt_kernel: dts[p] = CFL / sum_d (S_d / dx_d)
+// dt of every patch: dts[p] = CFL / sum_d (S_d / dx_d)
 static __global__ void dt_batched_kernel(const PatchGeom *__restrict__ pgs, int npatch,
                                          const unsigned long long *smax, double cfl, double *dts, double *dts_copy) {
     const int p = blockIdx.x * blockDim.x + threadIdx.x;
@@ -1033,8 +1057,7 @@ static __global__ void dt_batched_kernel(const PatchGeom *__restrict__ pgs, int 
     const double s1 = __longlong_as_double((long long)smax[3 * p + 1]);
     const double s2 = __longlong_as_double((long long)smax[3 * p + 2]);
     const PatchGeom pg = pgs[p];
-    const double sum = __dadd_rn(__dadd_rn(__ddiv_rn(s0, pg.dx), __ddiv_rn(s1, pg.dy)), __ddiv_rn(s2, pg.dz));
-    const double v = __ddiv_rn(cfl, sum);
+    const double v = cfl_dt(s0, s1, s2, cfl, pg.dx, pg.dy, pg.dz);
     dts[p] = v;
     if (dts_copy) dts_copy[p] = v;
 }
@@ -1042,19 +1065,6 @@ static __global__ void dt_batched_kernel(const PatchGeom *__restrict__ pgs, int 
 static __global__ void fill_kernel(double *dst, int n, double v) {
     const int p = blockIdx.x * blockDim.x + threadIdx.x;
     if (p < n) dst[p] = v;
-}
-
-// dt = CFL / sum_d (S_d / dx_d), with the same rounded operations as the
-// host-side w5ct_cfl_dt (no contraction), so both give the same dt
-static __global__ void dt_kernel(const unsigned long long *smax, double cfl, double dx, double dy, double dz,
-                                 double *dt, double *dt_copy) {
-    const double s0 = __longlong_as_double((long long)smax[0]);
-    const double s1 = __longlong_as_double((long long)smax[1]);
-    const double s2 = __longlong_as_double((long long)smax[2]);
-    const double sum = __dadd_rn(__dadd_rn(__ddiv_rn(s0, dx), __ddiv_rn(s1, dy)), __ddiv_rn(s2, dz));
-    const double v = __ddiv_rn(cfl, sum);
-    *dt = v;
-    if (dt_copy) *dt_copy = v;
 }
 
 static __global__ void set_scalar_kernel(double *dst, double v) { *dst = v; }
@@ -1153,6 +1163,7 @@ __global__ void __launch_bounds__(256) load_state_kernel(long long n, long long 
                                                          const double *bface, bool there, double *q0, double *b0,
                                                          Real *qs, Real *bs, Real *q0r, Real *b0r, int *flag,
                                                          unsigned long long *hits) {
+    chain_begin();
     constexpr bool kCopy = !std::is_same<Real, double>::value;
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         *flag = 0;
@@ -1180,9 +1191,9 @@ __global__ void __launch_bounds__(256) load_state_kernel(long long n, long long 
 // NULL), and the non-physical flag into mapped host memory: one launch
 // instead of 9 copies.
 static __global__ void __launch_bounds__(256) store_state_kernel(long long n, long long off, long long np,
-                                                                 const double *__restrict__ q0,
-                                                                 const double *__restrict__ b0, double *cons,
+                                                                 const double *q0, const double *b0, double *cons,
                                                                  double *bface, const int *flag, int *host_flag) {
+    chain_begin();
     if (blockIdx.x == 0 && threadIdx.x == 0) *host_flag = *flag;
     for (long long i = blockIdx.x * 256LL + threadIdx.x; i < np; i += 256LL * gridDim.x) {
         double v[8];
