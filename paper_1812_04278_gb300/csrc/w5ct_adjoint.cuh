@@ -36,6 +36,20 @@ constexpr int kAdjPrim = 77;                   // interface primitives (C_RHO ..
 constexpr int kAdjSide = 85;                   // (v_n, c_f, c_A, c_slow) of the lower cell, then of the upper
 constexpr int kAdjFacePlanes = 93;
 constexpr int kAdjFluxPlanes = 21;             // the first planes lie in the context's flux buffers
+// The planes are stored in runs of kAdjRun faces, plane after plane within a
+// run: a thread forms one address per face and part, and every plane is a
+// constant offset from it (with whole planes the 64-bit address arithmetic of
+// 93 stores and of about 120 loads was a tenth of both kernels in float).
+constexpr int kAdjRun = 128;
+constexpr size_t adj_run_cells(size_t n) { return (n + kAdjRun - 1) / kAdjRun * kAdjRun; }
+
+template <typename Real>
+struct AdjFaceRef {
+    Real *a, *b;
+    __device__ __forceinline__ Real &operator[](int k) const {
+        return k < kAdjFluxPlanes ? a[k * kAdjRun] : b[(k - kAdjFluxPlanes) * kAdjRun];
+    }
+};
 
 template <typename Real>
 struct AdjSweepArgs {
@@ -49,9 +63,9 @@ struct AdjSweepArgs {
     double *outq, *outb;       // 5 planes of the state's adjoint, 3 of the cell field's
     bool first;                // the first axis of the stage writes outq, outb, the others add
     Phys<Real> K;
-    __device__ __forceinline__ Real *face_plane(int k) const {
-        const size_t n = (size_t)nx * ny * nz;
-        return k < kAdjFluxPlanes ? fa + (size_t)k * n : fb + (size_t)(k - kAdjFluxPlanes) * n;
+    __device__ __forceinline__ AdjFaceRef<Real> face(size_t p) const {
+        const size_t run = p / kAdjRun, at = p % kAdjRun;
+        return {fa + run * (kAdjFluxPlanes * kAdjRun) + at, fb + run * ((kAdjFacePlanes - kAdjFluxPlanes) * kAdjRun) + at};
     }
 };
 
@@ -242,7 +256,7 @@ __global__ void __launch_bounds__(BX *T2, MINB) adj_face_kernel(AdjSweepArgs<R> 
         const int gx = wrapi(x0 - (AX == 0 ? 2 : 0) + cx, nx), gy = wrapi(y0 - (AX == 1 ? 2 : 0) + cy, ny),
                   gz = wrapi(z0 - (AX == 2 ? 2 : 0) + cz, nz);
         const size_t g = (size_t)gx + (size_t)nx * ((size_t)gy + (size_t)ny * (size_t)gz);
-        cell_fill<R, AX>(sm + c, TT::NC, a.q[0][g], a.q[1][g], a.q[2][g], a.q[3][g], a.q[4][g], a.bc[0][g],
+        cell_fill<R, AX>(sm, c, TT::NC, a.q[0][g], a.q[1][g], a.q[2][g], a.q[3][g], a.q[4][g], a.bc[0][g],
                          a.bc[1][g], a.bc[2][g], K, bad, hit);
     }
     __syncthreads();
@@ -271,6 +285,7 @@ __global__ void __launch_bounds__(BX *T2, MINB) adj_face_kernel(AdjSweepArgs<R> 
     constexpr int ST = TT::ST, NC = TT::NC;
     const size_t n = (size_t)nx * ny * nz;
     const size_t p = (size_t)gx + (size_t)nx * ((size_t)gy + (size_t)ny * (size_t)gz);
+    const AdjFaceRef<R> out_ = a.face(p);
 
 #define SMQ(q, k) box[(q) * NC + (k) * ST]
     // stencil pair (dF_c, du_c) at position j
@@ -482,8 +497,8 @@ __global__ void __launch_bounds__(BX *T2, MINB) adj_face_kernel(AdjSweepArgs<R> 
         transpose(X0, X4, X5, q, F[0][j], F[1][j], F[2][j], F[3][j], F[4][j], F[5][j], F[6][j], out);
 #pragma unroll
         for (int c = 0; c < 7; ++c) {
-            a.face_plane(kAdjDiff + (c * 5 + j) * 2)[p] = pair_x(out[c]);
-            a.face_plane(kAdjDiff + (c * 5 + j) * 2 + 1)[p] = pair_y(out[c]);
+            out_[kAdjDiff + (c * 5 + j) * 2] = pair_x(out[c]);
+            out_[kAdjDiff + (c * 5 + j) * 2 + 1] = pair_y(out[c]);
         }
     }
     if (!e.apart) {
@@ -516,9 +531,9 @@ __global__ void __launch_bounds__(BX *T2, MINB) adj_face_kernel(AdjSweepArgs<R> 
         Fe += u * (pair_x(Xc[0]) - tau * g);
     }
 #pragma unroll
-    for (int c = 0; c < 7; ++c) a.face_plane(kAdjCentral + c)[p] = lX0[c];
+    for (int c = 0; c < 7; ++c) out_[kAdjCentral + c] = lX0[c];
 #pragma unroll
-    for (int t = 0; t < 8; ++t) a.face_plane(kAdjSide + t)[p] = side[t];
+    for (int t = 0; t < 8; ++t) out_[kAdjSide + t] = side[t];
 #undef SMQ
 
     // ---- back-projection's scalars
@@ -616,7 +631,7 @@ __global__ void __launch_bounds__(BX *T2, MINB) adj_face_kernel(AdjSweepArgs<R> 
     lr -= ir * (ir * lir);
     const R lw[8] = {lr, lvn, lvt1, lvt2, R(2) * Bn * ir * lca2, lBt1, lBt2, lP};
 #pragma unroll
-    for (int t = 0; t < 8; ++t) a.face_plane(kAdjPrim + t)[p] = lw[t];
+    for (int t = 0; t < 8; ++t) out_[kAdjPrim + t] = lw[t];
 }
 
 // Reverse of cell_fill<R, AX>: given the adjoints lq of a cell's 23
@@ -749,14 +764,14 @@ __global__ void __launch_bounds__(256) adj_cell_kernel(AdjSweepArgs<R> a) {
         return (size_t)x + (size_t)nx * ((size_t)y + (size_t)ny * (size_t)z);
     };
     auto differences = [&](int x, int y, int z, int o, int row, int col) {
-        size_t f[5];
+        AdjFaceRef<R> f[5];
 #pragma unroll
-        for (int j = 0; j < 5; ++j) f[j] = at(x, y, z, o + 2 - j);
+        for (int j = 0; j < 5; ++j) f[j] = a.face(at(x, y, z, o + 2 - j));
 #pragma unroll
         for (int c = 0; c < 14; ++c) {
             R s = R(0);
 #pragma unroll
-            for (int j = 0; j < 5; ++j) s += a.face_plane(kAdjDiff + ((c % 7) * 5 + j) * 2 + c / 7)[f[j]];
+            for (int j = 0; j < 5; ++j) s += f[j][kAdjDiff + ((c % 7) * 5 + j) * 2 + c / 7];
             acc[c][row][col] = s;
         }
     };
@@ -772,7 +787,8 @@ __global__ void __launch_bounds__(256) adj_cell_kernel(AdjSweepArgs<R> a) {
     }
     __syncthreads();
     if (!in) return;
-    const size_t p = at(gx, gy, gz, 0), pm = at(gx, gy, gz, -1), pm2 = at(gx, gy, gz, -2), pp = at(gx, gy, gz, 1);
+    const size_t p = at(gx, gy, gz, 0), pm = at(gx, gy, gz, -1);
+    const AdjFaceRef<R> f0 = a.face(p), fm = a.face(pm), fm2 = a.face(at(gx, gy, gz, -2)), fp = a.face(at(gx, gy, gz, 1));
     constexpr int t1 = (AX + 1) % 3, t2 = (AX + 2) % 3;
     R cell[8], lq[NCQ];
 #pragma unroll
@@ -783,26 +799,25 @@ __global__ void __launch_bounds__(256) adj_cell_kernel(AdjSweepArgs<R> a) {
     constexpr int prim[8] = {C_RHO, C_VN, C_VT1, C_VT2, C_BN, C_BT1, C_BT2, C_P};
 #pragma unroll
     for (int t = 0; t < 8; ++t) {
-        const R *L = a.face_plane(kAdjPrim + t);
-        lq[prim[t]] = R(0.5) * (L[p] + L[pm]);
+        lq[prim[t]] = R(0.5) * (f0[kAdjPrim + t] + fm[kAdjPrim + t]);
     }
     auto D = [&](int c) {
         return AX == 0 ? acc[c][ty][tx] - acc[c][ty][tx + 1] : acc[c][ty][tx] - acc[c][ty + 1][tx];
     };
 #pragma unroll
     for (int c = 0; c < 7; ++c) {
-        const R *L = a.face_plane(kAdjCentral + c);
-        lq[C_F0 + c] = D(c) + (R(7) * (L[p] + L[pm]) - (L[pp] + L[pm2])) * R(1.0 / 12.0);
+        const int k = kAdjCentral + c;
+        lq[C_F0 + c] = D(c) + (R(7) * (f0[k] + fm[k]) - (fp[k] + fm2[k])) * R(1.0 / 12.0);
         if (c == 4 || c == 5)
             lq[qU[c]] += D(7 + c);
         else
             lq[qU[c]] = D(7 + c);
     }
     // lower cell of its face, upper cell of the one before
-    lq[C_VN] += a.face_plane(kAdjSide)[p] + a.face_plane(kAdjSide + 4)[pm];
-    lq[C_CF] = a.face_plane(kAdjSide + 1)[p] + a.face_plane(kAdjSide + 5)[pm];
-    lq[C_CA] = a.face_plane(kAdjSide + 2)[p] + a.face_plane(kAdjSide + 6)[pm];
-    lq[C_CSL] = a.face_plane(kAdjSide + 3)[p] + a.face_plane(kAdjSide + 7)[pm];
+    lq[C_VN] += f0[kAdjSide] + fm[kAdjSide + 4];
+    lq[C_CF] = f0[kAdjSide + 1] + fm[kAdjSide + 5];
+    lq[C_CA] = f0[kAdjSide + 2] + fm[kAdjSide + 6];
+    lq[C_CSL] = f0[kAdjSide + 3] + fm[kAdjSide + 7];
     // transport fluxes <B_n v_t>: half the sum of the two faces' adjoints
     {
         auto below = [&](int ax, int o) {
@@ -841,10 +856,17 @@ __device__ __forceinline__ bool adj_cell(const AdjGrid &g, int &i, int &j, int &
     const long long n = (long long)g.nx * g.ny * g.nz;
     const long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     if (q >= n) return false;
-    i = (int)(q % g.nx);
-    const long long r = q / g.nx;
-    j = (int)(r % g.ny);
-    k = (int)(r / g.ny);
+    if (n <= 0x7fffffffLL) {        // (a 64-bit division costs more than most of these kernels' cells)
+        const unsigned r = (unsigned)q / (unsigned)g.nx;
+        i = (int)((unsigned)q - r * (unsigned)g.nx);
+        k = (int)(r / (unsigned)g.ny);
+        j = (int)(r - (unsigned)k * (unsigned)g.ny);
+    } else {
+        const long long r = q / g.nx;
+        i = (int)(q - r * g.nx);
+        k = (int)(r / g.ny);
+        j = (int)(r - (long long)k * g.ny);
+    }
     p = (size_t)q;
     return true;
 }

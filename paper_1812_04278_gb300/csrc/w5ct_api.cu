@@ -886,9 +886,11 @@ int w5ct_init_grid(w5ct_ctx *c, int npatch, const int *n3, const double *dx3) {
     auto take = [&](size_t bytes) { size_t o = bytes_total; bytes_total += align256(bytes); return o; };
     const size_t o_q0 = take(5 * n * 8), o_b0 = take(3 * n * 8), o_acc = take(5 * n * 8), o_oacc = take(3 * n * 8);
     const size_t o_qs = take(5 * n * rs), o_bs = take(3 * n * rs), o_bc = take(3 * n * rs);
-    // Fx .. Sz: 21 planes in one run (the adjoint step uses them as such)
+    // Fx .. Sz: 21 planes in one piece, and room for their last incomplete run
+    // of faces (the adjoint step keeps face adjoints there)
     const size_t o_Fx = take(5 * n * rs), o_Fy = take(5 * n * rs), o_Fz = take(5 * n * rs);
     const size_t o_Sx = take(2 * n * rs), o_Sy = take(2 * n * rs), o_Sz = take(2 * n * rs);
+    take((size_t)kAdjFluxPlanes * kAdjRun * rs);
     const bool fp32 = !ctx_fp64(c);
     const size_t o_q0r = fp32 ? take(5 * n * rs) : 0, o_b0r = fp32 ? take(3 * n * rs) : 0;
     const size_t np = (size_t)npatch;
@@ -1309,7 +1311,8 @@ int autotune_measure(w5ct_ctx *c, int reps) {
 // planes of Real) and the face adjoints that do not fit the context's flux
 // buffers (free between the forward stages and the next step), then double
 // planes: two sets of stage adjoints (5 + 3 each), lamD (5), lamO (3), lamBc (3).
-constexpr int kAdjRealPlanes = 32 + kAdjFacePlanes - kAdjFluxPlanes;
+constexpr int kAdjFacePlanesOwn = kAdjFacePlanes - kAdjFluxPlanes;
+size_t adj_real_values(size_t n) { return 32 * n + kAdjFacePlanesOwn * adj_run_cells(n); }
 constexpr int kAdjDoublePlanes = 2 * 8 + 5 + 3 + 3;
 
 template <typename Real>
@@ -1317,7 +1320,7 @@ int ensure_adj(w5ct_ctx *c) {
     if (c->adj_slab) return W5CT_OK;
     W5_CUDA(c, c->cfg.weno_variant == W5CT_WENO_JS ? (prepare_adj_sweep<Real, 0>()) : (prepare_adj_sweep<Real, 1>()));
     const size_t n = (size_t)c->n;
-    const size_t bytes = align256(kAdjRealPlanes * n * sizeof(Real)) + (size_t)kAdjDoublePlanes * n * 8;
+    const size_t bytes = align256(adj_real_values(n) * sizeof(Real)) + (size_t)kAdjDoublePlanes * n * 8;
     W5_CUDA(c, cudaMalloc(&c->adj_slab, bytes));
     return W5CT_OK;
 }
@@ -1331,15 +1334,14 @@ int adjoint_step_impl(w5ct_ctx *c, double dt, const double *lq_fin, const double
     const size_t n = (size_t)nl;
     cudaStream_t st = c->stream;
     Real *stage = reinterpret_cast<Real *>(c->adj_slab);
-    double *w = reinterpret_cast<double *>((char *)c->adj_slab + align256(kAdjRealPlanes * n * sizeof(Real)));
+    double *w = reinterpret_cast<double *>((char *)c->adj_slab + align256(adj_real_values(n) * sizeof(Real)));
     double *set[2] = {w, w + 8 * n};           // stage adjoints: q (5 planes) then b (3 planes)
     double *lamD = w + 16 * n, *lamO = lamD + 5 * n, *lamBc = lamO + 3 * n;
 
-    unsigned long long hits0 = 0;
-    int flag0 = 0;
-    W5_CUDA(c, cudaMemcpyAsync(&hits0, c->hits, sizeof(hits0), cudaMemcpyDeviceToHost, st));
-    W5_CUDA(c, cudaMemcpyAsync(&flag0, c->flag, sizeof(flag0), cudaMemcpyDeviceToHost, st));
-    W5_CUDA(c, cudaStreamSynchronize(st));
+    // the floor counter and the flag are kept: aside in the reduction scratch
+    // (the recomputed stages touch them)
+    W5_CUDA(c, cudaMemcpyAsync(c->part, c->hits, sizeof(unsigned long long), cudaMemcpyDeviceToDevice, st));
+    W5_CUDA(c, cudaMemcpyAsync(c->part + 1, c->flag, sizeof(int), cudaMemcpyDeviceToDevice, st));
 
     // forward stages 0..2 from the current state, keeping the four stage states
     fill_kernel<<<1, 32, 0, st>>>(c->dt_dev, 1, dt);
@@ -1395,8 +1397,8 @@ int adjoint_step_impl(w5ct_ctx *c, double dt, const double *lq_fin, const double
         W5_CUDA(c, cudaGetLastError());
         next = cur;
     }
-    W5_CUDA(c, cudaMemcpyAsync(c->hits, &hits0, sizeof(hits0), cudaMemcpyHostToDevice, st));
-    W5_CUDA(c, cudaMemcpyAsync(c->flag, &flag0, sizeof(flag0), cudaMemcpyHostToDevice, st));
+    W5_CUDA(c, cudaMemcpyAsync(c->hits, c->part, sizeof(unsigned long long), cudaMemcpyDeviceToDevice, st));
+    W5_CUDA(c, cudaMemcpyAsync(c->flag, c->part + 1, sizeof(int), cudaMemcpyDeviceToDevice, st));
     W5_CUDA(c, cudaStreamSynchronize(st));
     return W5CT_OK;
 }

@@ -121,7 +121,7 @@ __device__ __forceinline__ void sweep_tile_at(const SweepArgs<Real> &a, const Pa
                                               Real *sm, int tx, int ty) {
     using TT = SweepTile<AX, T2, BX, FPT>;
     constexpr int NC = TT::template cells<Real>;      // elements between quantities
-    constexpr bool kFlat = std::is_same<Real, double>::value;
+    constexpr bool kFlat = std::is_same<Real, double>::value, kPaired = !kFlat;
     constexpr int pitch = TT::template pitch<Real>, st = TT::ST;
     const int nx = pg.nx, ny = pg.ny, nz = pg.nz;
     const size_t off = (size_t)pg.off;
@@ -166,7 +166,7 @@ __device__ __forceinline__ void sweep_tile_at(const SweepArgs<Real> &a, const Pa
         for (int j = 0; j < B; ++j) {
             const int c = tid + (it0 + j) * TT::NT;
             if (it0 + j < NIT && c < ncell)
-                cell_fill<Real, AX>(sm + at[j], NC, v[j][0], v[j][1], v[j][2], v[j][3], v[j][4], v[j][5], v[j][6],
+                cell_fill<Real, AX, kPaired>(sm, at[j], NC, v[j][0], v[j][1], v[j][2], v[j][3], v[j][4], v[j][5], v[j][6],
                                     v[j][7], a.K, bad, hit);
         }
     }
@@ -218,7 +218,7 @@ __device__ __forceinline__ void sweep_tile_at(const SweepArgs<Real> &a, const Pa
         if (kFlat || (gx < nx && gy < ny && gz < nz)) {
             Real Ff[7], s1, s2;
             // stencil cell i-2 of the face at bx + pitch t2
-            face_flux<Real, VAR, box_diff<Real>(), DWW>(sm + bx + pitch * t2, NC, st, a.K, Ff, s1, s2);
+            face_flux<Real, VAR, box_diff<Real>(), DWW, kPaired>(sm, bx + pitch * t2, NC, st, a.K, Ff, s1, s2);
             const size_t g = off + (size_t)gx + (size_t)nx * ((size_t)gy + (size_t)ny * (size_t)gz);
             a.F[0][g] = Ff[0];
             a.F[1 + AX][g] = Ff[1];
@@ -294,7 +294,7 @@ __device__ __forceinline__ void sweep_tile_rt(const SweepArgs<Real> &a, const Pa
             // stencil cell i-2 of the face: s = the face's position along the axis
             const int c0 = ax == 0 ? tx + CS * t2 : t2 + CS * tx;
             Real Ff[7], s1, s2;
-            face_flux<Real, VAR>(sm + c0, NQS, 1, a.K, Ff, s1, s2);
+            face_flux<Real, VAR>(sm, c0, NQS, 1, a.K, Ff, s1, s2);
             const size_t g = off + (size_t)gx + (size_t)nx * ((size_t)gy + (size_t)ny * (size_t)gz);
             // lab components of the frame momentum flux (n, t1, t2)
             Real *const fn = ax == 0 ? a.F[1] : (ax == 1 ? a.F[2] : a.F[3]);
