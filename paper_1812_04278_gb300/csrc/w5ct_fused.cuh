@@ -211,11 +211,11 @@ __device__ __forceinline__ void fused_cellb(const PatchGeom &g, int i, int j, in
                                             const Real *bz, Real *Bx, Real *By, Real *Bz) {
     const long long sy = g.nx, sz = (long long)g.nx * g.ny;
     const long long p = g.off + i + sy * j + sz * k;
-    const long long xm2 = wrapi(i - 2, g.nx) - i, xm1 = wrapi(i - 1, g.nx) - i, xp1 = wrapi(i + 1, g.nx) - i;
-    const long long ym2 = (wrapi(j - 2, g.ny) - j) * sy, ym1 = (wrapi(j - 1, g.ny) - j) * sy,
-                    yp1 = (wrapi(j + 1, g.ny) - j) * sy;
-    const long long zm2 = (wrapi(k - 2, g.nz) - k) * sz, zm1 = (wrapi(k - 1, g.nz) - k) * sz,
-                    zp1 = (wrapi(k + 1, g.nz) - k) * sz;
+    const long long xm2 = wrap_near(i - 2, g.nx) - i, xm1 = wrap_near(i - 1, g.nx) - i, xp1 = wrap_near(i + 1, g.nx) - i;
+    const long long ym2 = (wrap_near(j - 2, g.ny) - j) * sy, ym1 = (wrap_near(j - 1, g.ny) - j) * sy,
+                    yp1 = (wrap_near(j + 1, g.ny) - j) * sy;
+    const long long zm2 = (wrap_near(k - 2, g.nz) - k) * sz, zm1 = (wrap_near(k - 1, g.nz) - k) * sz,
+                    zp1 = (wrap_near(k + 1, g.nz) - k) * sz;
     Bx[p] = face_to_cell<Real>(bx[p + xm2], bx[p + xm1], bx[p], bx[p + xp1]);
     By[p] = face_to_cell<Real>(by[p + ym2], by[p + ym1], by[p], by[p + yp1]);
     Bz[p] = face_to_cell<Real>(bz[p + zm2], bz[p + zm1], bz[p], bz[p + zp1]);

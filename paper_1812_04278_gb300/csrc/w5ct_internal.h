@@ -116,9 +116,9 @@ struct SinglePatchSweep {
 // variant keeps 128 registers per thread in float: min blocks per SM = 512 /
 // threads per block.  One launch per axis and variant computes a float 32 x 16
 // tile as two halves, in blocks of 128 threads like the single-patch tiles.
-// Step of the 512-patch workload with one variant forced on every patch: 24.7,
-// 25.2, 24.0, 23.4 ms (model choice 23.6); 27.6 for whole 32 x 16 tiles in 256-thread blocks and 26.3 for 16 x 16
-// with one face per thread.
+// Step of the 512-patch workload with one variant forced on every patch: 24.1,
+// 23.4, 24.0, 23.4 ms, and 22.8 ms with the choice per patch and axis; before
+// the halves, whole 32 x 16 tiles in 256-thread blocks took 27.6 ms.
 constexpr int kMaxTileVariants = 4;
 
 #ifndef W5CT_ALL_WAVES32

@@ -72,8 +72,8 @@ constexpr int kStageBatch = 3;
 // unchanged.  In float the same numbering was 3-4% slower (its divisions, and
 // rows of a warp meeting in a shared-memory bank, which in double the FP64 pipe
 // hides), also where it fills lanes, so a float tile takes whole BX-wide rows,
-// its narrower tiles' x-boxes with a pitch that puts a warp's rows in different
-// banks.
+// the 8-wide x-box with a pitch that puts the two rows of an 8-byte load's
+// sixteen lanes in different banks.
 template <int AX, int T2, int BX_ = 32, int FPT_ = T2 / 8>
 struct SweepTile {
     static_assert(T2 % FPT_ == 0, "faces per thread must divide the tile height");
@@ -89,7 +89,7 @@ struct SweepTile {
     static constexpr int CZ = BZ + (AX == 2 ? 5 : 0);
     // elements between rows of the box and between quantities, and the stencil
     // stride
-    static constexpr int PITCH_F = AX != 0 || BX >= 32 ? CX : BX == 8 ? 24 : 48;
+    static constexpr int PITCH_F = AX == 0 && BX == 8 ? 24 : CX;
     template <typename Real>
     static constexpr int pitch = std::is_same<Real, float>::value ? PITCH_F : CX;
     static constexpr int NC = CX * CY * CZ;          // cells of the full box
@@ -115,13 +115,16 @@ struct PatchGeom {
 // One sweep tile (tile indices tbx, tby, tbz) of the patch described by g,
 // computed by the block's NT threads, numbered tx + BX ty.  sm: shared memory
 // of box_quantities<Real>() * cells<Real> elements.  SB: cells whose loads a
-// thread issues together when it stages the cell box.
-template <int AX, typename Real, int VAR, int T2, int BX, int FPT, int SB = kStageBatch, bool DWW = false>
+// thread issues together when it stages the cell box.  PAIR: the float box
+// with flux and state side by side (box_at); the one-face tiles of the batched
+// sweeps fit 128 registers without spills only unpaired, while the tiles of the
+// three-in-one launch gain by it (32^3: two steps, 182 -> 176 us).
+template <int AX, typename Real, int VAR, int T2, int BX, int FPT, int SB = kStageBatch, bool DWW = false, bool PAIR = (FPT > 1)>
 __device__ __forceinline__ void sweep_tile_at(const SweepArgs<Real> &a, const PatchGeom &pg, int tbx, int tby, int tbz,
                                               Real *sm, int tx, int ty) {
     using TT = SweepTile<AX, T2, BX, FPT>;
     constexpr int NC = TT::template cells<Real>;      // elements between quantities
-    constexpr bool kFlat = std::is_same<Real, double>::value, kPaired = !kFlat;
+    constexpr bool kFlat = std::is_same<Real, double>::value, kPaired = !kFlat && PAIR;
     constexpr int pitch = TT::template pitch<Real>, st = TT::ST;
     const int nx = pg.nx, ny = pg.ny, nz = pg.nz;
     const size_t off = (size_t)pg.off;
@@ -370,11 +373,11 @@ __global__ void __launch_bounds__(kAllThreads, sizeof(Real) == 4 ? 4 : DW ? 3 : 
     pg.nz = s.a[0].nz;
     pg.off = 0;
     if (ax == 0)
-        sweep_tile_at<0, Real, VAR, AllTile<0>::T2, AllTile<0>::BX, 1, kStageBatch, DW>(s.a[0], pg, tbx, t1, t2, sm, tid % AllTile<0>::BX, tid / AllTile<0>::BX);
+        sweep_tile_at<0, Real, VAR, AllTile<0>::T2, AllTile<0>::BX, 1, kStageBatch, DW, true>(s.a[0], pg, tbx, t1, t2, sm, tid % AllTile<0>::BX, tid / AllTile<0>::BX);
     else if (ax == 1)
-        sweep_tile_at<1, Real, VAR, AllTile<1>::T2, AllTile<1>::BX, 1, kStageBatch, DW>(s.a[1], pg, tbx, t1, t2, sm, tid % AllTile<1>::BX, tid / AllTile<1>::BX);
+        sweep_tile_at<1, Real, VAR, AllTile<1>::T2, AllTile<1>::BX, 1, kStageBatch, DW, true>(s.a[1], pg, tbx, t1, t2, sm, tid % AllTile<1>::BX, tid / AllTile<1>::BX);
     else
-        sweep_tile_at<2, Real, VAR, AllTile<2>::T2, AllTile<2>::BX, 1, kStageBatch, DW>(s.a[2], pg, tbx, t2, t1, sm, tid % AllTile<2>::BX, tid / AllTile<2>::BX);
+        sweep_tile_at<2, Real, VAR, AllTile<2>::T2, AllTile<2>::BX, 1, kStageBatch, DW, true>(s.a[2], pg, tbx, t2, t1, sm, tid % AllTile<2>::BX, tid / AllTile<2>::BX);
 }
 
 // Tile tables hold int4 (patch | axis << 28, tile x, tile y, tile z).
@@ -403,6 +406,13 @@ __global__ void __launch_bounds__(SweepTile<AX, T2, BX, FPT>::NT, MINB)
 // cell-centred field: fourth-order interpolation of the faces (Sec. 2.3)
 // ======================================================================
 
+// wrapi for -2 <= g <= n (n >= 1): selects instead of a division
+__device__ __forceinline__ int wrap_near(int g, int n) {
+    if (g < 0) g += n;
+    if (g < 0) g += n;
+    return g < n ? g : g - n;
+}
+
 // (9 (f_{-1/2} + f_{1/2}) - (f_{-3/2} + f_{3/2})) / 16: in double 3 FP64
 // instructions, the scaling of the outer sum being exact on the integer pipes
 template <typename Real>
@@ -420,9 +430,9 @@ __device__ __forceinline__ void cellb_cell(int nx, int ny, int nz, size_t off, i
     // index, small integer offsets)
     const long long sy = nx, sz = (long long)nx * ny;
     const long long p = (long long)off + i + sy * j + sz * k;
-    const long long xm2 = wrapi(i - 2, nx) - i, xm1 = wrapi(i - 1, nx) - i, xp1 = wrapi(i + 1, nx) - i;
-    const long long ym2 = (wrapi(j - 2, ny) - j) * sy, ym1 = (wrapi(j - 1, ny) - j) * sy, yp1 = (wrapi(j + 1, ny) - j) * sy;
-    const long long zm2 = (wrapi(k - 2, nz) - k) * sz, zm1 = (wrapi(k - 1, nz) - k) * sz, zp1 = (wrapi(k + 1, nz) - k) * sz;
+    const long long xm2 = wrap_near(i - 2, nx) - i, xm1 = wrap_near(i - 1, nx) - i, xp1 = wrap_near(i + 1, nx) - i;
+    const long long ym2 = (wrap_near(j - 2, ny) - j) * sy, ym1 = (wrap_near(j - 1, ny) - j) * sy, yp1 = (wrap_near(j + 1, ny) - j) * sy;
+    const long long zm2 = (wrap_near(k - 2, nz) - k) * sz, zm1 = (wrap_near(k - 1, nz) - k) * sz, zp1 = (wrap_near(k + 1, nz) - k) * sz;
     Bx[p] = face_to_cell<Real>(bx[p + xm2], bx[p + xm1], bx[p], bx[p + xp1]);
     By[p] = face_to_cell<Real>(by[p + ym2], by[p + ym1], by[p], by[p + yp1]);
     Bz[p] = face_to_cell<Real>(bz[p + zm2], bz[p + zm1], bz[p], bz[p + zp1]);
@@ -455,10 +465,10 @@ __global__ void __launch_bounds__(256) cellb_kernel(int nx, int ny, int nz, int 
     const int k0 = blockIdx.z * chunk, k1 = min(k0 + chunk, nz);
     if (i >= nx || j >= ny) return;
     const long long sy = nx, sz = (long long)nx * ny;
-    const long long xm2 = wrapi(i - 2, nx) - i, xm1 = wrapi(i - 1, nx) - i, xp1 = wrapi(i + 1, nx) - i;
-    const long long ym2 = (wrapi(j - 2, ny) - j) * sy, ym1 = (wrapi(j - 1, ny) - j) * sy, yp1 = (wrapi(j + 1, ny) - j) * sy;
+    const long long xm2 = wrap_near(i - 2, nx) - i, xm1 = wrap_near(i - 1, nx) - i, xp1 = wrap_near(i + 1, nx) - i;
+    const long long ym2 = (wrap_near(j - 2, ny) - j) * sy, ym1 = (wrap_near(j - 1, ny) - j) * sy, yp1 = (wrap_near(j + 1, ny) - j) * sy;
     const long long col = i + sy * j;
-    Real z0 = bz[col + sz * wrapi(k0 - 2, nz)], z1 = bz[col + sz * wrapi(k0 - 1, nz)], z2 = bz[col + sz * k0];
+    Real z0 = bz[col + sz * wrap_near(k0 - 2, nz)], z1 = bz[col + sz * wrap_near(k0 - 1, nz)], z2 = bz[col + sz * k0];
 #pragma unroll 4
     for (int k = k0; k < k1; ++k) {
         const long long p = col + sz * k;
