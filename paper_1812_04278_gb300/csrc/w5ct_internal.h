@@ -114,8 +114,10 @@ struct SinglePatchSweep {
 // that waste fewer lanes on patches whose sizes are not multiples of 32 or of
 // 16: (BX, T2, faces per thread) = (16, 16, 2), (8, 16, 1), (8, 8, 1).  Every
 // variant keeps 128 registers per thread in float: min blocks per SM = 512 /
-// threads per block.  One launch per axis and variant computes a float 32 x 16
-// tile as two halves, in blocks of 128 threads like the single-patch tiles.
+// threads per block.  One launch per axis and variant computes a float
+// or double 32 x 16 tile as two halves, in blocks of 128 threads like the
+// single-patch tiles (double: three of 168 registers per SM instead of one of 256
+// threads, 48 patches 50.6 -> 48.3 ms per step).
 // Step of the 512-patch workload with one variant forced on every patch: 24.1,
 // 23.4, 24.0, 23.4 ms, and 22.8 ms with the choice per patch and axis; before
 // the halves, whole 32 x 16 tiles in 256-thread blocks took 27.6 ms.
@@ -164,9 +166,9 @@ inline void tile_shape(int axis, int v, int &bx, int &t2) {
 template <int AX, typename Real, int VAR, int V>
 struct BatchedSweep {
     using C = TileV<AX, Real, V>;
-    static constexpr bool kHalves = std::is_same<Real, float>::value && V == 0;
+    static constexpr bool kHalves = V == 0;
     static constexpr int BX = kHalves && AX != 0 ? C::BX / 2 : C::BX, T2 = kHalves && AX == 0 ? C::T2 / 2 : C::T2,
-                         MINB = kHalves ? 2 * C::MINB : C::MINB;
+                         MINB = !kHalves ? C::MINB : std::is_same<Real, float>::value ? 2 * C::MINB : 3;
     using TT = SweepTile<AX, T2, BX, C::FPT>;
     static constexpr size_t smem = (size_t)TT::template cells<Real> * box_quantities<Real>() * sizeof(Real);
     static cudaError_t prepare() {

@@ -119,7 +119,8 @@ struct PatchGeom {
 // with flux and state side by side (box_at); the one-face tiles of the batched
 // sweeps fit 128 registers without spills only unpaired, while the tiles of the
 // three-in-one launch gain by it (32^3: two steps, 182 -> 176 us).
-template <int AX, typename Real, int VAR, int T2, int BX, int FPT, int SB = kStageBatch, bool DWW = false, bool PAIR = (FPT > 1)>
+template <int AX, typename Real, int VAR, int T2, int BX, int FPT, int SB = kStageBatch, bool DWW = false, bool PAIR = (FPT > 1),
+          typename MM = M<Real>>
 __device__ __forceinline__ void sweep_tile_at(const SweepArgs<Real> &a, const PatchGeom &pg, int tbx, int tby, int tbz,
                                               Real *sm, int tx, int ty) {
     using TT = SweepTile<AX, T2, BX, FPT>;
@@ -169,7 +170,7 @@ __device__ __forceinline__ void sweep_tile_at(const SweepArgs<Real> &a, const Pa
         for (int j = 0; j < B; ++j) {
             const int c = tid + (it0 + j) * TT::NT;
             if (it0 + j < NIT && c < ncell)
-                cell_fill<Real, AX, kPaired>(sm, at[j], NC, v[j][0], v[j][1], v[j][2], v[j][3], v[j][4], v[j][5], v[j][6],
+                cell_fill<Real, AX, kPaired, MM>(sm, at[j], NC, v[j][0], v[j][1], v[j][2], v[j][3], v[j][4], v[j][5], v[j][6],
                                     v[j][7], a.K, bad, hit);
         }
     }
@@ -221,7 +222,7 @@ __device__ __forceinline__ void sweep_tile_at(const SweepArgs<Real> &a, const Pa
         if (kFlat || (gx < nx && gy < ny && gz < nz)) {
             Real Ff[7], s1, s2;
             // stencil cell i-2 of the face at bx + pitch t2
-            face_flux<Real, VAR, box_diff<Real>(), DWW, kPaired>(sm, bx + pitch * t2, NC, st, a.K, Ff, s1, s2);
+            face_flux<Real, VAR, box_diff<Real>(), DWW, kPaired, MM>(sm, bx + pitch * t2, NC, st, a.K, Ff, s1, s2);
             const size_t g = off + (size_t)gx + (size_t)nx * ((size_t)gy + (size_t)ny * (size_t)gz);
             a.F[0][g] = Ff[0];
             a.F[1 + AX][g] = Ff[1];
@@ -354,12 +355,12 @@ struct AllTile {
     static constexpr int BX = AX == 0 ? 32 : 8, T2 = AX == 0 ? 4 : 16;
 };
 
-// Blocks per SM: float 4 (128 registers); double 2 (255 registers; three blocks
-// of 168 spill: 256^3 step 416.4 against 413.4 ms); double-word 3, whose chains
-// of dependent FP32 operations want the warps (128^3 step 37.0 -> 33.9 ms; four
-// blocks no faster).
+// Blocks per SM: float 4 (128 registers); double 3 of 168 registers: the chains
+// of integer products and of double-word operations want the warps (256^3 step
+// 388 -> 379 ms, with double-word weights at 128^3 37.0 -> 33.9 ms; four blocks
+// of 128 registers 359 against 353 ms, double-word no faster).
 template <typename Real, int VAR, bool DW>
-__global__ void __launch_bounds__(kAllThreads, sizeof(Real) == 4 ? 4 : DW ? 3 : 2) sweep_all_kernel(SweepAll<Real> s) {
+__global__ void __launch_bounds__(kAllThreads, sizeof(Real) == 4 ? 4 : 3) sweep_all_kernel(SweepAll<Real> s) {
     extern __shared__ __align__(16) unsigned char w5ct_smem[];
     chain_begin();
     Real *sm = reinterpret_cast<Real *>(w5ct_smem);
@@ -372,12 +373,18 @@ __global__ void __launch_bounds__(kAllThreads, sizeof(Real) == 4 ? 4 : DW ? 3 : 
     pg.ny = s.a[0].ny;
     pg.nz = s.a[0].nz;
     pg.off = 0;
+    using MM = std::conditional_t<std::is_same<Real, double>::value && !DW, MCalled, M<Real>>;
+    using X = AllTile<0>;
+    using Y = AllTile<1>;      // y and z alike
     if (ax == 0)
-        sweep_tile_at<0, Real, VAR, AllTile<0>::T2, AllTile<0>::BX, 1, kStageBatch, DW, true>(s.a[0], pg, tbx, t1, t2, sm, tid % AllTile<0>::BX, tid / AllTile<0>::BX);
+        sweep_tile_at<0, Real, VAR, X::T2, X::BX, 1, kStageBatch, DW, true, MM>(s.a[0], pg, tbx, t1, t2, sm, tid % X::BX,
+                                                                               tid / X::BX);
     else if (ax == 1)
-        sweep_tile_at<1, Real, VAR, AllTile<1>::T2, AllTile<1>::BX, 1, kStageBatch, DW, true>(s.a[1], pg, tbx, t1, t2, sm, tid % AllTile<1>::BX, tid / AllTile<1>::BX);
+        sweep_tile_at<1, Real, VAR, Y::T2, Y::BX, 1, kStageBatch, DW, true, MM>(s.a[1], pg, tbx, t1, t2, sm, tid % Y::BX,
+                                                                               tid / Y::BX);
     else
-        sweep_tile_at<2, Real, VAR, AllTile<2>::T2, AllTile<2>::BX, 1, kStageBatch, DW, true>(s.a[2], pg, tbx, t2, t1, sm, tid % AllTile<2>::BX, tid / AllTile<2>::BX);
+        sweep_tile_at<2, Real, VAR, Y::T2, Y::BX, 1, kStageBatch, DW, true, MM>(s.a[2], pg, tbx, t2, t1, sm, tid % Y::BX,
+                                                                               tid / Y::BX);
 }
 
 // Tile tables hold int4 (patch | axis << 28, tile x, tile y, tile z).

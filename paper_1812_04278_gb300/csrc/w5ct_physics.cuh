@@ -93,6 +93,93 @@ constexpr bool float_based = std::is_same<R, float>::value;
 
 // ---------------------------------------------------------------- math helpers
 template <typename Real> struct M;
+// ---------------------------------------------------------------- products
+// Products of doubles on the integer pipes, with the bits of an IEEE product
+// rounded to nearest even.  The FP64 sweeps are bound by the FP64 pipe (2 lanes
+// per SM and clock: 16 clocks for a warp's instruction) while the issue slots
+// are a tenth used, and the 30 integer instructions of a product issue in 8
+// clocks of an SM beside it: every product moved here is time off the bound.
+// (A fused multiply-add or a sum would take twice as many and stays where it
+// is.)  256^3 WENO-Z step, with the looped face function (face_flux): 413 ms
+// with all products in the FP64 multiplier, 388 with the products of the
+// weights moved, 371 with those of the quotients, 353 with those of the
+// projections, 331 with those of the eigenvectors, cells and roots.
+//
+// DFactor holds the magnitude of a factor: its 53-bit significand and its
+// exponent field less one, in place.  dmul_int multiplies two of them whose
+// product is normal: the first significand is shifted left by 11, so that the
+// upper half of the 128-bit product is the result's significand or half of it.
+struct DFactor {
+    unsigned lo, hi, e;
+    __device__ __forceinline__ explicit DFactor(double x) {
+        const unsigned h = (unsigned)__double2hiint(x) & 0x7fffffffu;
+        lo = (unsigned)__double2loint(x);
+        hi = (h & 0xfffffu) | 0x100000u;
+        e = h - hi;
+    }
+};
+
+__device__ __forceinline__ double dmul_int(const DFactor &a, const DFactor &b) {
+    using u64 = unsigned long long;
+    const unsigned ah = __funnelshift_l(a.lo, a.hi, 11), al = a.lo << 11;
+    const u64 p0 = (u64)al * b.lo;
+    const u64 p1 = (u64)ah * b.lo + (p0 >> 32);
+    const u64 p2 = (u64)al * b.hi + (unsigned)p1;
+    const u64 p3 = (u64)ah * b.hi + (p1 >> 32) + (p2 >> 32);
+    const unsigned h = (unsigned)(p3 >> 32), l = (unsigned)p3, f = (unsigned)p2, z = (unsigned)p0;
+    const unsigned s = (h >> 20) ^ 1u;   // 1: the upper half lacks its top bit
+    unsigned m1 = __funnelshift_l(l, h, s), m0 = __funnelshift_l(f, l, s);
+    const unsigned r = f << s;
+    // nearest even: add one half less a bit, plus the last place, to the
+    // remainder r : z, and its carry to the significand
+    const unsigned odd = m0 & 1u;
+    const unsigned e = a.e + b.e + ((h & 0x100000u) - (1022u << 20));
+    asm("{\n\t.reg .u32 t;\n\t"
+        "add.cc.u32 t, %2, %3;\n\t"
+        "addc.cc.u32 t, %4, %5;\n\t"
+        "addc.cc.u32 %0, %0, 0;\n\t"
+        "addc.u32 %1, %1, %6;\n\t}"
+        : "+r"(m0), "+r"(m1)
+        : "r"(z), "r"(odd - 1u), "r"(r), "r"(odd + 0x7fffffffu), "r"(e));
+    return __hiloint2double((int)m1, (int)m0);
+}
+
+// a product in the FP64 multiplier, out of line: inlined beside the integer form
+// it would issue there predicated off
+static __device__ __noinline__ double dmul_fp64(double a, double b) { return a * b; }
+
+__device__ __forceinline__ unsigned dmag_hi(double a) { return (unsigned)__double2hiint(a) & 0x7fffffffu; }
+
+// a b where the caller knows that both and the product are normal
+__device__ __forceinline__ double dmul_normal(double a, double b) {
+    const double p = dmul_int(DFactor(a), DFactor(b));
+    return __hiloint2double(__double2hiint(p) | ((__double2hiint(a) ^ __double2hiint(b)) & (int)0x80000000),
+                            __double2loint(p));
+}
+
+// 2^-510 <= |a| < 2^510: products of two such are normal (zero, subnormals,
+// infinities and NaN are outside)
+__device__ __forceinline__ bool dmid(double a) { return dmag_hi(a) - (513u << 20) < (1020u << 20); }
+
+// the exponent field of |a| less 767: below 2^9 << 20 for 2^-256 <= |a| < 2^256;
+// the form for several factors, whose results are joined by |
+__device__ __forceinline__ unsigned dwindow(double a) { return dmag_hi(a) - (767u << 20); }
+constexpr unsigned kInWindow = 512u << 20;
+
+// a b for any a and b: in the FP64 multiplier unless both are normal and the
+// exponents' sum leaves the product normal with a place to spare
+__device__ __forceinline__ double dmul_any(double a, double b) {
+    const unsigned u = dmag_hi(a), v = dmag_hi(b);
+    const bool fits = u - (1u << 20) < (2046u << 20) && v - (1u << 20) < (2046u << 20) &&
+                      u + v - (1026u << 20) < (2040u << 20);
+    return fits ? dmul_normal(a, b) : dmul_fp64(a, b);
+}
+
+// the same out of line, for the many products that appear once (inlined, the 70
+// of a face and a cell overrun the instruction cache: 100 x 70 x 50 WENO-JS
+// step 8.8 against 8.2 ms)
+static __device__ __noinline__ double dmul_call(double a, double b) { return dmul_any(a, b); }
+
 // Reciprocal of a positive finite double by Newton-Raphson iteration on
 // f(r) = 1/r - y (r' = r + r (1 - y r), quadratic convergence), started from
 // the hardware's approximate reciprocal (PTX rcp.approx.ftz.f64); two
@@ -118,8 +205,8 @@ __device__ __forceinline__ double drcp_newton(double y) {
 __device__ __forceinline__ double drsqrt_newton(double x) {
     double y;
     asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-    const double e = fma(-(x * y), y, 1.0);
-    return fma(fma(0.375, e, 0.5), y * e, y);
+    const double e = fma(-dmul_any(x, y), y, 1.0);
+    return fma(fma(0.375, e, 0.5), dmul_any(y, e), y);
 }
 
 // a / b, b > 0 finite and normal: the approximate quotient q0 = a r0 (r0
@@ -129,7 +216,7 @@ __device__ __forceinline__ double ddiv_newton(double a, double b) {
     double r;
     asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(b));
     const double e = fma(-b, r, 1.0);
-    const double q = a * r;
+    const double q = dmul_any(a, r);
     return fma(fma(e, e, e), q, q);
 }
 
@@ -162,6 +249,7 @@ __device__ __forceinline__ double dmax_nonneg(double a, double b) {
 
 template <> struct M<double> {
     static __device__ __forceinline__ double sqrt_(double x) { return sqrt(x); }
+    static __device__ __forceinline__ double mul_(double a, double b) { return a * b; }
     static __device__ __forceinline__ double div_(double a, double b) { return ddiv_newton(a, b); }
     static __device__ __forceinline__ double rcp_(double x) { return drcp_newton(x); }
     static __device__ __forceinline__ double rcp3_(double x) { return drcp_third(x); }
@@ -186,6 +274,7 @@ template <> struct M<double> {
 };
 template <> struct M<float> {
     static __device__ __forceinline__ float sqrt_(float x) { return sqrtf(x); }
+    static __device__ __forceinline__ float mul_(float a, float b) { return a * b; }
     static __device__ __forceinline__ float div_(float a, float b) { return __fdividef(a, b); }
     static __device__ __forceinline__ float rcp_(float x) { return __fdividef(1.0f, x); }
     static __device__ __forceinline__ float rcp3_(float x) { return __fdividef(1.0f, x); }
@@ -203,6 +292,15 @@ template <> struct M<float> {
     static __device__ __forceinline__ bool nonneg(float x) { return x >= 0.0f; }
     static __device__ __forceinline__ bool normal_pos(float x) { return !(x < 1.17549435e-38f); }
     static __device__ __forceinline__ bool finite_pos(float x) { return x > 0.0f && x < 3.0e38f; }
+};
+
+// The sweeps' choice for the products that appear once (MM of cell_fill and
+// face_flux): MCalled takes them through dmul_call.  Same bits; faster in the
+// three-in-one launch (256^3 WENO-Z step 342.6 -> 330.6 ms), slower where
+// another pipe or the tile's tail is the bound (128^3 step with double-word
+// weights 32.7 -> 34.2 ms; 48 patches 47.5 -> 48.6; adjoint 58.3 -> 58.8).
+struct MCalled : M<double> {
+    static __device__ __forceinline__ double mul_(double a, double b) { return dmul_call(a, b); }
 };
 
 // ---------------------------------------------------------------- wave speeds
@@ -235,22 +333,22 @@ __device__ __forceinline__ void speeds_fast(Real cs2, Real ca2, Real bt2, Real &
 // Fills the NCQ per-cell quantities of a cell from its state in the sweep
 // frame (n, t1, t2): momentum (mn, m1, m2), cell field (Bn, B1, B2), into the
 // box (box_at).
-template <typename Real, bool PAIRED = false>
+template <typename Real, bool PAIRED = false, typename MM = M<Real>>
 __device__ __forceinline__ void cell_fill_frame(Real *box, int cell, int stride, Real rho, Real mn, Real m1, Real m2, Real E,
                                                 Real Bn, Real B1, Real B2, const Phys<Real> &K, bool &bad, bool &hit) {
-    using m = M<Real>;
+    using m = MM;
     Real r = rho;
     if (K.floors && r < K.rho_min) { r = K.rho_min; hit = true; }
-    const Real isr = m::rsqrt_(r), ir = isr * isr;
-    const Real vn = mn * ir, v1 = m1 * ir, v2 = m2 * ir;
-    const Real vv = m::fma_(v2, v2, m::fma_(v1, v1, vn * vn));
-    const Real Bn2 = Bn * Bn, Bt2 = m::fma_(B2, B2, B1 * B1);
+    const Real isr = m::rsqrt_(r), ir = m::mul_(isr, isr);
+    const Real vn = m::mul_(mn, ir), v1 = m::mul_(m1, ir), v2 = m::mul_(m2, ir);
+    const Real vv = m::fma_(v2, v2, m::fma_(v1, v1, m::mul_(vn, vn)));
+    const Real Bn2 = m::mul_(Bn, Bn), Bt2 = m::fma_(B2, B2, m::mul_(B1, B1));
     const Real BB = Bn2 + Bt2;
     Real P = K.gm1 * m::fma_(Real(-0.5), m::fma_(r, vv, BB), E);
     if (K.floors && P < K.p_min) { P = K.p_min; hit = true; }
     if (!(r > Real(0)) || !m::finite_pos(P)) bad = true;
     const Real Pt = m::fma_(Real(0.5), BB, P);
-    const Real vB = m::fma_(v2, B2, m::fma_(v1, B1, vn * Bn));
+    const Real vB = m::fma_(v2, B2, m::fma_(v1, B1, m::mul_(vn, Bn)));
     box[box_at<PAIRED>(C_RHO, stride, cell)] = r;
     box[box_at<PAIRED>(C_VN, stride, cell)] = vn;
     box[box_at<PAIRED>(C_VT1, stride, cell)] = v1;
@@ -267,31 +365,31 @@ __device__ __forceinline__ void cell_fill_frame(Real *box, int cell, int stride,
     // rho v_n = m_n (v = m / rho with the same, possibly floored, rho)
     box[box_at<PAIRED>(C_F0, stride, cell)] = mn;
     box[box_at<PAIRED>(C_F1, stride, cell)] = m::fma_(mn, vn, Pt - Bn2);
-    box[box_at<PAIRED>(C_F2, stride, cell)] = m::fma_(mn, v1, -(Bn * B1));
-    box[box_at<PAIRED>(C_F3, stride, cell)] = m::fma_(mn, v2, -(Bn * B2));
-    box[box_at<PAIRED>(C_F4, stride, cell)] = m::fma_(B1, vn, -(Bn * v1));
-    box[box_at<PAIRED>(C_F5, stride, cell)] = m::fma_(B2, vn, -(Bn * v2));
-    box[box_at<PAIRED>(C_F6, stride, cell)] = m::fma_(E + Pt, vn, -(Bn * vB));
+    box[box_at<PAIRED>(C_F2, stride, cell)] = m::fma_(mn, v1, -m::mul_(Bn, B1));
+    box[box_at<PAIRED>(C_F3, stride, cell)] = m::fma_(mn, v2, -m::mul_(Bn, B2));
+    box[box_at<PAIRED>(C_F4, stride, cell)] = m::fma_(B1, vn, -m::mul_(Bn, v1));
+    box[box_at<PAIRED>(C_F5, stride, cell)] = m::fma_(B2, vn, -m::mul_(Bn, v2));
+    box[box_at<PAIRED>(C_F6, stride, cell)] = m::fma_(E + Pt, vn, -m::mul_(Bn, vB));
     // c_f, c_A and c_slow = c_s c_A / c_f, from reciprocal square roots
-    const Real cs2 = K.gamma * P * ir;
+    const Real cs2 = m::mul_(m::mul_(K.gamma, P), ir);
     Real fmc, cms, cf2;
-    speeds_fast<Real>(cs2, Bn2 * ir, Bt2 * ir, fmc, cms, cf2);
+    speeds_fast<Real>(cs2, m::mul_(Bn2, ir), m::mul_(Bt2, ir), fmc, cms, cf2);
     const Real icf = m::rsqrt_(cf2);
-    const Real ca = m::abs_(Bn) * isr;
-    box[box_at<PAIRED>(C_CF, stride, cell)] = cf2 * icf;
+    const Real ca = m::mul_(m::abs_(Bn), isr);
+    box[box_at<PAIRED>(C_CF, stride, cell)] = m::mul_(cf2, icf);
     box[box_at<PAIRED>(C_CA, stride, cell)] = ca;
-    box[box_at<PAIRED>(C_CSL, stride, cell)] = cs2 * m::rsqrt_(cs2) * (ca * icf);
+    box[box_at<PAIRED>(C_CSL, stride, cell)] = m::mul_(m::mul_(cs2, m::rsqrt_(cs2)), m::mul_(ca, icf));
 }
 
 // cell_fill_frame for a sweep along axis AX (frame (n, t1, t2) = (AX, AX+1,
 // AX+2) mod 3) from the lab components
-template <typename Real, int AX, bool PAIRED = false>
+template <typename Real, int AX, bool PAIRED = false, typename MM = M<Real>>
 __device__ __forceinline__ void cell_fill(Real *box, int cell, int stride, Real rho, Real mx, Real my, Real mz, Real E,
                                           Real Bx, Real By, Real Bz, const Phys<Real> &K, bool &bad, bool &hit) {
     constexpr int n = AX, t1 = (AX + 1) % 3, t2 = (AX + 2) % 3;
     const Real mm[3] = {mx, my, mz};
     const Real BB3[3] = {Bx, By, Bz};
-    cell_fill_frame<Real, PAIRED>(box, cell, stride, rho, mm[n], mm[t1], mm[t2], E, BB3[n], BB3[t1], BB3[t2], K, bad, hit);
+    cell_fill_frame<Real, PAIRED, MM>(box, cell, stride, rho, mm[n], mm[t1], mm[t2], E, BB3[n], BB3[t1], BB3[t2], K, bad, hit);
 }
 
 // the same with the axis known only at run time (selects, no indexed arrays)
@@ -406,20 +504,20 @@ __device__ __forceinline__ float phi_nf(float a, float b, float c, float d, floa
 
 // double: the weights times the common factor (s_0 s_1 s_2)^2, so that no
 // weight needs a division; phi_N = N / (12 D), and the two interpolants of
-// one field share a single division in weno_field.  29 FP64 instructions
-// (WENO-Z).
+// one field share a single division in weno_field.
+//
+// W0, V1, V2 are the alpha_k / d_k times that factor: weights_mul in the FP64
+// multiplier, weno_weights with the products on the integer pipes.  The
+// latter's range is checked once for all products: 2^-160 <= s_k < 2^96 by the
+// exponent fields, and (WENO-Z) tau != 0, so |tau| >= 2^-213.  The largest and
+// smallest are then q^2 in 2^-960 .. 2^576 and tau p_0 >= 2^-533.
 template <int VAR>
-__device__ __forceinline__ void phi_nd(double a, double b, double c, double d, double eps12, double &N, double &D) {
-    double s0, s1, s2, x0, y0, z0;
-    smoothness3<double>(a, b, c, d, eps12, s0, s1, s2, x0, y0, z0);
+static __device__ __noinline__ double3 weights_mul(double s0, double s1, double s2) {
     const double p0 = s1 * s2;
-    double W0, V1, V2;   // alpha_k / d_k times the common factor
     if constexpr (VAR == 0) {
         // alpha_k / d_k = 1 / s_k^2
         const double p1 = s0 * s2, p2 = s0 * s1;
-        W0 = p0 * p0;
-        V1 = p1 * p1;
-        V2 = p2 * p2;
+        return make_double3(p0 * p0, p1 * p1, p2 * p2);
     } else {
         // alpha_k / d_k = 1 + tau^2 / s_k^2: (s0 s1 s2)^2 + (tau prod_{j != k} s_j)^2,
         // tau = (IS_0 - IS_2) / 12 (its sign drops out)
@@ -427,14 +525,65 @@ __device__ __forceinline__ void phi_nd(double a, double b, double c, double d, d
         const double q = s0 * p0, t0 = tau * s0;
         const double A = tau * p0, B = t0 * s2, C = t0 * s1;
         const double Q = q * q;
-        W0 = fma(A, A, Q);
-        V1 = fma(B, B, Q);
-        V2 = fma(C, C, Q);
+        return make_double3(fma(A, A, Q), fma(B, B, Q), fma(C, C, Q));
     }
-    // D = W0 + 6 V1 + 3 V2, N = 4 W0 t1 + (6 V2 - D) t2
-    const double Y = fma(6.0, V1, W0);
-    D = fma(3.0, V2, Y);
-    N = fma(W0, dscale2<2>(x0 - y0), fma(3.0, V2, -Y) * (y0 - z0));
+}
+
+template <int VAR>
+__device__ __forceinline__ void weno_weights(double s0, double s1, double s2, double &W0, double &V1, double &V2) {
+    const unsigned c = 863u << 20;
+    const unsigned out = ((unsigned)__double2hiint(s0) - c) | ((unsigned)__double2hiint(s1) - c) |
+                         ((unsigned)__double2hiint(s2) - c);
+    if (out < (256u << 20) && (VAR == 0 || __double_as_longlong(s0) != __double_as_longlong(s2))) {
+        const DFactor f0(s0), f1(s1), f2(s2);
+        const DFactor p0(dmul_int(f1, f2));
+        if constexpr (VAR == 0) {
+            const DFactor p1(dmul_int(f0, f2)), p2(dmul_int(f0, f1));
+            W0 = dmul_int(p0, p0);
+            V1 = dmul_int(p1, p1);
+            V2 = dmul_int(p2, p2);
+        } else {
+            const DFactor ft(s0 - s2), q(dmul_int(f0, p0)), t0(dmul_int(ft, f0));
+            const double A = dmul_int(ft, p0), B = dmul_int(t0, f2), C = dmul_int(t0, f1);
+            const double Q = dmul_int(q, q);
+            W0 = fma(A, A, Q);
+            V1 = fma(B, B, Q);
+            V2 = fma(C, C, Q);
+        }
+    } else {
+        const double3 w = weights_mul<VAR>(s0, s1, s2);
+        W0 = w.x;
+        V1 = w.y;
+        V2 = w.z;
+    }
+}
+
+// The two interpolants of a field, phi_N(p_0 .. p_3) = Np / (12 Dp) and
+// phi_N(q_3 .. q_0) = Nm / (12 Dm), with D = W0 + 6 V1 + 3 V2 and
+// N = 4 W0 t1 + (6 V2 - D) t2
+template <int VAR>
+__device__ __forceinline__ void phi_nd(const double (&p)[4], const double (&q)[4], double eps12, double &Np, double &Dp,
+                                       double &Nm, double &Dm) {
+    double a0, a1, a2, ax, ay, az, b0, b1, b2, bx, by, bz;
+    smoothness3<double>(p[0], p[1], p[2], p[3], eps12, a0, a1, a2, ax, ay, az);
+    smoothness3<double>(q[3], q[2], q[1], q[0], eps12, b0, b1, b2, bx, by, bz);
+    double A0, A1, A2, B0, B1, B2;
+    weno_weights<VAR>(a0, a1, a2, A0, A1, A2);
+    weno_weights<VAR>(b0, b1, b2, B0, B1, B2);
+    const double YA = fma(6.0, A1, A0), YB = fma(6.0, B1, B0);
+    Dp = fma(3.0, A2, YA);
+    Dm = fma(3.0, B2, YB);
+    const double vA = fma(3.0, A2, -YA), vB = fma(3.0, B2, -YB), tA = ay - az, tB = by - bz;
+    double mA, mB;
+    if (dmid(vA) && dmid(vB) && dmid(tA) && dmid(tB)) {
+        mA = dmul_normal(vA, tA);
+        mB = dmul_normal(vB, tB);
+    } else {
+        mA = dmul_fp64(vA, tA);
+        mB = dmul_fp64(vB, tB);
+    }
+    Np = fma(A0, dscale2<2>(ax - ay), mA);
+    Nm = fma(B0, dscale2<2>(bx - by), mB);
 }
 
 // N_m / D_m - N_p / D_p where the product of the denominators leaves the
@@ -616,6 +765,39 @@ __device__ __forceinline__ Pair<float> pfma(float s, Pair<float> a, Pair<float> 
 __device__ __forceinline__ Pair<double> pfma(double s, Pair<double> a, Pair<double> c) {
     return {fma(s, a.x, c.x), fma(s, a.y, c.y)};
 }
+// s a, s b, -s c and s a, t a: in double one range check for all their products
+__device__ __forceinline__ void pmul3(float s, Pair<float> a, Pair<float> b, Pair<float> c, Pair<float> &x,
+                                      Pair<float> &y, Pair<float> &z) {
+    x = pmul(s, a);
+    y = pmul(s, b);
+    z = pmul(-s, c);
+}
+__device__ __forceinline__ void pmul2(float s, float t, Pair<float> a, Pair<float> &x, Pair<float> &y) {
+    x = pmul(s, a);
+    y = pmul(t, a);
+}
+__device__ __forceinline__ void pmul3(double s, Pair<double> a, Pair<double> b, Pair<double> c, Pair<double> &x,
+                                      Pair<double> &y, Pair<double> &z) {
+    const unsigned w = dwindow(s) | dwindow(a.x) | dwindow(a.y) | dwindow(b.x) | dwindow(b.y) | dwindow(c.x) | dwindow(c.y);
+    if (w < kInWindow) {
+        x = {dmul_normal(s, a.x), dmul_normal(s, a.y)};
+        y = {dmul_normal(s, b.x), dmul_normal(s, b.y)};
+        z = {dmul_normal(-s, c.x), dmul_normal(-s, c.y)};
+    } else {
+        x = {dmul_fp64(s, a.x), dmul_fp64(s, a.y)};
+        y = {dmul_fp64(s, b.x), dmul_fp64(s, b.y)};
+        z = {dmul_fp64(-s, c.x), dmul_fp64(-s, c.y)};
+    }
+}
+__device__ __forceinline__ void pmul2(double s, double t, Pair<double> a, Pair<double> &x, Pair<double> &y) {
+    if ((dwindow(s) | dwindow(t) | dwindow(a.x) | dwindow(a.y)) < kInWindow) {
+        x = {dmul_normal(s, a.x), dmul_normal(s, a.y)};
+        y = {dmul_normal(t, a.x), dmul_normal(t, a.y)};
+    } else {
+        x = {dmul_fp64(s, a.x), dmul_fp64(s, a.y)};
+        y = {dmul_fp64(t, a.x), dmul_fp64(t, a.y)};
+    }
+}
 // dF + alpha du and dF - alpha du
 __device__ __forceinline__ float psplit(Pair<float> a, float al) { return __fmaf_rn(al, a.v.y, a.v.x); }
 __device__ __forceinline__ double psplit(Pair<double> a, double al) { return fma(al, a.y, a.x); }
@@ -675,13 +857,19 @@ __device__ __forceinline__ Real weno_field(const Pair<Real> (&P)[5], Real alpha,
     }
     if constexpr (std::is_same<Real, double>::value) {
         double Np, Dp, Nm, Dm;
-        phi_nd<VAR>(p[0], p[1], p[2], p[3], eps3, Np, Dp);
-        phi_nd<VAR>(q[3], q[2], q[1], q[0], eps3, Nm, Dm);
-        const double prod = Dp * Dm;
+        phi_nd<VAR>(p, q, eps3, Np, Dp, Nm, Dm);
+        double prod, cross;
+        if (dmid(Dp) && dmid(Dm) && dmid(Np)) {
+            prod = dmul_normal(Dp, Dm);
+            cross = dmul_normal(Np, Dm);
+        } else {
+            prod = dmul_fp64(Dp, Dm);
+            cross = dmul_fp64(Np, Dm);
+        }
         // 2^-962 <= prod < 2^962 by its exponent field (positive, or NaN: outside)
         if ((unsigned)__double2hiint(prod) - 0x03d00000u < 0x78400000u)
             // -Np/Dp + Nm/Dm over the common denominator: one division
-            return ddiv_newton(fma(Nm, Dp, -(Np * Dm)), prod);
+            return ddiv_newton(fma(Nm, Dp, -cross), prod);
         return weno_quotients(Np, Dp, Nm, Dm);
     } else {
         static_assert(std::is_same<Real, float>::value, "weno_field takes float or double");
@@ -706,17 +894,17 @@ struct FaceEigen {
     bool apart;   // c_f > c_slow: a_f, a_s as above (else both 1, Appendix A)
 };
 
-template <typename Real>
+template <typename Real, typename MM = M<Real>>
 __device__ __forceinline__ FaceEigen<Real> face_eigen(Real r, Real v2, Real Bn, Real Bt1, Real Bt2, Real P,
                                                       const Phys<Real> &K) {
-    using m = M<Real>;
+    using m = MM;
     FaceEigen<Real> e;
     e.isr = m::rsqrt_(r);
-    const Real ir = e.isr * e.isr;
-    e.sr = r * e.isr;
-    const Real ca2 = Bn * Bn * ir;
-    const Real btm = m::fma_(Bt2, Bt2, Bt1 * Bt1);
-    const Real bt2 = btm * ir;
+    const Real ir = m::mul_(e.isr, e.isr);
+    e.sr = m::mul_(r, e.isr);
+    const Real ca2 = m::mul_(m::mul_(Bn, Bn), ir);
+    const Real btm = m::fma_(Bt2, Bt2, m::mul_(Bt1, Bt1));
+    const Real bt2 = m::mul_(btm, ir);
     // The slow and fast left eigenvectors carry 1/(2 c_s^2): the projection
     // amplifies the rounding of the data by about (v^2 + c_A^2 + b_t^2)/c_s^2.
     // In float, near a pressure floor, that reaches 1e9 and the split fluxes
@@ -724,35 +912,35 @@ __device__ __forceinline__ FaceEigen<Real> face_eigen(Real r, Real v2, Real Bn, 
     // no smaller than cs2_rel times that sum.  L and R stay exact inverses, so
     // the flux stays consistent and conservative; only the basis in which
     // WENO reconstructs changes.  cs2_rel = 0 in double.
-    e.cs2 = K.gamma * P * ir;
+    e.cs2 = m::mul_(m::mul_(K.gamma, P), ir);
     if constexpr (float_based<Real>) e.cs2 = m::max_(e.cs2, K.cs2_rel * (v2 + ca2 + bt2));
     const Real ics = m::rsqrt_(e.cs2);
-    e.cs = e.cs2 * ics;
-    e.ics2 = ics * ics;
-    const Real q = e.cs2 * bt2;
+    e.cs = m::mul_(e.cs2, ics);
+    e.ics2 = m::mul_(ics, ics);
+    const Real q = m::mul_(e.cs2, bt2);
     const Real aa = ca2 + bt2 - e.cs2;
     const Real dd = m::fma_(aa, aa, Real(4) * q);
     const bool some = m::normal_pos(dd);
     const Real isd = some ? m::rsqrt_(dd) : Real(0);
-    const Real sd = dd * isd;
+    const Real sd = m::mul_(dd, isd);
     const Real big = m::half_(sd + m::abs_(aa));
     const Real ibt = m::normal_pos(btm) ? m::rsqrt_(btm) : Real(0);
-    const Real bta = btm * ibt;   // |B_t|
-    const Real wb = big * isd;
+    const Real bta = m::mul_(btm, ibt);   // |B_t|
+    const Real wb = m::mul_(big, isd);
     const Real iwb = m::rsqrt_(wb);
-    const Real small_a = some ? (e.cs * (bta * e.isr)) * (isd * iwb) : Real(0);
+    const Real small_a = some ? m::mul_(m::mul_(e.cs, m::mul_(bta, e.isr)), m::mul_(isd, iwb)) : Real(0);
     e.apart = some && m::ge_pos(sd, K.eps_b2);
-    const Real ab = e.apart ? wb * iwb : Real(1), al = e.apart ? small_a : Real(1);
+    const Real ab = e.apart ? m::mul_(wb, iwb) : Real(1), al = e.apart ? small_a : Real(1);
     const bool fast_big = m::nonneg(aa);
     e.as = fast_big ? ab : al;
     e.af = fast_big ? al : ab;
     // c_f^2 = c_s^2 + (c_f^2 - c_s^2), the difference a_s^2 sqrt(d)
-    e.cf2 = e.cs2 + (fast_big ? big : (small_a * small_a) * sd);
+    e.cf2 = e.cs2 + (fast_big ? big : m::mul_(m::mul_(small_a, small_a), sd));
     const Real icf = m::rsqrt_(e.cf2);
-    e.cf = e.cf2 * icf;
+    e.cf = m::mul_(e.cf2, icf);
     // c_slow = c_s c_A / c_f (c_slow^2 = c_s^2 c_A^2 / c_f^2), c_A = |B_n| / sqrt(rho)
-    e.csl = e.cs * (m::abs_(Bn) * e.isr) * icf;
-    e.csl2 = e.csl * e.csl;
+    e.csl = m::mul_(m::mul_(e.cs, m::mul_(m::abs_(Bn), e.isr)), icf);
+    e.csl2 = m::mul_(e.csl, e.csl);
     if (m::gt_pos(btm, K.eps_b)) {   // b = B_t / |B_t|
         e.b1 = Bt1 * ibt;
         e.b2 = Bt2 * ibt;
@@ -786,32 +974,26 @@ __device__ __forceinline__ FaceEigen<Real> face_eigen(Real r, Real v2, Real Bn, 
 // float.  Against the form that projected eleven vectors on Appendix A's rows
 // in the lab frame: 535.0 -> 416.7 ms per 256^3 FP64 step (WENO-Z), 15.57 ->
 // 14.46 ms in FP32-bulk, 56.6 -> 49.3 ms per 128^3 step with double-word
-// weights; no larger error against 64-bit values in any of them.
-template <typename Real, int VAR, bool DIFF = false, bool DWW = false, bool PAIRED = false>
+// weights; no larger error against 64-bit values in any of them.  With the tiles
+// of today and the products on the integer pipes: 331 ms, FP64 pipe about 80%
+// busy, issue slots 20%.
+template <typename Real, int VAR, bool DIFF = false, bool DWW = false, bool PAIRED = false, typename MM = M<Real>>
 __device__ __forceinline__ void face_flux(const Real *__restrict__ box, int cell, int ncell, int st, const Phys<Real> &K,
                                           Real (&Ff)[7], Real &s1, Real &s2) {
-    using m = M<Real>;
+    using m = MM;
     using P2 = Pair<Real>;
 #define SMQ(q, k) box[box_at<PAIRED>(q, ncell, cell + (k) * st)]
     // stencil differences X[c][j] = (dF_c, du_c) at position j, and the
     // central combination (7 (f2 + f3) - (f1 + f4)) / 12 written as
     // f2 + (6 dF(2) + dF(1) - dF(3)) / 12
-    P2 X[7][5];
+    [[maybe_unused]] P2 X[7][5];
     Real X0[7];
 #pragma unroll
     for (int c = 0; c < 7; ++c) {
         if constexpr (DIFF) {
             // from the box's forward differences (its difference pass)
             const int qD = C_DF0 + c;
-            const int qU = c == 0 ? C_RHOQ : c == 1 ? C_MN : c == 2 ? C_MT1 : c == 3 ? C_MT2 : c == 4 ? C_DU4
-                           : c == 5 ? C_DU5 : C_E;
-            Real dF[5];
-#pragma unroll
-            for (int j = 0; j < 5; ++j) {
-                dF[j] = SMQ(qD, j);
-                X[c][j] = make_pair2(dF[j], SMQ(qU, j));
-            }
-            X0[c] = m::fma_(m::fma_(Real(6), dF[2], dF[1]) - dF[3], Real(1.0 / 12.0), SMQ(C_F0 + c, 2));
+            X0[c] = m::fma_(m::fma_(Real(6), SMQ(qD, 2), SMQ(qD, 1)) - SMQ(qD, 3), Real(1.0 / 12.0), SMQ(C_F0 + c, 2));
         } else if constexpr (PAIRED) {
             float2 f[6];
 #pragma unroll
@@ -848,12 +1030,11 @@ __device__ __forceinline__ void face_flux(const Real *__restrict__ box, int cell
     // twice the transport fluxes <B_n v_t> of the two cells
     const Real bvt1 = m::fma_(SMQ(C_BN, 2), SMQ(C_VT1, 2), SMQ(C_BN, 3) * SMQ(C_VT1, 3));
     const Real bvt2 = m::fma_(SMQ(C_BN, 2), SMQ(C_VT2, 2), SMQ(C_BN, 3) * SMQ(C_VT2, 3));
-#undef SMQ
 
     // ---- eigen scalars at the interface state (Appendix A)
     const Real v2 = m::fma_(vt2, vt2, m::fma_(vt1, vt1, vn * vn));
     const Real hv2 = m::half_(v2);
-    const FaceEigen<Real> e = face_eigen<Real>(r, v2, Bn, Bt1, Bt2, P, K);
+    const FaceEigen<Real> e = face_eigen<Real, MM>(r, v2, Bn, Bt1, Bt2, P, K);
     const Real b1 = e.b1, b2 = e.b2, sg = e.sg;
     const Real pre = m::half_(e.ics2);
     const Real tau = K.gm1 * e.ics2;
@@ -874,71 +1055,91 @@ __device__ __forceinline__ void face_flux(const Real *__restrict__ box, int cell
     // at most |B_t| |X_B| <= 1e-15 |X_B|.)  The Alfven fields are carried
     // without their factor sg/2: phi_N is linear up to epsilon, which scales
     // by 4 with them, and the factor joins the back-projection.
-    P2 fu[5], fl[5], su[5], sl[5], au[5], al[5], en[5];
+    P2 F[7][5];
     const Real cF = pre * (K.gm1 * e.af), cS = pre * (K.gm1 * e.as);
     const Real srcs = pre * (e.sr * e.cs);
     const Real hF = srcs * e.as, hS = -(srcs * e.af);
     const Real nF = -(pre * afcf), nS = -(pre * ascl), kF = pre * sas, kS = -(pre * saf);
     const Real ssr = sg * e.sr;
     const Real a5 = ssr * b1, a4 = -(ssr * b2);
-#pragma unroll
-    for (int j = 0; j < 5; ++j) {
-        const P2 Yn = pfma(-vn, X[0][j], X[1][j]);
-        const P2 Y1 = pfma(-vt1, X[0][j], X[2][j]);
-        const P2 Y2 = pfma(-vt2, X[0][j], X[3][j]);
-        const P2 h = pfma(b1, X[4][j], pmul(b2, X[5][j]));
-        const P2 k = pfma(b1, Y1, pmul(b2, Y2));
-        const P2 x = pfma(b1, Y2, pmul(-b2, Y1));
-        P2 g = pfma(-hv2, X[0][j], X[6][j]);
+    // The seven fields at one position of the stencil: the fast, slow and
+    // Alfven pairs (members u, l), entropy
+    auto project = [&](const P2 (&x7)[7], P2 (&f)[7]) {
+        const P2 Yn = pfma(-vn, x7[0], x7[1]);
+        const P2 Y1 = pfma(-vt1, x7[0], x7[2]);
+        const P2 Y2 = pfma(-vt2, x7[0], x7[3]);
+        P2 mh, mk, mx, mF, mS;
+        pmul3(b2, x7[5], Y2, Y1, mh, mk, mx);
+        const P2 h = pfma(b1, x7[4], mh);
+        const P2 k = pfma(b1, Y1, mk);
+        const P2 x = pfma(b1, Y2, mx);
+        pmul2(hF, hS, h, mF, mS);
+        P2 g = pfma(-hv2, x7[0], x7[6]);
         g = pfma(-vn, Yn, g);
         g = pfma(-vt1, Y1, g);
         g = pfma(-vt2, Y2, g);
         g = pfma(-e.bt, h, g);
-        mode_pair(pfma(cF, g, pmul(hF, h)), nF, Yn, kF, k, fu[j], fl[j]);
-        mode_pair(pfma(cS, g, pmul(hS, h)), nS, Yn, kS, k, su[j], sl[j]);
-        mode_pair(x, a4, X[4][j], a5, X[5][j], au[j], al[j]);
-        en[j] = pfma(-tau, g, X[0][j]);
-    }
-
+        mode_pair(pfma(cF, g, mF), nF, Yn, kF, k, f[0], f[1]);
+        mode_pair(pfma(cS, g, mS), nS, Yn, kS, k, f[2], f[3]);
+        mode_pair(x, a4, x7[4], a5, x7[5], f[4], f[5]);
+        f[6] = pfma(-tau, g, x7[0]);
+    };
     // ---- WENO parts of the fields: sums and differences of the pairs, upper
     // members m = 1 (v - c_f), 3 (v - c_slow), 2 (v - c_A)
     Real sf, df, ss, ds, sa, da, Fe;
-    [[maybe_unused]] auto fields = [&](const P2 (&u)[5], const P2 (&l)[5], Real cL, Real cR, Real ep, Real &sum, Real &dif) {
-        const Real Fu = weno_field<Real, VAR>(u, alpha(-cL, -cR), ep);
-        const Real Fl = weno_field<Real, VAR>(l, alpha(cL, cR), ep);
-        sum = Fu + Fl;
-        dif = Fu - Fl;
-    };
-    if constexpr (!DWW) {
-        fields(fu, fl, cfL, cfR, eps3, sf, df);
-        fields(su, sl, csL, csR, eps3, ss, ds);
-        fields(au, al, caL, caR, Real(4) * eps3, sa, da);
-        Fe = weno_field<Real, VAR>(en, m::max_nonneg(m::abs_(vL), m::abs_(vR)), eps3);
-    } else {
-        // double-word: one copy of the interpolants (about 1800 instructions
-        // for the two sides) in a loop over the fields, the projections in
-        // local memory.  Unrolled, the face function was 215 KB of code, which
-        // no instruction cache of an SM holds: 128^3 step 49.0 -> 39.7 ms.  (The
-        // IEEE form, 20 KB, is 1.6% faster unrolled.)
-        P2 F[7][5];
-        Real V[7];
-        const Real cL[7] = {-cfL, cfL, -csL, csL, -caL, caL, Real(0)}, cR[7] = {-cfR, cfR, -csR, csR, -caR, caR, Real(0)};
+    if constexpr (std::is_same<Real, float>::value) {
 #pragma unroll
         for (int j = 0; j < 5; ++j) {
-            F[0][j] = fu[j];
-            F[1][j] = fl[j];
-            F[2][j] = su[j];
-            F[3][j] = sl[j];
-            F[4][j] = au[j];
-            F[5][j] = al[j];
-            F[6][j] = en[j];
+            P2 x7[7], f[7];
+#pragma unroll
+            for (int c = 0; c < 7; ++c) x7[c] = X[c][j];
+            project(x7, f);
+#pragma unroll
+            for (int mo = 0; mo < 7; ++mo) F[mo][j] = f[mo];
         }
+        auto fields = [&](const P2 (&u)[5], const P2 (&l)[5], Real cL, Real cR, Real ep, Real &sum, Real &dif) {
+            const Real Fu = weno_field<Real, VAR>(u, alpha(-cL, -cR), ep);
+            const Real Fl = weno_field<Real, VAR>(l, alpha(cL, cR), ep);
+            sum = Fu + Fl;
+            dif = Fu - Fl;
+        };
+        fields(F[0], F[1], cfL, cfR, eps3, sf, df);
+        fields(F[2], F[3], csL, csR, eps3, ss, ds);
+        fields(F[4], F[5], caL, caR, Real(4) * eps3, sa, da);
+        Fe = weno_field<Real, VAR>(F[6], m::max_nonneg(m::abs_(vL), m::abs_(vR)), eps3);
+    } else {
+        // double: loops over the positions and over the fields, the projections
+        // in local memory.  With integer products and double-word interpolants
+        // the unrolled face function is 100 to 200 KB of code, which no
+        // instruction cache of an SM holds, and the loops need no more than 168
+        // registers, three blocks per SM without spills: 256^3 WENO-Z step 388
+        // ms unrolled, 353 looped with the products of the projections and
+        // quotients on the integer pipes (396 and more unrolled); 128^3 step
+        // with double-word weights 49.0 -> 39.7 ms.
+#pragma unroll 1
+        for (int j = 0; j < 5; ++j) {
+            P2 x7[7], f[7];
+#pragma unroll
+            for (int c = 0; c < 7; ++c) {
+                const int qU = c == 0 ? C_RHOQ : c == 1 ? C_MN : c == 2 ? C_MT1 : c == 3 ? C_MT2
+                               : c == 4 ? (DIFF ? (int)C_DU4 : (int)C_BT1) : c == 5 ? (DIFF ? (int)C_DU5 : (int)C_BT2) : C_E;
+                if constexpr (DIFF)
+                    x7[c] = make_pair2(SMQ(C_DF0 + c, j), SMQ(qU, j));
+                else
+                    x7[c] = make_pair2(SMQ(C_F0 + c, j + 1) - SMQ(C_F0 + c, j), SMQ(qU, j + 1) - SMQ(qU, j));
+            }
+            project(x7, f);
+#pragma unroll
+            for (int mo = 0; mo < 7; ++mo) F[mo][j] = f[mo];
+        }
+        Real V[7];
+        const Real cL[7] = {-cfL, cfL, -csL, csL, -caL, caL, Real(0)}, cR[7] = {-cfR, cfR, -csR, csR, -caR, caR, Real(0)};
 #pragma unroll 1
         for (int mo = 0; mo < 7; ++mo) {
             P2 f[5];
 #pragma unroll
             for (int j = 0; j < 5; ++j) f[j] = F[mo][j];
-            V[mo] = weno_field<Real, VAR, true>(f, alpha(cL[mo], cR[mo]), mo == 4 || mo == 5 ? Real(4) * eps3 : eps3);
+            V[mo] = weno_field<Real, VAR, DWW>(f, alpha(cL[mo], cR[mo]), mo == 4 || mo == 5 ? Real(4) * eps3 : eps3);
         }
         sf = V[0] + V[1];
         df = V[0] - V[1];
@@ -948,6 +1149,7 @@ __device__ __forceinline__ void face_flux(const Real *__restrict__ box, int cell
         da = V[4] - V[5];
         Fe = V[6];
     }
+#undef SMQ
     if (!e.apart) {
         // Appendix A's fallback: the central part through L and R, in the
         // units of the WENO parts, in place of the unprojected one
