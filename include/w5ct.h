@@ -284,7 +284,8 @@ int w5ct_status(w5ct_ctx *ctx, long long *floor_hits, int *nonphysical);
 int w5ct_synchronize(w5ct_ctx *ctx);
 
 /* Kernel timing: when enabled, each launch of the characteristic sweep
- * kernel is bracketed by CUDA events on the context's stream.
+ * kernel (one axis, or the three axes of a stage where they share a launch) is
+ * bracketed by CUDA events on the context's stream.
  * w5ct_sweep_timing returns the number of sweep launches and their summed
  * device time in milliseconds since timing was last enabled (synchronises). */
 int w5ct_set_timing(w5ct_ctx *ctx, int enable);

@@ -975,8 +975,8 @@ __device__ __forceinline__ FaceEigen<Real> face_eigen(Real r, Real v2, Real Bn, 
 // in the lab frame: 535.0 -> 416.7 ms per 256^3 FP64 step (WENO-Z), 15.57 ->
 // 14.46 ms in FP32-bulk, 56.6 -> 49.3 ms per 128^3 step with double-word
 // weights; no larger error against 64-bit values in any of them.  With the tiles
-// of today and the products on the integer pipes: 331 ms, FP64 pipe about 80%
-// busy, issue slots 20%.
+// of today and the products on the integer pipes: 331 ms, FP64 pipe 83%
+// busy, issue slots 24%.
 template <typename Real, int VAR, bool DIFF = false, bool DWW = false, bool PAIRED = false, typename MM = M<Real>>
 __device__ __forceinline__ void face_flux(const Real *__restrict__ box, int cell, int ncell, int st, const Phys<Real> &K,
                                           Real (&Ff)[7], Real &s1, Real &s2) {
