@@ -355,12 +355,13 @@ struct AllTile {
     static constexpr int BX = AX == 0 ? 32 : 8, T2 = AX == 0 ? 4 : 16;
 };
 
-// Blocks per SM: float 4 (128 registers); double 3 of 168 registers: the chains
-// of integer products and of double-word operations want the warps (256^3 step
-// 388 -> 379 ms, with double-word weights at 128^3 37.0 -> 33.9 ms; four blocks
-// of 128 registers 359 against 353 ms, double-word no faster).
+// Blocks per SM: float 4 (128 registers); double 3 of 168 registers, as the chains
+// of integer products want the warps (256^3 step 388 -> 379 ms; four blocks of
+// 128 registers 337 against 330 ms with every product there); double-word 4, whose
+// chains of FP32 operations are longer still (128^3 step, two to four blocks:
+// 37.0, 33.9, and of the present form 32.7 at three, 31.7 ms at four).
 template <typename Real, int VAR, bool DW>
-__global__ void __launch_bounds__(kAllThreads, sizeof(Real) == 4 ? 4 : 3) sweep_all_kernel(SweepAll<Real> s) {
+__global__ void __launch_bounds__(kAllThreads, sizeof(Real) == 4 || DW ? 4 : 3) sweep_all_kernel(SweepAll<Real> s) {
     extern __shared__ __align__(16) unsigned char w5ct_smem[];
     chain_begin();
     Real *sm = reinterpret_cast<Real *>(w5ct_smem);
