@@ -945,10 +945,16 @@ __device__ __forceinline__ bool float_speeds(const double (&q)[8], const FloatPh
         const float aa = ca2 + bt2 - cs2;
         const float cf2 = 0.5f * (cs2 + ca2 + bt2 + sqrtf(__fmaf_rn(aa, aa, 4.0f * cs2 * bt2)));
         const float s = fabsf(u[d]) + sqrtf(cf2);
-        lo[d] = ok ? s * (1.0f - w) : 0.0f;
+        lo[d] = s * (1.0f - w);
         up[d] = s * (1.0f + w);
     }
-    return ok && up[0] < 1e18f && up[1] < 1e18f && up[2] < 1e18f;
+    // lo goes into the maxima that rule other cells out: it is 0 wherever the
+    // cell cannot be trusted, also when only the speeds themselves (squares of
+    // squares) leave float's range
+    const bool trust = ok && up[0] < 1e18f && up[1] < 1e18f && up[2] < 1e18f;
+#pragma unroll
+    for (int d = 0; d < 3; ++d) lo[d] = trust ? lo[d] : 0.0f;
+    return trust;
 }
 
 // dt = CFL / sum_d (S_d / dx_d), with the same rounded operations as the
