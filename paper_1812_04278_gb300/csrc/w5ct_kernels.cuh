@@ -909,13 +909,17 @@ __device__ __forceinline__ float d2f_trunc(double x) {
 
 // Float bounds on a cell's double signal speeds: S_d lies in [lo[d], up[d]].
 // Returns false where float cannot tell (a pressure that is a small
-// difference, a state that is not physical or out of float's range).
+// difference, a state that is not physical or out of float's range), with lo = 0.
 // With h = 2^-18, more than 8 float roundings (inputs truncated to 2^-23,
 // then at most 8 operations each on positive terms): the pressure is off by
 // at most h (gamma - 1)(|E| + kinetic + magnetic energy) =: ep P, v, c_A^2 and
 // b_t^2 by h.  c_f^2 is increasing and homogeneous of degree 1 in (c_s^2,
 // c_A^2, b_t^2), so it is off by at most a factor 1 + ep + 2 h, plus h for its
-// own evaluation, whose error is a few roundings of c_s^2 + c_A^2 + b_t^2 <= 2 c_f^2.
+// own evaluation, whose error is a few roundings of t = c_s^2 + c_A^2 + b_t^2 <=
+// 2 c_f^2.  The discriminant squares its arguments, so it is formed from
+// c_s^2 / t, c_A^2 / t and b_t^2 / t, which are at most 1 and sum to 1: its
+// underflows are below 2^-126 of the result at any scale of the speeds (without
+// the scaling, c_f came out sqrt 2 too small for c_f below 5e-12).
 struct FloatPhys {
     float gamma, gm1, rho_min, p_min;   // rho_min, p_min: 0 without floors
 };
@@ -938,20 +942,21 @@ __device__ __forceinline__ bool float_speeds(const double (&q)[8], const FloatPh
     const float ep = h * gm1 * (fabsf(E) + half) / P;
     const bool ok = r > 1e-30f && r < 1e30f && P > 1e-30f && P < 1e30f && ep < 0.25f;
     const float cs2 = K.gamma * P * ir;
+    const float t = cs2 + a2[0] + a2[1] + a2[2], it = __fdividef(1.0f, t);
+    const float cs2t = cs2 * it;
     const float w = ep + 4.0f * h;
 #pragma unroll
     for (int d = 0; d < 3; ++d) {
-        const float ca2 = a2[d], bt2 = a2[(d + 1) % 3] + a2[(d + 2) % 3];
-        const float aa = ca2 + bt2 - cs2;
-        const float cf2 = 0.5f * (cs2 + ca2 + bt2 + sqrtf(__fmaf_rn(aa, aa, 4.0f * cs2 * bt2)));
-        const float s = fabsf(u[d]) + sqrtf(cf2);
+        const float ca2 = a2[d] * it, bt2 = (a2[(d + 1) % 3] + a2[(d + 2) % 3]) * it;
+        const float aa = ca2 + bt2 - cs2t;
+        const float cf2 = 0.5f * (cs2t + ca2 + bt2 + sqrtf(__fmaf_rn(aa, aa, 4.0f * cs2t * bt2)));
+        const float s = fabsf(u[d]) + sqrtf(t * cf2);
         lo[d] = s * (1.0f - w);
         up[d] = s * (1.0f + w);
     }
     // lo goes into the maxima that rule other cells out: it is 0 wherever the
-    // cell cannot be trusted, also when only the speeds themselves (squares of
-    // squares) leave float's range
-    const bool trust = ok && up[0] < 1e18f && up[1] < 1e18f && up[2] < 1e18f;
+    // cell cannot be trusted, also when only the speeds leave the range
+    const bool trust = ok && t > 1e-30f && t < 1e30f && up[0] < 1e18f && up[1] < 1e18f && up[2] < 1e18f;
 #pragma unroll
     for (int d = 0; d < 3; ++d) lo[d] = trust ? lo[d] : 0.0f;
     return trust;

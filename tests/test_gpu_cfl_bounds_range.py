@@ -1,8 +1,9 @@
 """The float bounds of speed_kernel's double CFL maxima hold over the whole
 range of units.  Against the oracle's maxima, 1e-13 relative (the parity bar of
 one evaluation): a cell whose squared speeds overflow float when squared once
-more must not shadow the others.  Several iterations of a warp, so that published
-maxima are read."""
+more must not shadow the others (overflow), and states whose speeds are so
+small that their fourth powers underflow must keep a bound above the speed
+(small).  Several iterations of a warp, so that published maxima are read."""
 import numpy as np
 import pytest
 
@@ -39,3 +40,24 @@ def test_overflow(pressure, velocity, at):
     for d in range(3):
         v[d].reshape(-1)[at + 8 * d] = velocity
     check(rho, v, P, (0.0, 0.0, 0.0))
+
+
+# speeds within 30% of one another, the scale of their squares from 1e-26 to 1e34
+@pytest.mark.parametrize("exponent", range(-26, 35, 5))
+@pytest.mark.parametrize("field", [0.0, 0.7])
+def test_small(exponent, field):
+    n = SHAPE[::-1]
+    rng = np.random.default_rng(exponent + 100)
+    scale = 10.0 ** exponent
+    v = rng.uniform(-0.3, 0.3, (3,) + n) * scale ** 0.5
+    P = scale * rng.uniform(1.0, 1.2, n)
+    check(np.ones(n), v, P, tuple(field * scale ** 0.5 * w for w in (0.6, 0.5, -0.4)))
+
+
+# the pressure alone sets the speed, and one cell of the last iteration wins by 10%
+@pytest.mark.parametrize("exponent", [-26, -24, -22, -20])
+def test_small_winner(exponent):
+    n = SHAPE[::-1]
+    P = np.full(n, 10.0 ** exponent)
+    P.reshape(-1)[-100] *= 1.21
+    check(np.ones(n), np.zeros((3,) + n), P, (0.0, 0.0, 0.0))
