@@ -77,35 +77,44 @@ template <typename R>
 __device__ __forceinline__ void speeds_rev(R cs2, R ca2, R bt2, R lfmc, R lcms, R lcf2, R lcsl2, R &lcs2, R &lca2,
                                            R &lbt2) {
     using m = M<R>;
-    const R q = cs2 * bt2;
     const R aa = ca2 + bt2 - cs2;
-    const R dd = m::fma_(aa, aa, R(4) * q);
-    const R isd = m::normal_pos(dd) ? m::rsqrt_(dd) : R(0);
-    const R big = m::half_(dd * isd + m::abs_(aa));
+    const R dd = m::fma_(aa, aa, R(4) * (cs2 * bt2));
+    R isd, sd;
+    if (disc_normal(dd)) {
+        isd = m::rsqrt_(dd);
+        sd = dd * isd;
+    } else {
+        const Disc<R> d = disc_small(aa, cs2, bt2);
+        isd = d.isd;
+        sd = d.sd;
+    }
+    const R big = m::half_(sd + m::abs_(aa));
     const R ibig = m::normal_pos(big) ? m::rcp3_(big) : R(0);
-    const R oth = q * ibig;
+    // ratios of speeds first: products of two squared speeds, or of their
+    // adjoints and a reciprocal, may leave the range
+    const R ci = cs2 * ibig, bi = bt2 * ibig, oth = cs2 * bi;
     const bool fast_big = m::nonneg(aa);
     const R cf2 = cs2 + (fast_big ? big : oth);
     const R icf2 = m::normal_pos(cf2) ? m::rcp3_(cf2) : R(0);
-    lcs2 += lcsl2 * (ca2 * icf2);
-    lca2 += lcsl2 * (cs2 * icf2);
-    lcf2 -= lcsl2 * (cs2 * ca2 * icf2) * icf2;
+    const R cc = cs2 * icf2, ac = ca2 * icf2;
+    lcs2 += lcsl2 * ac;
+    lca2 += lcsl2 * cc;
+    lcf2 -= lcsl2 * (cc * ac);
     lcs2 += lcf2;
     lfmc += lcf2;
-    // big = (sqrt(dd) + |aa|) / 2, oth = q / big
+    // big = (sqrt(dd) + |aa|) / 2, oth = c_s^2 b_t^2 / big
     const R loth = fast_big ? lcms : lfmc;
     R lbig = fast_big ? lfmc : lcms;
-    const R lq = loth * ibig;
-    lbig -= loth * oth * ibig;
-    lcs2 += lq * bt2;
-    lbt2 += lq * cs2;
-    const R laa = m::half_(fast_big ? lbig : -lbig);
-    const R ldd = m::half_(lbig) * m::half_(isd);
-    // dd = aa^2 + 4 q, aa = ca2 + bt2 - cs2
-    const R la = laa + R(2) * ldd * aa;
+    lbig -= loth * (ci * bi);
+    lcs2 += loth * bi;
+    lbt2 += loth * ci;
+    const R hb = m::half_(lbig);
+    const R laa = fast_big ? hb : -hb;
+    // dd = aa^2 + 4 c_s^2 b_t^2, aa = ca2 + bt2 - cs2
+    const R la = laa + hb * (aa * isd);
     lca2 += la;
-    lbt2 += la + R(4) * ldd * cs2;
-    lcs2 += R(4) * ldd * bt2 - la;
+    lbt2 += la + lbig * (cs2 * isd);
+    lcs2 += lbig * (bt2 * isd) - la;
 }
 
 // One interpolant phi~ = N / D = 12 phi_N(a, b, c, d) (the weights of the
@@ -696,7 +705,7 @@ __device__ __forceinline__ void cell_fill_adjoint(const R (&in)[8], const R (&lq
         R fmc, cms, cf2;
         speeds_fast<R>(cs2, ca2, bt2, fmc, cms, cf2);
         const R icf2 = m::normal_pos(cf2) ? m::rcp3_(cf2) : R(0);
-        const R csl2 = cs2 * ca2 * icf2;
+        const R csl2 = (cs2 * icf2) * ca2;
         const R lcf2 = m::normal_pos(cf2) ? m::half_(lcf * m::rsqrt_(cf2)) : R(0);
         const R lcsl2 = m::normal_pos(csl2) ? m::half_(lcs * m::rsqrt_(csl2)) : R(0);
         R lcs2 = R(0), lca2 = R(0), lbt2 = R(0);

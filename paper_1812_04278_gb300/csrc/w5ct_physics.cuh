@@ -304,6 +304,46 @@ struct MCalled : M<double> {
 };
 
 // ---------------------------------------------------------------- wave speeds
+// The discriminant d = aa^2 + 4 c_s^2 b_t^2 (aa = c_A^2 + b_t^2 - c_s^2) of the
+// fast and slow speeds is a square of squared speeds: speeds below 3e-10 in
+// float (1e-77 in double) take it below the normal range, where its root
+// c_f^2 - c_slow^2 still has all its digits.  Below disc_normal, where either
+// square may have lost some of them (2^28, 2^61 times the smallest normal
+// number: a flushed c_s^2 b_t^2 is then below rounding), it is formed from aa and
+// 2 c_s b_t times 2^100 (2^900).  sd = sqrt(d), isd = 1 / sd, small = c_s^2 b_t^2 / big
+// with big = (sd + |aa|) / 2; all 0 where sd itself is below the normal range.
+__device__ __forceinline__ bool disc_normal(float dd) { return !(dd < 0x1p-98f); }
+__device__ __forceinline__ bool disc_normal(double dd) { return __double2hiint(dd) >= 63 << 20; }   // 2^-960
+template <typename Real>
+struct Disc {
+    Real sd, isd, small;
+};
+template <typename Real>
+__device__ __forceinline__ Disc<Real> disc_scaled(Real aa, Real cs2, Real bt2) {
+    using m = M<Real>;
+    constexpr Real S = std::is_same<Real, float>::value ? Real(0x1p100) : Real(0x1p900);
+    constexpr Real iS = std::is_same<Real, float>::value ? Real(0x1p-100) : Real(0x1p-900);
+    const Real cs = m::normal_pos(cs2) ? cs2 * m::rsqrt_(cs2) : Real(0);
+    const Real bt = m::normal_pos(bt2) ? bt2 * m::rsqrt_(bt2) : Real(0);
+    const Real a = aa * S, h = (cs * bt) * S;
+    const Real dd = m::fma_(a, a, Real(4) * (h * h));
+    if (!m::normal_pos(dd)) return {Real(0), Real(0), Real(0)};
+    const Real isd = m::rsqrt_(dd), sd = dd * isd;
+    if (!m::normal_pos(sd * iS)) return {Real(0), Real(0), Real(0)};
+    return {sd * iS, isd * S, m::div_(h * iS, m::half_(sd + m::abs_(a))) * h};
+}
+// (double: out of line, so that its rare instructions do not issue, predicated
+// off, on the FP64 pipe)
+static __device__ __noinline__ double3 disc_scaled_call(double aa, double cs2, double bt2) {
+    const Disc<double> d = disc_scaled<double>(aa, cs2, bt2);
+    return make_double3(d.sd, d.isd, d.small);
+}
+__device__ __forceinline__ Disc<float> disc_small(float aa, float cs2, float bt2) { return disc_scaled<float>(aa, cs2, bt2); }
+__device__ __forceinline__ Disc<double> disc_small(double aa, double cs2, double bt2) {
+    const double3 d = disc_scaled_call(aa, cs2, bt2);
+    return {d.x, d.y, d.z};
+}
+
 // c_f^2 - c_s^2 (fmc), c_s^2 - c_slow^2 (cms) without cancellation, and c_f^2.
 // The larger of the two differences is (sd + |aa|) / 2 (aa = c_A^2 + b_t^2 -
 // c_s^2), the other c_s^2 b_t^2 over it; the discriminant is the same one as
@@ -315,16 +355,23 @@ __device__ __forceinline__ void speeds_fast(Real cs2, Real ca2, Real bt2, Real &
     const Real q = cs2 * bt2;
     const Real aa = ca2 + bt2 - cs2;
     const Real dd = m::fma_(aa, aa, Real(4) * q);
-    const Real sd = m::normal_pos(dd) ? dd * m::rsqrt_(dd) : Real(0);
-    const Real big = m::half_(sd + m::abs_(aa));
-    // a branch, not a select: the callers that use only fmc skip the division
-    // where it is the larger one
-    if (m::nonneg(aa)) {
-        fmc = big;
-        cms = m::normal_pos(big) ? m::div_(q, big) : Real(0);
+    if (disc_normal(dd)) {
+        const Real sd = dd * m::rsqrt_(dd);
+        const Real big = m::half_(sd + m::abs_(aa));
+        // a branch, not a select: the callers that use only fmc skip the division
+        // where it is the larger one
+        if (m::nonneg(aa)) {
+            fmc = big;
+            cms = m::normal_pos(big) ? m::div_(q, big) : Real(0);
+        } else {
+            cms = big;
+            fmc = m::normal_pos(big) ? m::div_(q, big) : Real(0);
+        }
     } else {
-        cms = big;
-        fmc = m::normal_pos(big) ? m::div_(q, big) : Real(0);
+        const Disc<Real> d = disc_small(aa, cs2, bt2);
+        const Real big = m::half_(d.sd + m::abs_(aa));
+        fmc = m::nonneg(aa) ? big : d.small;
+        cms = m::nonneg(aa) ? d.small : big;
     }
     cf2 = cs2 + fmc;
 }
@@ -920,9 +967,17 @@ __device__ __forceinline__ FaceEigen<Real> face_eigen(Real r, Real v2, Real Bn, 
     const Real q = m::mul_(e.cs2, bt2);
     const Real aa = ca2 + bt2 - e.cs2;
     const Real dd = m::fma_(aa, aa, Real(4) * q);
-    const bool some = m::normal_pos(dd);
-    const Real isd = some ? m::rsqrt_(dd) : Real(0);
-    const Real sd = m::mul_(dd, isd);
+    Real sd, isd;
+    bool some = true;
+    if (disc_normal(dd)) {
+        isd = m::rsqrt_(dd);
+        sd = m::mul_(dd, isd);
+    } else {
+        const Disc<Real> d = disc_small(aa, e.cs2, bt2);
+        sd = d.sd;
+        isd = d.isd;
+        some = m::normal_pos(sd);
+    }
     const Real big = m::half_(sd + m::abs_(aa));
     const Real ibt = m::normal_pos(btm) ? m::rsqrt_(btm) : Real(0);
     const Real bta = m::mul_(btm, ibt);   // |B_t|
