@@ -1123,7 +1123,7 @@ static __global__ void __launch_bounds__(kRedThreads) divb_partial_kernel(int nx
         const long long pym = p + (long long)nx * ((j > 0 ? j - 1 : ny - 1) - j);
         const long long pzm = p + (long long)nx * ny * ((k > 0 ? k - 1 : nz - 1) - k);
         const double d = (bx[p] - bx[pxm]) * rdx + (by[p] - by[pym]) * rdy + (bz[p] - bz[pzm]) * rdz;
-        v[0] = dmax_nonneg(v[0], fabs(d));   // (a NaN is kept)
+        v[0] = dmax_number(v[0], fabs(d));   // (cells with a NaN do not count)
         v[1] += d * d;
     }
     bool ismax[2] = {true, false};

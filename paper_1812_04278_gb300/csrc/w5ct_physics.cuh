@@ -247,6 +247,12 @@ __device__ __forceinline__ double dmax_nonneg(double a, double b) {
     return __double_as_longlong(a) > __double_as_longlong(b) ? a : b;
 }
 
+// the same with a NaN b left out (fmax of non-negative doubles)
+__device__ __forceinline__ double dmax_number(double a, double b) {
+    const long long v = __double_as_longlong(b);
+    return v > __double_as_longlong(a) && v <= 0x7ff0000000000000LL ? b : a;
+}
+
 template <> struct M<double> {
     static __device__ __forceinline__ double sqrt_(double x) { return sqrt(x); }
     static __device__ __forceinline__ double mul_(double a, double b) { return a * b; }
