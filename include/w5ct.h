@@ -221,7 +221,9 @@ int w5ct_tile_variant(w5ct_ctx *ctx, int axis, int patch, int out[3]);
  * eigenvectors + LF splitting + WENO, Sec. 2.2) contracted with the flux
  * adjoints.  At max(), |.| and the eps_B switches the derivative is that of
  * the branch the forward step takes.  The arithmetic type of the forward
- * path is kept (float Jacobians for FP32_BULK), accumulation is double.
+ * path is kept (float Jacobians for FP32_BULK); the sums over the faces of a
+ * cell are kept in double (FP32_BULK: in pairs of floats, 48 bits, rounded
+ * once), those over axes and stages in double.
  * The state is not changed; the floor-hit counter and flag are kept.
  * Synchronises.  W5CT_ERR_UNSUPPORTED for npatch > 1.  (No counterpart in
  * the paper.) */

@@ -750,17 +750,72 @@ __device__ __forceinline__ void cell_fill_adjoint(const R (&in)[8], const R (&lq
     out[5 + t2] = lB2;
 }
 
+// A sum over faces.  The face adjoints that meet in a cell cancel (a difference's
+// sum against its neighbour's above all), so a float sum would lose what float
+// adjoints hold: in double a plain sum; in float the running sum and the sum of
+// its rounding errors (TwoSum), which together keep 48 bits until value()
+// rounds once.  64^3 FP32 gradient, three steps: 6.67 ms with float sums, 6.92 with
+// these pairs, 15.8 with sums in double (conversions and the FP64 pipe), the
+// gradient 3.3e-6 from 64 bits in all three.  The rounding errors of an infinite
+// sum are not numbers and are left out.
+template <typename R> struct FaceSum;
+template <> struct FaceSum<double> {
+    double s;
+    static __device__ __forceinline__ FaceSum of(double x) { return {x}; }
+    __device__ __forceinline__ void add(double x) { s += x; }
+    __device__ __forceinline__ void add(const FaceSum &x) { s += x.s; }
+    __device__ __forceinline__ FaceSum minus(const FaceSum &x) const { return {s - x.s}; }
+    __device__ __forceinline__ double value() const { return s; }
+    // (7 (a + b) - (c + d)) / 12
+    static __device__ __forceinline__ FaceSum central(double a, double b, double c, double d) {
+        return {(7.0 * (a + b) - (c + d)) * (1.0 / 12.0)};
+    }
+};
+template <> struct FaceSum<float> {
+    float s, e;
+    static __device__ __forceinline__ FaceSum of(float x) { return {x, 0.0f}; }
+    __device__ __forceinline__ void add(float x) {
+        const dw t = ef_twosum(s, x);
+        s = t.hi;
+        e = __fadd_rn(e, t.lo);
+    }
+    __device__ __forceinline__ void add(const FaceSum &x) {
+        add(x.s);
+        e = __fadd_rn(e, x.e);
+    }
+    __device__ __forceinline__ FaceSum minus(const FaceSum &x) const {
+        FaceSum d = *this;
+        d.add(FaceSum{-x.s, -x.e});
+        return d;
+    }
+    __device__ __forceinline__ float value() const {
+        const float v = __fadd_rn(s, e);
+        return v == v ? v : s;
+    }
+    static __device__ __forceinline__ FaceSum central(float a, float b, float c, float d) {
+        const dw p = ef_twoprod(7.0f, a), q = ef_twoprod(7.0f, b);
+        FaceSum t = {p.hi, __fadd_rn(p.lo, q.lo)};
+        t.add(q.hi);
+        t.add(-c);
+        t.add(-d);
+        const float k = 1.0f / 12.0f;
+        const dw r = ef_twoprod(t.s, k);
+        return {r.hi, __fmaf_rn(t.e, k, r.lo)};
+    }
+};
+
 // Cell p of a 32 x 8 tile (x and the axis, or y for the x-sweep): the adjoint
 // of the difference between cells d and d + 1 is the sum of the face adjoints
 // at position j over the five faces d + 2 - j that read it, formed once per
 // difference (a tile's first cell also needs the one below it) and kept in
 // shared memory; a flux or conserved component of cell i then takes D(i-1) -
 // D(i), plus, for the flux, the central combinations of four faces.  Fixed
-// order throughout.
+// order throughout; every sum over faces is a FaceSum.
 template <int AX, typename R>
 __global__ void __launch_bounds__(256) adj_cell_kernel(AdjSweepArgs<R> a) {
     constexpr int W = AX == 0 ? 33 : 32, H = AX == 0 ? 8 : 9;
-    __shared__ R acc[14][H][W];
+    using Sum = FaceSum<R>;
+    __shared__ Sum acc[14][H][W];
     const int nx = a.nx, ny = a.ny, nz = a.nz;
     const size_t n = (size_t)nx * ny * nz;
     const int tx = threadIdx.x, ty = threadIdx.y;
@@ -779,9 +834,9 @@ __global__ void __launch_bounds__(256) adj_cell_kernel(AdjSweepArgs<R> a) {
         for (int j = 0; j < 5; ++j) f[j] = a.face(at(x, y, z, o + 2 - j));
 #pragma unroll
         for (int c = 0; c < 14; ++c) {
-            R s = R(0);
+            Sum s = Sum::of(f[0][kAdjDiff + (c % 7) * 10 + c / 7]);
 #pragma unroll
-            for (int j = 0; j < 5; ++j) s += f[j][kAdjDiff + ((c % 7) * 5 + j) * 2 + c / 7];
+            for (int j = 1; j < 5; ++j) s.add(f[j][kAdjDiff + ((c % 7) * 5 + j) * 2 + c / 7]);
             acc[c][row][col] = s;
         }
     };
@@ -805,30 +860,21 @@ __global__ void __launch_bounds__(256) adj_cell_kernel(AdjSweepArgs<R> a) {
     for (int f = 0; f < 5; ++f) cell[f] = a.q[f][p];
 #pragma unroll
     for (int f = 0; f < 3; ++f) cell[5 + f] = a.bc[f][p];
-    constexpr int qU[7] = {C_RHOQ, C_MN, C_MT1, C_MT2, C_BT1, C_BT2, C_E};
-    constexpr int prim[8] = {C_RHO, C_VN, C_VT1, C_VT2, C_BN, C_BT1, C_BT2, C_P};
-#pragma unroll
-    for (int t = 0; t < 8; ++t) {
-        lq[prim[t]] = R(0.5) * (f0[kAdjPrim + t] + fm[kAdjPrim + t]);
-    }
-    auto D = [&](int c) {
-        return AX == 0 ? acc[c][ty][tx] - acc[c][ty][tx + 1] : acc[c][ty][tx] - acc[c][ty + 1][tx];
+    auto D = [&](int c) { return acc[c][ty][tx].minus(AX == 0 ? acc[c][ty][tx + 1] : acc[c][ty + 1][tx]); };
+    // a primitive in the interface means, and a speed of the cell: the lower cell
+    // of its own face, the upper one of the face before
+    auto mean = [&](int t) {
+        Sum v = Sum::of(R(0.5) * f0[kAdjPrim + t]);
+        v.add(R(0.5) * fm[kAdjPrim + t]);
+        return v;
     };
-#pragma unroll
-    for (int c = 0; c < 7; ++c) {
-        const int k = kAdjCentral + c;
-        lq[C_F0 + c] = D(c) + (R(7) * (f0[k] + fm[k]) - (fp[k] + fm2[k])) * R(1.0 / 12.0);
-        if (c == 4 || c == 5)
-            lq[qU[c]] += D(7 + c);
-        else
-            lq[qU[c]] = D(7 + c);
-    }
-    // lower cell of its face, upper cell of the one before
-    lq[C_VN] += f0[kAdjSide] + fm[kAdjSide + 4];
-    lq[C_CF] = f0[kAdjSide + 1] + fm[kAdjSide + 5];
-    lq[C_CA] = f0[kAdjSide + 2] + fm[kAdjSide + 6];
-    lq[C_CSL] = f0[kAdjSide + 3] + fm[kAdjSide + 7];
+    auto side = [&](int k) {
+        Sum v = Sum::of(f0[kAdjSide + k]);
+        v.add(fm[kAdjSide + 4 + k]);
+        return v;
+    };
     // transport fluxes <B_n v_t>: half the sum of the two faces' adjoints
+    R tn, tv1, tv2;
     {
         auto below = [&](int ax, int o) {
             const int x = ax == 0 ? wrapi(gx - 1, nx) : gx, y = ax == 1 ? wrapi(gy - 1, ny) : gy,
@@ -839,10 +885,34 @@ __global__ void __launch_bounds__(256) adj_cell_kernel(AdjSweepArgs<R> a) {
         const R l1 = from_double<R>(-0.25 * ((On[p] + On[below(t1, 0)]) + (On[pm] + On[below(t1, -1)])));
         const R l2 = from_double<R>(0.25 * ((O2[p] + O2[below(t2, 0)]) + (O2[pm] + O2[below(t2, -1)])));
         const R ir = M<R>::rcp3_(a.K.floors ? M<R>::max_(cell[0], a.K.rho_min) : cell[0]);
-        lq[C_BN] += (l1 * cell[1 + t1] + l2 * cell[1 + t2]) * ir;
-        lq[C_VT1] += l1 * cell[5 + AX];
-        lq[C_VT2] += l2 * cell[5 + AX];
+        tn = (l1 * cell[1 + t1] + l2 * cell[1 + t2]) * ir;
+        tv1 = l1 * cell[5 + AX];
+        tv2 = l2 * cell[5 + AX];
     }
+    constexpr int qU[7] = {C_RHOQ, C_MN, C_MT1, C_MT2, C_BT1, C_BT2, C_E};
+    constexpr int prim[8] = {C_RHO, C_VN, C_VT1, C_VT2, C_BN, C_BT1, C_BT2, C_P};
+#pragma unroll
+    for (int t = 0; t < 8; ++t) {
+        Sum v = mean(t);
+        if (prim[t] == C_VN) v.add(side(0));
+        if (prim[t] == C_VT1) v.add(tv1);
+        if (prim[t] == C_VT2) v.add(tv2);
+        if (prim[t] == C_BN) v.add(tn);
+        if (prim[t] == C_BT1) v.add(D(7 + 4));
+        if (prim[t] == C_BT2) v.add(D(7 + 5));
+        lq[prim[t]] = v.value();
+    }
+#pragma unroll
+    for (int c = 0; c < 7; ++c) {
+        const int k = kAdjCentral + c;
+        Sum v = D(c);
+        v.add(Sum::central(f0[k], fm[k], fp[k], fm2[k]));
+        lq[C_F0 + c] = v.value();
+        if (c != 4 && c != 5) lq[qU[c]] = D(7 + c).value();
+    }
+    lq[C_CF] = side(1).value();
+    lq[C_CA] = side(2).value();
+    lq[C_CSL] = side(3).value();
     R g[8];
     cell_fill_adjoint<R, AX>(cell, lq, a.K, g);
 #pragma unroll
