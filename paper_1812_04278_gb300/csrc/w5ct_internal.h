@@ -123,10 +123,6 @@ struct SinglePatchSweep {
 // the halves, whole 32 x 16 tiles in 256-thread blocks took 27.6 ms.
 constexpr int kMaxTileVariants = 4;
 
-#ifndef W5CT_ALL_WAVES32
-#define W5CT_ALL_WAVES32 8
-#endif
-
 template <int AX, typename Real, int V>
 struct TileV;
 template <int AX, typename Real>
@@ -401,16 +397,23 @@ inline long long sweep_blocks(int axis, int t2, int bx, int nx, int ny, int nz) 
 // boxes: step of 32^3 1.93 -> 1.01 ms against three launches of 32 x 16 and 16 x
 // 32 tiles, 64^3 7.68 -> 6.60, 100 x 70 x 50 10.26 -> 9.80 (WENO5), 160^3 101.4 ->
 // 100.4, 256^3 413.4 -> 411.4 ms.
-// FP32: below 8 waves of the default tiles' blocks on the device, where the
-// tails of three launches cost more than the one face per thread: 32^3 0.140 ->
-// 0.092 ms, 64^3 0.279 -> 0.255, 96^3 (5.7 waves) 0.798 -> 0.790, but 112^3 (9
-// waves) 1.260 -> 1.262 and 160^3 3.26 -> 3.37.
+// FP32: one launch saves two launches' latency and tail; its blocks are twice as
+// many and cost more each, also where an axis is thin and they hold one row of
+// faces (512 x 512 x 1).  So it is taken up to 12 waves of its blocks (four per
+// SM), and to more where nx leaves lanes of 16-wide tiles empty that its 8-wide
+// ones fill (`lanes`: 1 for none, 1/2 for nx <= 8).  us a step, three launches against
+// one (waves): 48^3 150, 128 (4.7); 64^3 236, 230 (10); 192 x 192 x 1 141, 128 (8.5);
+// 208 x 1 x 208 171, 174 (12); 256 x 256 x 1 185, 194 (15); 80^3 473, 482 (21);
+// 512 x 512 x 1 500, 658 (61); 256^2 x 16 845, 897 (40); with lanes 0.9 72^3 387, 379
+// (17), 66 x 200 x 200 2615, 2713 (126); 0.83 40 x 200 x 100 878, 857 (39); 0.75 24 x
+// 200 x 200 1003, 926 (42), 4 x 512 x 512 (0.5) 4342, 3794 (162).
 inline bool sweeps_in_one_f32(int nx, int ny, int nz, int sms) {
-    using X = SweepCfg<0, float>;
-    using YZ = SweepCfg<1, float>;
-    const long long least = (long long)W5CT_ALL_WAVES32 * sms * X::MINB;
-    return sweep_blocks(0, X::T2, X::BX, nx, ny, nz) < least || sweep_blocks(1, YZ::T2, YZ::BX, nx, ny, nz) < least ||
-           sweep_blocks(2, YZ::T2, YZ::BX, nx, ny, nz) < least;
+    using X = AllTile<0>;
+    using YZ = AllTile<1>;
+    const double waves = (double)(sweep_blocks(0, X::T2, X::BX, nx, ny, nz) + sweep_blocks(1, YZ::T2, YZ::BX, nx, ny, nz) +
+                                  sweep_blocks(2, YZ::T2, YZ::BX, nx, ny, nz)) / (4.0 * sms);
+    const double lanes = (double)((nx + 7) / 8) / (2 * ((nx + 15) / 16));
+    return waves * (lanes - 0.8) <= 2.4;
 }
 
 // Whether W5CT_FP64_DW sweeps a patch in double-word arithmetic: where each
