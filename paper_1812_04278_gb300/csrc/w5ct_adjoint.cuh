@@ -15,6 +15,7 @@
 #pragma once
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <type_traits>
 
 #include "w5ct_kernels.cuh"
@@ -52,6 +53,36 @@ struct AdjFaceRef {
     }
 };
 
+// Division of 0 <= n < 2^31 by d > 0: with 2^(s - 1) < d <= 2^s and mul =
+// ceil(2^(31 + s) / d) <= 2^32 - 1 (d = 1: s = 0, mul = 2^31) the quotient is the
+// top of n mul, whose excess over n 2^(31 + s) / d is below n < 2^31, less than the
+// 2^(31 + s) / d >= 2^31 that separates two quotients.
+struct IntDiv {
+    unsigned mul, shift;
+    int d;
+    __device__ __forceinline__ int div(int n) const { return (int)(((unsigned long long)(unsigned)n * mul) >> shift); }
+};
+inline IntDiv int_div(int d) {
+    int s = 0;
+    while (s < 31 && (1LL << s) < d) ++s;
+    return {(unsigned)(((1ULL << (31 + s)) + (unsigned)d - 1) / (unsigned)d), (unsigned)(31 + s), d};
+}
+
+// Tiles of the two kernels.  The pencils of a sweep (lines of cells along its
+// axis) are numbered flat over the other two directions, and cut into nseg
+// segments of len positions.  A block computes `per` units: for the x-sweep a
+// unit is a segment of one pencil, for the others the same segment of BX
+// consecutive pencils, so that neither a narrow x nor a thin axis leaves lanes
+// or rows empty (chosen by adj_tile; tiles cut in x and one other direction
+// left most of a block idle there: gradient of 256 x 256 x 1 in float 1.45 -> 0.78 ms, 1 x
+// 128 x 128 1.56 -> 0.67, in double 19.7 -> 10.1 and 29.5 -> 4.5; 64^3 1.875 -> 1.895 and
+// 23.4 -> 23.2).
+struct AdjTile {
+    int len, nseg, per;
+    int units;                       // of the whole sweep
+    IntDiv rows, positions, segments, cross;   // by a segment's rows, by len, nseg, and the pencils' faster direction
+};
+
 template <typename Real>
 struct AdjSweepArgs {
     int nx, ny, nz;
@@ -64,6 +95,7 @@ struct AdjSweepArgs {
     double *outq, *outb;       // 5 planes of the state's adjoint, 3 of the cell field's
     bool first;                // the first axis of the stage writes outq, outb, the others add
     Phys<Real> K;
+    AdjTile face_tile, cell_tile;   // (adj_tiles)
     __device__ __forceinline__ AdjFaceRef<Real> face(size_t p) const {
         const size_t run = p / kAdjRun, at = p % kAdjRun;
         return {fa + run * (kAdjFluxPlanes * kAdjRun) + at, fb + run * ((kAdjFacePlanes - kAdjFluxPlanes) * kAdjRun) + at};
@@ -230,6 +262,38 @@ __device__ __forceinline__ R field_rev(Pair<R> (&P)[5], R alpha, R eps3, R l, R 
     return fq - fp;
 }
 
+// One pencil of a sweep along AX: position i lies at base + i * stride of a plane.
+template <int AX>
+struct Pencil {
+    size_t base;
+    int n;
+    size_t stride;
+    __device__ __forceinline__ Pencil(int id, int nx, int ny, int nz, const IntDiv &cross) {
+        n = AX == 0 ? nx : AX == 1 ? ny : nz;
+        stride = AX == 0 ? 1 : AX == 1 ? (size_t)nx : (size_t)nx * ny;
+        const int z = AX == 1 ? cross.div(id) : 0;
+        base = AX == 0 ? (size_t)id * nx : AX == 1 ? (size_t)(id - z * nx) + (size_t)nx * ny * z : (size_t)id;
+    }
+    __device__ __forceinline__ size_t at(int i) const { return base + stride * (size_t)i; }
+};
+// pencils of a sweep
+template <int AX>
+__device__ __forceinline__ int pencils(int nx, int ny, int nz) {
+    return AX == 0 ? ny * nz : AX == 1 ? nx * nz : nx * ny;
+}
+
+// Elements between the cells of the face kernel's box (odd multiples of a
+// bank's width, so that neighbouring lanes' cells lie in different banks), and
+// the most cells of a box.
+template <typename R>
+__host__ __device__ constexpr int adj_box_pitch() {
+    return float_based<R> ? NCQ : NBQ + 1;
+}
+template <typename R>
+__host__ __device__ constexpr int adj_box_cells() {
+    return float_based<R> ? 512 : 768;
+}
+
 // Reverse mode of the face function (face_flux and face_eigen: same
 // quantities, same branches).  Its outputs are the five lab-order face fluxes
 // and the two transport fluxes; their adjoints come from lamD and lamO by the
@@ -247,57 +311,61 @@ __device__ __forceinline__ R field_rev(Pair<R> (&P)[5], R alpha, R eps3, R l, R 
 // 45.1 to 18.7 ms in its face and cell kernels (FP64, WENO-Z) and from 2.6 to
 // 1.35 ms (FP32-bulk, WENO5); the whole 2-step rollout gradient 127.8 -> 66.3 ms,
 // in float (3 steps) 12.1 -> 7.8 ms, no larger error against 64-bit gradients.
-template <int AX, typename R, int VAR, int T2, int BX, int MINB>
-__global__ void __launch_bounds__(BX *T2, MINB) adj_face_kernel(AdjSweepArgs<R> a) {
+template <int AX, typename R, int VAR, int BX, int NT, int MINB>
+__global__ void __launch_bounds__(NT, MINB) adj_face_kernel(AdjSweepArgs<R> a) {
     using m = M<R>;
     using P2 = Pair<R>;
-    using TT = SweepTile<AX, T2, BX, 1>;
     constexpr bool DIFF = box_diff<R>();
+    constexpr int ST = BX, PQ = adj_box_pitch<R>();      // (BX = 1 for the x-sweep)
     extern __shared__ __align__(16) unsigned char w5ct_smem[];
     R *sm = reinterpret_cast<R *>(w5ct_smem);
-    const int nx = a.nx, ny = a.ny, nz = a.nz;
-    const int tx = threadIdx.x, ty = threadIdx.y, tid = tx + BX * ty;
-    const int x0 = blockIdx.x * TT::BX, y0 = blockIdx.y * TT::BY, z0 = blockIdx.z * TT::BZ;
+    const int nx = a.nx, ny = a.ny, nz = a.nz, tid = threadIdx.x;
+    const AdjTile &t = a.face_tile;
+    const int len = t.len, rows = len + 5, np = pencils<AX>(nx, ny, nz), first = (int)blockIdx.x * t.per;
     const Phys<R> K = a.K;
-    // cell box
+    // cell box: per segments of len + 5 cells, BX pencils side by side (y, z),
+    // a cell's quantities together.  Pencils and units past the last repeat it.
+    const int ncell = BX * t.per * rows;
     bool bad = false, hit = false;
-    for (int c = tid; c < TT::NC; c += TT::NT) {
-        const int cx = c % TT::CX, cy = (c / TT::CX) % TT::CY, cz = c / (TT::CX * TT::CY);
-        const int gx = wrapi(x0 - (AX == 0 ? 2 : 0) + cx, nx), gy = wrapi(y0 - (AX == 1 ? 2 : 0) + cy, ny),
-                  gz = wrapi(z0 - (AX == 2 ? 2 : 0) + cz, nz);
-        const size_t g = (size_t)gx + (size_t)nx * ((size_t)gy + (size_t)ny * (size_t)gz);
-        cell_fill<R, AX>(sm, c, TT::NC, a.q[0][g], a.q[1][g], a.q[2][g], a.q[3][g], a.q[4][g], a.bc[0][g],
-                         a.bc[1][g], a.bc[2][g], K, bad, hit);
+    for (int c = tid; c < ncell; c += NT) {
+        const int row = c / BX, u = t.rows.div(row);
+        const int unit = min(first + u, t.units - 1), group = t.segments.div(unit), seg = unit - group * t.nseg;
+        const Pencil<AX> pen(min(group * BX + c % BX, np - 1), nx, ny, nz, t.cross);
+        const size_t g = pen.at(wrapi(seg * len + (row - u * rows) - 2, pen.n));
+        cell_fill<R, AX>(sm + c * PQ, 0, 1, a.q[0][g], a.q[1][g], a.q[2][g], a.q[3][g], a.q[4][g], a.bc[0][g], a.bc[1][g],
+                         a.bc[2][g], K, bad, hit);
     }
     __syncthreads();
     if constexpr (DIFF) {
-        constexpr int NIT = (TT::NC + TT::NT - 1) / TT::NT;
-        constexpr int LAST = (AX == 0 ? TT::CX : AX == 1 ? TT::CY : TT::CZ) - 1;
+        // (a segment's last cell has no successor, and none is read)
+        constexpr int NIT = (adj_box_cells<R>() + NT - 1) / NT;
         CellDiff<R> d[NIT];
-        bool has[NIT];
 #pragma unroll
         for (int it = 0; it < NIT; ++it) {
-            const int c = tid + it * TT::NT;
-            const int ca = AX == 0 ? c % TT::CX : AX == 1 ? (c / TT::CX) % TT::CY : c / (TT::CX * TT::CY);
-            has[it] = c < TT::NC && ca < LAST;
-            if (has[it]) box_diff_load<R>(sm, TT::NC, c, TT::ST, d[it]);
+            const int c = tid + it * NT;
+            if (c + ST < ncell) box_diff_load<R>(sm + c * PQ, 1, 0, ST * PQ, d[it]);
         }
         __syncthreads();
 #pragma unroll
-        for (int it = 0; it < NIT; ++it)
-            if (has[it]) box_diff_store<R>(sm, TT::NC, tid + it * TT::NT, d[it]);
+        for (int it = 0; it < NIT; ++it) {
+            const int c = tid + it * NT;
+            if (c + ST < ncell) box_diff_store<R>(sm + c * PQ, 1, 0, d[it]);
+        }
         __syncthreads();
     }
-    const int gx = x0 + tx, gy = y0 + (AX == 2 ? 0 : ty), gz = z0 + (AX == 2 ? ty : 0);
-    if (gx >= nx || gy >= ny || gz >= nz) return;
-    const int c0 = tx + TT::CX * ((AX == 2 ? 0 : ty) + TT::CY * (AX == 2 ? ty : 0));   // stencil cell i-2
-    const R *box = sm + c0;
-    constexpr int ST = TT::ST, NC = TT::NC;
+    // this thread's face
+    const int trow = tid / BX, u = t.positions.div(trow), unit = first + u;
+    const int group = t.segments.div(unit), id = group * BX + tid % BX;
+    const int at = (unit - group * t.nseg) * len + (trow - u * len);
+    if (u >= t.per || unit >= t.units || id >= np || at >= (AX == 0 ? nx : AX == 1 ? ny : nz)) return;
+    const R *box = sm + ((trow + 5 * u) * BX + tid % BX) * PQ;       // stencil cell i-2
     const size_t n = (size_t)nx * ny * nz;
-    const size_t p = (size_t)gx + (size_t)nx * ((size_t)gy + (size_t)ny * (size_t)gz);
+    const size_t p = Pencil<AX>(id, nx, ny, nz, t.cross).at(at);
+    const int slow = t.cross.div(id), fast = id - slow * t.cross.d;   // the other two directions
+    const int gx = AX == 0 ? at : fast, gy = AX == 0 ? fast : AX == 1 ? at : slow, gz = AX == 2 ? at : slow;
     const AdjFaceRef<R> out_ = a.face(p);
 
-#define SMQ(q, k) box[(q) * NC + (k) * ST]
+#define SMQ(q, k) box[(k) * (ST * PQ) + (q)]
     // stencil pair (dF_c, du_c) at position j
     auto X = [&](int c, int j) -> P2 {
         const int qU = c == 0 ? C_RHOQ : c == 1 ? C_MN : c == 2 ? C_MT1 : c == 3 ? C_MT2
@@ -804,63 +872,61 @@ template <> struct FaceSum<float> {
     }
 };
 
-// Cell p of a 32 x 8 tile (x and the axis, or y for the x-sweep): the adjoint
-// of the difference between cells d and d + 1 is the sum of the face adjoints
-// at position j over the five faces d + 2 - j that read it, formed once per
-// difference (a tile's first cell also needs the one below it) and kept in
-// shared memory; a flux or conserved component of cell i then takes D(i-1) -
+// A cell of a tile of segments (AdjTile): the adjoint of the difference between
+// cells d and d + 1 is the sum of the face adjoints at position j over the five
+// faces d + 2 - j that read it, formed once per difference (a segment's first
+// cell also needs the one below it) and kept in shared memory; a flux or conserved component of cell i then takes D(i-1) -
 // D(i), plus, for the flux, the central combinations of four faces.  Fixed
 // order throughout; every sum over faces is a FaceSum.
+constexpr int kAdjCellEntries = 384;       // differences of a block
 template <int AX, typename R>
 __global__ void __launch_bounds__(256) adj_cell_kernel(AdjSweepArgs<R> a) {
-    constexpr int W = AX == 0 ? 33 : 32, H = AX == 0 ? 8 : 9;
     using Sum = FaceSum<R>;
-    __shared__ Sum acc[14][H][W];
-    const int nx = a.nx, ny = a.ny, nz = a.nz;
+    constexpr int BX = AX == 0 ? 1 : 32;
+    __shared__ Sum acc[14][kAdjCellEntries];
+    const int nx = a.nx, ny = a.ny, nz = a.nz, tid = threadIdx.x;
     const size_t n = (size_t)nx * ny * nz;
-    const int tx = threadIdx.x, ty = threadIdx.y;
-    const int gx = blockIdx.x * 32 + tx, gy = AX == 2 ? (int)blockIdx.y : (int)blockIdx.y * 8 + ty,
-              gz = AX == 2 ? (int)blockIdx.z * 8 + ty : (int)blockIdx.z;
-    // index of the cell `o` cells along the axis from (x, y, z)
-    auto at = [&](int x, int y, int z, int o) {
-        if (AX == 0) x = wrapi(x + o, nx);
-        if (AX == 1) y = wrapi(y + o, ny);
-        if (AX == 2) z = wrapi(z + o, nz);
-        return (size_t)x + (size_t)nx * ((size_t)y + (size_t)ny * (size_t)z);
-    };
-    auto differences = [&](int x, int y, int z, int o, int row, int col) {
+    const AdjTile &t = a.cell_tile;
+    const int len = t.len, rows = len + 1, np = pencils<AX>(nx, ny, nz), first = (int)blockIdx.x * t.per;
+    // entry (unit u, row r, pencil b) at (u rows + r) BX + b: the difference
+    // between positions r - 1 and r of the unit's segment
+    const int entries = BX * t.per * rows;
+    for (int e = tid; e < entries; e += 256) {
+        const int row = e / BX, u = t.rows.div(row), unit = first + u, group = t.segments.div(unit);
+        const int id = group * BX + e % BX, at = (unit - group * t.nseg) * len + (row - u * rows) - 1;
+        if (unit >= t.units || id >= np) continue;
+        const Pencil<AX> pen(id, nx, ny, nz, t.cross);
+        if (at >= pen.n) continue;
         AdjFaceRef<R> f[5];
 #pragma unroll
-        for (int j = 0; j < 5; ++j) f[j] = a.face(at(x, y, z, o + 2 - j));
+        for (int j = 0; j < 5; ++j) f[j] = a.face(pen.at(wrapi(at + 2 - j, pen.n)));
 #pragma unroll
         for (int c = 0; c < 14; ++c) {
             Sum s = Sum::of(f[0][kAdjDiff + (c % 7) * 10 + c / 7]);
 #pragma unroll
             for (int j = 1; j < 5; ++j) s.add(f[j][kAdjDiff + ((c % 7) * 5 + j) * 2 + c / 7]);
-            acc[c][row][col] = s;
-        }
-    };
-    const bool in = gx < nx && gy < ny && gz < nz;
-    if (in) differences(gx, gy, gz, 0, AX == 0 ? ty : ty + 1, AX == 0 ? tx + 1 : tx);
-    if (ty == 0) {      // the differences below the tile: one warp
-        if (AX == 0) {
-            const int y = blockIdx.y * 8 + tx;
-            if (tx < 8 && y < ny) differences((int)blockIdx.x * 32, y, gz, -1, tx, 0);
-        } else if (in) {
-            differences(gx, gy, gz, -1, 0, tx);
+            acc[c][e] = s;
         }
     }
     __syncthreads();
-    if (!in) return;
-    const size_t p = at(gx, gy, gz, 0), pm = at(gx, gy, gz, -1);
-    const AdjFaceRef<R> f0 = a.face(p), fm = a.face(pm), fm2 = a.face(at(gx, gy, gz, -2)), fp = a.face(at(gx, gy, gz, 1));
+    const int trow = tid / BX, u = t.positions.div(trow), unit = first + u, group = t.segments.div(unit);
+    const int id = group * BX + tid % BX, at = (unit - group * t.nseg) * len + (trow - u * len);
+    if (u >= t.per || unit >= t.units || id >= np) return;
+    const Pencil<AX> pen(id, nx, ny, nz, t.cross);
+    if (at >= pen.n) return;
+    const int below_ = (trow + u) * BX + tid % BX;         // D(i - 1); D(i) one row on
+    const size_t p = pen.at(at), pm = pen.at(wrapi(at - 1, pen.n));
+    const AdjFaceRef<R> f0 = a.face(p), fm = a.face(pm), fm2 = a.face(pen.at(wrapi(at - 2, pen.n))),
+                        fp = a.face(pen.at(wrapi(at + 1, pen.n)));
+    const int slow = t.cross.div(id), fast = id - slow * t.cross.d;
+    const int gx = AX == 0 ? at : fast, gy = AX == 0 ? fast : AX == 1 ? at : slow, gz = AX == 2 ? at : slow;
     constexpr int t1 = (AX + 1) % 3, t2 = (AX + 2) % 3;
     R cell[8], lq[NCQ];
 #pragma unroll
     for (int f = 0; f < 5; ++f) cell[f] = a.q[f][p];
 #pragma unroll
     for (int f = 0; f < 3; ++f) cell[5 + f] = a.bc[f][p];
-    auto D = [&](int c) { return acc[c][ty][tx].minus(AX == 0 ? acc[c][ty][tx + 1] : acc[c][ty + 1][tx]); };
+    auto D = [&](int c) { return acc[c][below_].minus(acc[c][below_ + BX]); };
     // a primitive in the interface means, and a speed of the cell: the lower cell
     // of its own face, the upper one of the face before
     auto mean = [&](int t) {
@@ -876,10 +942,12 @@ __global__ void __launch_bounds__(256) adj_cell_kernel(AdjSweepArgs<R> a) {
     // transport fluxes <B_n v_t>: half the sum of the two faces' adjoints
     R tn, tv1, tv2;
     {
+        // of the cell `o` along the sweep (0 or -1), the neighbour below along ax
         auto below = [&](int ax, int o) {
-            const int x = ax == 0 ? wrapi(gx - 1, nx) : gx, y = ax == 1 ? wrapi(gy - 1, ny) : gy,
-                      z = ax == 2 ? wrapi(gz - 1, nz) : gz;
-            return at(x, y, z, o);
+            const int x = ax == 0 ? wrapi(gx - 1, nx) : AX == 0 ? wrapi(gx + o, nx) : gx;
+            const int y = ax == 1 ? wrapi(gy - 1, ny) : AX == 1 ? wrapi(gy + o, ny) : gy;
+            const int z = ax == 2 ? wrapi(gz - 1, nz) : AX == 2 ? wrapi(gz + o, nz) : gz;
+            return (size_t)x + (size_t)nx * ((size_t)y + (size_t)ny * (size_t)z);
         };
         const double *On = a.lamO + (size_t)AX * n, *O2 = a.lamO + (size_t)t2 * n;
         const R l1 = from_double<R>(-0.25 * ((On[p] + On[below(t1, 0)]) + (On[pm] + On[below(t1, -1)])));
@@ -1165,31 +1233,84 @@ static __global__ void __launch_bounds__(256) ic_curl_adjoint_kernel(AdjGrid g, 
     lA[2 * n + p] = (bx[p] - bx[g.at(i, j + 1, k)]) * g.rdy - (by[p] - by[g.at(i + 1, j, k)]) * g.rdx;
 }
 
-// Tiles of the face kernel, one face per thread at up to 255 registers, eight
-// warps per SM: in double 256 threads (32 x 8 faces along x, 16 x 16 in the
-// other two sweeps), in float two blocks of 128 (32 x 4 and 8 x 16).  64^3
-// WENO5 rollout in float, three steps: 7.76 ms; one block of 256 threads 7.82,
-// three blocks of 128 (168 registers) 7.96, four (128 registers) 8.49.
+// The tile of a kernel whose block has `rows` positions to give (of BX pencils
+// each) and room for `room` rows, `extra` of them per segment beside its
+// positions: the segment length that takes the fewest blocks, a block's cells
+// counting a sixteenth of a face each.  Of blocks that leave some of the `slots`
+// (SMs times blocks on each) empty, those with the fewest positions, down to a
+// warp's, that still fit in the slots.
+inline AdjTile adj_tile(int ax, int nx, int ny, int nz, int BX, int rows, int room, int extra, int slots) {
+    const int na = ax == 0 ? nx : ax == 1 ? ny : nz;
+    const long long n = (long long)nx * ny * nz, groups = (n / na + BX - 1) / BX;
+    AdjTile best = {};
+    for (int r = rows; r * BX >= 32; r /= 2) {
+        AdjTile tile = {};
+        long long fewest = 0;
+        double cost = 1e300;
+        for (int most = std::min(r, na); most > 0; --most) {
+            const int nseg = (na + most - 1) / most, len = (na + nseg - 1) / nseg;      // (nearly equal segments)
+            const int per = std::min(r / len, room / (len + extra));
+            const long long units = groups * nseg, blocks = (units + per - 1) / per;
+            const double c = (double)blocks * (r + per * (len + extra) / 16.0);
+            if (c < 0.999 * cost) {
+                cost = c;
+                fewest = blocks;
+                tile.len = len;
+                tile.nseg = nseg;
+                tile.per = per;
+                tile.units = (int)units;
+            }
+        }
+        if (r < rows && fewest > slots) break;
+        best = tile;
+    }
+    best.rows = int_div(best.len + extra);
+    best.positions = int_div(best.len);
+    best.segments = int_div(best.nseg);
+    best.cross = int_div(ax == 0 ? ny : nx);
+    return best;
+}
+
+// The face kernel: one face per thread at up to 255 registers, eight warps per
+// SM: in double 256 threads (16 pencils side by side along y and z), in float two
+// blocks of 128 (8 pencils).  64^3 WENO5 rollout in float, three steps: 7.76 ms;
+// one block of 256 threads 7.82, three blocks of 128 (168 registers) 7.96, four
+// (128 registers) 8.49.
 template <int AX, typename R, int VAR>
 struct AdjFace {
     static constexpr bool kF = float_based<R>;
-    static constexpr int BX = AX == 0 ? 32 : kF ? 8 : 16, T2 = AX == 0 ? (kF ? 4 : 8) : 16, MINB = kF ? 2 : 1;
-    using TT = SweepTile<AX, T2, BX, 1>;
-    static constexpr size_t smem = (size_t)TT::NC * box_quantities<R>() * sizeof(R);
+    static constexpr int BX = AX == 0 ? 1 : kF ? 8 : 16, NT = kF ? 128 : 256, MINB = kF ? 2 : 1;
+    static constexpr size_t cell_bytes = adj_box_pitch<R>() * sizeof(R);
     static cudaError_t prepare() {
-        return cudaFuncSetAttribute(adj_face_kernel<AX, R, VAR, T2, BX, MINB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    (int)smem);
+        return cudaFuncSetAttribute(adj_face_kernel<AX, R, VAR, BX, NT, MINB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    (int)(adj_box_cells<R>() * cell_bytes));
+    }
+    static AdjTile tile(int nx, int ny, int nz) {
+        return adj_tile(AX, nx, ny, nz, BX, NT / BX, adj_box_cells<R>() / BX, 5, 152 * MINB);
     }
     static cudaError_t launch(const AdjSweepArgs<R> &a, cudaStream_t s) {
-        const dim3 grid = AX == 2 ? dim3((a.nx + BX - 1) / BX, a.ny, (a.nz + T2 - 1) / T2)
-                                  : dim3((a.nx + BX - 1) / BX, (a.ny + T2 - 1) / T2, a.nz);
-        adj_face_kernel<AX, R, VAR, T2, BX, MINB><<<grid, dim3(BX, T2), smem, s>>>(a);
-        const dim3 cells = AX == 2 ? dim3((a.nx + 31) / 32, a.ny, (a.nz + 7) / 8)
-                                   : dim3((a.nx + 31) / 32, (a.ny + 7) / 8, a.nz);
-        adj_cell_kernel<AX, R><<<cells, dim3(32, 8), 0, s>>>(a);
+        const AdjTile &f = a.face_tile, &c = a.cell_tile;
+        const size_t smem = (size_t)BX * f.per * (f.len + 5) * cell_bytes;
+        adj_face_kernel<AX, R, VAR, BX, NT, MINB><<<(f.units + f.per - 1) / f.per, NT, smem, s>>>(a);
+        adj_cell_kernel<AX, R><<<(c.units + c.per - 1) / c.per, 256, 0, s>>>(a);
         return cudaGetLastError();
     }
 };
+
+inline AdjTile adj_cell_tile(int ax, int nx, int ny, int nz) {
+    const int BX = ax == 0 ? 1 : 32;
+    return adj_tile(ax, nx, ny, nz, BX, 256 / BX, kAdjCellEntries / BX, 1, 152 * 2);
+}
+
+// The tiles of the sweep along each axis over a grid (a few hundred trial
+// divisions each: once per grid, not per launch).
+template <typename R>
+void adj_tiles(int nx, int ny, int nz, AdjTile (&face)[3], AdjTile (&cell)[3]) {
+    face[0] = AdjFace<0, R, 0>::tile(nx, ny, nz);
+    face[1] = AdjFace<1, R, 0>::tile(nx, ny, nz);
+    face[2] = AdjFace<2, R, 0>::tile(nx, ny, nz);
+    for (int ax = 0; ax < 3; ++ax) cell[ax] = adj_cell_tile(ax, nx, ny, nz);
+}
 
 // Defined in w5ct_adjoint{32,64}{js,z}.cu (one translation unit per
 // arithmetic type and WENO variant, compiled in parallel): the face and cell

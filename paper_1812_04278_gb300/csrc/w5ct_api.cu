@@ -82,6 +82,7 @@ struct w5ct_ctx {
     int ncells = 0;
     // adjoint work buffers (w5ct_adjoint_step): allocated on first use
     void *adj_slab = nullptr;
+    AdjTile adj_face_tile[3] = {}, adj_cell_tile[3] = {};   // set with adj_slab
     // captured step (w5ct_step_graph)
     cudaStream_t cap_stream = nullptr;
     cudaGraphExec_t gexec = nullptr;
@@ -1319,6 +1320,7 @@ template <typename Real>
 int ensure_adj(w5ct_ctx *c) {
     if (c->adj_slab) return W5CT_OK;
     W5_CUDA(c, c->cfg.weno_variant == W5CT_WENO_JS ? (prepare_adj_sweep<Real, 0>()) : (prepare_adj_sweep<Real, 1>()));
+    adj_tiles<Real>(c->nx, c->ny, c->nz, c->adj_face_tile, c->adj_cell_tile);
     const size_t n = (size_t)c->n;
     const size_t bytes = align256(adj_real_values(n) * sizeof(Real)) + (size_t)kAdjDoublePlanes * n * 8;
     W5_CUDA(c, cudaMalloc(&c->adj_slab, bytes));
@@ -1385,6 +1387,8 @@ int adjoint_step_impl(w5ct_ctx *c, double dt, const double *lq_fin, const double
             aa.outq = cur;
             aa.outb = lamBc;
             aa.first = ax == 0;
+            aa.face_tile = c->adj_face_tile[ax];
+            aa.cell_tile = c->adj_cell_tile[ax];
             aa.K = K;
             const cudaError_t ea = c->cfg.weno_variant == W5CT_WENO_JS ? launch_adj_sweep<Real, 0>(ax, aa, st)
                                                                        : launch_adj_sweep<Real, 1>(ax, aa, st);

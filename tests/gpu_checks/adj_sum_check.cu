@@ -47,8 +47,8 @@ static double run(int nx, int ny, int nz) {
     a.outq = (double *)up(nullptr, 5 * n * 8), a.outb = (double *)up(nullptr, 3 * n * 8);
     a.K = Phys<R>{};
     a.K.gamma = R(5.0 / 3.0), a.K.gm1 = R(2.0 / 3.0);
-    const dim3 cells = AX == 2 ? dim3((nx + 31) / 32, ny, (nz + 7) / 8) : dim3((nx + 31) / 32, (ny + 7) / 8, nz);
-    adj_cell_kernel<AX, R><<<cells, dim3(32, 8)>>>(a);
+    const AdjTile &t = a.cell_tile = adj_cell_tile(AX, nx, ny, nz);
+    adj_cell_kernel<AX, R><<<(t.units + t.per - 1) / t.per, 256>>>(a);
     if (cudaDeviceSynchronize() != cudaSuccess) exit(3);
     std::vector<double> out(n);
     cudaMemcpy(out.data(), a.outq + 4 * n, n * 8, cudaMemcpyDeviceToHost);
