@@ -127,6 +127,8 @@ __device__ __forceinline__ void sweep_tile_at(const SweepArgs<Real> &a, const Pa
     constexpr int NC = TT::template cells<Real>;      // elements between quantities
     constexpr bool kFlat = std::is_same<Real, double>::value, kPaired = !kFlat && PAIR;
     constexpr int pitch = TT::template pitch<Real>, st = TT::ST;
+    // (div_by's range)
+    static_assert(!kFlat || (TT::NC <= 1024 && TT::CX <= 64 && T2 * BX <= 1024), "tile too large for div_by");
     const int nx = pg.nx, ny = pg.ny, nz = pg.nz;
     const size_t off = (size_t)pg.off;
     const int ntx = (nx + BX - 1) / BX, w0 = kFlat ? (nx + ntx - 1) / ntx : BX;
