@@ -481,7 +481,7 @@ def run_native(args):
         "dtype": "f64",
         "data": "synthetic",
         "config": workload_config(n),
-        "roofline": {"kernel": "sweep_kernel (FP64)", "bound": "alu", "achieved": ach64, "peak": PEAK_FP64_TFLOPS,
+        "roofline": {"kernel": "sweep_all_kernel (FP64)", "bound": "alu", "achieved": ach64, "peak": PEAK_FP64_TFLOPS,
                      "unit": "TFLOP/s", "frac": ach64 / PEAK_FP64_TFLOPS,
                      "traffic": sweep_traffic("fp64", zones), "launch_ms": swms64 / nsw64,
                      "algorithmic_flops_per_launch": sweep_flops,
@@ -509,7 +509,7 @@ def run_native(args):
             "dtype": "f64; WENO indicators, weights and interpolants in double-word f32 pairs (48-bit significand)",
             "speedup_vs_fp64": valuedw / value64, "max_rel_vs_fp64": reldw, "error_steps": nlog,
             "div_b_linf": divbdw,
-            "roofline": {"kernel": "sweep_kernel (FP64, double-word WENO)", "bound": "alu", "achieved": achdw,
+            "roofline": {"kernel": "sweep_all_kernel (FP64, double-word WENO)", "bound": "alu", "achieved": achdw,
                          "peak": PEAK_FP64_TFLOPS, "unit": "TFLOP/s", "frac": achdw / PEAK_FP64_TFLOPS,
                          "traffic": sweep_traffic("fp64dw", zones), "launch_ms": swmsdw / nswdw,
                          "hbm_gbs": hbm_gbs(sweep_traffic("fp64dw", zones), swmsdw / nswdw),

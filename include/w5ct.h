@@ -67,12 +67,15 @@ extern "C" {
                                       interpolants of the LF-split differences;
                                       Sec. 2.2) in double-word arithmetic (pairs
                                       of floats, 48-bit significand) on the FP32
-                                      pipe, in the single-patch sweeps of the
-                                      default tiles; everything else, every
+                                      pipe, in the single-patch sweeps, along
+                                      all three axes or none: where each of
+                                      ceil(nx/32) ceil(ny/16) nz, ceil(nx/16)
+                                      ceil(ny/32) nz and ceil(nx/16) ny
+                                      ceil(nz/32) is at least twice the number
+                                      of SMs (152: 304).  Everything else, every
                                       stored value and every other kernel
-                                      (grids too small for those tiles, the
-                                      batched, fused and adjoint paths) as
-                                      W5CT_FP64 */
+                                      (smaller grids, the batched, fused and
+                                      adjoint paths) as W5CT_FP64 */
 
 typedef struct w5ct_ctx w5ct_ctx;
 

@@ -26,8 +26,10 @@ CFLAGS = ["-O3", "-std=c++17", "-lineinfo", "-Xcompiler", "-fPIC", "-I", INCLUDE
 # reciprocal / square root and flushes subnormals; every double operation
 # and every other translation unit stays IEEE.
 FAST_FLOAT = ["-ftz=true", "-prec-div=false", "-prec-sqrt=false"]
-# The sweeps write every FMA out and contract nothing else, so that all copies
-# of the face arithmetic (tiles, variants, single patch and batch) round alike.
+# The sweeps write every FMA out and contract nothing else, so that all their
+# copies of the face arithmetic (tiles, variants, single patch and batch) round
+# alike.  The fused step and the adjoint contract as the compiler sees fit and
+# agree with them to rounding.
 NO_CONTRACT = ["-fmad=false"]
 TU_FLAGS = {"w5ct_sweep32.cu": FAST_FLOAT + NO_CONTRACT, "w5ct_sweep64.cu": NO_CONTRACT, "w5ct_sweep64dw.cu": NO_CONTRACT,
             "w5ct_adjoint32z.cu": FAST_FLOAT, "w5ct_adjoint32js.cu": FAST_FLOAT,

@@ -116,8 +116,9 @@ struct SinglePatchSweep {
 // variant keeps 128 registers per thread in float: min blocks per SM = 512 /
 // threads per block.  One launch per axis and variant computes a float
 // or double 32 x 16 tile as two halves, in blocks of 128 threads like the
-// single-patch tiles (double: three of 168 registers per SM instead of one of 256
-// threads, 48 patches 50.6 -> 48.3 ms per step).
+// single-patch tiles (double, 168 registers: three per SM along x, two along y and
+// z, whose boxes of 84 KB fill it, instead of one of 256 threads; 48 patches 50.6 ->
+// 48.3 ms per step).
 // Step of the 512-patch workload with one variant forced on every patch: 24.1,
 // 23.4, 24.0, 23.4 ms, and 22.8 ms with the choice per patch and axis; before
 // the halves, whole 32 x 16 tiles in 256-thread blocks took 27.6 ms.

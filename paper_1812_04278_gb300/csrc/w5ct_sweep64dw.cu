@@ -1,5 +1,6 @@
-// w5ct_sweep64dw.cu -- the FP64 single-patch sweeps with the WENO part of every characteristic field's flux in
-// double-word arithmetic (w5ct_physics.cuh, weno_field): the smoothness
+// w5ct_sweep64dw.cu -- the FP64 single-patch sweeps with the WENO part of
+// every characteristic field's flux in double-word arithmetic
+// (w5ct_physics.cuh, weno_field): the smoothness
 // indicators, the nonlinear weights and the two interpolants of the LF-split
 // differences run on the FP32 pipe, while the cell box, the eigenvectors,
 // the projections, the split itself, the back-projection and every stored
