@@ -194,11 +194,11 @@ def kernel_source_hash():
     return h.hexdigest()[:16]
 
 
-# DRAM bytes (read + write) per zone of one sweep launch, from ncu captures
+# DRAM bytes (read + write) per zone and axis of the sweeps, from ncu captures
 # at 128^3 (dram__bytes_read.sum + dram__bytes_write.sum / 128^3), valid for
-# the sweep source with the given hash; scaled to a launch by the zone count
+# sweep source with the given hash; scaled to a sweep by the zone count
 # (traffic grows with the zones: one tile pass per zone).
-SWEEP_TRAFFIC = {"src": "94dd87415640b72f", "fp64": 103.51, "fp32": 43.84, "fp64dw": 105.32}
+SWEEP_TRAFFIC = {"src": "70008e903e757ab9", "fp64": 226.0, "fp32": 43.9, "fp64dw": 626.4}
 
 
 def hbm_gbs(traffic, launch_ms):

@@ -55,7 +55,8 @@ struct SweepTuning;
 // 27.36 ms for two 256^3 WENO-Z steps and 109.8 ms for a 512^3 WENO5 step, against
 // 27.95 and 113.1 for 256-thread blocks of 32 x 16 (a barrier stalls half an
 // SM's warps there), 27.47 and 110.8 for 8 x 32, 28.17 and 113.9 for one face
-// per thread, 28.1 and 112.8 for three, 28.7 and 116.2 for four.
+// per thread, 28.1 and 112.8 for three, 28.7 and 116.2 for four (26.5 and 108.3 for
+// the chosen one with the later forms of the box and the eigenvectors).
 #ifndef W5CT_F32_T2X
 #define W5CT_F32_T2X 8
 #endif

@@ -1041,8 +1041,9 @@ __device__ __forceinline__ FaceEigen<Real> face_eigen(Real r, Real v2, Real Bn, 
 // in the lab frame: 535.0 -> 416.7 ms per 256^3 FP64 step (WENO-Z), 15.57 ->
 // 14.46 ms in FP32-bulk, 56.6 -> 49.3 ms per 128^3 step with double-word
 // weights; no larger error against 64-bit values in any of them.  With the tiles
-// of today and the products on the integer pipes: 331 ms, FP64 pipe 83%
-// busy, issue slots 24%.
+// of today and the products on the integer pipes: 330 ms, FP64 pipe 88% busy on
+// 861 FP64 instructions per interface with its share of the cells (128^3
+// WENO-Z), issue slots 25%; FP32-bulk 13.2 ms, issue slots 74-76%.
 template <typename Real, int VAR, bool DIFF = false, bool DWW = false, bool PAIRED = false, typename MM = M<Real>>
 __device__ __forceinline__ void face_flux(const Real *__restrict__ box, int cell, int ncell, int st, const Phys<Real> &K,
                                           Real (&Ff)[7], Real &s1, Real &s2) {
