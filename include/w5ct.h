@@ -282,7 +282,10 @@ int w5ct_div_b_norm(w5ct_ctx *ctx, int patch, double *linf, double *l2);
 int w5ct_conserved_totals(w5ct_ctx *ctx, int patch, double out[8]);
 
 /* Number of floor activations (when floors = 1) and the non-physical flag
- * since the last set_state; either pointer may be NULL.  Synchronises. */
+ * since the last set_state; either pointer may be NULL.  Synchronises.  The
+ * number is positive exactly if a floor acted; it counts the sweeps' recoveries,
+ * of cells that neighbouring tiles share more than once, and so depends on the
+ * tiles and the schedule. */
 int w5ct_status(w5ct_ctx *ctx, long long *floor_hits, int *nonphysical);
 
 /* Block the host until all work of the context's stream is done. */
